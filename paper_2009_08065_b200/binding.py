@@ -1,5 +1,9 @@
-"""ctypes binding of libbsp.so.  Same names as the C entry points; arguments are torch CUDA
+"""Binding of libbsp.so.  Same names as the C entry points; arguments are torch CUDA
 tensors (or None) whose device pointers are handed to the library unchanged.
+
+The calls that a program makes once per matrix and step go through `_bsp_native` (csrc/bsp_native.cpp),
+which marshals the arguments in C++: with ctypes a call costs 8 to 12 us of host time, more than most of
+the kernels run for on one matrix.  Size queries, one-off calls and the raw C functions (`lib`) use ctypes.
 
 bf16 tensors may be passed either as torch.bfloat16 or as raw bit patterns (torch.uint16 /
 torch.int16); the library only sees the pointer.  There is no CPU fallback: if the shared
@@ -41,6 +45,7 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+from . import _bsp_native as _native  # noqa: E402  (links against libbsp.so, which is loaded by now)
 
 _vp, _i, _f, _d = ctypes.c_void_p, ctypes.c_int, ctypes.c_float, ctypes.c_double
 _sz, _szp = ctypes.c_size_t, ctypes.POINTER(ctypes.c_size_t)
@@ -164,17 +169,13 @@ def bsp_group_norms(W: torch.Tensor, block: int, orient: int = ORIENT_C, eps: fl
                     gamma_out: Optional[torch.Tensor] = None, penalty: Optional[torch.Tensor] = None,
                     stream=None) -> None:
     """norms / gamma_out: float32 per-group tensors; penalty: one-element float64 tensor (all optional outputs)."""
-    rows, cols = W.shape
-    _check(lib.bsp_group_norms(_ptr(W), rows, cols, _ld(W), block, orient, eps, pen, _ptr(norms), _ptr(gamma_in),
-                               _ptr(gamma_out), _ptr(penalty), _stream(stream)), "bsp_group_norms")
+    _check(_native.group_norms(W, block, orient, eps, pen, norms, gamma_in, gamma_out, penalty, stream), "bsp_group_norms")
 
 
 def bsp_penalty_grad(W: torch.Tensor, block: int, orient: int, pen: int, gamma: torch.Tensor, scale: float,
                      grad: torch.Tensor, accumulate: bool = False, stream=None) -> None:
     """grad: float32 [rows, cols]; gamma: float32 per-group tensor."""
-    rows, cols = W.shape
-    _check(lib.bsp_penalty_grad(_ptr(W), rows, cols, _ld(W), block, orient, pen, _ptr(gamma), scale, _ptr(grad),
-                                _ld(grad), int(accumulate), _stream(stream)), "bsp_penalty_grad")
+    _check(_native.penalty_grad(W, block, orient, pen, gamma, scale, grad, int(accumulate), stream), "bsp_penalty_grad")
 
 
 def bsp_pack_bound(rows: int, cols: int, block: int, orient: int = ORIENT_C) -> Tuple[int, int, int]:
@@ -223,11 +224,8 @@ class PackedMatrix:
 
 def bsp_prune_pack(W: torch.Tensor, out: PackedMatrix, threshold: float = 0.0,
                    threshold_dev: Optional[torch.Tensor] = None, keep_per_block: int = -1, stream=None) -> None:
-    rows, cols = W.shape
-    _check(lib.bsp_prune_pack(_ptr(W), rows, cols, _ld(W), out.block, out.orient, threshold, _ptr(threshold_dev),
-                              keep_per_block, _ptr(out.keep), _ptr(out.blk_ptr), _ptr(out.idx), _ptr(out.vals),
-                              _ptr(out.kept_weights), _ptr(out.ws), out.ws.numel(), _stream(stream)),
-           "bsp_prune_pack")
+    _check(_native.prune_pack(W, out.block, out.orient, threshold, threshold_dev, keep_per_block, out.keep, out.blk_ptr,
+                              out.idx, out.vals, out.kept_weights, out.ws, stream), "bsp_prune_pack")
 
 
 def bsp_prune_pack_static(W: torch.Tensor, out: PackedMatrix, threshold: float = 0.0,
@@ -242,15 +240,11 @@ def bsp_prune_pack_static(W: torch.Tensor, out: PackedMatrix, threshold: float =
 
 def bsp_percentile_threshold(W: torch.Tensor, block: int, orient: int, rate: float, threshold_out: torch.Tensor,
                              ws: torch.Tensor, stream=None) -> None:
-    rows, cols = W.shape
-    _check(lib.bsp_percentile_threshold(_ptr(W), rows, cols, _ld(W), block, orient, rate, _ptr(threshold_out),
-                                        _ptr(ws), ws.numel(), _stream(stream)), "bsp_percentile_threshold")
+    _check(_native.percentile_threshold(W, block, orient, rate, threshold_out, ws, stream), "bsp_percentile_threshold")
 
 
 def bsp_apply_mask(W: torch.Tensor, block: int, orient: int, keep: torch.Tensor, stream=None) -> None:
-    rows, cols = W.shape
-    _check(lib.bsp_apply_mask(_ptr(W), rows, cols, _ld(W), block, orient, _ptr(keep), _stream(stream)),
-           "bsp_apply_mask")
+    _check(_native.apply_mask(W, block, orient, keep, stream), "bsp_apply_mask")
 
 
 @dataclass
@@ -286,14 +280,15 @@ def make_job_array(jobs):
 def bsp_prepare_batched(jobs, block: int, eps: float = 1e-3, pen: int = PEN_L2, stream=None) -> None:
     """jobs: a list of LayerJob, or an array made by make_job_array."""
     arr = jobs if isinstance(jobs, ctypes.Array) else make_job_array(jobs)
-    _check(lib.bsp_prepare_batched(arr, len(arr), block, eps, pen, _stream(stream)), "bsp_prepare_batched")
+    _check(_native.prepare_batched(ctypes.addressof(arr), len(arr), block, eps, pen, stream), "bsp_prepare_batched")
 
 
 def bsp_percentile_threshold_batched(jobs, block: int, rates, stream=None) -> None:
     """Per-matrix percentile thresholds for a job array (each job's threshold_dev tensor receives its threshold)."""
     arr = jobs if isinstance(jobs, ctypes.Array) else make_job_array(jobs)
     r = (_d * len(arr))(*[float(v) for v in rates])
-    _check(lib.bsp_percentile_threshold_batched(arr, len(arr), block, r, _stream(stream)), "bsp_percentile_threshold_batched")
+    _check(_native.percentile_threshold_batched(ctypes.addressof(arr), len(arr), block, ctypes.addressof(r), stream),
+           "bsp_percentile_threshold_batched")
 
 
 def bsp_linear_plan_bytes(n_out: int, k_in: int, block: int) -> int:
@@ -304,34 +299,25 @@ def bsp_linear_plan_bytes(n_out: int, k_in: int, block: int) -> int:
 
 def bsp_linear_plan(packed: PackedMatrix, plan: torch.Tensor, stream=None) -> None:
     """Execution layout of a packed matrix of either orientation."""
-    if packed.orient == ORIENT_R:
-        _check(lib.bsp_linear_plan_r(_ptr(packed.blk_ptr), _ptr(packed.idx), _ptr(packed.vals), packed.rows, packed.cols,
-                                     packed.block, _ptr(plan), plan.numel() * plan.element_size(), _stream(stream)),
-               "bsp_linear_plan_r")
-        return
-    _check(lib.bsp_linear_plan(_ptr(packed.blk_ptr), _ptr(packed.idx), _ptr(packed.vals), packed.rows, packed.cols,
-                               packed.block, _ptr(plan), plan.numel() * plan.element_size(), _stream(stream)),
-           "bsp_linear_plan")
+    _check(_native.linear_plan(packed.orient, packed.blk_ptr, packed.idx, packed.vals, packed.rows, packed.cols, packed.block,
+                               plan, stream), "bsp_linear_plan_r" if packed.orient == ORIENT_R else "bsp_linear_plan")
 
 
 def bsp_linear_plan_t(packed: PackedMatrix, plan_t: torch.Tensor, stream=None) -> None:
     """Transposed execution layout (orientation C): the operand of dX = dY (W * Mask)."""
-    _check(lib.bsp_linear_plan_t(_ptr(packed.blk_ptr), _ptr(packed.idx), _ptr(packed.vals), packed.rows, packed.cols,
-                                 packed.block, _ptr(plan_t), plan_t.numel() * plan_t.element_size(), _stream(stream)),
-           "bsp_linear_plan_t")
+    _check(_native.linear_plan(2, packed.blk_ptr, packed.idx, packed.vals, packed.rows, packed.cols, packed.block, plan_t,
+                               stream), "bsp_linear_plan_t")
 
 
 def bsp_linear_backward_weight(dY: torch.Tensor, X: torch.Tensor, block: int, keep: Optional[torch.Tensor],
                                dW: torch.Tensor, stream=None) -> None:
     """dW = (dY^T X) * Mask; dY [tokens, n_out], X [tokens, k_in], dW [n_out, k_in], all bf16."""
-    _check(lib.bsp_linear_backward_weight(_ptr(dY), _ld(dY), _ptr(X), _ld(X), dY.shape[0], dY.shape[1], X.shape[1], block,
-                                          _ptr(keep), _ptr(dW), _ld(dW), _stream(stream)), "bsp_linear_backward_weight")
+    _check(_native.linear_backward_weight(dY, X, block, keep, dW, stream), "bsp_linear_backward_weight")
 
 
 def bsp_linear_planned(plan: torch.Tensor, n_out: int, k_in: int, block: int, X: torch.Tensor,
                        bias: Optional[torch.Tensor], act: int, Y: torch.Tensor, stream=None) -> None:
-    _check(lib.bsp_linear_planned(_ptr(plan), n_out, k_in, block, _ptr(X), X.shape[0], _ld(X), _ptr(bias), act,
-                                  _ptr(Y), _ld(Y), _stream(stream)), "bsp_linear_planned")
+    _check(_native.linear_planned(plan, n_out, k_in, block, X, bias, act, Y, LINEAR_AUTO, stream), "bsp_linear_planned")
 
 
 LINEAR_AUTO, LINEAR_ONE_CTA, LINEAR_CTA_PAIR = 0, 1, 2
@@ -342,15 +328,13 @@ LINEAR_OUT_TRANSPOSED = 0x200  # OR into `algo`: Y is written as [n_out, tokens]
 def bsp_linear_planned_ex(plan: torch.Tensor, n_out: int, k_in: int, block: int, X: torch.Tensor,
                           bias: Optional[torch.Tensor], act: int, Y: torch.Tensor, algo: int = LINEAR_AUTO,
                           stream=None) -> None:
-    _check(lib.bsp_linear_planned_ex(_ptr(plan), n_out, k_in, block, _ptr(X), X.shape[0], _ld(X), _ptr(bias), act,
-                                     _ptr(Y), _ld(Y), algo, _stream(stream)), "bsp_linear_planned_ex")
+    _check(_native.linear_planned(plan, n_out, k_in, block, X, bias, act, Y, algo, stream), "bsp_linear_planned_ex")
 
 
 def bsp_linear(packed: PackedMatrix, X: torch.Tensor, bias: Optional[torch.Tensor], act: int, Y: torch.Tensor,
                ws: Optional[torch.Tensor], stream=None) -> None:
-    _check(lib.bsp_linear(_ptr(packed.blk_ptr), _ptr(packed.idx), _ptr(packed.vals), packed.rows, packed.cols,
-                          packed.block, _ptr(X), X.shape[0], _ld(X), _ptr(bias), act, _ptr(Y), _ld(Y), _ptr(ws),
-                          0 if ws is None else ws.numel() * ws.element_size(), _stream(stream)), "bsp_linear")
+    _check(_native.linear_packed(packed.blk_ptr, packed.idx, packed.vals, packed.rows, packed.cols, packed.block, X, bias, act,
+                                 Y, ws, stream), "bsp_linear")
 
 
 def bsp_masked_adam_step(W: torch.Tensor, grad: torch.Tensor, m: torch.Tensor, v: torch.Tensor,
@@ -358,10 +342,8 @@ def bsp_masked_adam_step(W: torch.Tensor, grad: torch.Tensor, m: torch.Tensor, v
                          eps: float, weight_decay: float, step: int, W_bf16: Optional[torch.Tensor] = None,
                          stream=None) -> None:
     """W, m, v, grad: float32 [rows, cols]; keep: per-group uint8 flags or None; W_bf16: optional bf16 output."""
-    rows, cols = W.shape
-    _check(lib.bsp_masked_adam_step(_ptr(W), _ptr(grad), _ptr(m), _ptr(v), rows, cols, _ld(W), _ld(grad), _ptr(keep),
-                                    block, orient, lr, beta1, beta2, eps, weight_decay, step, _ptr(W_bf16),
-                                    0 if W_bf16 is None else _ld(W_bf16), _stream(stream)), "bsp_masked_adam_step")
+    _check(_native.masked_adam_step(W, grad, m, v, keep, block, orient, lr, beta1, beta2, eps, weight_decay, step, W_bf16,
+                                    stream), "bsp_masked_adam_step")
 
 
 def bsp_dense_mask(W: torch.Tensor, mask: torch.Tensor, stream=None) -> None:
@@ -372,8 +354,7 @@ def bsp_dense_mask(W: torch.Tensor, mask: torch.Tensor, stream=None) -> None:
 
 def bsp_repack_values(W: torch.Tensor, packed: PackedMatrix, stream=None) -> None:
     """Refreshes packed.vals from an updated bf16 W; blk_ptr and idx stay as they are."""
-    _check(lib.bsp_repack_values(_ptr(W), W.shape[0], W.shape[1], _ld(W), packed.block, _ptr(packed.blk_ptr),
-                                 _ptr(packed.idx), _ptr(packed.vals), _stream(stream)), "bsp_repack_values")
+    _check(_native.repack_values(W, packed.block, packed.blk_ptr, packed.idx, packed.vals, stream), "bsp_repack_values")
 
 
 def bsp_linear_gather_plan_bytes(n_out: int, k_in: int, block: int) -> int:
@@ -389,23 +370,21 @@ def bsp_linear_gather_plan(packed: PackedMatrix, gplan: torch.Tensor, stream=Non
 
 
 def bsp_transpose(X: torch.Tensor, XT: torch.Tensor, stream=None) -> None:
-    _check(lib.bsp_transpose(_ptr(X), X.shape[0], X.shape[1], _ld(X), _ptr(XT), _ld(XT), _stream(stream)),
-           "bsp_transpose")
+    _check(_native.transpose(X, XT, stream), "bsp_transpose")
 
 
 def bsp_linear_gathered(gplan: torch.Tensor, n_out: int, k_in: int, block: int, XT: torch.Tensor,
                         bias: Optional[torch.Tensor], act: int, Y: torch.Tensor, stream=None) -> None:
     """XT is [k_in, tokens] (the transposed activations); Y is [tokens, n_out]."""
-    _check(lib.bsp_linear_gathered(_ptr(gplan), n_out, k_in, block, _ptr(XT), XT.shape[1], _ld(XT), _ptr(bias), act,
-                                   _ptr(Y), _ld(Y), _stream(stream)), "bsp_linear_gathered")
+    _check(_native.linear_gathered(gplan, n_out, k_in, block, XT, bias, act, Y, 0, stream), "bsp_linear_gathered")
 
 
 def bsp_linear_gathered_ex(gplan: torch.Tensor, n_out: int, k_in: int, block: int, XT: torch.Tensor,
                            bias: Optional[torch.Tensor], act: int, Y: torch.Tensor, out_transposed: bool = False,
                            stream=None) -> None:
     """As bsp_linear_gathered; with out_transposed the output tensor is [n_out, tokens]."""
-    _check(lib.bsp_linear_gathered_ex(_ptr(gplan), n_out, k_in, block, _ptr(XT), XT.shape[1], _ld(XT), _ptr(bias), act,
-                                      _ptr(Y), _ld(Y), int(out_transposed), _stream(stream)), "bsp_linear_gathered_ex")
+    _check(_native.linear_gathered(gplan, n_out, k_in, block, XT, bias, act, Y, int(out_transposed), stream),
+           "bsp_linear_gathered_ex")
 
 
 @dataclass
@@ -499,9 +478,10 @@ def bsp_linear_route(call) -> int:
 
 def bsp_linear_run(call, route: int = ROUTE_AUTO, stream=None) -> int:
     """Runs the layer; returns the route taken (ROUTE_ZERO_EXPANDED or ROUTE_GATHERED)."""
-    r = _i(0)
-    _check(lib.bsp_linear_run(ctypes.byref(call), route, ctypes.byref(r), _stream(stream)), "bsp_linear_run")
-    return r.value
+    r = _native.linear_run(ctypes.addressof(call), route, stream)     # the route, or a negative status
+    if r < 0:
+        _check(r, "bsp_linear_run")
+    return r
 
 
 def bsp_linear_tune(call, reps: int = 3, stream=None) -> Tuple[int, float, float]:
