@@ -18,15 +18,19 @@ namespace {
 
 constexpr int kRowsPerPass = 4;   // rows staged in shared memory at a time
 
-struct Batch {
+// The job table travels as a kernel parameter; a single-matrix call gets a table of one job (0.2 KB instead
+// of the 15 KB of a full batch, which every launch has to copy).
+template <int N>
+struct BatchT {
   int n_jobs, block, squared;
   float eps;
-  int first_block[kFusedMaxJobs + 1];   // CTA index of each job's first row-block
-  FusedJob job[kFusedMaxJobs];
+  int first_block[N + 1];   // CTA index of each job's first row-block
+  FusedJob job[N];
 };
 
 // Job that owns CTA `cta`: the last j with first_block[j] <= cta (binary search).
-__device__ __forceinline__ int find_job(const Batch& B, int cta) {
+template <int N>
+__device__ __forceinline__ int find_job(const BatchT<N>& B, int cta) {
   int lo = 0, hi = B.n_jobs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -35,10 +39,13 @@ __device__ __forceinline__ int find_job(const Batch& B, int cta) {
   return lo;
 }
 
+template <int N>
 __global__ void __launch_bounds__(256)
-fused_stage1_kernel(const __grid_constant__ Batch B) {
+fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
   __shared__ int s_cnt[8];
   __shared__ double s_pen[8];
+  pdl_wait();
+  pdl_launch_dependents();
   const int j = find_job(B, blockIdx.x);
   const FusedJob& J = B.job[j];
   const int b = blockIdx.x - B.first_block[j];
@@ -137,12 +144,15 @@ __host__ __device__ inline int rows_per_cta(int cols, int d) {
   return r > d ? d : r;
 }
 
+template <int N>
 __global__ void __launch_bounds__(256)
-fused_stage2_kernel(const __grid_constant__ Batch B) {
+fused_stage2_kernel(const __grid_constant__ BatchT<N> B) {
   extern __shared__ __align__(16) uint8_t s_raw[];
   __shared__ int s_warp[32];
   __shared__ double s_red[8];
   __shared__ int s_base;
+  pdl_wait();
+  pdl_launch_dependents();
   const int j = find_job(B, blockIdx.x);
   const FusedJob& J = B.job[j];
   const int b = blockIdx.x - B.first_block[j];
@@ -286,59 +296,74 @@ fused_stage2_kernel(const __grid_constant__ Batch B) {
   }
 }
 
-template <typename Fill>
-int run_batches(const FusedJob* jobs, int n_jobs, int block, Fill launch) {
-  for (int j0 = 0; j0 < n_jobs; j0 += kFusedMaxJobs) {
-    Batch B;
-    B.n_jobs = n_jobs - j0 < kFusedMaxJobs ? n_jobs - j0 : kFusedMaxJobs;
-    B.block = block;
-    int total = 0, max_cols = 0;
-    for (int i = 0; i < B.n_jobs; ++i) {
-      B.job[i] = jobs[j0 + i];
-      B.first_block[i] = total;
-      total += jobs[j0 + i].n_blocks;
-      if (jobs[j0 + i].cols > max_cols) max_cols = jobs[j0 + i].cols;
-    }
-    B.first_block[B.n_jobs] = total;
-    int st = launch(B, total, max_cols);
-    if (st != BSP_OK) return st;
+template <int N>
+void fill_batch(BatchT<N>& B, const FusedJob* jobs, int n_jobs, int block, int* total, int* max_cols) {
+  B.n_jobs = n_jobs;
+  B.block = block;
+  *total = 0;
+  *max_cols = 0;
+  for (int i = 0; i < n_jobs; ++i) {
+    B.job[i] = jobs[i];
+    B.first_block[i] = *total;
+    *total += jobs[i].n_blocks;
+    if (jobs[i].cols > *max_cols) *max_cols = jobs[i].cols;
   }
+  B.first_block[n_jobs] = *total;
+}
+
+template <int N>
+int launch_stage1(const FusedJob* jobs, int n_jobs, int block, float eps, int squared, cudaStream_t s) {
+  BatchT<N> B;
+  int total, max_cols;
+  fill_batch(B, jobs, n_jobs, block, &total, &max_cols);
+  B.eps = eps;
+  B.squared = squared;
+  int threads = ((max_cols >> 3) + 31) / 32 * 32;
+  threads = threads > 256 ? 256 : threads;
+  BSP_CUDA_TRY(launch_pdl(fused_stage1_kernel<N>, dim3(total), dim3(threads), 0, s, B));
+  return BSP_OK;
+}
+
+template <int N>
+int launch_stage2(const FusedJob* jobs, int n_jobs, int block, cudaStream_t s) {
+  BatchT<N> B;
+  int total, max_cols;
+  fill_batch(B, jobs, n_jobs, block, &total, &max_cols);
+  B.eps = 0.0f;
+  B.squared = 0;
+  int splits = 1;
+  size_t smem = 0;
+  for (int i = 0; i < n_jobs; ++i) {
+    const int per = rows_per_cta(B.job[i].cols, block);
+    const int need = (block + per - 1) / per;
+    if (need > splits) splits = need;
+    const size_t bytes = static_cast<size_t>(B.job[i].cols) * (rows_per_pass(B.job[i].cols) * 2 + 4);
+    if (bytes > smem) smem = bytes;
+  }
+  BSP_CUDA_TRY(launch_pdl(fused_stage2_kernel<N>, dim3(total, splits), dim3(256), smem, s, B));
   return BSP_OK;
 }
 
 }  // namespace
 
 int fused_stage1(const FusedJob* jobs, int n_jobs, int block, float eps, int squared, cudaStream_t s) {
-  return run_batches(jobs, n_jobs, block, [&](Batch& B, int total, int max_cols) -> int {
-    B.eps = eps;
-    B.squared = squared;
-    int threads = ((max_cols >> 3) + 31) / 32 * 32;
-    threads = threads > 256 ? 256 : threads;
-    fused_stage1_kernel<<<total, threads, 0, s>>>(B);
-    BSP_LAUNCH_CHECK();
-    return BSP_OK;
-  });
+  if (n_jobs == 1) return launch_stage1<1>(jobs, 1, block, eps, squared, s);
+  for (int j0 = 0; j0 < n_jobs; j0 += kFusedMaxJobs) {
+    const int n = n_jobs - j0 < kFusedMaxJobs ? n_jobs - j0 : kFusedMaxJobs;
+    const int st = launch_stage1<kFusedMaxJobs>(jobs + j0, n, block, eps, squared, s);
+    if (st != BSP_OK) return st;
+  }
+  return BSP_OK;
 }
 
 int fused_stage2(const FusedJob* jobs, int n_jobs, int block, cudaStream_t s) {
-  return run_batches(jobs, n_jobs, block, [&](Batch& B, int total, int max_cols) -> int {
-    B.eps = 0.0f;
-    B.squared = 0;
-    int splits = 1;
-    for (int i = 0; i < B.n_jobs; ++i) {
-      const int per = rows_per_cta(B.job[i].cols, block);
-      const int need = (block + per - 1) / per;
-      if (need > splits) splits = need;
-    }
-    size_t smem = 0;
-    for (int i = 0; i < B.n_jobs; ++i) {
-      const size_t need = static_cast<size_t>(B.job[i].cols) * (rows_per_pass(B.job[i].cols) * 2 + 4);
-      if (need > smem) smem = need;
-    }
-    fused_stage2_kernel<<<dim3(total, splits), 256, smem, s>>>(B);
-    BSP_LAUNCH_CHECK();
-    return BSP_OK;
-  });
+  if (n_jobs == 1) return launch_stage2<1>(jobs, 1, block, s);
+  for (int j0 = 0; j0 < n_jobs; j0 += kFusedMaxJobs) {
+    const int n = n_jobs - j0 < kFusedMaxJobs ? n_jobs - j0 : kFusedMaxJobs;
+    const int st = launch_stage2<kFusedMaxJobs>(jobs + j0, n, block, s);
+    if (st != BSP_OK) return st;
+  }
+  return BSP_OK;
 }
 
 }  // namespace bsp

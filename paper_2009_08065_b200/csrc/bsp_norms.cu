@@ -20,12 +20,20 @@ __device__ __forceinline__ void add_penalty(const NormOut& o, double local) {
   if ((threadIdx.x & 31) == 0 && local != 0.0) atomicAdd(o.penalty, local);
 }
 
+__global__ void __launch_bounds__(32) clear_penalty_kernel(double* penalty) {
+  pdl_wait();
+  pdl_launch_dependents();
+  if (threadIdx.x == 0) *penalty = 0.0;
+}
+
 // Any geometry: one thread per group.  C: lanes run along columns (each row is read
 // contiguously by the warp).  R: lanes run along the strips of one row (adjacent groups are
 // adjacent in memory).
 __global__ void __launch_bounds__(256)
-norms_generic_kernel(const uint16_t* __restrict__ W, int rows, int cols, int ldw, int block, int orient,
+norms_generic_kernel(const uint16_t* __restrict__ W, int rows, int cols, int ldw, int block, int orient, int vec,
                      NormOut o) {
+  pdl_wait();
+  pdl_launch_dependents();
   const long long n_groups = (orient == BSP_ORIENT_C) ? static_cast<long long>(rows / block) * cols
                                                       : static_cast<long long>(rows) * (cols / block);
   const long long g = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -40,7 +48,7 @@ norms_generic_kernel(const uint16_t* __restrict__ W, int rows, int cols, int ldw
       const int per_row = cols / block;
       const long long i = g / per_row;
       const int a = static_cast<int>(g - i * per_row);
-      S = group_sumsq_strided(W + static_cast<size_t>(i) * ldw + static_cast<size_t>(a) * block, block, 1);
+      S = group_sumsq_contig(W + static_cast<size_t>(i) * ldw + static_cast<size_t>(a) * block, block, vec);
     }
     local = finish_group(o, static_cast<size_t>(g), S);
   }
@@ -75,7 +83,8 @@ extern "C" int bsp_group_norms(const void* W, int rows, int cols, int ldw, int b
   if (!(eps >= 0.0f)) return BSP_ERR_ARG;
   if (norms == nullptr && gamma_out == nullptr && penalty == nullptr) return BSP_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (penalty) BSP_CUDA_TRY(cudaMemsetAsync(penalty, 0, sizeof(double), s));
+  // (a kernel, not a memset: a memset node keeps the kernels on both sides of it from overlapping, 3 us)
+  if (penalty) BSP_CUDA_TRY(launch_pdl(clear_penalty_kernel, dim3(1), dim3(32), 0, s, penalty));
 
   NormOut o{norms, gamma_in, gamma_out, penalty, eps, pen == BSP_PEN_L2SQ ? 1 : 0};
   const uint16_t* w = static_cast<const uint16_t*>(W);
@@ -92,8 +101,8 @@ extern "C" int bsp_group_norms(const void* W, int rows, int cols, int ldw, int b
     geometry(rows, cols, block, orient, &nb, &ng);
     const long long groups = static_cast<long long>(nb) * ng;
     const unsigned grid = static_cast<unsigned>((groups + 255) / 256);
-    norms_generic_kernel<<<grid, 256, 0, s>>>(w, rows, cols, ldw, block, orient, o);
+    BSP_CUDA_TRY(launch_pdl(norms_generic_kernel, dim3(grid), dim3(256), 0, s, w, rows, cols, ldw, block, orient,
+                            contig_vec(W, ldw, block), o));
   }
-  BSP_LAUNCH_CHECK();
   return BSP_OK;
 }

@@ -1,4 +1,4 @@
-// bsp_prune_pack, bsp_percentile_threshold, bsp_apply_mask: Algorithm 1's keep decision per
+// bsp_prune_pack, bsp_apply_mask: Algorithm 1's keep decision per
 // group, Algorithm 2's mask, and the compaction of the kept groups into the canonical
 // block-structured storage (Section 3.1).
 //
@@ -7,10 +7,8 @@
 // ascending order and gather the dense tile of kept values.  W is read from HBM once by (1);
 // (2) re-reads it from L2.  Orientation C with 8-element alignment runs the vectorised
 // two-stage kernels of bsp_fused.cu; this file holds the generic kernels (any alignment,
-// orientation R, with a single-CTA scan between (1) and (2)), the keep-count and percentile
-// kernels, and the entry points.
+// orientation R), the keep-count kernel and the entry points.
 #include <mutex>
-#include <new>
 
 #include "bsp_common.cuh"
 
@@ -21,6 +19,7 @@ constexpr int kPackThreads = 256;
 
 struct Geometry {
   int rows, cols, ldw, block, orient, n_blocks, n_groups;
+  int vec;            // widest vector that reads whole pieces: of a group (R), of 8 adjacent columns (C)
 };
 
 // Pointer to element 0 of group g of block b, and the stride between the group's elements.
@@ -40,13 +39,22 @@ __device__ __forceinline__ size_t group_slot(const Geometry& G, int b, int g) {
                                   : static_cast<size_t>(g) * G.n_blocks + b;
 }
 
-// (1a) threshold mode.
-__global__ void __launch_bounds__(kPackThreads)
+// Float32 sum of squares of group g of block b.
+__device__ __forceinline__ float group_sum(const uint16_t* __restrict__ W, const Geometry& G, int b, int g) {
+  size_t stride;
+  const uint16_t* p = group_ptr(W, G, b, g, &stride);
+  return G.orient == BSP_ORIENT_C ? group_sumsq_strided(p, G.block, stride) : group_sumsq_contig(p, G.block, G.vec);
+}
+
+// (1a) threshold mode, one CTA per block.
+__global__ void __launch_bounds__(1024)
 flags_threshold_kernel(const uint16_t* __restrict__ W, Geometry G, float threshold,
                        const float* __restrict__ threshold_dev, uint8_t* __restrict__ keep,
                        int32_t* __restrict__ counts) {
   __shared__ int s_count;
   if (threadIdx.x == 0) s_count = 0;
+  pdl_wait();
+  pdl_launch_dependents();
   __syncthreads();
   const float t = threshold_dev ? *threshold_dev : threshold;
   const bool keep_all = t < 0.0f;
@@ -54,9 +62,7 @@ flags_threshold_kernel(const uint16_t* __restrict__ W, Geometry G, float thresho
   const int b = blockIdx.x;
   int local = 0;
   for (int g = threadIdx.x; g < G.n_groups; g += blockDim.x) {
-    size_t stride;
-    const uint16_t* p = group_ptr(W, G, b, g, &stride);
-    const float S = group_sumsq_strided(p, G.block, stride);
+    const float S = group_sum(W, G, b, g);
     const bool k = keep_all || (S > t2);
     keep[group_slot(G, b, g)] = k ? 1 : 0;
     local += k ? 1 : 0;
@@ -67,35 +73,102 @@ flags_threshold_kernel(const uint16_t* __restrict__ W, Geometry G, float thresho
   if (threadIdx.x == 0) counts[b] = s_count;
 }
 
-// (1b) keep-count mode: rank every group of the block by (larger S first, lower index first).
+// (1b) keep-count mode, one CTA per block: the keep_count largest sums, ties towards the lower index.  The
+// block's sums stay in shared memory as float bit patterns (monotone, they are not negative); a radix
+// select of three digits finds the smallest kept one, and a scan in index order decides which of its equals
+// are kept.  O(groups) work per digit; ranking every sum against every other one (O(groups^2)) took
+// 0.5-1 ms on the larger matrices.
+constexpr int kTopkDigit = 11;                       // 31 bits = 11 + 10 + 10
+constexpr int kTopkBins = 1 << kTopkDigit;
 __global__ void __launch_bounds__(kPackThreads)
 flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
                   uint8_t* __restrict__ keep, int32_t* __restrict__ counts) {
-  extern __shared__ float s_S[];
-  const int b = blockIdx.x;
-  for (int g = threadIdx.x; g < G.n_groups; g += blockDim.x) {
-    size_t stride;
-    const uint16_t* p = group_ptr(W, G, b, g, &stride);
-    s_S[g] = group_sumsq_strided(p, G.block, stride);
+  extern __shared__ uint32_t s_key[];                // [n_groups]
+  __shared__ uint32_t hist[kTopkBins];
+  __shared__ int s_warp[32];
+  __shared__ uint32_t s_pick[2];
+  constexpr int kPer = kTopkBins / kPackThreads;
+  const int b = blockIdx.x, n = G.n_groups;
+  pdl_wait();
+  pdl_launch_dependents();
+  if (keep_count <= 0 || keep_count >= n) {
+    const uint8_t all = keep_count > 0 ? 1 : 0;
+    for (int g = threadIdx.x; g < n; g += kPackThreads) keep[group_slot(G, b, g)] = all;
+    if (threadIdx.x == 0) counts[b] = all ? n : 0;
+    return;
   }
-  __syncthreads();
-  for (int g = threadIdx.x; g < G.n_groups; g += blockDim.x) {
-    const float mine = s_S[g];
-    int rank = 0;
-    for (int o = 0; o < G.n_groups; ++o) {
-      const float other = s_S[o];
-      rank += (other > mine || (other == mine && o < g)) ? 1 : 0;
+  if (G.orient == BSP_ORIENT_C && G.vec == 8) {
+    for (int q = threadIdx.x; q < (n >> 3); q += kPackThreads) {
+      float acc[8];
+      sumsq8(W + static_cast<size_t>(b) * G.block * G.ldw + (q << 3), G.block, G.ldw, acc);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s_key[(q << 3) + i] = __float_as_uint(acc[i]);
     }
-    keep[group_slot(G, b, g)] = rank < keep_count ? 1 : 0;
+  } else {
+    for (int g = threadIdx.x; g < n; g += kPackThreads) s_key[g] = __float_as_uint(group_sum(W, G, b, g));
   }
-  if (threadIdx.x == 0) counts[b] = keep_count < G.n_groups ? keep_count : G.n_groups;
+  uint32_t want = static_cast<uint32_t>(n - keep_count + 1);   // the smallest kept sum is the want-th smallest
+  uint32_t prefix = 0u;
+  int shift = 31;
+#pragma unroll 1
+  for (int pass = 0; pass < 3; ++pass) {
+    const int bits = pass == 0 ? kTopkDigit : 10;
+    const int above = shift;                         // bits above `above` are decided
+    shift -= bits;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) hist[threadIdx.x + i * kPackThreads] = 0u;
+    __syncthreads();
+    const uint32_t mask = (1u << bits) - 1u;
+    for (int g = threadIdx.x; g < n; g += kPackThreads) {
+      const uint32_t u = s_key[g];
+      if (above >= 31 || (u >> above) == prefix) atomicAdd(&hist[(u >> shift) & mask], 1u);
+    }
+    __syncthreads();
+    uint32_t c[kPer], mine = 0u;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) { c[i] = hist[threadIdx.x * kPer + i]; mine += c[i]; }
+    int total;
+    uint32_t before = static_cast<uint32_t>(block_exclusive_scan(static_cast<int>(mine), s_warp, &total));
+    if (before < want && want <= before + mine) {    // exactly one thread
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        if (before < want && want <= before + c[i]) { s_pick[0] = threadIdx.x * kPer + i; s_pick[1] = want - before; }
+        before += c[i];
+      }
+    }
+    __syncthreads();
+    prefix = (prefix << bits) | s_pick[0];
+    want = s_pick[1];
+    __syncthreads();
+  }
+  // groups above the smallest kept sum stay; of the e groups equal to it the first e - want + 1 do
+  // (the select counted want - 1 of them as smaller)
+  int larger = 0;
+  for (int g = threadIdx.x; g < n; g += kPackThreads) larger += s_key[g] > prefix ? 1 : 0;
+  int total;
+  block_exclusive_scan(larger, s_warp, &total);
+  const int equals_kept = keep_count - total;
+  int seen = 0;
+  for (int g0 = 0; g0 < n; g0 += kPackThreads) {
+    const int g = g0 + threadIdx.x;
+    const uint32_t u = g < n ? s_key[g] : 0u;
+    const int eq = g < n && u == prefix ? 1 : 0;
+    int round;
+    const int rank = seen + block_exclusive_scan(eq, s_warp, &round);
+    seen += round;
+    if (g < n) keep[group_slot(G, b, g)] = u > prefix || (eq && rank < equals_kept) ? 1 : 0;
+  }
+  if (threadIdx.x == 0) counts[b] = keep_count;
 }
 
-// (2) counts -> blk_ptr (exclusive scan) and the kept-weight total.
+// (2) counts -> blk_ptr (exclusive scan) and the kept-weight total: matrices with more blocks than the
+// compaction kernel adds up by itself.
 __global__ void __launch_bounds__(1024)
 scan_counts_kernel(const int32_t* __restrict__ counts, int n_blocks, int block,
                    int32_t* __restrict__ blk_ptr, int64_t* __restrict__ kept_weights) {
   __shared__ int s_warp[32];
+  pdl_wait();
+  pdl_launch_dependents();
   int running = 0;
   for (int base = 0; base < n_blocks; base += blockDim.x) {
     const int i = base + threadIdx.x;
@@ -111,17 +184,39 @@ scan_counts_kernel(const int32_t* __restrict__ counts, int n_blocks, int block,
   }
 }
 
-// (3) compaction: ascending index list and the dense tile of kept values of one block.
-__global__ void __launch_bounds__(kPackThreads)
-compact_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep,
-               const int32_t* __restrict__ blk_ptr, int32_t* __restrict__ idx,
-               uint16_t* __restrict__ vals) {
+// (3) compaction: ascending index list and the dense tile of kept values of one block.  With `counts` the
+// CTA adds up the counts before its block itself and writes blk_ptr (one launch less; 4 bytes per block and
+// CTA from L2), without it blk_ptr is there already.  Orientation R: a thread moves its whole group, by
+// vectors of G.vec elements; the kept groups of a warp are neighbours in the tile.
+__global__ void __launch_bounds__(1024)
+compact_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep, const int32_t* __restrict__ counts,
+               int32_t* __restrict__ blk_ptr, int32_t* __restrict__ idx, uint16_t* __restrict__ vals,
+               int64_t* __restrict__ kept_weights) {
   __shared__ int s_warp[32];
   const int b = blockIdx.x;
-  const int base = blk_ptr[b];
-  const int kc = blk_ptr[b + 1] - base;
+  pdl_wait();
+  pdl_launch_dependents();
+  int base, kc;
+  if (counts != nullptr) {
+    int part = 0;
+    for (int i = threadIdx.x; i < b; i += blockDim.x) part += counts[i];
+    block_exclusive_scan(part, s_warp, &base);
+    kc = counts[b];
+    if (threadIdx.x == 0) {
+      blk_ptr[b] = base;
+      if (b == G.n_blocks - 1) {
+        blk_ptr[G.n_blocks] = base + kc;
+        if (kept_weights) *kept_weights = static_cast<int64_t>(base + kc) * G.block;
+      }
+    }
+  } else {
+    base = blk_ptr[b];
+    kc = blk_ptr[b + 1] - base;
+  }
   if (kc == 0) return;
   uint16_t* tile = vals + static_cast<size_t>(G.block) * base;
+  // (values are stored at multiples of the block from an array that is only known to be 2-byte aligned)
+  const int vec = G.orient == BSP_ORIENT_R && (reinterpret_cast<uintptr_t>(vals) & 15) == 0 ? G.vec : 1;
   int running = 0;
   for (int g0 = 0; g0 < G.n_groups; g0 += blockDim.x) {
     const int g = g0 + threadIdx.x;
@@ -133,131 +228,48 @@ compact_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __rest
       idx[base + p] = g;
       size_t stride;
       const uint16_t* src = group_ptr(W, G, b, g, &stride);
+      uint16_t* dst = tile + static_cast<size_t>(p) * G.block;
       if (G.orient == BSP_ORIENT_C) {
         // tile [d, kc]: element r of the group goes to row r, position p
         for (int r = 0; r < G.block; ++r) tile[static_cast<size_t>(r) * kc + p] = src[static_cast<size_t>(r) * stride];
+      } else if (vec == 8) {
+#pragma unroll 4
+        for (int c = 0; c < G.block; c += 8) *reinterpret_cast<uint4*>(dst + c) = __ldg(reinterpret_cast<const uint4*>(src + c));
+      } else if (vec == 4) {
+#pragma unroll 4
+        for (int c = 0; c < G.block; c += 4) *reinterpret_cast<uint2*>(dst + c) = __ldg(reinterpret_cast<const uint2*>(src + c));
       } else {
-        // tile [kc, h]: the group's h contiguous elements form row p
-        for (int c = 0; c < G.block; ++c) tile[static_cast<size_t>(p) * G.block + c] = src[c];
+        for (int c = 0; c < G.block; ++c) dst[c] = src[c];
       }
     }
   }
 }
 
-
-// Float32 sums of squares of all groups, flattened in per-group-array order.
-__global__ void __launch_bounds__(kPackThreads)
-sumsq_kernel(const uint16_t* __restrict__ W, Geometry G, float* __restrict__ S) {
-  const int b = blockIdx.x;
-  for (int g = threadIdx.x; g < G.n_groups; g += blockDim.x) {
-    size_t stride;
-    const uint16_t* p = group_ptr(W, G, b, g, &stride);
-    S[group_slot(G, b, g)] = group_sumsq_strided(p, G.block, stride);
-  }
-}
-
-// r-th smallest (1-based) of n non-negative floats by a 4-pass radix select on their bit
-// patterns (monotone for non-negative floats), one CTA of 1024 threads; then the threshold whose
-// float32 square is >= that value.  Sums of squares of one matrix share their leading byte, so a
-// single shared histogram would serialise on two or three counters: every warp counts into its own
-// 256-bin histogram and the lanes of a warp that hit the same bin add once (match_any).
-__device__ void select_threshold(const float* __restrict__ S, long long n, long long r, float* __restrict__ out,
-                                 unsigned int (*hist)[256], unsigned int* s_prefix, long long* s_remaining) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
-  if (r <= 0) {
-    if (threadIdx.x == 0) *out = -1.0f;
-    return;
-  }
-  if (threadIdx.x == 0) { *s_prefix = 0u; *s_remaining = r; }
-  for (int pass = 3; pass >= 0; --pass) {
-    for (int i = lane; i < 256; i += 32) hist[warp][i] = 0u;
-    __syncthreads();
-    const unsigned int prefix = *s_prefix;
-    const int shift = pass * 8;
-    const unsigned int high_mask = pass == 3 ? 0u : (0xffffffffu << (shift + 8));
-    for (long long i0 = 0; i0 < n; i0 += blockDim.x) {
-      const long long i = i0 + threadIdx.x;
-      unsigned int bin = 0xffffffffu;                    // lanes without an element, or outside the prefix, sit out
-      if (i < n) {
-        const unsigned int u = __float_as_uint(S[i]);
-        if ((u & high_mask) == prefix) bin = (u >> shift) & 0xffu;
-      }
-      const unsigned int peers = __match_any_sync(0xffffffffu, bin);
-      if (bin != 0xffffffffu && lane == __ffs(peers) - 1) hist[warp][bin] += static_cast<unsigned int>(__popc(peers));
+// Orientation C, 8 adjacent columns per thread: nothing is read but the flags, and only pieces with a
+// pruned group are written.
+__global__ void __launch_bounds__(256)
+apply_mask_c_kernel(uint16_t* __restrict__ W, int rows, int cols, int ldw, int block, const uint8_t* __restrict__ keep) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (cols >> 3)) return;
+  for (int i = blockIdx.y; i < rows; i += gridDim.y) {
+    const uint2 f = __ldg(reinterpret_cast<const uint2*>(keep + static_cast<size_t>(i / block) * cols + (q << 3)));
+    if (((f.x - 0x01010101u) & ~f.x & 0x80808080u) == 0u && ((f.y - 0x01010101u) & ~f.y & 0x80808080u) == 0u) continue;   // no zero byte
+    uint16_t* w = W + static_cast<size_t>(i) * ldw + (q << 3);
+    if ((f.x | f.y) == 0u) {
+      *reinterpret_cast<uint4*>(w) = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if ((((c < 4 ? f.x : f.y) >> (8 * (c & 3))) & 0xffu) == 0u) w[c] = 0;
     }
-    __syncthreads();
-    if (threadIdx.x < 256) {                             // fold the warps' histograms into the first one
-      unsigned int c = 0;
-      for (int w = 0; w < n_warps; ++w) c += hist[w][threadIdx.x];
-      hist[0][threadIdx.x] = c;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      long long rem = *s_remaining;
-      unsigned int d = 0;
-      for (; d < 256; ++d) {
-        if (rem <= static_cast<long long>(hist[0][d])) break;
-        rem -= hist[0][d];
-      }
-      *s_prefix = prefix | (d << shift);
-      *s_remaining = rem;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const float s_r = __uint_as_float(*s_prefix);
-    float t = __fsqrt_rn(s_r);
-    while (__fmul_rn(t, t) < s_r) t = __uint_as_float(__float_as_uint(t) + 1u);  // next float up (t >= 0)
-    *out = t;
   }
 }
-
-__global__ void __launch_bounds__(1024)
-select_threshold_kernel(const float* __restrict__ S, long long n, long long r, float* __restrict__ out) {
-  __shared__ unsigned int hist[32][256];
-  __shared__ unsigned int s_prefix;
-  __shared__ long long s_remaining;
-  select_threshold(S, n, r, out, hist, &s_prefix, &s_remaining);
-}
-
-// The same for a batch of matrices: sums of squares of every row-block of every matrix in one launch
-// (orientation C, one CTA per row-block), then one selecting CTA per matrix.
-constexpr int kSelectBatch = 96;
-struct SelectJob {
-  const uint16_t* W;
-  int cols, ldw, n_blocks, first_block;
-  float* S;
-  float* out;
-  long long n, r;
-};
-struct SelectBatch {
-  int n_jobs, block;
-  SelectJob job[kSelectBatch];
-};
-__global__ void __launch_bounds__(kPackThreads)
-sumsq_batched_kernel(const __grid_constant__ SelectBatch B) {
-  int lo = 0, hi = B.n_jobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (B.job[mid].first_block <= static_cast<int>(blockIdx.x)) lo = mid; else hi = mid - 1;
-  }
-  const SelectJob& J = B.job[lo];
-  const int b = static_cast<int>(blockIdx.x) - J.first_block;
-  const uint16_t* wblk = J.W + static_cast<size_t>(b) * B.block * J.ldw;
-  for (int g = threadIdx.x; g < J.cols; g += blockDim.x)
-    J.S[static_cast<size_t>(b) * J.cols + g] = group_sumsq_strided(wblk + g, B.block, J.ldw);
-}
-__global__ void __launch_bounds__(1024)
-select_threshold_batched_kernel(const __grid_constant__ SelectBatch B) {
-  __shared__ unsigned int hist[32][256];
-  __shared__ unsigned int s_prefix;
-  __shared__ long long s_remaining;
-  const SelectJob& J = B.job[blockIdx.x];
-  select_threshold(J.S, J.n, J.r, J.out, hist, &s_prefix, &s_remaining);
-}
-
 __global__ void __launch_bounds__(256)
 apply_mask_kernel(uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep) {
+  pdl_wait();
+  pdl_launch_dependents();
   const long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= static_cast<long long>(G.rows) * G.cols) return;
   const int i = static_cast<int>(e / G.cols), j = static_cast<int>(e - static_cast<long long>(i) * G.cols);
@@ -306,8 +318,10 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
   if (blk_ptr == nullptr || idx == nullptr || vals == nullptr || ws == nullptr) return BSP_ERR_ARG;
   if (!aligned_to(ws, 256) || !aligned_to(vals, 2) || !aligned_to(blk_ptr, 4) || !aligned_to(idx, 4)) return BSP_ERR_ARG;
   if (threshold != threshold) return BSP_ERR_ARG;  // NaN
-  Geometry G{rows, cols, ldw, block, orient, 0, 0};
+  Geometry G{rows, cols, ldw, block, orient, 0, 0, 1};
   geometry(rows, cols, block, orient, &G.n_blocks, &G.n_groups);
+  if (orient == BSP_ORIENT_R) G.vec = contig_vec(W, ldw, block);
+  else if (cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16)) G.vec = 8;
   const WsLayout L = ws_layout(G.n_blocks, G.n_groups);
   if (ws_bytes < L.sumsq_off) return BSP_ERR_WORKSPACE;   // counts and flags; the float32 region is the percentile call's
   if (keep_per_block >= 0 && G.n_groups > BSP_TOPK_MAX_GROUPS) return BSP_ERR_UNSUPPORTED;
@@ -324,99 +338,29 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
     FusedJob j{w, rows, cols, ldw, G.n_blocks, threshold, threshold_dev, nullptr, nullptr, nullptr, nullptr, nullptr,
                flags, counts, blk_ptr, idx, static_cast<uint16_t*>(vals), kept_weights, nullptr};
     if (keep_per_block >= 0) {
-      flags_topk_kernel<<<G.n_blocks, kPackThreads, sizeof(float) * G.n_groups, s>>>(w, G, keep_per_block, flags, counts);
-      BSP_LAUNCH_CHECK();
+      BSP_CUDA_TRY(launch_pdl(flags_topk_kernel, dim3(G.n_blocks), dim3(kPackThreads), sizeof(uint32_t) * G.n_groups, s, w, G,
+                              keep_per_block, flags, counts));
     } else {
       st = fused_stage1(&j, 1, block, 0.0f, 0, s);
       if (st != BSP_OK) return st;
     }
     return fused_stage2(&j, 1, block, s);
   }
+  // a CTA per block, threads for its groups: up to 1024 of them, since a matrix of few tall blocks has few CTAs
+  const int threads = G.n_groups >= 1024 ? 1024 : G.n_groups <= 128 ? 128 : (G.n_groups + 31) / 32 * 32;
   if (keep_per_block >= 0) {
-    flags_topk_kernel<<<G.n_blocks, kPackThreads, sizeof(float) * G.n_groups, s>>>(w, G, keep_per_block, flags, counts);
+    BSP_CUDA_TRY(launch_pdl(flags_topk_kernel, dim3(G.n_blocks), dim3(kPackThreads), sizeof(uint32_t) * G.n_groups, s, w, G,
+                            keep_per_block, flags, counts));
   } else {
-    flags_threshold_kernel<<<G.n_blocks, kPackThreads, 0, s>>>(w, G, threshold, threshold_dev, flags, counts);
+    BSP_CUDA_TRY(launch_pdl(flags_threshold_kernel, dim3(G.n_blocks), dim3(threads), 0, s, w, G, threshold, threshold_dev, flags, counts));
   }
-  BSP_LAUNCH_CHECK();
-  scan_counts_kernel<<<1, 1024, 0, s>>>(counts, G.n_blocks, block, blk_ptr, kept_weights);
-  BSP_LAUNCH_CHECK();
-  compact_kernel<<<G.n_blocks, kPackThreads, 0, s>>>(w, G, flags, blk_ptr, idx, static_cast<uint16_t*>(vals));
-  BSP_LAUNCH_CHECK();
+  // every CTA of the compaction adds up the counts before its block; past 4096 blocks that costs more than a
+  // scan of its own (it grows with the square of the block count)
+  const bool own_scan = G.n_blocks > 4096;
+  if (own_scan) BSP_CUDA_TRY(launch_pdl(scan_counts_kernel, dim3(1), dim3(1024), 0, s, counts, G.n_blocks, block, blk_ptr, kept_weights));
+  BSP_CUDA_TRY(launch_pdl(compact_kernel, dim3(G.n_blocks), dim3(threads), 0, s, w, G, flags, own_scan ? nullptr : counts, blk_ptr, idx,
+                          static_cast<uint16_t*>(vals), kept_weights));
   return BSP_OK;
-}
-
-extern "C" int bsp_percentile_threshold(const void* W, int rows, int cols, int ldw, int block,
-                                        int orient, double rate, float* threshold_out, void* ws,
-                                        size_t ws_bytes, void* stream) {
-  using namespace bsp;
-  int st = check_matrix_args(W, rows, cols, ldw, block, orient);
-  if (st != BSP_OK) return st;
-  if (threshold_out == nullptr || ws == nullptr || !aligned_to(ws, 256)) return BSP_ERR_ARG;
-  if (!(rate >= 1.0)) return BSP_ERR_ARG;
-  Geometry G{rows, cols, ldw, block, orient, 0, 0};
-  geometry(rows, cols, block, orient, &G.n_blocks, &G.n_groups);
-  const WsLayout L = ws_layout(G.n_blocks, G.n_groups);
-  if (ws_bytes < L.total) return BSP_ERR_WORKSPACE;
-  const long long groups = static_cast<long long>(G.n_blocks) * G.n_groups;
-  // r = floor(G * (1 - 1/c)) in float64, as the definition states it
-  const long long r = static_cast<long long>(static_cast<double>(groups) * (1.0 - 1.0 / rate));
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  float* S = reinterpret_cast<float*>(static_cast<char*>(ws) + L.sumsq_off);
-  sumsq_kernel<<<G.n_blocks, kPackThreads, 0, s>>>(static_cast<const uint16_t*>(W), G, S);
-  BSP_LAUNCH_CHECK();
-  select_threshold_kernel<<<1, 1024, 0, s>>>(S, groups, r, threshold_out);
-  BSP_LAUNCH_CHECK();
-  return BSP_OK;
-}
-
-extern "C" int bsp_percentile_threshold_batched(const bsp_layer_job* jobs, int n_jobs, int block, const double* rates,
-                                                void* stream) {
-  using namespace bsp;
-  if (jobs == nullptr || rates == nullptr || n_jobs <= 0 || block <= 0) return BSP_ERR_ARG;
-  if (n_jobs > 4096) return BSP_ERR_UNSUPPORTED;
-  for (int i = 0; i < n_jobs; ++i) {                       // everything is checked before the first launch
-    const bsp_layer_job& u = jobs[i];
-    int st = check_matrix_args(u.W, u.rows, u.cols, u.ldw, block, BSP_ORIENT_C);
-    if (st != BSP_OK) return st;
-    if (u.threshold_dev == nullptr || u.ws == nullptr || !aligned_to(u.ws, 256)) return BSP_ERR_ARG;
-    if (!(rates[i] >= 1.0)) return BSP_ERR_ARG;
-    if (u.ws_bytes < ws_layout(u.rows / block, u.cols).total) return BSP_ERR_WORKSPACE;
-  }
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  SelectBatch* B = new (std::nothrow) SelectBatch;
-  if (B == nullptr) return BSP_ERR_ARG;
-  int st = BSP_OK;
-  for (int j0 = 0; j0 < n_jobs && st == BSP_OK; j0 += kSelectBatch) {
-    const int n = n_jobs - j0 < kSelectBatch ? n_jobs - j0 : kSelectBatch;
-    B->n_jobs = n;
-    B->block = block;
-    int blocks = 0;
-    for (int i = 0; i < n; ++i) {
-      const bsp_layer_job& u = jobs[j0 + i];
-      const int nb = u.rows / block;
-      const long long groups = static_cast<long long>(nb) * u.cols;
-      SelectJob& J = B->job[i];
-      J.W = static_cast<const uint16_t*>(u.W);
-      J.cols = u.cols;
-      J.ldw = u.ldw;
-      J.n_blocks = nb;
-      J.first_block = blocks;
-      J.S = reinterpret_cast<float*>(static_cast<char*>(u.ws) + ws_layout(nb, u.cols).sumsq_off);
-      J.out = const_cast<float*>(u.threshold_dev);
-      J.n = groups;
-      J.r = static_cast<long long>(static_cast<double>(groups) * (1.0 - 1.0 / rates[j0 + i]));   // as the single-matrix call
-      blocks += nb;
-    }
-    sumsq_batched_kernel<<<blocks, kPackThreads, 0, s>>>(*B);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) {
-      select_threshold_batched_kernel<<<n, 1024, 0, s>>>(*B);
-      e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) st = cuda_fail(e);
-  }
-  delete B;
-  return st;
 }
 
 extern "C" int bsp_apply_mask(void* W, int rows, int cols, int ldw, int block, int orient,
@@ -425,12 +369,18 @@ extern "C" int bsp_apply_mask(void* W, int rows, int cols, int ldw, int block, i
   int st = check_matrix_args(W, rows, cols, ldw, block, orient);
   if (st != BSP_OK) return st;
   if (keep == nullptr) return BSP_ERR_ARG;
-  Geometry G{rows, cols, ldw, block, orient, 0, 0};
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  uint16_t* w = static_cast<uint16_t*>(W);
+  if (orient == BSP_ORIENT_C && cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && aligned_to(keep, 8)) {
+    const dim3 grid((cols / 8 + 255) / 256, rows < 65535 ? rows : 65535);
+    const int threads = cols / 8 >= 256 ? 256 : (cols / 8 + 31) / 32 * 32;
+    BSP_CUDA_TRY(launch_pdl(apply_mask_c_kernel, grid, dim3(threads), 0, s, w, rows, cols, ldw, block, keep));
+    return BSP_OK;
+  }
+  Geometry G{rows, cols, ldw, block, orient, 0, 0, 1};
   geometry(rows, cols, block, orient, &G.n_blocks, &G.n_groups);
   const long long elems = static_cast<long long>(rows) * cols;
-  apply_mask_kernel<<<static_cast<unsigned>((elems + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<uint16_t*>(W), G, keep);
-  BSP_LAUNCH_CHECK();
+  BSP_CUDA_TRY(launch_pdl(apply_mask_kernel, dim3(static_cast<unsigned>((elems + 255) / 256)), dim3(256), 0, s, w, G, keep));
   return BSP_OK;
 }
 
