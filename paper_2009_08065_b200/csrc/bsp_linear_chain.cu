@@ -129,55 +129,69 @@ linear_chain_kernel(const __grid_constant__ ChainMaps M, const __grid_constant__
     return s_tile[r];
   };
 
-  if (warp == 0 && lane == 0) {
+  // the same for a whole warp, with one answer for its lanes
+  auto read_ticket_warp = [&](int seq) -> int {
+    const int r = seq % kRing;
+    if (!mbar_wait_warp(posted_bar(r), static_cast<uint32_t>((seq / kRing) & 1), P.status)) return -2;
+    return s_tile[r];
+  };
+
+  if (warp == 0) {
     // ---------------------------------------------------------------- tickets, and TMA producer of the X tiles
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
     for (int seq = 0; ok; ++seq) {
       const int r = seq % kRing;
-      if (!mbar_wait(taken_bar(r), static_cast<uint32_t>(((seq / kRing) & 1) ^ 1), P.status)) { ok = false; break; }
-      int tile = atomicAdd(P.ticket, 1);
-      if (tile >= P.total_tiles) tile = -1;
-      s_tile[r] = tile;
-      mbar_arrive(posted_bar(r));             // (release: the readers' waits acquire the slot's content)
+      if (!mbar_wait_warp(taken_bar(r), static_cast<uint32_t>(((seq / kRing) & 1) ^ 1), P.status)) { ok = false; break; }
+      int tile = 0;
+      if (lane == 0) {
+        tile = atomicAdd(P.ticket, 1);
+        if (tile >= P.total_tiles) tile = -1;
+        s_tile[r] = tile;
+        mbar_arrive(posted_bar(r));           // (release: the readers' waits acquire the slot's content)
+      }
+      tile = __shfl_sync(0xffffffffu, tile, 0);
       if (tile < 0) break;
       const TileRef T = decode_tile(P, tile);
       const ChainOp& op = P.op[T.g];
       if (op.dep >= 0) {
         // the rows this tile reads were written by other CTAs' TMA stores
-        if (!wait_counter(P.done + op.dep * P.m_tiles + T.m, op.dep_need, P.status)) { ok = false; break; }
+        int there = lane == 0 ? wait_counter(P.done + op.dep * P.m_tiles + T.m, op.dep_need, P.status) : 0;
+        there = __shfl_sync(0xffffffffu, there, 0);
+        __syncwarp();
+        if (!there) { ok = false; break; }
         asm volatile("fence.proxy.async;" ::: "memory");   // order the acquire before the async-proxy reads below
       }
       for (int kb = 0; kb < op.k_blocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
-        mbar_arrive_expect_tx(full_bar(stage), Cfg::kStageA);
-        tma_load_2d(smem_base + stage * Cfg::kStage, &M.x[T.g], kb * kBlockK, T.m * kBlockM, full_bar(stage));
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+        tma_stage_load(smem_base + stage * Cfg::kStage, &M.x[T.g], kb * kBlockK, T.m * kBlockM, full_bar(stage), Cfg::kStageA);
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
     }
-    if (!ok) record_timeout(P.status, timed_out);
-  } else if (warp == 10 && lane == 0) {
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 10) {
     // ---------------------------------------------------------------- TMA producer of the weight tiles
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
     for (int seq = 0; ok; ++seq) {
-      const int tile = read_ticket(seq);
+      const int tile = read_ticket_warp(seq);
       if (tile == -2) { ok = false; break; }
-      mbar_arrive(taken_bar(seq % kRing));
+      __syncwarp();                           // every lane has read the slot
+      if (lane == 0) mbar_arrive(taken_bar(seq % kRing));
       if (tile < 0) break;
       const TileRef T = decode_tile(P, tile);
       const ChainOp& op = P.op[T.g];
       for (int kb = 0; kb < op.k_blocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
-        mbar_arrive_expect_tx(full_bar(stage), static_cast<uint32_t>(op.bn) * kBlockK * 2u);
-        tma_load_2d(smem_base + stage * Cfg::kStage + Cfg::kStageA, &M.w[T.g], kb * kBlockK, T.n * op.bn, full_bar(stage));
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+        tma_stage_load(smem_base + stage * Cfg::kStage + Cfg::kStageA, &M.w[T.g], kb * kBlockK, T.n * op.bn, full_bar(stage),
+                       static_cast<uint32_t>(op.bn) * kBlockK * 2u);
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
     }
-    if (!ok) record_timeout(P.status, timed_out);
-  } else if (warp == 1 && lane == 0) {
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
     int stage = 0;
     uint32_t phase = 0;
@@ -185,33 +199,30 @@ linear_chain_kernel(const __grid_constant__ ChainMaps M, const __grid_constant__
     int acc = 0;
     bool ok = true;
     for (int seq = 0; ok; ++seq) {
-      const int tile = read_ticket(seq);
+      const int tile = read_ticket_warp(seq);
       if (tile == -2) { ok = false; break; }
-      mbar_arrive(taken_bar(seq % kRing));
+      __syncwarp();                           // every lane has read the slot
+      if (lane == 0) mbar_arrive(taken_bar(seq % kRing));
       if (tile < 0) break;
       const ChainOp& op = P.op[decode_tile(P, tile).g];
       const uint32_t idesc = instr_desc_bf16(op.bn);
-      if (!mbar_wait(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
       tcgen05_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * kMaxBN);
       for (int kb = 0; kb < op.k_blocks; ++kb) {
-        if (!mbar_wait(full_bar(stage), phase, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(full_bar(stage), phase, P.status)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t a_addr = smem_base + stage * Cfg::kStage;
         const uint32_t b_addr = a_addr + Cfg::kStageA;
-#pragma unroll
-        for (int k = 0; k < kBlockK / kUmmaK; ++k)
-          tcgen05_mma_bf16(d_tmem, smem_desc_sw128(a_addr + k * kUmmaK * 2), smem_desc_sw128(b_addr + k * kUmmaK * 2),
-                           idesc, (kb | k) != 0 ? 1u : 0u);
-        tcgen05_commit(empty_bar(stage));
+        mma_stage<2, 2>(d_tmem, smem_desc_sw128(a_addr), smem_desc_sw128(b_addr), idesc, kb != 0 ? 1u : 0u, empty_bar(stage));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
       if (!ok) break;
-      tcgen05_commit(acc_full_bar(acc));
+      tcgen05_commit_elect(acc_full_bar(acc));
       acc_phase[acc] ^= 1u;
       acc ^= 1;
     }
-    if (!ok) record_timeout(P.status, timed_out);
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
   } else if (warp >= 2 && warp < 10) {
     // ---------------------------------------------------------------- epilogue (two groups of four warps)
     const int group = (warp - 2) >> 2;

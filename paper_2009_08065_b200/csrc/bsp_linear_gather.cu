@@ -218,6 +218,37 @@ __device__ __forceinline__ void tmem_load_16cols(uint32_t taddr, uint32_t (&v)[1
       : "memory");
 }
 
+// Four rows of XT x 64 tokens, for both 64-token halves of a tile, by an elected lane of a converged warp.
+__device__ __forceinline__ void gather4_elect(uint32_t dst, const CUtensorMap* map, int x, int r0, int r1, int r2, int r3, uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t.reg .b32 d2, x2;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "add.u32 d2, %0, %8;\n\tadd.s32 x2, %2, 64;\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes "
+      "[d2], [%1, {x2, %3, %4, %5, %6}], [%7];\n\t}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(bar), "n"(kGStageK * 128)
+      : "memory");
+}
+// The MMAs of one stage, one per real group of 16 columns, then the commit that frees it.
+__device__ __forceinline__ void mma_gather_stage(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
+                                                 uint32_t groups, uint32_t free_bar) {
+  asm volatile(
+      "{\n\t.reg .pred p, t, e, e1, e2, e3;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "setp.gt.and.u32 e1, %5, 1, e;\n\tsetp.gt.and.u32 e2, %5, 2, e;\n\tsetp.gt.and.u32 e3, %5, 3, e;\n\t"
+      "add.s64 a1, %1, 128;\n\tadd.s64 a2, %1, 256;\n\tadd.s64 a3, %1, 384;\n\t"
+      "add.s64 b1, %2, 2;\n\tadd.s64 b2, %2, 4;\n\tadd.s64 b3, %2, 6;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "@e1 tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, t;\n\t"
+      "@e2 tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, t;\n\t"
+      "@e3 tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, t;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(groups), "r"(free_bar)
+      : "memory");
+}
+
 template <int D>
 __global__ void __launch_bounds__(kGThreads, 1)
 linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_constant__ GatherParams P) {
@@ -266,15 +297,14 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
     // four consecutive rows): one TMA gather4 per lane brings four kept columns (rows of XT) x 64
     // tokens into the stage with the 128-byte swizzle.  A row number equal to k_in is out of range
     // and reads as zeros (padding rows); tokens beyond the end read as zeros too.
-    const int half = lane >> 4, quad4 = lane & 15;
-    const uint32_t dst_lane = static_cast<uint32_t>(half * (kGStageK * 128) + quad4 * 512);
+    const int quad4 = lane & 15;                     // this lane holds the numbers of columns 4 quad4 .. 4 quad4 + 3
     long long n0 = 0;                                // stages before this unit, over all units of this CTA
     bool ok = true;
     for (int unit = blockIdx.x; unit < total_units && ok; unit += gridDim.x) {
       const int m = unit / P.n_chunks, ch = unit - m * P.n_chunks;
       const int rb0 = ch * P.rb_per_chunk, rb1 = min(P.n_blocks, rb0 + P.rb_per_chunk);
       const int g_begin = __ldg(P.soff + rb0), g_end = __ldg(P.soff + rb1);
-      const int x = m * kBlockM + half * 64;
+      const int x = m * kBlockM;
       const int first = g_begin + static_cast<int>(((warp - n0) % 4 + 4) % 4);   // this warp's first stage of the unit
       // column numbers and stage bytes are loaded two of the warp's stages (eight stages) ahead
       uint2 cq[2];
@@ -292,7 +322,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
             const long long n = n0 + (g - g_begin);
             const int stage = static_cast<int>(n % S);
             const uint32_t phase = static_cast<uint32_t>((n / S) & 1);
-            if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; }
+            if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; }
             if (ok) {
               const uint2 cv = cq[q];
               const uint32_t mt = mq[q];
@@ -309,20 +339,15 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
                              : "memory");
               }
               __syncwarp();
-              if (quad4 * 4 < groups * 16) {
-                int r[4];
-                r[0] = static_cast<int16_t>(cv.x & 0xffffu);
-                r[1] = static_cast<int16_t>(cv.x >> 16);
-                r[2] = static_cast<int16_t>(cv.y & 0xffffu);
-                r[3] = static_cast<int16_t>(cv.y >> 16);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) r[i] = r[i] < 0 ? P.k_in : r[i];
-                asm volatile(
-                    "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes "
-                    "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
-                    ::"r"(a_dst + dst_lane), "l"(reinterpret_cast<uint64_t>(&map_xt)), "r"(x), "r"(r[0]), "r"(r[1]),
-                      "r"(r[2]), "r"(r[3]), "r"(full_bar(stage))
-                    : "memory");
+              int r01 = static_cast<int>(cv.x), r23 = static_cast<int>(cv.y);
+              for (int q4 = 0; q4 < groups * 4; ++q4) {          // four rows of XT at a time, both 64-token halves
+                const int c01 = __shfl_sync(0xffffffffu, r01, q4), c23 = __shfl_sync(0xffffffffu, r23, q4);
+                int r0 = static_cast<int16_t>(c01 & 0xffff), r1 = c01 >> 16, r2 = static_cast<int16_t>(c23 & 0xffff), r3 = c23 >> 16;
+                r0 = r0 < 0 ? P.k_in : r0;
+                r1 = r1 < 0 ? P.k_in : r1;
+                r2 = r2 < 0 ? P.k_in : r2;
+                r3 = r3 < 0 ? P.k_in : r3;
+                gather4_elect(a_dst + static_cast<uint32_t>(q4) * 512u, &map_xt, x, r0, r1, r2, r3, full_bar(stage));
               }
             }
           }
@@ -333,7 +358,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
     if (!ok && lane == 0) record_timeout(P.status, timed_out);
   } else if (warp == 4) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc = gather_idesc(D);
       int stage = 0;
       uint32_t phase = 0;
@@ -345,34 +370,29 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
         const int rb0 = ch * P.rb_per_chunk, rb1 = min(P.n_blocks, rb0 + P.rb_per_chunk);
         const int g_begin = __ldg(P.soff + rb0), g_end = __ldg(P.soff + rb1);
         for (int g = g_begin; g < g_end; ++g) {
-          if (!mbar_wait(full_bar(stage), phase, P.status)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(stage), phase, P.status)) { ok = false; break; }
           tcgen05_fence_after();
           const uint32_t mt = s_meta[stage];
           const int groups = static_cast<int>(mt & 7u);
           const bool first = (mt & 0x10u) != 0, last = (mt & 0x20u) != 0;
           if (first) {
-            if (!mbar_wait(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
+            if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
             tcgen05_fence_after();
           }
           const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * D);
           const uint32_t a_addr = smem_base + stage * Cfg::kStage;
           const uint32_t b_addr = a_addr + kGStageA;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (k < groups)
-              tcgen05_mma_bf16(d_tmem, gather_desc_a(a_addr + k * 2048), smem_desc_sw128(b_addr + k * 32), idesc,
-                               (first && k == 0) ? 0u : 1u);
-          }
-          tcgen05_commit(empty_bar(stage));
+          mma_gather_stage(d_tmem, gather_desc_a(a_addr), smem_desc_sw128(b_addr), idesc, first ? 0u : 1u, static_cast<uint32_t>(groups),
+                           empty_bar(stage));
           if (last) {
-            tcgen05_commit(acc_full_bar(acc));
+            tcgen05_commit_elect(acc_full_bar(acc));
             acc_phase[acc] ^= 1u;
             acc ^= 1;
           }
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
       }
-      if (!ok) record_timeout(P.status, timed_out);
+      if (!ok && lane == 0) record_timeout(P.status, timed_out);
     }
   } else {
     // ---------------------------------------------------------------- epilogue

@@ -11,9 +11,9 @@
 // stays the storage format; the plan is private scratch derived from it.
 //
 // Kernel.  Persistent CTAs (one per SM) walk output tiles of 128 tokens x BN outputs.
-//   warp 0 (one lane): TMA producer, X tile [128 x 64] and W tile [BN x 64] per pipeline stage
+//   warps 0 and 10   : TMA producers, X tile [128 x 64] and W tile [BN x 64] per pipeline stage
 //                      (128-byte swizzle), completion on an mbarrier;
-//   warp 1 (one lane): issues tcgen05.mma (M=128, N=BN, K=16) into one of two TMEM accumulators
+//   warp 1           : issues tcgen05.mma (M=128, N=BN, K=16) into one of two TMEM accumulators
 //                      and commits stage release / accumulator ready to mbarriers;
 //   warps 2..9       : epilogue, two groups of four warps; group g takes the 32-column pieces of
 //                      the tile with index = g (mod 2).  Each warp tcgen05.ld's its 32 TMEM lanes
@@ -51,6 +51,7 @@ __device__ __align__(16) int g_linear_status[8];
 struct LinearParams {
   int tokens, n_out, k_in, act;
   int plan_stable;      // the plan was complete before the kernel preceding this one in the stream began
+  int a_bytes;          // bytes of one copy of an activation tile (copy_rows)
   int transposed;       // the output is written as [n_out, tokens] (map_y describes that matrix)
   const uint16_t* bias;
   int* status;
@@ -143,7 +144,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
   const int total_tiles = m_tiles * n_tiles;
   const int k_blocks = (P.k_in + kBlockK - 1) / kBlockK;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of the X tiles
     // (the two operands of a stage are issued by two warps, this one and the last one, so neither waits
     // behind the other's copy)
@@ -153,15 +154,14 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
       const int m0 = (tile / n_tiles) * kBlockM;
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
         const uint32_t a_dst = smem_base + stage * Cfg::kStage;
-        mbar_arrive_expect_tx(full_bar(stage), Cfg::kStageA);
-        tma_load_2d(a_dst, &map_x, kb * kBlockK, m0, full_bar(stage));
+        tma_stage_load(a_dst, &map_x, kb * kBlockK, m0, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
     }
-    if (!ok) record_timeout(P.status, timed_out);
-  } else if (warp == kWeightWarp && lane == 0) {
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == kWeightWarp) {
     // ---------------------------------------------------------------- TMA producer of the weight tiles
     int stage = 0;
     uint32_t phase = 0;
@@ -169,14 +169,13 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
       const int n0 = (tile % n_tiles) * BN;
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
-        mbar_arrive_expect_tx(full_bar(stage), Cfg::kStageB);
-        tma_load_2d(smem_base + stage * Cfg::kStage + Cfg::kStageA, &map_w, kb * kBlockK, n0, full_bar(stage));
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+        tma_stage_load(smem_base + stage * Cfg::kStage + Cfg::kStageA, &map_w, kb * kBlockK, n0, full_bar(stage), Cfg::kStageB);
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
     }
-    if (!ok) record_timeout(P.status, timed_out);
-  } else if (warp == 1 && lane == 0) {
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
     constexpr uint32_t idesc = instr_desc_bf16(BN);
     int stage = 0;
@@ -185,29 +184,29 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     int acc = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      if (!mbar_wait(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
       tcgen05_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * BN);
+      bool ready = false;
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(full_bar(stage), phase, P.status)) { ok = false; break; }
+        if (!mbar_wait_probed(ready, full_bar(stage), phase, P.status)) { ok = false; break; }
         tcgen05_fence_after();
+        const int next = stage + 1 == S ? 0 : stage + 1;
+        const uint32_t next_phase = next ? phase : phase ^ 1u;
+        ready = kb + 1 < k_blocks && mbar_try_wait(full_bar(next), next_phase);
         const uint32_t a_addr = smem_base + stage * Cfg::kStage;
         const uint32_t b_addr = a_addr + Cfg::kStageA;
-#pragma unroll
-        for (int k = 0; k < kBlockK / kUmmaK; ++k) {
-          const uint64_t a_desc = smem_desc_sw128(a_addr + k * kUmmaK * 2);
-          const uint64_t b_desc = smem_desc_sw128(b_addr + k * kUmmaK * 2);
-          tcgen05_mma_bf16(d_tmem, a_desc, b_desc, idesc, (kb | k) != 0 ? 1u : 0u);
-        }
-        tcgen05_commit(empty_bar(stage));  // stage reusable once these MMAs have read it
-        if (++stage == S) { stage = 0; phase ^= 1u; }
+        // the stage is reusable once these MMAs have read it
+        mma_stage<2, 2>(d_tmem, smem_desc_sw128(a_addr), smem_desc_sw128(b_addr), idesc, kb != 0 ? 1u : 0u, empty_bar(stage));
+        stage = next;
+        phase = next_phase;
       }
       if (!ok) break;
-      tcgen05_commit(acc_full_bar(acc));   // accumulator complete
+      tcgen05_commit_elect(acc_full_bar(acc));   // accumulator complete
       acc_phase[acc] ^= 1u;
       acc ^= 1;
     }
-    if (!ok) record_timeout(P.status, timed_out);
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
   } else if (warp >= 2 && warp < kWeightWarp) {
     // ---------------------------------------------------------------- epilogue
     const int group = (warp - 2) >> 2;
@@ -529,7 +528,7 @@ int launch_tc(TcDevice* dev, int slot, const void* plan, const void* X, void* Y,
   static_assert(Cfg::kStages >= 3, "pipeline too shallow");
   static_assert(BN % kEpiCols == 0, "tile width must be a multiple of the epilogue piece");
   CUtensorMap map_x, map_w, map_y;
-  if (!make_map(&map_x, X, P.k_in, P.tokens, ldx, kBlockM)) return BSP_ERR_CUDA;
+  if (!make_map(&map_x, X, P.k_in, P.tokens, ldx, copy_rows(P.tokens))) return BSP_ERR_CUDA;
   if (!make_map(&map_w, plan, P.k_in, P.n_out, P.k_in, BN)) return BSP_ERR_CUDA;
   if (P.transposed) {     // Y is [n_out, tokens]: pieces of 32 output rows x 128 tokens
     if (!make_map(&map_y, Y, P.tokens, P.n_out, ldy, kEpiCols, kBlockM)) return BSP_ERR_CUDA;
@@ -688,9 +687,11 @@ extern "C" int bsp_linear_planned_ex(const void* plan, int n_out, int k_in, int 
   const bool pair = algo == BSP_LINEAR_CTA_PAIR ||
                     (algo == BSP_LINEAR_AUTO && 4 * pair_tiles >= 5LL * dev->sms && act == BSP_ACT_NONE && !transposed);
   if (pair) return launch_tc_pair(dev, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy, s);
-  LinearParams P{tokens, n_out, k_in, act, (algo_flags & BSP_LINEAR_PLAN_STABLE) ? 1 : 0, transposed ? 1 : 0,
+  LinearParams P{tokens, n_out, k_in, act, (algo_flags & BSP_LINEAR_PLAN_STABLE) ? 1 : 0, copy_rows(tokens) * kBlockK * 2,
+                 transposed ? 1 : 0,
                  static_cast<const uint16_t*>(bias), dev->status};
-  switch (choose_bn(tokens, n_out, dev->sms)) {
+  const int bn = choose_bn(tokens, n_out, dev->sms);
+  switch (bn) {
     case 256: return launch_tc<256>(dev, 0, plan, X, Y, P, ldx, ldy, s);
     case 192: return launch_tc<192>(dev, 1, plan, X, Y, P, ldx, ldy, s);
     case 128: return launch_tc<128>(dev, 2, plan, X, Y, P, ldx, ldy, s);

@@ -47,20 +47,35 @@ __device__ __forceinline__ void cluster_sync_all() {
 // TMA load whose completion bytes are counted on an mbarrier that may live in the peer CTA.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar_cluster) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster)
       : "memory");
 }
-__device__ __forceinline__ void tcgen05_commit_pair(uint32_t bar_cluster) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_cluster) : "memory");
-}
-__device__ __forceinline__ void tcgen05_mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                      uint32_t accumulate) {
+// Commits to the same barrier of both CTAs (by an elected lane of a converged warp).
+__device__ __forceinline__ void tcgen05_commit_pair(uint32_t bar_own, uint32_t bar_peer) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}" ::"r"(bar_own), "r"(bar_peer)
+      : "memory");
+}
+// One pipeline stage for the pair: four K = 16 steps, then the commits that free the stage in both CTAs.
+__device__ __forceinline__ void mma_stage_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
+                                               uint32_t free_own, uint32_t free_peer) {
+  asm volatile(
+      "{\n\t.reg .pred p, t, e;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "add.s64 a1, %1, 2;\n\tadd.s64 a2, %1, 4;\n\tadd.s64 a3, %1, 6;\n\t"
+      "add.s64 b1, %2, 2;\n\tadd.s64 b2, %2, 4;\n\tadd.s64 b3, %2, 6;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a1, b1, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a2, b2, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a3, b3, %3, t;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(free_own), "r"(free_peer)
       : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
@@ -126,7 +141,7 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   const int total_tiles = m_tiles * n_tiles;
   const int k_blocks = (P.k_in + kBlockK - 1) / kBlockK;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer (both CTAs)
     int stage = 0;
     uint32_t phase = 0;
@@ -135,18 +150,19 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
       const int m0 = (tile / n_tiles) * 256 + static_cast<int>(rank) * kBlockM;
       const int w0 = (tile % n_tiles) * kPairBN + static_cast<int>(rank) * (kPairBN / 2);
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
         const uint32_t a_dst = smem_base + stage * kPairStage;
         const uint32_t b_dst = a_dst + kPairStageA;
         const uint32_t leader_full = map_to_cta(full_bar(stage), 0);
-        if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * kPairStage);   // both CTAs' bytes
+        if (rank == 0 && lane == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * kPairStage);   // both CTAs' bytes
+        __syncwarp();
         tma_load_2d_pair(a_dst, &map_x, kb * kBlockK, m0, leader_full);
         tma_load_2d_pair(b_dst, &map_w, kb * kBlockK, w0, leader_full);
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
     }
-    if (!ok) record_timeout(P.status, timed_out);
-  } else if (warp == 1 && lane == 0 && rank == 0) {
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 1 && rank == 0) {
     // ---------------------------------------------------------------- MMA issuer (leader CTA only)
     int stage = 0;
     uint32_t phase = 0;
@@ -154,30 +170,25 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     int acc = 0;
     bool ok = true;
     for (int tile = pair; tile < total_tiles && ok; tile += n_pairs) {
-      if (!mbar_wait(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
       tcgen05_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * kPairBN);
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(full_bar(stage), phase, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(full_bar(stage), phase, P.status)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t a_addr = smem_base + stage * kPairStage;
         const uint32_t b_addr = a_addr + kPairStageA;
-#pragma unroll
-        for (int k = 0; k < kBlockK / kUmmaK; ++k)
-          tcgen05_mma_bf16_pair(d_tmem, smem_desc_sw128(a_addr + k * kUmmaK * 2), smem_desc_sw128(b_addr + k * kUmmaK * 2),
-                                kPairIdesc, (kb | k) != 0 ? 1u : 0u);
         // the stage is free in both CTAs once these MMAs have read it
-        tcgen05_commit_pair(empty_bar(stage));
-        tcgen05_commit_pair(map_to_cta(empty_bar(stage), 1));
+        mma_stage_pair(d_tmem, smem_desc_sw128(a_addr), smem_desc_sw128(b_addr), kPairIdesc, kb != 0 ? 1u : 0u, empty_bar(stage),
+                       map_to_cta(empty_bar(stage), 1));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
       if (!ok) break;
-      tcgen05_commit_pair(acc_full_bar(acc));
-      tcgen05_commit_pair(map_to_cta(acc_full_bar(acc), 1));
+      tcgen05_commit_pair(acc_full_bar(acc), map_to_cta(acc_full_bar(acc), 1));
       acc_phase[acc] ^= 1u;
       acc ^= 1;
     }
-    if (!ok) record_timeout(P.status, timed_out);
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
   } else if (warp >= 2) {
     // ---------------------------------------------------------------- epilogue of this CTA's 128 rows
     const int group = (warp - 2) >> 2;

@@ -88,6 +88,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const i
     if (global_timer_ns() - start > limit) return false;
   }
 }
+// The same wait by a whole warp, with one answer for all of its lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const int* status) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const unsigned long long limit = wait_limit_ns(status);
+  const unsigned long long start = global_timer_ns();
+  for (;;) {
+#pragma unroll 1
+    for (int i = 0; i < 256; ++i)
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, global_timer_ns() - start > limit)) return false;
+  }
+}
 // The same wait for many threads at once (a whole CTA waiting for its bulk copies): each probe lets
 // the hardware suspend the thread for up to `kSuspendNs` or until the phase completes, so the
 // waiting warps leave the issue slots to the CTAs that share the SM instead of polling.
@@ -162,6 +174,60 @@ __device__ __forceinline__ void tcgen05_mma_bf16(uint32_t d_tmem, uint64_t a_des
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// A warp's wait for a barrier that it has already probed once (`ready`): the probe of the next stage goes out before
+// the current stage's MMAs are issued, so that its latency is hidden behind them.
+__device__ __forceinline__ bool mbar_wait_probed(bool ready, uint32_t bar, uint32_t parity, const int* status) {
+  return __all_sync(0xffffffffu, ready) || mbar_wait_warp(bar, parity, status);
+}
+
+// ---- issue by an elected lane of a converged warp
+// The tensor core's and the copy engine's instructions take their operands from the warp-uniform registers.  Issued
+// inside `if (lane == 0)` every operand is first moved there as a per-thread value: 72 cycles per tcgen05.mma and
+// 63 per commit, about 420 cycles per 64-deep stage for the issuing thread, which is what bounded every tile
+// narrower than 256 outputs (a stage of a 128 x 64 tile is 128 cycles of tensor work).  With the whole warp in the
+// loop and the lane elected inside the statement: 34 and 49.
+// One pipeline stage: four K = 16 steps, descriptors STEP_A / STEP_B (16-byte units) apart, then the commit that
+// frees the stage, all by the same lane.
+template <int STEP_A, int STEP_B>
+__device__ __forceinline__ void mma_stage(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
+                                          uint32_t free_bar) {
+  asm volatile(
+      "{\n\t.reg .pred p, t, e;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "add.s64 a1, %1, %6;\n\tadd.s64 a2, a1, %6;\n\tadd.s64 a3, a2, %6;\n\t"
+      "add.s64 b1, %2, %7;\n\tadd.s64 b2, b1, %7;\n\tadd.s64 b3, b2, %7;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, t;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(free_bar), "n"(STEP_A), "n"(STEP_B)
+      : "memory");
+}
+__device__ __forceinline__ void tcgen05_commit_elect(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+      : "memory");
+}
+// Arms a stage's barrier for `bytes` and starts its first copy.
+__device__ __forceinline__ void tma_stage_load(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar, uint32_t bytes) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%4], %5;\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "r"(bytes)
+      : "memory");
+}
+// A further copy of the same stage.
+__device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
 __device__ __forceinline__ void tmem_load_32cols(uint32_t taddr, uint32_t (&v)[32]) {
@@ -399,6 +465,12 @@ inline bool make_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+
+// Rows of one copy of an activation tile: 128, or the whole matrix rounded up to 8 rows where it has fewer.  The
+// rows of the tile behind it keep whatever shared memory holds: they only reach output rows that do not exist.
+// (Filling them with zeros costs as much of the copy engine's time as fetching them: with 8 tokens a 64-wide stage
+// took 0.3 us, three quarters of it zeros.)
+inline int copy_rows(int tokens) { return tokens >= kBlockM ? kBlockM : (tokens + 7) / 8 * 8; }
 
 }  // namespace tc
 
