@@ -1,0 +1,523 @@
+// Split contraction for tensor-core products with fewer output tiles than SMs: a cluster of C CTAs shares one
+// 128 x BN output tile, CTA r multiplies the r-th part of the contraction, and the partial tiles are added
+// through distributed shared memory.  Two operand forms:
+//   linear   Y = act(X plan^T + b): K-major operands, the contraction runs over the input features.  With few
+//            tokens a layer's product has 12 to 60 tiles of 64 outputs; FFN-down at 8 tokens was 12 CTAs
+//            working through 48 stages, 15.7 us of which nearly all was the latency of one CTA's loads.
+//   tn       dW = (dY^T X) * Mask: MN-major operands, the contraction runs over the tokens; the 18 to 72 tiles
+//            of 128 x 256 of a BERT-base weight left half to seven eighths of the SMs idle.
+// A CTA: warps 0 and 10 TMA producers of the two operands, warp 1 MMA issuer, warps
+// 2-9 the exchange and epilogue, in two groups of four warps (a warp per quarter of the TMEM lanes).  Each CTA owns
+// BN / C columns of the tile: once every CTA of the cluster has finished multiplying (first cluster barrier: the
+// operand stages are free) each sends the others their columns as float32 straight from tensor memory into their
+// stages (16 bytes per lane, 512 contiguous bytes per warp), and after the second barrier each adds its columns in
+// rank order (the result does not depend on timing), applies bias, GELU or mask, and stores bf16 rows: by TMA where
+// a warp group has 32 columns, from registers otherwise.  (Bulk copies between the CTAs' shared memories instead of
+// the stores, with an mbarrier instead of the second cluster barrier, were 0.6 us slower on the small tiles.)
+// A CTA asks for more than half of an SM's shared memory even where a few stages would do: two CTAs of a cluster
+// on one SM share its path to L2 (768 outputs x 768 inputs, C = 4: 4.2 us against 3.7).
+// All waits are bounded; a CTA whose wait ran out still takes part in the cluster barriers.
+#include <atomic>
+
+#include "bsp_tc.cuh"
+
+namespace bsp {
+using namespace tc;
+
+namespace {
+
+constexpr int kSplitThreads = 352;
+constexpr int kAtomBytes = 64 * kBlockK * 2;       // MN-major: 64 elements x 64 contraction rows = 8 KB
+
+struct SplitParams {
+  int rows, cols;            // output matrix
+  int n_tiles, k_blocks, stages;
+  int a_bytes;               // bytes of one A copy: fewer than 128 rows where the matrix has fewer
+  int bars_off;              // offset of the mbarriers behind the operand stages
+  int plan_stable, act;
+  int transposed;            // linear: the output is written as [cols, rows]
+  const uint16_t* bias;      // linear
+  const uint8_t* keep;       // tn: per-group flags [rows / block, cols], or null
+  int block;
+  uint16_t* Y;
+  int ldy;
+  int* status;
+};
+
+__device__ __forceinline__ uint32_t split_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void split_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t split_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d));
+}
+template <int N>
+__device__ __forceinline__ void tmem_load_cols(uint32_t taddr, uint32_t (&v)[N]) {
+  static_assert(N == 8 || N == 16 || N == 32, "columns per load");
+  if constexpr (N == 32) {
+    tmem_load_32cols(taddr, v);
+  } else if constexpr (N == 16) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+          "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+  } else {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr)
+                 : "memory");
+  }
+}
+// The registers of a TMEM load pass through an empty statement behind the wait, so that no use of them moves above it.
+template <int N>
+__device__ __forceinline__ void tmem_loaded(uint32_t (&v)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(v[i]));
+}
+// MN-major operand tile with the 128-byte swizzle: 8-row atoms 1024 bytes apart along the contraction,
+// 64-element groups 8 KB apart along M / N.
+__device__ __forceinline__ uint64_t split_desc_mn(uint32_t smem_addr) {
+  uint64_t d = 0;
+  d |= static_cast<uint64_t>((smem_addr & 0x3ffff) >> 4);
+  d |= static_cast<uint64_t>(kAtomBytes >> 4) << 16;             // leading byte offset / 16
+  d |= static_cast<uint64_t>(1024 >> 4) << 32;                   // stride byte offset / 16
+  d |= static_cast<uint64_t>(1) << 46;
+  d |= static_cast<uint64_t>(2) << 61;
+  return d;
+}
+
+template <int BN, int C, bool kTn>
+__global__ void __launch_bounds__(kSplitThreads, 1)
+gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                  const __grid_constant__ CUtensorMap map_y, const __grid_constant__ SplitParams P) {
+  constexpr int kStageA = kBlockM * kBlockK * 2, kStageB = BN * kBlockK * 2, kStage = kStageA + kStageB;
+  constexpr uint32_t kTmemCols = BN;
+  constexpr int W = BN / C;                            // columns a CTA owns: [rank * W, +W) of the tile
+  constexpr int UW = W >= 16 ? W / 2 : 8;              // of these, the columns of one epilogue group (W = 8: group 0 only)
+  constexpr int PC = UW < 32 / (C > 4 ? 2 : 1) ? UW : 32 / (C > 4 ? 2 : 1);   // columns a thread handles at a time
+  constexpr uint32_t kSlot = kBlockM * W * 4;          // receive buffer of one source CTA
+  constexpr bool kTmaStore = UW % kEpiCols == 0;
+  static_assert(W % 8 == 0 && UW % PC == 0, "column pieces");
+  constexpr uint32_t kIdesc = kTn ? (instr_desc_bf16(BN) | (1u << 15) | (1u << 16)) : instr_desc_bf16(BN);
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P.bars_off);       // [8] full, [8] empty, accumulator
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 17);
+  float* s_bias = reinterpret_cast<float*>(bars + 20);                   // [W]
+  volatile uint32_t* timed_out = tmem_holder + 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t smem_base = smem_u32(smem), bar_base = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (8 + s); };
+  const uint32_t acc_bar = bar_base + 8u * 16;
+  const int S = P.stages;
+  const uint32_t rank = split_rank();
+
+  if (threadIdx.x == 0) {
+    *timed_out = 0u;
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
+    for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1); }
+    mbar_init(acc_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tcgen05_fence_before();
+  __syncthreads();
+  tcgen05_fence_after();
+  const uint32_t tmem_base = *tmem_holder;
+
+  // The weights of a stable plan are older than the kernel before this one: their producer does not wait.
+  if (!(P.plan_stable && warp == 10)) pdl_wait();
+  pdl_launch_dependents();
+
+  const int tile = static_cast<int>(blockIdx.x) / C;
+  const int m0 = (tile / P.n_tiles) * kBlockM, n0 = (tile % P.n_tiles) * BN;
+  const int kb0 = static_cast<int>(static_cast<long long>(P.k_blocks) * rank / C);
+  const int kb1 = static_cast<int>(static_cast<long long>(P.k_blocks) * (rank + 1) / C);
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- TMA producer of the A tiles
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+      const uint32_t dst = smem_base + stage * kStage;
+      if constexpr (kTn) {
+        tma_stage_load(dst, &map_a, m0, kb * kBlockK, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
+        tma_load_2d_elect(dst + kAtomBytes, &map_a, m0 + 64, kb * kBlockK, full_bar(stage));
+      } else {
+        tma_stage_load(dst, &map_a, kb * kBlockK, m0, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
+      }
+      if (++stage == S) { stage = 0; phase ^= 1u; }
+    }
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 10) {
+    // ---------------------------------------------------------------- TMA producer of the B tiles
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+      const uint32_t dst = smem_base + stage * kStage + kStageA;
+      if constexpr (kTn) {
+        tma_stage_load(dst, &map_b, n0, kb * kBlockK, full_bar(stage), kStageB);
+#pragma unroll
+        for (int g = 1; g < BN / 64; ++g) tma_load_2d_elect(dst + g * kAtomBytes, &map_b, n0 + 64 * g, kb * kBlockK, full_bar(stage));
+      } else {
+        tma_stage_load(dst, &map_b, kb * kBlockK, n0, full_bar(stage), kStageB);
+      }
+      if (++stage == S) { stage = 0; phase ^= 1u; }
+    }
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true, ready = false;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_probed(ready, full_bar(stage), phase, P.status)) { ok = false; break; }
+      tcgen05_fence_after();
+      const int next = stage + 1 == S ? 0 : stage + 1;
+      const uint32_t next_phase = next ? phase : phase ^ 1u;
+      ready = kb + 1 < kb1 && mbar_try_wait(full_bar(next), next_phase);
+      const uint32_t a_addr = smem_base + stage * kStage, b_addr = a_addr + kStageA;
+      if constexpr (kTn)     // 16 contraction rows = two 8-row atoms = 2048 bytes per step
+        mma_stage<128, 128>(tmem_base, split_desc_mn(a_addr), split_desc_mn(b_addr), kIdesc, kb != kb0 ? 1u : 0u, empty_bar(stage));
+      else                   // 16 columns = 32 bytes
+        mma_stage<2, 2>(tmem_base, smem_desc_sw128(a_addr), smem_desc_sw128(b_addr), kIdesc, kb != kb0 ? 1u : 0u, empty_bar(stage));
+      stage = next;
+      phase = next_phase;
+    }
+    if (ok) tcgen05_commit_elect(acc_bar);
+    else if (lane == 0) record_timeout(P.status, timed_out);
+  }
+  __syncwarp();
+  const bool epilogue = warp >= 2 && warp < 10;
+  const int group = (warp - 2) >> 2, quad = warp & 3;
+  const int row = quad * 32 + lane, m = m0 + row;
+  const bool mine = epilogue && group * UW < W;        // this warp has columns
+  const int n_own = n0 + static_cast<int>(rank) * W + group * UW;   // its first output column
+  // the accumulator is complete: every MMA has read its operands, the stages are free
+  bool ok = true;
+  uint2 flags[kTn ? UW / 8 : 1];
+  if (epilogue) {
+    if constexpr (!kTn) {
+      const int c = static_cast<int>(threadIdx.x) - 64, n = n0 + static_cast<int>(rank) * W + c;
+      if (c < W) s_bias[c] = P.bias != nullptr && n < P.cols ? bf16_bits_to_float(__ldg(P.bias + n)) : 0.0f;
+    } else {
+#pragma unroll
+      for (int i = 0; i < UW / 8; ++i) {               // (cols is a multiple of 8: eight columns are inside or outside)
+        flags[i] = make_uint2(0x01010101u, 0x01010101u);
+        if (P.keep != nullptr && mine && m < P.rows && n_own + 8 * i < P.cols)
+          flags[i] = __ldg(reinterpret_cast<const uint2*>(P.keep + static_cast<size_t>(m / P.block) * P.cols + n_own + 8 * i));
+      }
+    }
+    ok = mbar_wait(acc_bar, 0u, P.status);
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+    tcgen05_fence_after();
+  }
+  __syncwarp();
+  split_cluster_sync();
+
+  const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+  // receive buffer of a CTA: [source, own rank left out][4-column group][row][4 floats], then the output staging
+  const uint32_t row_at = static_cast<uint32_t>(row) * 16u;
+  if (mine) {
+    // ---------------------------------------------------------------- partial columns to their owners
+#pragma unroll 1
+    for (int c0 = group * UW; c0 < (group + 1) * UW; c0 += PC) {
+      uint32_t v[C - 1][PC];
+#pragma unroll
+      for (int o = 1; o < C; ++o) tmem_load_cols<PC>(taddr + ((rank + o) % C) * W + c0, v[o - 1]);
+      tmem_load_wait();
+#pragma unroll
+      for (int o = 1; o < C; ++o) {
+        tmem_loaded<PC>(v[o - 1]);
+        const uint32_t q = (rank + o) % C, slot = rank < q ? rank : rank - 1;
+        const uint32_t dst = split_map(smem_base + slot * kSlot + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at, q);
+#pragma unroll
+        for (int j = 0; j < PC / 4; ++j)
+          st_cluster_v4(dst + j * (kBlockM * 16u), v[o - 1][4 * j], v[o - 1][4 * j + 1], v[o - 1][4 * j + 2], v[o - 1][4 * j + 3]);
+      }
+    }
+  }
+  __syncwarp();
+  split_cluster_sync();
+
+  // ---------------------------------------------------------------- this CTA's columns
+  if (epilogue) ok = epilogue_all_ok(ok);              // one decision: nobody is left alone at a named barrier
+  if (mine && ok) {
+    const uint32_t out_base = smem_base + (C - 1) * kSlot + static_cast<uint32_t>(group) * 2u * kEpiStage;
+#pragma unroll 1
+    for (int p = 0; p < UW / PC; ++p) {
+      const int c0 = group * UW + p * PC;
+      uint32_t own[PC];
+      tmem_load_cols<PC>(taddr + rank * W + c0, own);
+      tmem_load_wait();
+      tmem_loaded<PC>(own);
+      float f[PC];
+#pragma unroll
+      for (int i = 0; i < PC; ++i) f[i] = __uint_as_float(own[i]);
+      const uint32_t at = smem_base + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at;
+#pragma unroll
+      for (int src = 0; src < C - 1; ++src) {          // own part first, then the others in rank order
+        uint4 a[PC / 4];
+#pragma unroll
+        for (int j = 0; j < PC / 4; ++j) a[j] = ld_shared_v4(at + src * kSlot + j * (kBlockM * 16u));
+#pragma unroll
+        for (int j = 0; j < PC / 4; ++j) {
+          f[4 * j] += __uint_as_float(a[j].x);
+          f[4 * j + 1] += __uint_as_float(a[j].y);
+          f[4 * j + 2] += __uint_as_float(a[j].z);
+          f[4 * j + 3] += __uint_as_float(a[j].w);
+        }
+      }
+      if constexpr (!kTn) {
+#pragma unroll
+        for (int i = 0; i < PC; ++i) f[i] += s_bias[c0 + i];
+        if (P.act == BSP_ACT_GELU) {
+#pragma unroll
+          for (int i = 0; i < PC; i += 2) gelu_erf_pair(f[i], f[i + 1]);
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < PC / 8; ++u) {
+          uint2 fl = flags[0];
+#pragma unroll
+          for (int i = 1; i < UW / 8; ++i)
+            if (i == p * (PC / 8) + u) fl = flags[i];
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if ((((i < 4 ? fl.x : fl.y) >> (8 * (i & 3))) & 0xffu) == 0u) f[8 * u + i] = 0.0f;
+        }
+      }
+      uint32_t o[PC / 2];
+#pragma unroll
+      for (int i = 0; i < PC / 2; ++i) o[i] = pack_bf16x2(f[2 * i], f[2 * i + 1]);
+      if (!kTn && P.transposed) {
+        // lanes are neighbouring tokens: 64 contiguous bytes per output row
+        if (m < P.rows) {
+          uint16_t* out = P.Y + static_cast<size_t>(n0 + static_cast<int>(rank) * W + c0) * P.ldy + m;
+#pragma unroll
+          for (int i = 0; i < PC; ++i)
+            if (n_own + p * PC + i < P.cols) out[static_cast<size_t>(i) * P.ldy] = static_cast<uint16_t>(i & 1 ? o[i >> 1] >> 16 : o[i >> 1] & 0xffffu);
+        }
+      } else if constexpr (kTmaStore) {
+        // PC = 32: a 128 x 32 piece of this group, staged as the tensor map's 64-byte swizzle expects it
+        const uint32_t buf = out_base + (p & 1) * kEpiStage;
+        const bool issuer = (threadIdx.x & 127) == 64;   // first thread of warps 2 and 6
+        if (p >= 2) {
+          if (issuer) tma_store_wait_read<1>();
+          group_sync(group);
+        }
+        const uint32_t row_xor = static_cast<uint32_t>((row >> 1) & 3);
+#pragma unroll
+        for (int j = 0; j < PC / 8; ++j)
+          st_shared_v4(buf + static_cast<uint32_t>(row) * 64u + ((static_cast<uint32_t>(j) ^ row_xor) << 4), o[4 * j], o[4 * j + 1],
+                       o[4 * j + 2], o[4 * j + 3]);
+        fence_async_smem();
+        group_sync(group);
+        if (issuer) {
+          const int n = n0 + static_cast<int>(rank) * W + c0;
+          if (n < P.cols) tma_store_2d(&map_y, n, m0, buf);
+          tma_store_commit();
+        }
+      } else if (m < P.rows) {
+        uint16_t* out = P.Y + static_cast<size_t>(m) * P.ldy + n0 + static_cast<int>(rank) * W + c0;
+#pragma unroll
+        for (int u = 0; u < PC / 8; ++u)
+          if (n_own + p * PC + 8 * u < P.cols)
+            *reinterpret_cast<uint4*>(out + 8 * u) = make_uint4(o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]);
+      }
+    }
+    if (kTmaStore && (threadIdx.x & 127) == 64) tma_store_wait_read<0>();
+  }
+
+  tcgen05_fence_before();
+  __syncthreads();
+  quiet_period(timed_out);
+  if (warp == 1) {
+    tcgen05_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+  }
+}
+
+template <int BN, int C, bool kTn>
+int launch_split(TcDevice* dev, const CUtensorMap& map_a, const CUtensorMap& map_b, SplitParams P, cudaStream_t s) {
+  CUtensorMap map_y;
+  if (P.transposed) map_y = map_a;                                   // (not used)
+  else if (!make_map(&map_y, P.Y, P.cols, P.rows, P.ldy, kBlockM, kEpiCols)) return BSP_ERR_CUDA;
+  constexpr int kStage = (kBlockM + BN) * kBlockK * 2;
+  constexpr int kTail = 1024 + 160 + BN / C * 4 + 32;                // alignment slack, barriers, bias
+  constexpr int kFit = (kSmemLimit - kTail) / kStage;
+  constexpr bool kTmaStore = BN / C >= 64;
+  constexpr int kExchange = (C - 1) * kBlockM * (BN / C) * 4 + (kTmaStore ? kEpiBytes : 0);
+  constexpr int kAlone = kSmemLimit / 2 + 1024;                      // one CTA per SM
+  static_assert(kExchange + kTail <= kSmemLimit, "exchange areas");
+  const int per_cta = (P.k_blocks + C - 1) / C;
+  P.stages = per_cta < kFit ? per_cta : kFit;
+  if (P.stages > 8) P.stages = 8;
+  P.bars_off = P.stages * kStage > kExchange ? P.stages * kStage : kExchange;
+  if (P.bars_off < kAlone) P.bars_off = kAlone;
+  P.status = dev->status;
+  static std::atomic<bool> attr_set[64];
+  int device = 0;
+  BSP_CUDA_TRY(cudaGetDevice(&device));
+  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
+  if (!attr_set[device].load(std::memory_order_acquire)) {
+    BSP_CUDA_TRY(cudaFuncSetAttribute(gemm_split_kernel<BN, C, kTn>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
+    attr_set[device].store(true, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((P.rows + kBlockM - 1) / kBlockM * P.n_tiles * C);
+  cfg.blockDim = dim3(kSplitThreads);
+  cfg.dynamicSmemBytes = P.bars_off + kTail;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  BSP_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_split_kernel<BN, C, kTn>, map_a, map_b, map_y, P));
+  return BSP_OK;
+}
+template <int BN, bool kTn>
+int launch_split_c(TcDevice* dev, int c, const CUtensorMap& map_a, const CUtensorMap& map_b, const SplitParams& P, cudaStream_t s) {
+  return c == 2 ? launch_split<BN, 2, kTn>(dev, map_a, map_b, P, s)
+       : c == 4 ? launch_split<BN, 4, kTn>(dev, map_a, map_b, P, s)
+                : launch_split<BN, 8, kTn>(dev, map_a, map_b, P, s);
+}
+
+}  // namespace
+
+bool query_split_ctas(int (&ctas)[3]) {
+  // GPCs of different sizes hold different numbers of whole clusters: ask, with the shared memory of a real launch
+  if (cudaFuncSetAttribute(gemm_split_kernel<64, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
+    return false;
+  for (int i = 0; i < 3; ++i) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(8);
+    cfg.blockDim = dim3(kSplitThreads);
+    cfg.dynamicSmemBytes = kSmemLimit;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2u << i;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_split_kernel<64, 2, false>, &cfg) != cudaSuccess) return false;
+    ctas[i] = n << (i + 1);
+  }
+  return true;
+}
+
+// The choices below compare times in nanoseconds fitted to single launches on B200 (graphs of one launch, operands in
+// L2): a fixed part per kernel and a part per 64-deep stage.  They hold for grids of one wave only; a split is
+// considered where its clusters all run at once.
+//   whole tile, 64 / 128 / 192 / 256 wide: 2850 / 3200 / 3750 / 4400 + 158 / 168 / 250 / 320 per stage
+//   64-wide tile split 2 / 4 / 8:          3350 / 3450 / 3750       + 165
+//   128-wide tile split 2 / 4 / 8:         4600 / 4600 / 4600       + 170
+// (768 outputs x 3072 inputs at 128 tokens: 10.1 us whole, 4.8 us as 64-wide tiles split 8; 1024 x 4096 at 1003
+// tokens: 13.4 us whole, 128-wide tiles split 2; 768 x 768: 4.6 and 3.9; 304 inputs: not split.)
+int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, int bn_whole, int* bn) {
+  const long long m_tiles = (tokens + kBlockM - 1) / kBlockM;
+  const int kb = (k_in + kBlockK - 1) / kBlockK;
+  if (m_tiles * ((n_out + bn_whole - 1) / bn_whole) > dev.sms) return -1;
+  static const int fixed_whole[4] = {2850, 3200, 3750, 4400}, stage_whole[4] = {158, 168, 250, 320};
+  static const int fixed_split[2][3] = {{3350, 3450, 3750}, {4600, 4600, 4600}}, stage_split[2] = {165, 170};
+  const int w = bn_whole / 64 - 1;
+  int best = fixed_whole[w] + kb * stage_whole[w] - 100, choice = -1;      // a split has to win by more than noise
+  for (int b = 0; b < 2; ++b) {
+    const long long tiles = m_tiles * ((n_out + 64 * (b + 1) - 1) / (64 * (b + 1)));
+    for (int i = 0; i < 3; ++i) {
+      const int c = 2 << i;
+      if (c > kb || tiles * c > dev.split_ctas[i]) continue;
+      const int t = fixed_split[b][i] + (kb + c - 1) / c * stage_split[b];
+      if (t < best) { best = t; choice = i; *bn = 64 * (b + 1); }
+    }
+  }
+  return choice;
+}
+// dW, 128 x 256 tiles: 4600 + 360 per stage and wave whole, 6500 / 6300 / 6300 + 310 split 2 / 4 / 8.
+int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in) {
+  const long long tiles = static_cast<long long>((n_out + kBlockM - 1) / kBlockM) * ((k_in + 255) / 256);
+  const int kb = (tokens + kBlockK - 1) / kBlockK;
+  if (tiles > dev.sms) return -1;
+  static const int fixed_split[3] = {6500, 6300, 6300};
+  int best = 4600 + 360 * kb, choice = -1;
+  for (int i = 0; i < 3; ++i) {
+    const int c = 2 << i;
+    if (c > kb || tiles * c > dev.split_ctas[i]) continue;
+    const int t = fixed_split[i] + (kb + c - 1) / c * 310;
+    if (t < best) { best = t; choice = i; }
+  }
+  return choice;
+}
+
+// Y = act(X plan^T + b) with a cluster of c = 2, 4 or 8 CTAs per 128 x bn tile (arguments already validated).
+int launch_linear_split(TcDevice* dev, int bn, int c, const void* plan, const void* X, void* Y, int tokens, int n_out, int k_in,
+                        int act, const void* bias, int ldx, int ldy, bool plan_stable, bool transposed, cudaStream_t s) {
+  CUtensorMap map_x, map_w;
+  const int box = copy_rows(tokens);
+  if (!make_map(&map_x, X, k_in, tokens, ldx, box)) return BSP_ERR_CUDA;
+  if (!make_map(&map_w, plan, k_in, n_out, k_in, bn)) return BSP_ERR_CUDA;
+  SplitParams P{};
+  P.rows = tokens;
+  P.cols = n_out;
+  P.n_tiles = (n_out + bn - 1) / bn;
+  P.k_blocks = (k_in + kBlockK - 1) / kBlockK;
+  P.a_bytes = box * kBlockK * 2;
+  P.plan_stable = plan_stable ? 1 : 0;
+  P.transposed = transposed ? 1 : 0;
+  P.act = act;
+  P.bias = static_cast<const uint16_t*>(bias);
+  P.Y = static_cast<uint16_t*>(Y);
+  P.ldy = ldy;
+  return bn == 64 ? launch_split_c<64, false>(dev, c, map_x, map_w, P, s) : launch_split_c<128, false>(dev, c, map_x, map_w, P, s);
+}
+
+// dW = (dY^T X) * Mask with a cluster of c = 2, 4 or 8 CTAs per 128 x 256 tile (arguments already validated; keep
+// 8-byte aligned or null).
+int launch_tn_split(TcDevice* dev, int c, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
+                    int block, const uint8_t* keep, void* dW, int lddw, cudaStream_t s) {
+  CUtensorMap map_dy, map_x;
+  if (!make_map(&map_dy, dY, n_out, tokens, ldy, kBlockK)) return BSP_ERR_CUDA;
+  if (!make_map(&map_x, X, k_in, tokens, ldx, kBlockK)) return BSP_ERR_CUDA;
+  SplitParams P{};
+  P.rows = n_out;
+  P.cols = k_in;
+  P.n_tiles = (k_in + 255) / 256;
+  P.k_blocks = (tokens + kBlockK - 1) / kBlockK;
+  P.a_bytes = kBlockM * kBlockK * 2;
+  P.keep = keep;
+  P.block = block;
+  P.Y = static_cast<uint16_t*>(dW);
+  P.ldy = lddw;
+  return launch_split_c<256, true>(dev, c, map_dy, map_x, P, s);
+}
+
+}  // namespace bsp

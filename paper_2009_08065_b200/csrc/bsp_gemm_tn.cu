@@ -10,7 +10,8 @@
 // stride byte offset = distance between 8-row groups).  Everything else (persistent CTAs, TMA
 // producers, one MMA-issuing thread, two TMEM accumulators, two epilogue groups, TMA stores,
 // bounded waits) is the pipeline of bsp_linear_tc.cu with a 128 x 256 output tile.
-// The mask is applied afterwards by the mask kernel (pruned groups of dW are written as zero).
+// The epilogue applies the mask (pruned groups of dW are written as zero).  A weight of fewer tiles than SMs goes
+// to the split contraction of bsp_gemm_split.cu instead where that is faster.
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -40,6 +41,8 @@ constexpr uint32_t kTnIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | 
 
 struct TnParams {
   int tokens, n_out, k_in;
+  const uint8_t* keep;       // per-group flags [n_out / block, k_in], 8-byte aligned, or null
+  int block;
   int* status;
 };
 
@@ -88,7 +91,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
   const int total_tiles = m_tiles * n_tiles;
   const int k_blocks = (P.tokens + kBlockK - 1) / kBlockK;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of the dY tiles
     int stage = 0;
     uint32_t phase = 0;
@@ -96,17 +99,15 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
       const int m0 = (tile / n_tiles) * kBlockM;
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
         const uint32_t a_dst = smem_base + stage * Cfg::kStage;
-        mbar_arrive_expect_tx(full_bar(stage), Cfg::kStageA);
-#pragma unroll
-        for (int g = 0; g < kBlockM / 64; ++g)
-          tma_load_2d(a_dst + g * kAtomGroup, &map_dy, m0 + 64 * g, kb * kBlockK, full_bar(stage));
+        tma_stage_load(a_dst, &map_dy, m0, kb * kBlockK, full_bar(stage), Cfg::kStageA);
+        tma_load_2d_elect(a_dst + kAtomGroup, &map_dy, m0 + 64, kb * kBlockK, full_bar(stage));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
     }
-    if (!ok) record_timeout(P.status, timed_out);
-  } else if (warp == 10 && lane == 0) {
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 10) {
     // ---------------------------------------------------------------- TMA producer of the X tiles
     int stage = 0;
     uint32_t phase = 0;
@@ -114,17 +115,17 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
       const int n0 = (tile % n_tiles) * kTnBN;
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
         const uint32_t b_dst = smem_base + stage * Cfg::kStage + Cfg::kStageA;
-        mbar_arrive_expect_tx(full_bar(stage), Cfg::kStageB);
+        tma_stage_load(b_dst, &map_x, n0, kb * kBlockK, full_bar(stage), Cfg::kStageB);
 #pragma unroll
-        for (int g = 0; g < kTnBN / 64; ++g)
-          tma_load_2d(b_dst + g * kAtomGroup, &map_x, n0 + 64 * g, kb * kBlockK, full_bar(stage));
+        for (int g = 1; g < kTnBN / 64; ++g)
+          tma_load_2d_elect(b_dst + g * kAtomGroup, &map_x, n0 + 64 * g, kb * kBlockK, full_bar(stage));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
     }
-    if (!ok) record_timeout(P.status, timed_out);
-  } else if (warp == 1 && lane == 0) {
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
+  } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
     int stage = 0;
     uint32_t phase = 0;
@@ -132,27 +133,24 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     int acc = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      if (!mbar_wait(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
       tcgen05_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * kTnBN);
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(full_bar(stage), phase, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(full_bar(stage), phase, P.status)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t a_addr = smem_base + stage * Cfg::kStage;
         const uint32_t b_addr = a_addr + Cfg::kStageA;
-#pragma unroll
-        for (int k = 0; k < kBlockK / kUmmaK; ++k)     // 16 token rows = two 8-row atoms = 2048 bytes per step
-          tcgen05_mma_bf16(d_tmem, smem_desc_mn_sw128(a_addr + k * 2048), smem_desc_mn_sw128(b_addr + k * 2048), kTnIdesc,
-                           (kb | k) != 0 ? 1u : 0u);
-        tcgen05_commit(empty_bar(stage));
+        // 16 token rows = two 8-row atoms = 2048 bytes per step
+        mma_stage<128, 128>(d_tmem, smem_desc_mn_sw128(a_addr), smem_desc_mn_sw128(b_addr), kTnIdesc, kb != 0 ? 1u : 0u, empty_bar(stage));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
       if (!ok) break;
-      tcgen05_commit(acc_full_bar(acc));
+      tcgen05_commit_elect(acc_full_bar(acc));
       acc_phase[acc] ^= 1u;
       acc ^= 1;
     }
-    if (!ok) record_timeout(P.status, timed_out);
+    if (!ok && lane == 0) record_timeout(P.status, timed_out);
   } else if (warp >= 2 && warp < 10) {
     // ---------------------------------------------------------------- epilogue (as in bsp_linear_tc.cu, no bias)
     const int group = (warp - 2) >> 2;
@@ -183,7 +181,20 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
         if (issuer) tma_store_wait_read<1>();
         group_sync(group);
         EpiloguePiece piece;
+        uint2 flags[kEpiCols / 8];
+#pragma unroll
+        for (int j = 0; j < kEpiCols / 8; ++j) {     // (k_in is a multiple of 8: eight columns are inside or outside)
+          flags[j] = make_uint2(0x01010101u, 0x01010101u);
+          const int n = n0 + c0 + 8 * j;
+          if (P.keep != nullptr && m0 + row < P.n_out && n < P.k_in)
+            flags[j] = __ldg(reinterpret_cast<const uint2*>(P.keep + static_cast<size_t>((m0 + row) / P.block) * P.k_in + n));
+        }
         piece_load(taddr + c0, smem_u32(s_zero), piece);
+        if (P.keep != nullptr) {
+#pragma unroll
+          for (int i = 0; i < kEpiCols; ++i)
+            if ((((i & 4 ? flags[i >> 3].y : flags[i >> 3].x) >> (8 * (i & 3))) & 0xffu) == 0u) piece.v[i] = 0u;
+        }
         if (pc + 2 >= pieces) {
           tcgen05_fence_before();
           __syncwarp();
@@ -235,6 +246,15 @@ extern "C" int bsp_linear_backward_weight(const void* dY, int ldy, const void* X
     return BSP_ERR_UNSUPPORTED;
   TcDevice* dev = tc_device();
   if (dev == nullptr) return BSP_ERR_CUDA;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // (flags that are not 8-byte aligned are applied by the mask kernel afterwards)
+  const uint8_t* flags = keep != nullptr && aligned_to(keep, 8) ? keep : nullptr;
+  const int split = choose_tn_split(*dev, tokens, n_out, k_in);
+  if (split >= 0) {
+    const int st = launch_tn_split(dev, 2 << split, dY, ldy, X, ldx, tokens, n_out, k_in, block, flags, dW, lddw, s);
+    if (st != BSP_OK || keep == flags) return st;
+    return bsp_apply_mask(dW, n_out, k_in, lddw, block, BSP_ORIENT_C, keep, stream);
+  }
   // operands as [token rows, features]: inner dimension = features, boxes of 64 features x 64 token rows
   CUtensorMap map_dy, map_x, map_dw;
   if (!make_map(&map_dy, dY, n_out, tokens, ldy, kBlockK)) return BSP_ERR_CUDA;
@@ -244,9 +264,8 @@ extern "C" int bsp_linear_backward_weight(const void* dY, int ldy, const void* X
     BSP_CUDA_TRY(cudaFuncSetAttribute(gemm_tn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
     dev->attr_set[6] = true;
   }
-  TnParams P{tokens, n_out, k_in, dev->status};
+  TnParams P{tokens, n_out, k_in, flags, block, dev->status};
   const int tiles = ((n_out + kBlockM - 1) / kBlockM) * ((k_in + kTnBN - 1) / kTnBN);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles < dev->sms ? tiles : dev->sms);
   cfg.blockDim = dim3(kTnThreads);
@@ -258,6 +277,6 @@ extern "C" int bsp_linear_backward_weight(const void* dY, int ldy, const void* X
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   BSP_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_tn_kernel, map_dy, map_x, map_dw, P));
-  if (keep != nullptr) return bsp_apply_mask(dW, n_out, k_in, lddw, block, BSP_ORIENT_C, keep, stream);
+  if (keep != flags) return bsp_apply_mask(dW, n_out, k_in, lddw, block, BSP_ORIENT_C, keep, stream);
   return BSP_OK;
 }

@@ -13,7 +13,7 @@
 // been handed out belongs to a running CTA that got it without waiting for a larger one, and a CTA
 // works through its tiles in the order it took them, so the smallest unfinished tile can always
 // proceed: no co-residency of all CTAs is needed.  The dependency wait, like the mbarrier waits,
-// has a deadline.
+// has a deadline.  Few tokens are served by single launches instead (see the entry point).
 //
 // Inside a CTA the pipeline is the one of bsp_linear_tc.cu (X producer, weight producer, MMA
 // issuer, two epilogue groups of four warps, two TMEM accumulators, operand stages sized for the
@@ -340,6 +340,7 @@ extern "C" int bsp_linear_chain(const bsp_chain_op* ops, int n_ops, const void* 
   P.m_tiles = m_tiles;
   P.tokens = tokens;
   int tile_begin = 0;
+  bool split = false;
   for (int i = 0; i < n_ops; ++i) {
     const bsp_chain_op& u = ops[i];
     const void* src = X;
@@ -353,6 +354,8 @@ extern "C" int bsp_linear_chain(const bsp_chain_op* ops, int n_ops, const void* 
       return BSP_ERR_UNSUPPORTED;
     if (tokens == 0) continue;
     const int bn = choose_bn(tokens, u.n_out, dev->sms);
+    int bn_split;
+    split = split || (u.k_in <= 12288 && choose_linear_split(*dev, tokens, u.n_out, u.k_in, bn, &bn_split) >= 0);
     const uint16_t* src_base = static_cast<const uint16_t*>(src) + u.src_col;
     if (!make_map(&M.x[i], src_base, u.k_in, tokens, src_ld, kBlockM)) return BSP_ERR_CUDA;
     if (!make_map(&M.w[i], u.plan, u.k_in, u.n_out, u.k_in, bn)) return BSP_ERR_CUDA;
@@ -370,6 +373,18 @@ extern "C" int bsp_linear_chain(const bsp_chain_op* ops, int n_ops, const void* 
     tile_begin += o.n_tiles * m_tiles;
   }
   if (tokens == 0) return BSP_OK;
+  // With so few tokens that single launches would split a contraction over a cluster, single launches are what is
+  // fastest (a layer at 8 tokens: 17 us against 45), and the outputs are theirs bit for bit.
+  if (split) {
+    for (int i = 0; i < n_ops; ++i) {
+      const bsp_chain_op& u = ops[i];
+      const uint16_t* src = static_cast<const uint16_t*>(u.src >= 0 ? ops[u.src].Y : X) + u.src_col;
+      st = bsp_linear_planned(u.plan, u.n_out, u.k_in, u.block, src, tokens, u.src >= 0 ? ops[u.src].ldy : ldx, u.bias, u.act, u.Y,
+                              u.ldy, stream);
+      if (st != BSP_OK) return st;
+    }
+    return BSP_OK;
+  }
   P.total_tiles = tile_begin;
 
   P.status = dev->status;

@@ -580,6 +580,7 @@ TcDevice* tc_device() {
     int init[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     memcpy(&init[2], &limit, sizeof(limit));
     if (cudaMemcpy(p, init, sizeof(init), cudaMemcpyHostToDevice) != cudaSuccess) return nullptr;
+    if (!query_split_ctas(d.split_ctas)) return nullptr;
     d.status = static_cast<int*>(p);
     d.sms = sms;
   }
@@ -691,6 +692,14 @@ extern "C" int bsp_linear_planned_ex(const void* plan, int n_out, int k_in, int 
                  transposed ? 1 : 0,
                  static_cast<const uint16_t*>(bias), dev->status};
   const int bn = choose_bn(tokens, n_out, dev->sms);
+  if (algo == BSP_LINEAR_AUTO) {
+    // few output tiles: a cluster of CTAs per tile, each with a part of the contraction
+    int bn_split = 0;
+    const int c = choose_linear_split(*dev, tokens, n_out, k_in, bn, &bn_split);
+    if (c >= 0)
+      return launch_linear_split(dev, bn_split, 2 << c, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy,
+                                 (algo_flags & BSP_LINEAR_PLAN_STABLE) != 0, transposed, s);
+  }
   switch (bn) {
     case 256: return launch_tc<256>(dev, 0, plan, X, Y, P, ldx, ldy, s);
     case 192: return launch_tc<192>(dev, 1, plan, X, Y, P, ldx, ldy, s);

@@ -156,26 +156,8 @@ __device__ __forceinline__ void quiet_period(const volatile uint32_t* cta_flag) 
   }
   __syncthreads();
 }
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
 __device__ __forceinline__ void tcgen05_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tcgen05_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tcgen05_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tcgen05_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                 uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 // A warp's wait for a barrier that it has already probed once (`ready`): the probe of the next stage goes out before
 // the current stage's MMAs are issued, so that its latency is hidden behind them.
 __device__ __forceinline__ bool mbar_wait_probed(bool ready, uint32_t bar, uint32_t parity, const int* status) {
@@ -480,7 +462,18 @@ struct TcDevice {
   int sms = 0;
   int* status = nullptr;
   bool attr_set[8] = {false, false, false, false, false, false, false, false};
+  int split_ctas[3] = {0, 0, 0};     // CTAs of bsp_gemm_split.cu's kernel that run at once in clusters of 2, 4, 8
 };
 TcDevice* tc_device();
+// Fills split_ctas (bsp_gemm_split.cu).
+bool query_split_ctas(int (&ctas)[3]);
+// Cluster size (2, 4, 8) index of dW's split contraction, or -1: the persistent kernel (bsp_gemm_split.cu).
+int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in);
+// The same for the linear layer; *bn = tile width.  bn_whole is the tile width of the one-CTA kernel.
+int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, int bn_whole, int* bn);
+int launch_linear_split(TcDevice* dev, int bn, int c, const void* plan, const void* X, void* Y, int tokens, int n_out, int k_in,
+                        int act, const void* bias, int ldx, int ldy, bool plan_stable, bool transposed, cudaStream_t s);
+int launch_tn_split(TcDevice* dev, int c, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
+                    int block, const uint8_t* keep, void* dW, int lddw, cudaStream_t s);
 
 }  // namespace bsp
