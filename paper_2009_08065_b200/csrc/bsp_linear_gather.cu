@@ -23,8 +23,12 @@
 //               lane 0 also issues the bulk copy of the weight tile and hands the stage's byte on;
 //   warp 4    : one lane issues tcgen05.mma (M=128, N=d, K=16) into one of two TMEM accumulators,
 //               commits stage release and, at the end of a row-block, accumulator ready;
-//   warps 5-8 : epilogue; each warp reads its 32 TMEM lanes (tokens), adds bias, optional GELU,
-//               rounds to bf16 and stores its row's d outputs (2 d contiguous bytes).
+//   warps 5-12: epilogue, two groups of four warps that take the row-blocks in turn (group = accumulator);
+//               each warp reads its 32 TMEM lanes (tokens), adds bias, optional GELU, rounds to bf16, and the
+//               group's 128 x 32 pieces leave through staging buffers as TMA stores (blocks of 16 rows:
+//               straight from registers).  With one group storing from registers a row-block of 128 outputs
+//               with GELU, written transposed, took longer than its two stages of 64 columns: 54 us for
+//               4096 x 1024 at 8 times compression and 8192 tokens, 27 us for the same work without either.
 // Every wait is bounded; on expiry the role records BSP_ERR_TIMEOUT and leaves its loop.
 //
 // What bounds it: every gathered element crosses L2 -> shared memory once per row-block and feeds
@@ -42,7 +46,7 @@ using namespace tc;
 
 namespace {
 
-constexpr int kGThreads = 288;              // 4 producer warps, MMA warp, 4 epilogue warps
+constexpr int kGThreads = 416;              // 4 producer warps, MMA warp, 2 x 4 epilogue warps
 constexpr int kGStageK = 64;                // kept columns per pipeline stage
 constexpr int kGStageA = kGStageK * kBlockM * 2;   // 16 KB: 64 rows of 128 tokens
 constexpr int kGQueue = 12;                 // a producer warp loads its column numbers up to this many stages ahead
@@ -52,7 +56,9 @@ template <int D>
 struct GatherCfg {
   static constexpr int kStageB = D * 128;                       // d rows of 64 bf16
   static constexpr int kStage = kGStageA + kStageB;
-  static constexpr int kFixed = 1024 /*alignment slack*/ + 512 /*barriers, stage bytes*/;
+  static constexpr bool kStaged = D >= kEpiCols;                // outputs leave through staging buffers and TMA stores
+  static constexpr int kStaging = kStaged ? kEpiBytes : 0;
+  static constexpr int kFixed = 1024 /*alignment slack*/ + 512 /*barriers, stage bytes*/ + 2 * D * 2 /*bias, two blocks*/ + kStaging;
   static constexpr int kStagesRaw = (kSmemLimit - kFixed) / kStage;
   static constexpr int kStages = kStagesRaw > 12 ? 12 : kStagesRaw;
   static constexpr int kTmemCols = 2 * D < 32 ? 32 : 2 * D;     // 32, 64, 128, 256
@@ -151,6 +157,8 @@ gather_plan_fill_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __re
 __global__ void __launch_bounds__(256)
 transpose_kernel(const uint16_t* __restrict__ X, int rows, int cols, int ldx, uint16_t* __restrict__ XT, int ldxt) {
   __shared__ uint16_t s_t[64][66];
+  pdl_wait();
+  pdl_launch_dependents();
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   for (int e = threadIdx.x; e < 512; e += 256) {
     const int r = e >> 3, q = e & 7;
@@ -249,15 +257,32 @@ __device__ __forceinline__ void mma_gather_stage(uint32_t d_tmem, uint64_t a_des
       : "memory");
 }
 
+// The 128 threads of an epilogue group agree on whether all of their waits succeeded (named barrier 3 + group); also
+// the barrier behind the group's bias writes.
+__device__ __forceinline__ bool group_all_ok(int group, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %1, 0;\n\t"
+      "barrier.cta.red.and.pred q, %2, 128, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(ok ? 1u : 0u), "r"(3 + group)
+      : "memory");
+  return r != 0u;
+}
+
 template <int D>
 __global__ void __launch_bounds__(kGThreads, 1)
-linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_constant__ GatherParams P) {
+linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_constant__ CUtensorMap map_y,
+                     const __grid_constant__ GatherParams P) {
   using Cfg = GatherCfg<D>;
   constexpr int S = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  // [S stages: A 16 KB, B D*128][mbarriers][stage bytes][TMEM base]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * Cfg::kStage);
+  // [S stages: A 16 KB, B D*128][output staging][bias of two row-blocks][mbarriers][stage bytes][TMEM base]
+  uint16_t* s_bias = reinterpret_cast<uint16_t*>(smem + S * Cfg::kStage + Cfg::kStaging);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_bias + 2 * D);
   // bars[0..S) full, [S..2S) empty, [2S..2S+2) accumulator full, [2S+2..2S+4) accumulator empty
   uint8_t* s_meta = reinterpret_cast<uint8_t*>(bars + 2 * S + 4);
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(s_meta + 16);
@@ -290,6 +315,8 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
   const uint32_t tmem_base = *tmem_holder;
 
   const int total_units = P.m_tiles * P.n_chunks;
+  pdl_wait();
+  pdl_launch_dependents();
 
   if (warp < 4) {
     // ---------------------------------------------------------------- producers
@@ -396,40 +423,61 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
     }
   } else {
     // ---------------------------------------------------------------- epilogue
+    const int group = (warp - 5) >> 2;       // takes accumulator `group`: every other row-block of this CTA's sequence
     const int quad = warp & 3;               // TMEM lanes [32*quad, 32*quad+32) belong to this warp
-    uint32_t acc_phase[2] = {0u, 0u};
-    int acc = 0;
+    const int row = quad * 32 + lane;
+    const int tid = static_cast<int>(threadIdx.x) - 160 - group * 128;
+    const bool issuer = tid == 0;            // the thread that owns the group's TMA stores
+    const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(group * D);
+    const uint32_t buf0 = smem_base + S * Cfg::kStage + static_cast<uint32_t>(group) * 2u * kEpiStage;
+    uint16_t* my_bias = s_bias + group * D;
+    uint32_t phase = 0u, piece_no = 0u;
+    int seq = 0;                             // row-blocks of this CTA so far
     bool ok = true;
     for (int unit = blockIdx.x; unit < total_units && ok; unit += gridDim.x) {
       const int m = unit / P.n_chunks, ch = unit - m * P.n_chunks;
       const int rb0 = ch * P.rb_per_chunk, rb1 = min(P.n_blocks, rb0 + P.rb_per_chunk);
-      const int t = m * kBlockM + quad * 32 + lane;
-      uint16_t* yrow = P.Y + static_cast<size_t>(t) * P.ldy;
-      for (int rb = rb0; rb < rb1; ++rb) {
-        // the bias of this row-block first, so that its latency overlaps the wait for the accumulator
-        uint4 bv[D / 8];
-#pragma unroll
-        for (int j = 0; j < D / 8; ++j) bv[j] = make_uint4(0u, 0u, 0u, 0u);
-        if (P.bias != nullptr) {
-          const uint4* bp = reinterpret_cast<const uint4*>(P.bias + static_cast<size_t>(rb) * D);
-#pragma unroll
-          for (int j = 0; j < D / 8; ++j) bv[j] = __ldg(bp + j);
-        }
-        if (!mbar_wait(acc_full_bar(acc), acc_phase[acc], P.status)) { ok = false; break; }
+      for (int rb = rb0; rb < rb1; ++rb, ++seq) {
+        if ((seq & 1) != group) continue;
+        // the bias first, so that its latency overlaps the wait for the accumulator (its last readers are behind
+        // the group's last barrier)
+        if (tid < D) my_bias[tid] = P.bias != nullptr ? __ldg(P.bias + static_cast<size_t>(rb) * D + tid) : static_cast<uint16_t>(0);
+        // one decision for the group: nobody is left alone at its barriers
+        if (!group_all_ok(group, mbar_wait(acc_full_bar(group), phase, P.status))) { ok = false; break; }
+        phase ^= 1u;
         tcgen05_fence_after();
-        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(acc * D);
-        constexpr int kPiece = 16;
-#pragma unroll
-        for (int c0 = 0; c0 < D; c0 += kPiece) {
-          uint32_t v[16];
-          tmem_load_16cols(taddr + c0, v);
-          tmem_load_wait();
-          if (c0 + kPiece >= D) {              // this warp's last read of the accumulator
-            tcgen05_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty_bar(acc));
+        if constexpr (Cfg::kStaged) {
+#pragma unroll 1
+          for (int c0 = 0; c0 < D; c0 += kEpiCols) {
+            const uint32_t buf = buf0 + (piece_no & 1u) * kEpiStage;
+            ++piece_no;
+            EpiloguePiece piece;
+            piece_load(taddr + c0, smem_u32(my_bias + c0), piece);
+            if (issuer) tma_store_wait_read<1>();   // the store issued two pieces ago has read this buffer
+            group_sync(group);
+            if (c0 + kEpiCols >= D) {               // this warp's last read of the accumulator
+              tcgen05_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(acc_empty_bar(group));
+            }
+            if (P.transposed) piece_store_transposed(piece, P.act, buf, row);
+            else piece_store(piece, P.act, buf + static_cast<uint32_t>(row) * 64u, static_cast<uint32_t>((row >> 1) & 3));
+            fence_async_smem();
+            group_sync(group);
+            if (issuer) {
+              if (P.transposed) tma_store_2d(&map_y, m * kBlockM, rb * D + c0, buf);
+              else tma_store_2d(&map_y, rb * D + c0, m * kBlockM, buf);
+              tma_store_commit();
+            }
           }
-          const uint4 b0 = bv[c0 / 8], b1 = bv[c0 / 8 + 1];
+        } else {
+          uint32_t v[16];
+          tmem_load_16cols(taddr, v);
+          const uint4 b0 = ld_shared_v4(smem_u32(my_bias)), b1 = ld_shared_v4(smem_u32(my_bias) + 16u);
+          tmem_load_wait();
+          tcgen05_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_empty_bar(group));
           const uint32_t bw[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
           float f[16];
 #pragma unroll
@@ -441,28 +489,28 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
 #pragma unroll
             for (int i = 0; i < 16; i += 2) gelu_erf_pair(f[i], f[i + 1]);
           }
-          if (P.transposed) {
-            // output row n = rb * D + c0 + i holds this thread's token in column t: the 32 lanes of a warp
-            // write 64 contiguous bytes per output row
-            if (t < P.tokens) {
-              uint16_t* col = P.Y + (static_cast<size_t>(rb) * D + c0) * P.ldy + t;
+          const int t = m * kBlockM + row;
+          if (t < P.tokens) {
+            uint32_t w[8];
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const uint32_t w = pack_bf16x2(f[2 * i], f[2 * i + 1]);
-                col[static_cast<size_t>(2 * i) * P.ldy] = static_cast<uint16_t>(w & 0xffffu);
-                col[static_cast<size_t>(2 * i + 1) * P.ldy] = static_cast<uint16_t>(w >> 16);
-              }
+            for (int i = 0; i < 8; ++i) w[i] = pack_bf16x2(f[2 * i], f[2 * i + 1]);
+            if (P.transposed) {
+              // output row n = rb * D + i holds this thread's token in column t: the 32 lanes of a warp write 64
+              // contiguous bytes per output row
+              uint16_t* col = P.Y + static_cast<size_t>(rb) * D * P.ldy + t;
+#pragma unroll
+              for (int i = 0; i < 16; ++i) col[static_cast<size_t>(i) * P.ldy] = static_cast<uint16_t>(i & 1 ? w[i >> 1] >> 16 : w[i >> 1] & 0xffffu);
+            } else {
+              uint4* out = reinterpret_cast<uint4*>(P.Y + static_cast<size_t>(t) * P.ldy + static_cast<size_t>(rb) * D);
+              out[0] = make_uint4(w[0], w[1], w[2], w[3]);
+              out[1] = make_uint4(w[4], w[5], w[6], w[7]);
             }
-          } else if (t < P.tokens) {
-            uint4* out = reinterpret_cast<uint4*>(yrow + static_cast<size_t>(rb) * D + c0);
-            out[0] = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
-            out[1] = make_uint4(pack_bf16x2(f[8], f[9]), pack_bf16x2(f[10], f[11]), pack_bf16x2(f[12], f[13]), pack_bf16x2(f[14], f[15]));
           }
+          group_sync(group);                        // everyone has read the bias
         }
-        acc_phase[acc] ^= 1u;
-        acc ^= 1;
       }
     }
+    if (issuer) tma_store_wait_read<0>();
     if (!ok && lane == 0) record_timeout(P.status, timed_out);
   }
 
@@ -492,10 +540,17 @@ int launch_gather(TcDevice* dev, int slot, const GatherParams& P, cudaStream_t s
   CUtensorMap map_xt;      // XT as [k_in rows, tokens]; box = one row of 64 tokens, 128-byte swizzle, zeros out of range
   // (no L2 promotion: a gathered row is 128 bytes, and fetching 256 would read every line twice)
   if (!make_map(&map_xt, P.XT, P.tokens, P.k_in, P.ldxt, 1, 64, CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) return BSP_ERR_CUDA;
+  CUtensorMap map_y = map_xt;       // (blocks of 16 rows store without it)
+  if (Cfg::kStaged) {
+    if (P.transposed) {
+      if (!make_map(&map_y, P.Y, P.tokens, P.n_out, P.ldy, kEpiCols, kBlockM)) return BSP_ERR_CUDA;
+    } else if (!make_map(&map_y, P.Y, P.n_out, P.tokens, P.ldy, kBlockM, kEpiCols)) {
+      return BSP_ERR_CUDA;
+    }
+  }
   const int units = P.m_tiles * P.n_chunks;
   const int grid = units < dev->sms ? units : dev->sms;
-  linear_gather_kernel<D><<<grid, kGThreads, Cfg::kSmemBytes, s>>>(map_xt, P);
-  BSP_LAUNCH_CHECK();
+  BSP_CUDA_TRY(launch_pdl(linear_gather_kernel<D>, dim3(grid), dim3(kGThreads), Cfg::kSmemBytes, s, map_xt, map_y, P));
   return BSP_OK;
 }
 
@@ -545,9 +600,8 @@ extern "C" int bsp_transpose(const void* X, int rows, int cols, int ldx, void* X
   if (rows == 0) return BSP_OK;
   const dim3 grid((cols + 63) / 64, (rows + 63) / 64);
   if (grid.y > 65535) return BSP_ERR_UNSUPPORTED;
-  transpose_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const uint16_t*>(X), rows, cols, ldx,
-                                                                        static_cast<uint16_t*>(XT), ldxt);
-  BSP_LAUNCH_CHECK();
+  BSP_CUDA_TRY(launch_pdl(transpose_kernel, grid, dim3(256), 0, static_cast<cudaStream_t>(stream), static_cast<const uint16_t*>(X), rows,
+                          cols, ldx, static_cast<uint16_t*>(XT), ldxt));
   return BSP_OK;
 }
 
