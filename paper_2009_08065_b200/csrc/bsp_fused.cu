@@ -5,10 +5,9 @@
 //            squares (the defined decision quantity), then any of: norms / gamma (two 16-byte
 //            stores each), penalty partial, keep flags (one 8-byte store) and the block's count.
 //   stage 2  grid (row-blocks, row ranges of about 16K weights): blk_ptr from the counts before
-//            the block, the ascending index list from the flags, then 4 rows at a time staged in
-//            shared memory (16-byte loads) and from there (a) the zero-expanded execution
-//            layout, (b) the packed tile, written as 16-byte vectors wherever the output is
-//            16-byte aligned.
+//            the block, the ascending index list from the flags, and the rows, staged in shared
+//            memory by asynchronous copies; from there (a) the zero-expanded execution layout,
+//            (b) the packed tile, two values per 4-byte store.
 #include <new>
 
 #include "bsp_common.cuh"
@@ -149,45 +148,78 @@ __global__ void __launch_bounds__(256)
 fused_stage2_kernel(const __grid_constant__ BatchT<N> B) {
   extern __shared__ __align__(16) uint8_t s_raw[];
   __shared__ int s_warp[32];
+  __shared__ int s_part[8];
   __shared__ double s_red[8];
-  __shared__ int s_base;
-  pdl_wait();
-  pdl_launch_dependents();
   const int j = find_job(B, blockIdx.x);
   const FusedJob& J = B.job[j];
   const int b = blockIdx.x - B.first_block[j];
   const int d = B.block;
   const int per_cta = rows_per_cta(J.cols, d);
   const int r_begin = blockIdx.y * per_cta;
+  pdl_wait();
+  pdl_launch_dependents();
   if (r_begin >= d) return;
   const int r_end = min(d, r_begin + per_cta);
-  uint16_t* s_w = reinterpret_cast<uint16_t*>(s_raw);                                    // [rows_per_pass][cols]
-  int32_t* s_idx = reinterpret_cast<int32_t*>(s_raw + static_cast<size_t>(rows_per_pass(J.cols)) * J.cols * 2);  // [cols]
+  const int pass_rows = rows_per_pass(J.cols);
+  uint16_t* s_w = reinterpret_cast<uint16_t*>(s_raw);                                                   // [pass_rows][cols]
+  uint16_t* s_idx = reinterpret_cast<uint16_t*>(s_raw + static_cast<size_t>(pass_rows) * J.cols * 2);  // [cols]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
+  const uint16_t* wblk = J.W + static_cast<size_t>(b) * d * J.ldw;
+  const uint8_t* flags = J.flags + static_cast<size_t>(b) * J.cols;
+  const int chunks = J.cols >> 3;
+
+  // Rows of a pass into shared memory, one warp per row, by asynchronous copies: the first pass's rows, the counts
+  // before the block and the flags are all on their way at once, so the CTA pays one trip to memory before it
+  // writes (it used to be four in a row, 8 us for a 3072 x 768 matrix of 16-row blocks).
+  auto fetch_rows = [&](int r_lo) {
+    const int n_rows = min(pass_rows, r_end - r_lo);
+    for (int rr = warp; rr < n_rows; rr += n_warps) {
+      const uint16_t* src = wblk + static_cast<size_t>(r_lo + rr) * J.ldw;
+      const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(s_w + rr * J.cols));
+      for (int q = lane; q < chunks; q += 32)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + static_cast<uint32_t>(q) * 16u), "l"(src + (q << 3)) : "memory");
+    }
+  };
+  fetch_rows(r_begin);
+  const int q_first = static_cast<int>(threadIdx.x);
+  uint2 f = q_first < chunks ? *reinterpret_cast<const uint2*>(flags + (q_first << 3)) : make_uint2(0u, 0u);
+  const int kc = J.counts[b];
+  int part = 0;                                              // blk_ptr[b] = sum of counts[0..b)
+  for (int i = threadIdx.x; i < b; i += blockDim.x) part += J.counts[i];
 
   // penalty total of the job: its first CTA adds the per-block partials in a fixed order
   if (b == 0 && blockIdx.y == 0 && J.penalty != nullptr && J.partial != nullptr) {
     double p = 0.0;
     for (int i = threadIdx.x; i < J.n_blocks; i += blockDim.x) p += J.partial[i];
     p = warp_sum(p);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = p;
+    if (lane == 0) s_red[warp] = p;
     __syncthreads();
     if (threadIdx.x == 0) {
       double tot = 0.0;
-      for (int w = 0; w < (blockDim.x >> 5); ++w) tot += s_red[w];
+      for (int w = 0; w < n_warps; ++w) tot += s_red[w];
       *J.penalty = tot;
     }
   }
 
-  // blk_ptr[b] = sum of counts[0..b)
-  int part = 0;
-  for (int i = threadIdx.x; i < b; i += blockDim.x) part += J.counts[i];
+  // the sum of the counts and the first round of the list (each thread inspects 8 flags) share one barrier
   part = warp_sum(part);
-  if (threadIdx.x == 0) s_base = 0;
+  int incl = __popc(f.x) + __popc(f.y);
+  const int mine = incl;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  if (lane == 0) s_part[warp] = part;
   __syncthreads();
-  if ((threadIdx.x & 31) == 0 && part) atomicAdd(&s_base, part);
-  __syncthreads();
-  const int base = s_base;
-  const int kc = J.counts[b];
+  int base = 0, running = 0, p0 = incl - mine;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    base += s_part[w];
+    if (w < warp) p0 += s_warp[w];
+    running += s_warp[w];
+  }
   if (blockIdx.y == 0 && threadIdx.x == 0) {
     J.blk_ptr[b] = base;
     if (b == J.n_blocks - 1) {
@@ -195,104 +227,80 @@ fused_stage2_kernel(const __grid_constant__ BatchT<N> B) {
       if (J.kept_weights) *J.kept_weights = static_cast<int64_t>(base + kc) * d;
     }
   }
-
-  const uint16_t* wblk = J.W + static_cast<size_t>(b) * d * J.ldw;
-  const uint8_t* flags = J.flags + static_cast<size_t>(b) * J.cols;
-  const int chunks = J.cols >> 3;
-
-  // ascending list of kept columns: each thread inspects 8 flags per round
-  if (kc > 0) {
-    int running = 0;
-    for (int q0 = 0; q0 < chunks; q0 += blockDim.x) {
-      const int q = q0 + threadIdx.x;
-      uint2 f = make_uint2(0u, 0u);
-      if (q < chunks) f = *reinterpret_cast<const uint2*>(flags + (q << 3));
-      const int mine = __popc(f.x) + __popc(f.y);
-      int total;
-      int p = running + block_exclusive_scan(mine, s_warp, &total);
-      running += total;
+  auto list8 = [&](uint2 fl, int q, int p) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const uint32_t bit = ((i < 4 ? f.x : f.y) >> (8 * (i & 3))) & 1u;
-        if (bit) s_idx[p++] = (q << 3) + i;
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t bit = ((i < 4 ? fl.x : fl.y) >> (8 * (i & 3))) & 1u;
+      if (bit) {
+        s_idx[p] = static_cast<uint16_t>((q << 3) + i);
+        if (blockIdx.y == 0) J.idx[base + p] = (q << 3) + i;
+        ++p;
       }
     }
-    __syncthreads();
-    if (blockIdx.y == 0)
-      for (int p = threadIdx.x; p < kc; p += blockDim.x) J.idx[base + p] = s_idx[p];
+  };
+  list8(f, q_first, p0);
+  for (int q0 = blockDim.x; q0 < chunks; q0 += blockDim.x) {
+    const int q = q0 + threadIdx.x;
+    f = q < chunks ? *reinterpret_cast<const uint2*>(flags + (q << 3)) : make_uint2(0u, 0u);
+    int total;
+    __syncthreads();                                         // s_warp of the round before has been read
+    const int p = running + block_exclusive_scan(__popc(f.x) + __popc(f.y), s_warp, &total);
+    running += total;
+    list8(f, q, p);
   }
-  if (kc == 0 && J.plan == nullptr) return;
+  // (no return before this point: other threads' copies are in flight)
 
-  const bool vec_ok = (reinterpret_cast<uintptr_t>(J.vals) & 15) == 0;
-  const long long tile0 = static_cast<long long>(d) * base;      // element offset of the block's tile in vals
-  const int pass_rows = rows_per_pass(J.cols);
+  const long long tile0 = static_cast<long long>(d) * base;  // element offset of the block's tile in vals
+  const bool pair_ok = (reinterpret_cast<uintptr_t>(J.vals) & 3) == 0;
   for (int r_lo = r_begin; r_lo < r_end; r_lo += pass_rows) {
     const int n_rows = min(pass_rows, r_end - r_lo);
-    // this pass's rows, one warp per row (rows warp, warp + n_warps, ...), lanes along the row:
-    // 16-byte loads kept in shared memory; the execution layout is the same data with the pruned
-    // columns zeroed.  No index arithmetic beyond adds, so the loop stays load-bound.
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
-    for (int rr = warp; rr < n_rows; rr += n_warps) {
-      const uint16_t* src = wblk + static_cast<size_t>(r_lo + rr) * J.ldw;
-      uint16_t* dst = s_w + rr * J.cols;
-      // (a plan that IS W: in-place mode, only pieces that change are written)
-      const bool in_place = J.plan == J.W;
-      uint16_t* pdst = J.plan ? J.plan + (static_cast<size_t>(b) * d + r_lo + rr) * (in_place ? J.ldw : J.cols) : nullptr;
-      for (int q0 = lane; q0 < chunks; q0 += 128) {
-        uint4 w[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (q0 + 32 * u < chunks) w[u] = __ldg(reinterpret_cast<const uint4*>(src + ((q0 + 32 * u) << 3)));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q = q0 + 32 * u;
-          if (q >= chunks) break;
-          *reinterpret_cast<uint4*>(dst + (q << 3)) = w[u];
-          if (pdst != nullptr) {
-            const uint2 f = *reinterpret_cast<const uint2*>(flags + (q << 3));
-            uint4 m;   // a flag byte is 0 or 1: flag * 0xffff masks the matching 16-bit element
-            m.x = w[u].x & (((f.x & 0xffu) * 0xffffu) | (((f.x >> 8) & 0xffu) * 0xffff0000u));
-            m.y = w[u].y & ((((f.x >> 16) & 0xffu) * 0xffffu) | (((f.x >> 24) & 0xffu) * 0xffff0000u));
-            m.z = w[u].z & (((f.y & 0xffu) * 0xffffu) | (((f.y >> 8) & 0xffu) * 0xffff0000u));
-            m.w = w[u].w & ((((f.y >> 16) & 0xffu) * 0xffffu) | (((f.y >> 24) & 0xffu) * 0xffff0000u));
-            if (!in_place || ((m.x ^ w[u].x) | (m.y ^ w[u].y) | (m.z ^ w[u].z) | (m.w ^ w[u].w)) != 0u)
-              *reinterpret_cast<uint4*>(pdst + (q << 3)) = m;
-          }
-        }
-      }
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();   // s_w (and, on the first pass, s_idx) complete
-    // packed tile rows of this pass, again one warp per row: row r occupies
-    // vals[tile0 + r*kc, tile0 + (r+1)*kc); whole 16-byte vectors in the middle, ragged ends by element
-    if (kc > 0) {
+    // execution layout: the rows with the pruned columns zeroed
+    // (a plan that IS W: in-place mode, only pieces that change are written)
+    if (J.plan != nullptr) {
+      const bool in_place = J.plan == J.W;
       for (int rr = warp; rr < n_rows; rr += n_warps) {
-        const uint16_t* srow = s_w + rr * J.cols;
-        const long long e0 = tile0 + static_cast<long long>(r_lo + rr) * kc;
-        uint16_t* out_row = J.vals + e0;                               // element p of the row goes to out_row[p]
-        if (vec_ok) {
-          const int head = static_cast<int>((8 - (e0 & 7)) & 7);       // elements before the first aligned vector
-          const int n_vec = kc > head ? (kc - head) >> 3 : 0;
-          for (int v = lane; v < n_vec; v += 32) {
-            const int p = head + (v << 3);
-            uint32_t o[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              o[i] = static_cast<uint32_t>(srow[s_idx[p + 2 * i]]) | (static_cast<uint32_t>(srow[s_idx[p + 2 * i + 1]]) << 16);
-            *reinterpret_cast<uint4*>(out_row + p) = make_uint4(o[0], o[1], o[2], o[3]);
-          }
-          const int tail0 = head + (n_vec << 3);
-          if (lane < 8) {
-            if (lane < head && lane < kc) out_row[lane] = srow[s_idx[lane]];
-          } else if (lane < 16) {
-            const int p = tail0 + (lane - 8);
-            if (p >= head && p < kc) out_row[p] = srow[s_idx[p]];
-          }
-        } else {
-          for (int p = lane; p < kc; p += 32) out_row[p] = srow[s_idx[p]];
+        uint16_t* pdst = J.plan + (static_cast<size_t>(b) * d + r_lo + rr) * (in_place ? J.ldw : J.cols);
+        for (int q = lane; q < chunks; q += 32) {
+          const uint4 w = *reinterpret_cast<const uint4*>(s_w + rr * J.cols + (q << 3));
+          const uint2 fl = *reinterpret_cast<const uint2*>(flags + (q << 3));
+          uint4 m;   // a flag byte is 0 or 1: flag * 0xffff masks the matching 16-bit element
+          m.x = w.x & (((fl.x & 0xffu) * 0xffffu) | (((fl.x >> 8) & 0xffu) * 0xffff0000u));
+          m.y = w.y & ((((fl.x >> 16) & 0xffu) * 0xffffu) | (((fl.x >> 24) & 0xffu) * 0xffff0000u));
+          m.z = w.z & (((fl.y & 0xffu) * 0xffffu) | (((fl.y >> 8) & 0xffu) * 0xffff0000u));
+          m.w = w.w & ((((fl.y >> 16) & 0xffu) * 0xffffu) | (((fl.y >> 24) & 0xffu) * 0xffff0000u));
+          if (!in_place || ((m.x ^ w.x) | (m.y ^ w.y) | (m.z ^ w.z) | (m.w ^ w.w)) != 0u)
+            *reinterpret_cast<uint4*>(pdst + (q << 3)) = m;
         }
       }
     }
-    __syncthreads();   // s_w is overwritten by the next pass
+    // packed tile rows of this pass, one warp per row: row r occupies vals[tile0 + r*kc, tile0 + (r+1)*kc).  A lane
+    // takes two neighbouring positions (two values a few columns apart: different banks from lane to lane) and
+    // stores them as one word; a row that starts at an odd element has its first one stored alone.
+    for (int rr = warp; rr < n_rows; rr += n_warps) {
+      const uint16_t* srow = s_w + rr * J.cols;
+      const long long e0 = tile0 + static_cast<long long>(r_lo + rr) * kc;
+      uint16_t* out_row = J.vals + e0;                               // element p of the row goes to out_row[p]
+      if (pair_ok) {
+        const int head = static_cast<int>(e0 & 1);
+        const int n_pairs = kc > head ? (kc - head) >> 1 : 0;
+        uint32_t* out32 = reinterpret_cast<uint32_t*>(out_row + head);
+#pragma unroll 4
+        for (int p = lane; p < n_pairs; p += 32) {
+          const int at = head + 2 * p;
+          out32[p] = static_cast<uint32_t>(srow[s_idx[at]]) | (static_cast<uint32_t>(srow[s_idx[at + 1]]) << 16);
+        }
+        if (lane == 0 && head && kc > 0) out_row[0] = srow[s_idx[0]];
+        if (lane == 1 && head + 2 * n_pairs < kc) out_row[kc - 1] = srow[s_idx[kc - 1]];
+      } else {
+        for (int p = lane; p < kc; p += 32) out_row[p] = srow[s_idx[p]];
+      }
+    }
+    if (r_lo + pass_rows < r_end) {
+      __syncthreads();   // s_w is overwritten by the next pass
+      fetch_rows(r_lo + pass_rows);
+    }
   }
 }
 
