@@ -45,7 +45,8 @@ namespace {
 // [0]: 0, or BSP_ERR_TIMEOUT once a bounded wait expired; [1]: a counter nothing ever bumps (self-test);
 // [2..3]: the limit of one wait in nanoseconds; [4]: waits that ran out in the last self-test;
 // [6..7]: how long its mbarrier wait lasted, nanoseconds
-__device__ __align__(16) int g_linear_status[8];
+__device__ __align__(16) int g_linear_status[8] = {0, 0, static_cast<int>(kDefaultWaitLimitNs & 0xffffffffull),
+                                                   static_cast<int>(kDefaultWaitLimitNs >> 32), 0, 0, 0, 0};
 
 
 struct LinearParams {
@@ -331,39 +332,63 @@ __global__ void __launch_bounds__(128, 1) wait_selftest_kernel(int* status) {
 }
 
 // Plan: put the packed tiles of one row-block back at their natural column positions, zero
-// elsewhere.  grid = (row-blocks, row splits); one thread produces 8 adjacent columns of a row
-// (one 16-byte store), looking the columns up in a shared column -> kept-position table.
+// elsewhere.  grid = (row-blocks, row ranges); a CTA brings its rows' packed values (one contiguous run) and the
+// index list into shared memory together, makes a column -> kept-position table, and each thread produces 8
+// adjacent columns of a row (one 16-byte store).  Latency-bound: block pointers, then values and list, then stores.
+// Looking the values up in global memory instead, eight dependent 2-byte loads per store, took 4.2 us for a
+// 3072 x 768 matrix of 16-row blocks.
+constexpr int kPlanSmem = 48 * 1024;
+__host__ __device__ inline int plan_rows_per_cta(int k_in) {
+  const int r = kPlanSmem / (2 * k_in) - 1;     // rows of at most k_in values, and the table
+  return r > 4 ? 4 : r < 1 ? 1 : r;
+}
 __global__ void __launch_bounds__(256)
 plan_expand_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restrict__ idx,
                    const uint16_t* __restrict__ vals, int k_in, int block, uint16_t* __restrict__ Wx) {
-  extern __shared__ int16_t s_pos[];      // column -> position in the kept list, or -1 (k_in < 32768)
+  extern __shared__ __align__(16) int16_t s_pos[];   // [k_in] column -> position in the kept list, or -1 (k_in < 32768)
   const int b = blockIdx.x;
-  for (int k = threadIdx.x; k < k_in; k += blockDim.x) s_pos[k] = -1;
+  const int rows_per = plan_rows_per_cta(k_in);
+  const int r_lo = blockIdx.y * rows_per, n_rows = min(rows_per, block - r_lo);
+  uint16_t* s_val = reinterpret_cast<uint16_t*>(s_pos + k_in);   // [n_rows][kc]
+  const int chunks = k_in >> 3;
+  for (int k = threadIdx.x; k < chunks; k += 256) reinterpret_cast<uint4*>(s_pos)[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
   pdl_wait();
   pdl_launch_dependents();
-  const int lo = blk_ptr[b], kc = blk_ptr[b + 1] - lo;
+  const int lo = __ldg(blk_ptr + b), kc = __ldg(blk_ptr + b + 1) - lo;
+  const uint16_t* run = vals + static_cast<size_t>(block) * lo + static_cast<size_t>(r_lo) * kc;
+  int col[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) col[u] = static_cast<int>(threadIdx.x) + u * 256 < kc ? __ldg(idx + lo + threadIdx.x + u * 256) : -1;
+  const int n_val = n_rows * kc;
+  for (int e0 = threadIdx.x; e0 < n_val; e0 += 8 * 256) {
+    uint16_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (e0 + u * 256 < n_val) v[u] = __ldg(run + e0 + u * 256);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (e0 + u * 256 < n_val) s_val[e0 + u * 256] = v[u];
+  }
+  __syncthreads();                                   // the table is cleared
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (col[u] >= 0) s_pos[col[u]] = static_cast<int16_t>(threadIdx.x + u * 256);
+  for (int j = threadIdx.x + 1024; j < kc; j += 256) s_pos[__ldg(idx + lo + j)] = static_cast<int16_t>(j);
   __syncthreads();
-  for (int j = threadIdx.x; j < kc; j += blockDim.x) s_pos[idx[lo + j]] = static_cast<int16_t>(j);
-  __syncthreads();
-  const uint16_t* tile = vals + static_cast<size_t>(block) * lo;
-  const int rows_per = (block + gridDim.y - 1) / gridDim.y;
-  const int r_lo = blockIdx.y * rows_per;
-  const int r_hi = min(block, r_lo + rows_per);
-  const int chunks = k_in >> 3;
-  for (int e = threadIdx.x; e < (r_hi - r_lo) * chunks; e += blockDim.x) {
-    const int r = r_lo + e / chunks, q = e % chunks;
+  for (int e = threadIdx.x; e < n_rows * chunks; e += 256) {
+    const int r = e / chunks, q = e - r * chunks;
     const uint4 pos4 = *reinterpret_cast<const uint4*>(s_pos + (q << 3));
     const uint32_t pw[4] = {pos4.x, pos4.y, pos4.z, pos4.w};
-    const uint16_t* trow = tile + static_cast<size_t>(r) * kc;
+    const uint16_t* row = s_val + r * kc;
     uint32_t out[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int p0 = static_cast<int16_t>(pw[i] & 0xffffu), p1 = static_cast<int16_t>(pw[i] >> 16);
-      const uint32_t v0 = p0 >= 0 ? __ldg(trow + p0) : 0u;
-      const uint32_t v1 = p1 >= 0 ? __ldg(trow + p1) : 0u;
+      const uint32_t v0 = p0 >= 0 ? row[p0] : 0u;
+      const uint32_t v1 = p1 >= 0 ? row[p1] : 0u;
       out[i] = v0 | (v1 << 16);
     }
-    *reinterpret_cast<uint4*>(Wx + (static_cast<size_t>(b) * block + r) * k_in + (q << 3)) =
+    *reinterpret_cast<uint4*>(Wx + (static_cast<size_t>(b) * block + r_lo + r) * k_in + (q << 3)) =
         make_uint4(out[0], out[1], out[2], out[3]);
   }
 }
@@ -576,10 +601,6 @@ TcDevice* tc_device() {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_linear_status) != cudaSuccess) return nullptr;
-    const unsigned long long limit = kDefaultWaitLimitNs;
-    int init[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    memcpy(&init[2], &limit, sizeof(limit));
-    if (cudaMemcpy(p, init, sizeof(init), cudaMemcpyHostToDevice) != cudaSuccess) return nullptr;
     if (!query_split_ctas(d.split_ctas)) return nullptr;
     d.status = static_cast<int*>(p);
     d.sms = sms;
@@ -607,8 +628,10 @@ extern "C" int bsp_linear_plan(const int32_t* blk_ptr, const int32_t* idx, const
   if (plan_bytes < need) return BSP_ERR_WORKSPACE;
   if (k_in > 12288) return BSP_ERR_UNSUPPORTED;
   if (k_in % 8) return BSP_ERR_UNSUPPORTED;
-  const int splits = block >= 4 ? 4 : 1;
-  BSP_CUDA_TRY(launch_pdl(plan_expand_kernel, dim3(n_out / block, splits), dim3(256), sizeof(int16_t) * k_in,
+  const int rows_per = plan_rows_per_cta(k_in);
+  const dim3 grid(n_out / block, (block + rows_per - 1) / rows_per);
+  if (grid.y > 65535) return BSP_ERR_UNSUPPORTED;
+  BSP_CUDA_TRY(launch_pdl(plan_expand_kernel, grid, dim3(256), static_cast<size_t>(k_in) * 2 * (1 + rows_per),
                           static_cast<cudaStream_t>(stream), blk_ptr, idx, static_cast<const uint16_t*>(vals), k_in, block,
                           static_cast<uint16_t*>(plan)));
   return BSP_OK;
