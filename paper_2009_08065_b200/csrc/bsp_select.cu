@@ -1,18 +1,21 @@
 // bsp_percentile_threshold and its batched form: the threshold that a target compression rate implies
 // (Section 3.1's percentile), a radix select on the bit patterns of the groups' float32 sums of squares
 // (monotone, they are not negative).  Three launches for any number of matrices:
-//   clear    the matrix's histogram and counters (in the part of the workspace that holds flags elsewhere);
+//   clear    the matrix's histogram (in the part of the workspace that holds flags elsewhere);
 //   sums     the sum of every group, W read once (HBM-bound: 2 bytes per weight in, 4 per group out, 16-byte
 //            loads wherever the geometry allows), and a histogram of their upper 12 bits: in shared memory
 //            per CTA, then one global addition per bin that was hit (a hundred or so);
-//   select   every CTA looks the answer's bin up in the histogram, lists its keys of that bin (a few per
-//            cent) in the workspace, and the last CTA of a matrix to do so finds the answer among them in two
-//            more digits (10 and 9 bits).
-// Matrices whose flag region is too small for histogram and list are selected by one CTA straight from the
-// sums, and so is what overflows the list (a matrix of equal groups).  Latency bounds all of this: 3 us for
-// the sums of a 3072 x 768 matrix and 5 us for the select, against 197 us for one CTA with four 8-bit digits
-// over all keys and 12 us for a cluster of eight that merged its histograms through distributed shared memory.
-#include "bsp_common.cuh"
+//   select   one thread-block cluster per matrix: every CTA looks the answer's bin up in the histogram and
+//            lists its keys of that bin (a few per cent) in shared memory; CTA 0 gathers the lists through
+//            distributed shared memory and finds the answer among them in two more digits (10 and 9 bits).
+// Matrices whose flag region is too small for the histogram are selected by one CTA straight from the sums, and
+// so is what overflows a list (a matrix of equal groups).  Latency bounds all of this.  Measured on 147456
+// groups: one CTA with four 8-bit digits over all keys 197 us; a cluster that also made the histogram 12 us;
+// many CTAs with their lists in global memory, the last one finishing, 9 us (fences and atomics through L2
+// instead of cluster barriers).
+#include <atomic>
+
+#include "bsp_tc.cuh"
 
 namespace bsp {
 namespace {
@@ -20,26 +23,33 @@ namespace {
 constexpr int kSelThreads = 1024;
 constexpr int kBits1 = 12, kBits2 = 10, kBits3 = 9;          // 31 bits: the sign of a sum of squares is 0
 constexpr int kBins1 = 1 << kBits1, kBins2 = 1 << kBits2, kBins3 = 1 << kBits3;
-constexpr int kHeadWords = kBins1 + 64;                      // histogram, then list length and finished CTAs
+constexpr int kList = 4096, kCandidates = 12288;              // keys on a CTA's list, and that CTA 0 gathers
+constexpr int kSelSmem = (kList + kCandidates) * 4;
+constexpr int kSelMaxCluster = 8;
+// Copies of a histogram: a CTA of the sums adds to one of them (its number modulo the copies).  A sum of squares
+// falls into a hundred bins or so, and 192 CTAs adding to the same words kept the next launch waiting for 1 us.
+constexpr int kReplicas = 4;
 constexpr int kSelectBatch = 96;                             // matrices per launch; the table is a kernel parameter
 constexpr int kSumThreads = 128;
+constexpr int kSumRowBytes = 24 * 1024;                      // rows of one item of the streaming sums kernel
+constexpr int kSumPerSm = 3;                                 // its CTAs per SM: two row buffers and a histogram each
 
 struct SelectJob {
   const uint16_t* W;
   int cols, ldw, n_blocks, vec;
+  int parts, part_cols;      // streaming sums kernel: column ranges of a row-block
   float* S;
   float* out;
   long long n, r;
-  uint32_t* head;            // histogram and counters, or null: one CTA selects straight from the sums
-  uint32_t list_cap;         // keys that fit behind them
-  int chunks;                // CTAs of the select
+  uint32_t* head;            // histograms, or null: one CTA selects straight from the sums
+  int replicas;              // 1 or kReplicas histograms
 };
 template <int N>
 struct SelectBatchT {
   int n_jobs, block;
-  int loads;                 // 16-byte loads per thread and CTA of the select
+  int max_part_cols, total_items;   // streaming sums kernel
+  int* status;
   int first_block[N];        // apart from the wide records: a search stays within a few lines of the constant cache
-  int first_chunk[N];
   SelectJob job[N];
 };
 template <int N>
@@ -57,9 +67,9 @@ __global__ void __launch_bounds__(kSelThreads)
 select_clear_kernel(const __grid_constant__ SelectBatchT<N> B) {
   pdl_wait();
   pdl_launch_dependents();
-  uint32_t* head = B.job[blockIdx.x].head;
-  if (head == nullptr) return;
-  for (int i = threadIdx.x; i < kHeadWords; i += kSelThreads) head[i] = 0u;
+  const SelectJob& J = B.job[blockIdx.x];
+  if (J.head == nullptr) return;
+  for (int i = threadIdx.x; i < J.replicas * (kBins1 / 4); i += kSelThreads) reinterpret_cast<uint4*>(J.head)[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // ------------------------------------------------------------------------------------------ sums
@@ -114,13 +124,120 @@ sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
   }
   if (!count) return;
   __syncthreads();
-  add_bins(hist, J.head);
+  add_bins(hist, J.head + (blockIdx.x % J.replicas) * kBins1);
+}
+
+// The same for batches of many row-blocks: a CTA works through a run of items (a row-block, or a column range of
+// it whose rows fit 24 KB) with the next item's rows on their way into a second buffer (bulk copies, one per row)
+// while the current item is summed, and adds its histogram once per matrix.  One CTA per row-block, as above, loads,
+// sums and leaves, and with 10 CTAs per SM coming and going a third of the time nothing was in flight: 72 matrices
+// of a BERT-base stack (170 MB) 46 us, 3.7 TB/s.
+template <int N>
+__global__ void __launch_bounds__(kSumThreads)
+sums_stream_kernel(const __grid_constant__ SelectBatchT<N> B) {
+  extern __shared__ __align__(128) uint8_t s_raw[];          // [2][block rows][max_part_cols], then the histogram
+  __shared__ __align__(8) uint64_t s_bar[2];
+  const int d = B.block;
+  const uint32_t buf_bytes = static_cast<uint32_t>((d * B.max_part_cols * 2 + 127) / 128 * 128);
+  uint32_t* hist = reinterpret_cast<uint32_t*>(s_raw + 2 * buf_bytes);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    tc::mbar_init(tc::smem_u32(&s_bar[0]), 1);
+    tc::mbar_init(tc::smem_u32(&s_bar[1]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  clear_bins(hist);
+  const long long total = B.total_items;
+  const int i0 = static_cast<int>(total * blockIdx.x / gridDim.x), i1 = static_cast<int>(total * (blockIdx.x + 1) / gridDim.x);
+  // an item: matrix, row-block, first column and columns (first_block counts items here)
+  auto locate = [&](int item, int& jn, int& b, int& c0, int& pc) {
+    while (jn + 1 < B.n_jobs && B.first_block[jn + 1] <= item) ++jn;
+    const SelectJob& J = B.job[jn];
+    const int at = item - B.first_block[jn];
+    b = at / J.parts;
+    c0 = (at - b * J.parts) * J.part_cols;
+    pc = min(J.part_cols, J.cols - c0);
+  };
+  auto fetch = [&](int jn, int b, int c0, int pc, int slot) {   // by warp 0
+    const SelectJob& J = B.job[jn];
+    const uint32_t bar = tc::smem_u32(&s_bar[slot]), dst = tc::smem_u32(s_raw) + static_cast<uint32_t>(slot) * buf_bytes;
+    const uint32_t row_bytes = static_cast<uint32_t>(pc) * 2u;
+    if (lane == 0) tc::mbar_arrive_expect_tx(bar, row_bytes * static_cast<uint32_t>(d));
+    __syncwarp();
+    const uint16_t* src = J.W + static_cast<size_t>(b) * d * J.ldw + c0;
+    for (int r = lane; r < d; r += 32)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   ::"r"(dst + static_cast<uint32_t>(r) * row_bytes),
+                     "l"(reinterpret_cast<uint64_t>(src + static_cast<size_t>(r) * J.ldw)), "r"(row_bytes), "r"(bar)
+                   : "memory");
+  };
+  int jn = owner(B.first_block, B.n_jobs, i0), b, c0, pc;
+  pdl_wait();
+  pdl_launch_dependents();
+  __syncthreads();
+  locate(i0, jn, b, c0, pc);
+  if (warp == 0 && i0 < i1) fetch(jn, b, c0, pc, 0);
+  uint32_t parity[2] = {0u, 0u};
+  for (int item = i0; item < i1; ++item) {
+    const int slot = (item - i0) & 1;
+    int jn2 = jn, b2 = 0, c2 = 0, pc2 = 0;
+    if (item + 1 < i1) {
+      locate(item + 1, jn2, b2, c2, pc2);
+      if (warp == 0) fetch(jn2, b2, c2, pc2, slot ^ 1);       // (its readers are behind the barrier below)
+    }
+    if (!__syncthreads_and(tc::mbar_wait_suspended(tc::smem_u32(&s_bar[slot]), parity[slot], B.status) ? 1 : 0)) {
+      // the rows never arrived: record it, hold the buffers a millisecond for copies still on their way, leave
+      if (threadIdx.x == 0) atomicExch(B.status, BSP_ERR_TIMEOUT);
+      const unsigned long long start = tc::global_timer_ns();
+      while (tc::global_timer_ns() - start < tc::kQuietNs) __nanosleep(2000);
+      return;
+    }
+    parity[slot] ^= 1u;
+    const SelectJob& J = B.job[jn];
+    const uint16_t* s_w = reinterpret_cast<const uint16_t*>(s_raw + static_cast<size_t>(slot) * buf_bytes);
+    const bool count = J.head != nullptr;
+    for (int k = threadIdx.x; k < (pc >> 3); k += kSumThreads) {
+      float acc[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+#pragma unroll 8
+      for (int r = 0; r < d; ++r) {                           // rows in increasing order: the defined decision quantity
+        const uint4 v = *reinterpret_cast<const uint4*>(s_w + r * pc + (k << 3));
+        const uint32_t w32[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float lo = __uint_as_float(w32[i] << 16), hi = __uint_as_float(w32[i] & 0xffff0000u);
+          acc[2 * i] = __fmaf_rn(lo, lo, acc[2 * i]);
+          acc[2 * i + 1] = __fmaf_rn(hi, hi, acc[2 * i + 1]);
+        }
+      }
+      float4* dst = reinterpret_cast<float4*>(J.S + static_cast<size_t>(b) * J.cols + c0 + (k << 3));
+      dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+      if (count) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) count_key(hist, acc[i]);
+      }
+    }
+    __syncthreads();                                          // the buffer and, before a flush, the bins are complete
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (count && (item + 1 == i1 || jn2 != jn)) {
+      add_bins(hist, J.head + (blockIdx.x % J.replicas) * kBins1);
+      if (item + 1 < i1) {
+        __syncthreads();
+        clear_bins(hist);
+        __syncthreads();
+      }
+    }
+    jn = jn2; b = b2; c0 = c2; pc = pc2;
+  }
 }
 
 // Orientation R: one thread per group, neighbouring threads on neighbouring groups of a row.
 __global__ void __launch_bounds__(256)
 sums_r_kernel(const uint16_t* __restrict__ W, int rows, int per_row, int ldw, int block, int vec, float* __restrict__ S,
-              uint32_t* head) {
+              uint32_t* head, int replicas) {
   __shared__ __align__(16) uint32_t hist[kBins1];
   if (head != nullptr) clear_bins(hist);
   pdl_wait();
@@ -136,7 +253,7 @@ sums_r_kernel(const uint16_t* __restrict__ W, int rows, int per_row, int ldw, in
   }
   if (head == nullptr) return;
   __syncthreads();
-  add_bins(hist, head);
+  add_bins(hist, head + (blockIdx.x % replicas) * kBins1);
 }
 
 // ---------------------------------------------------------------------------------------- select
@@ -215,115 +332,169 @@ __device__ __forceinline__ void for_matching(const uint32_t* __restrict__ keys, 
   }
 }
 
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Shared memory of CTA `rank` of the cluster, at the address that p has in this CTA.
+__device__ __forceinline__ uint32_t map_to_cta(const void* p, uint32_t rank) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(tc::smem_u32(p)), "r"(rank));
+  return remote;
+}
+__device__ __forceinline__ uint32_t ld_cluster(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
 template <int N>
 __global__ void __launch_bounds__(kSelThreads)
 select_kernel(const __grid_constant__ SelectBatchT<N> B) {
   __shared__ __align__(16) uint32_t hist[kBins1];
   __shared__ uint32_t s_sum[32];
   __shared__ uint32_t s_pick[2];
-  __shared__ uint32_t s_n, s_base;
+  __shared__ uint32_t s_n;
+  extern __shared__ uint32_t s_list[];                       // [kList], then in CTA 0 [kCandidates]
+  uint32_t* s_cand = s_list + kList;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int jn = owner(B.first_chunk, B.n_jobs, static_cast<int>(blockIdx.x));
-  const SelectJob& J = B.job[jn];
-  const int chunk = static_cast<int>(blockIdx.x) - B.first_chunk[jn];
+  const uint32_t rank = cluster_rank(), n_cta = cluster_size();
+  const SelectJob& J = B.job[blockIdx.x / n_cta];
   const uint32_t* keys = reinterpret_cast<const uint32_t*>(J.S);
   const long long n = J.n;
   if (threadIdx.x == 0) s_n = 0u;
   pdl_wait();
   pdl_launch_dependents();
-  if (J.r <= 0) {
-    if (chunk == 0 && threadIdx.x == 0) *J.out = -1.0f;
+  if (J.r <= 0) {                                            // the same for the whole cluster
+    if (rank == 0 && threadIdx.x == 0) *J.out = -1.0f;
     return;
   }
   Pick p{0u, static_cast<uint32_t>(J.r)};
-  uint32_t prefix;
-  uint32_t found = 0xffffffffu;                              // keys on the list; too many to use it where there is none
+  uint32_t prefix = 0u;
+  uint32_t found = 0xffffffffu;                              // keys on the lists; all ones: read them all
   if (J.head != nullptr) {
-    // this CTA's keys are on their way while the histogram is looked at
-    uint32_t k[16], valid = 0u;
+    // this CTA's first keys are on their way while the histogram is looked at
     const uint4* v4 = reinterpret_cast<const uint4*>(keys);
-    const long long n4 = n >> 2, i0 = static_cast<long long>(chunk) * B.loads * kSelThreads + threadIdx.x;
+    const long long n4 = n >> 2, step = static_cast<long long>(n_cta) * kSelThreads;
+    long long i0 = static_cast<long long>(rank) * kSelThreads;
+    uint32_t k[16], valid = 0u;
+    auto load = [&]() {
+      valid = 0u;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (u < B.loads && i0 + u * kSelThreads < n4) {
-        const uint4 v = __ldcg(v4 + i0 + u * kSelThreads);
-        k[4 * u] = v.x; k[4 * u + 1] = v.y; k[4 * u + 2] = v.z; k[4 * u + 3] = v.w;
-        valid |= 0xfu << (4 * u);
+      for (int u = 0; u < 4; ++u) {
+        if (i0 + u * step + threadIdx.x < n4) {
+          const uint4 v = __ldcg(v4 + i0 + u * step + threadIdx.x);
+          k[4 * u] = v.x; k[4 * u + 1] = v.y; k[4 * u + 2] = v.z; k[4 * u + 3] = v.w;
+          valid |= 0xfu << (4 * u);
+        }
       }
-    }
-    reinterpret_cast<uint4*>(hist)[threadIdx.x] = __ldcg(reinterpret_cast<const uint4*>(J.head) + threadIdx.x);
+    };
+    load();
+    uint4 h[kReplicas];
+#pragma unroll
+    for (int r = 0; r < kReplicas; ++r)
+      h[r] = r < J.replicas ? __ldcg(reinterpret_cast<const uint4*>(J.head + r * kBins1) + threadIdx.x) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int r = 1; r < kReplicas; ++r) { h[0].x += h[r].x; h[0].y += h[r].y; h[0].z += h[r].z; h[0].w += h[r].w; }
+    reinterpret_cast<uint4*>(hist)[threadIdx.x] = h[0];
     static_assert(kBins1 == 4 * kSelThreads, "a 16-byte piece of the histogram per thread");
     __syncthreads();
     p = pick_bin<kBins1>(hist, p.want, s_sum, s_pick);
-    uint32_t hit = 0u;
+    prefix = p.bin;
+    for (;;) {
+      uint32_t hit = 0u;
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if ((valid >> i & 1u) && (k[i] >> (kBits2 + kBits3)) == p.bin) hit |= 1u << i;
-    uint32_t tail = 0u;                                      // the last n mod 4 keys: the last CTA's
-    const bool has_tail = chunk == J.chunks - 1 && threadIdx.x < static_cast<unsigned>(n & 3);
-    if (has_tail) tail = __ldcg(keys + (n4 << 2) + threadIdx.x);
-    const bool hit_tail = has_tail && (tail >> (kBits2 + kBits3)) == p.bin;
-    const uint32_t mine = __popc(hit) + (hit_tail ? 1u : 0u);
-    uint32_t incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += up;
-    }
-    if (lane == 31) s_sum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      const uint32_t w = s_sum[lane];
-      uint32_t in = w;
+      for (int i = 0; i < 16; ++i)
+        if ((valid >> i & 1u) && (k[i] >> (kBits2 + kBits3)) == prefix) hit |= 1u << i;
+      const uint32_t mine = __popc(hit);
+      uint32_t incl = mine;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t up = __shfl_up_sync(0xffffffffu, in, o);
-        if (lane >= o) in += up;
+        const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
       }
-      s_sum[lane] = in - w;
-      if (lane == 31) s_base = in ? atomicAdd(J.head + kBins1, in) : 0u;
-    }
-    __syncthreads();
-    uint32_t at = s_base + s_sum[warp] + incl - mine;
-    uint32_t* list = J.head + kHeadWords;
+      uint32_t at = 0u;
+      if (lane == 31 && incl) at = atomicAdd(&s_n, incl);
+      at = __shfl_sync(0xffffffffu, at, 31) + incl - mine;
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if (hit >> i & 1u) {
-        if (at < J.list_cap) list[at] = k[i];
-        ++at;
-      }
-    if (hit_tail && at < J.list_cap) list[at] = tail;
-    // the last CTA of the matrix goes on (every CTA's part of the list is visible to it)
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      s_n = atomicAdd(J.head + kBins1 + 1, 1u);
-      __threadfence();
+      for (int i = 0; i < 16; ++i)
+        if (hit >> i & 1u) {
+          if (at < kList) s_list[at] = k[i];
+          ++at;
+        }
+      i0 += 4 * step;
+      if (i0 >= n4) break;
+      load();
     }
-    __syncthreads();
-    if (s_n + 1u != static_cast<uint32_t>(J.chunks)) return;
-    found = __ldcg(J.head + kBins1);
-    prefix = p.bin;
+    if (rank == 0 && threadIdx.x < static_cast<unsigned>(n & 3)) {   // the last n mod 4 keys
+      const uint32_t tail = __ldcg(keys + (n4 << 2) + threadIdx.x);
+      if ((tail >> (kBits2 + kBits3)) == prefix) {
+        const uint32_t at = atomicAdd(&s_n, 1u);
+        if (at < kList) s_list[at] = tail;
+      }
+    }
+    cluster_sync();                                          // the lists are complete
+    if (rank == 0) {
+      const uint32_t length = lane < static_cast<int>(n_cta) ? ld_cluster(map_to_cta(&s_n, lane)) : 0u;
+      found = __reduce_add_sync(0xffffffffu, length);
+      if (__any_sync(0xffffffffu, length > kList) || found > kCandidates) {
+        found = 0xffffffffu;
+      } else {
+        // four lists at a time, eight warps each; a list's keys go behind those of the lists before it
+        uint32_t at = 0u;
+        for (uint32_t q = 0; q < n_cta; ++q) {
+          const uint32_t len = __shfl_sync(0xffffffffu, length, static_cast<int>(q));
+          if ((q & 3u) == static_cast<uint32_t>(warp & 3)) {
+            const uint32_t src = map_to_cta(s_list, q);
+            for (uint32_t i = static_cast<uint32_t>((warp >> 2) * 32 + lane); i < len; i += kSelThreads / 4) s_cand[at + i] = ld_cluster(src + 4u * i);
+          }
+          at += len;
+        }
+      }
+    }
   } else {
-    clear_bins(hist);
-    __syncthreads();
-    for_matching(keys, n, 31, 0u, [&](uint32_t k) { atomicAdd(&hist[k >> (kBits2 + kBits3)], 1u); });
-    __syncthreads();
-    p = pick_bin<kBins1>(hist, p.want, s_sum, s_pick);
-    prefix = p.bin;
+    if (rank == 0) {
+      clear_bins(hist);
+      __syncthreads();
+      for_matching(keys, n, 31, 0u, [&](uint32_t k) { atomicAdd(&hist[k >> (kBits2 + kBits3)], 1u); });
+      __syncthreads();
+      p = pick_bin<kBins1>(hist, p.want, s_sum, s_pick);
+      prefix = p.bin;
+    }
+    cluster_sync();
   }
-  const bool listed = J.head != nullptr && found <= J.list_cap;
-  if (listed) keys = J.head + kHeadWords;
-  const long long left = listed ? static_cast<long long>(found) : n;
-  hist[threadIdx.x] = 0u;                                    // two digits more, each with bins of its own
+  if (rank != 0) {
+    cluster_sync();                                          // CTA 0 has read this CTA's list
+    return;
+  }
+  // two digits more, each with bins of its own, over the listed keys or all of them
+  __syncthreads();
+  hist[threadIdx.x] = 0u;
   if (threadIdx.x < kBins3) hist[kBins2 + threadIdx.x] = 0u;
   __syncthreads();
-  for_matching(keys, left, kBits2 + kBits3, prefix, [&](uint32_t k) { atomicAdd(&hist[(k >> kBits3) & (kBins2 - 1)], 1u); });
+  auto over_keys = [&](int above, uint32_t upper, auto f) {
+    if (found != 0xffffffffu) {
+      for (uint32_t i = threadIdx.x; i < found; i += kSelThreads)
+        if ((s_cand[i] >> above) == upper) f(s_cand[i]);
+    } else {
+      for_matching(keys, n, above, upper, f);
+    }
+  };
+  over_keys(kBits2 + kBits3, prefix, [&](uint32_t k) { atomicAdd(&hist[(k >> kBits3) & (kBins2 - 1)], 1u); });
   __syncthreads();
   p = pick_bin<kBins2>(hist, p.want, s_sum, s_pick);
   prefix = (prefix << kBits2) | p.bin;
-  __syncthreads();
-  for_matching(keys, left, kBits3, prefix, [&](uint32_t k) { atomicAdd(&hist[kBins2 + (k & (kBins3 - 1))], 1u); });
+  over_keys(kBits3, prefix, [&](uint32_t k) { atomicAdd(&hist[kBins2 + (k & (kBins3 - 1))], 1u); });
   __syncthreads();
   p = pick_bin<kBins3>(hist + kBins2, p.want, s_sum, s_pick);
   if (threadIdx.x == 0) {
@@ -332,6 +503,7 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
     while (__fmul_rn(t, t) < s_r) t = __uint_as_float(__float_as_uint(t) + 1u);  // next float up (t >= 0)
     *J.out = t;
   }
+  cluster_sync();
 }
 
 // r = floor(G * (1 - 1/c)) in float64, as the definition states it
@@ -354,35 +526,95 @@ SelectJob select_job(const void* W, int cols, int ldw, int n_blocks, int n_group
   J.out = out;
   J.n = groups;
   J.r = groups_to_remove(groups, rate);
-  // the region of the flags: one byte per group.  Below 1024 list entries (20 thousand groups) one CTA reads
-  // all keys three times instead.
-  const size_t words = (L.sumsq_off - L.keep_off) / 4;
-  if (words >= kHeadWords + 1024) {
-    J.head = reinterpret_cast<uint32_t*>(base + L.keep_off);
-    J.list_cap = static_cast<uint32_t>(words - kHeadWords);
-  }
+  // the region of the flags: one byte per group
+  J.replicas = L.sumsq_off - L.keep_off >= kReplicas * kBins1 * sizeof(uint32_t) ? kReplicas : 1;
+  if (L.sumsq_off - L.keep_off >= kBins1 * sizeof(uint32_t)) J.head = reinterpret_cast<uint32_t*>(base + L.keep_off);
   return J;
 }
 
 // The select counts in 32 bits.
 bool too_many_groups(long long groups) { return groups >= (1LL << 32); }
 
+// CTAs per matrix: as many as fit the GPU at once (one per SM: 1024 threads of 48 registers), up to the portable
+// cluster size, but not so many that a CTA has fewer than 2048 keys.
+int select_cluster(int n_jobs, long long largest, int sms) {
+  int c = kSelMaxCluster;
+  while (c > 1 && (static_cast<long long>(n_jobs) * c > sms || largest < 2048LL * c)) c >>= 1;
+  return c;
+}
 template <int N>
-int launch_select(SelectBatchT<N>& B, int sms, cudaStream_t s) {
-  // 4096 keys per CTA and 16-byte load of a thread: as few loads as keep the grid to two CTAs per SM, at most four
-  long long keys = 0;
-  for (int i = 0; i < B.n_jobs; ++i) keys += B.job[i].n;
-  B.loads = 1;
-  while (B.loads < 4 && keys > 2LL * sms * B.loads * 4 * kSelThreads) B.loads *= 2;
-  const long long per_cta = 4LL * kSelThreads * B.loads;
-  int chunks = 0;
+int launch_select(const SelectBatchT<N>& B, int sms, cudaStream_t s) {
+  long long largest = 0;
+  for (int i = 0; i < B.n_jobs; ++i)
+    if (B.job[i].n > largest) largest = B.job[i].n;
+  const int c = select_cluster(B.n_jobs, largest, sms);
+  static std::atomic<bool> attr_set[64];            // per device; setting the attribute twice does no harm
+  int device = 0;
+  BSP_CUDA_TRY(cudaGetDevice(&device));
+  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
+  if (!attr_set[device].load(std::memory_order_acquire)) {
+    BSP_CUDA_TRY(cudaFuncSetAttribute(select_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmem));
+    attr_set[device].store(true, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(B.n_jobs * c));
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.dynamicSmemBytes = kSelSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = c;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  BSP_CUDA_TRY(cudaLaunchKernelEx(&cfg, select_kernel<N>, B));
+  return BSP_OK;
+}
+
+// Sums of a batch in orientation C: streaming where there are several items for every CTA and every matrix can be
+// copied in 16-byte pieces, one CTA per row-block otherwise (its single trip to memory is what a small batch needs).
+template <int N>
+int launch_sums_c(SelectBatchT<N>& B, int sms, cudaStream_t s) {
+  const int max_cols = kSumRowBytes / (2 * B.block) / 8 * 8;
+  bool stream = max_cols >= 8;
+  int blocks = 0, items = 0;
+  B.max_part_cols = 0;
   for (int i = 0; i < B.n_jobs; ++i) {
     SelectJob& J = B.job[i];
-    J.chunks = J.head == nullptr ? 1 : static_cast<int>((J.n + per_cta - 1) / per_cta);
-    B.first_chunk[i] = chunks;
-    chunks += J.chunks;
+    stream = stream && J.vec;
+    blocks += J.n_blocks;
+    if (!stream) continue;
+    J.parts = (J.cols + max_cols - 1) / max_cols;
+    J.part_cols = ((J.cols + J.parts - 1) / J.parts + 7) / 8 * 8;
+    J.parts = (J.cols + J.part_cols - 1) / J.part_cols;
+    items += J.n_blocks * J.parts;
+    if (J.part_cols > B.max_part_cols) B.max_part_cols = J.part_cols;
   }
-  BSP_CUDA_TRY(launch_pdl(select_kernel<N>, dim3(chunks), dim3(kSelThreads), 0, s, B));
+  if (stream && items >= 2 * kSumPerSm * sms) {
+    TcDevice* dev = tc_device();
+    if (dev == nullptr) return BSP_ERR_CUDA;
+    B.status = dev->status;
+    B.total_items = items;
+    int at = 0;
+    for (int i = 0; i < B.n_jobs; ++i) { B.first_block[i] = at; at += B.job[i].n_blocks * B.job[i].parts; }
+    const size_t smem = 2 * round_up(static_cast<size_t>(B.block) * B.max_part_cols * 2, 128) + kBins1 * 4;
+    static std::atomic<bool> attr_set[64];
+    int device = 0;
+    BSP_CUDA_TRY(cudaGetDevice(&device));
+    if (device < 0 || device >= 64) return BSP_ERR_CUDA;
+    if (!attr_set[device].load(std::memory_order_acquire)) {
+      BSP_CUDA_TRY(cudaFuncSetAttribute(sums_stream_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSumRowBytes + 256 + kBins1 * 4));
+      attr_set[device].store(true, std::memory_order_release);
+    }
+    BSP_CUDA_TRY(launch_pdl(sums_stream_kernel<N>, dim3(kSumPerSm * sms), dim3(kSumThreads), smem, s, B));
+    return BSP_OK;
+  }
+  int at = 0;
+  for (int i = 0; i < B.n_jobs; ++i) { B.first_block[i] = at; at += B.job[i].n_blocks; }
+  BSP_CUDA_TRY(launch_pdl(sums_c_kernel<N>, dim3(blocks), dim3(kSumThreads), 0, s, B));
   return BSP_OK;
 }
 
@@ -417,14 +649,15 @@ extern "C" int bsp_percentile_threshold(const void* W, int rows, int cols, int l
   SelectBatchT<1> B;
   B.n_jobs = 1;
   B.block = block;
-  B.first_block[0] = 0;
   B.job[0] = select_job(W, cols, ldw, nb, ng, rate, ws, threshold_out);
   if (B.job[0].head != nullptr) BSP_CUDA_TRY(launch_pdl(select_clear_kernel<1>, dim3(1), dim3(kSelThreads), 0, s, B));
   if (orient == BSP_ORIENT_C) {
-    BSP_CUDA_TRY(launch_pdl(sums_c_kernel<1>, dim3(nb), dim3(kSumThreads), 0, s, B));
+    st = launch_sums_c(B, sms, s);
+    if (st != BSP_OK) return st;
   } else {
     BSP_CUDA_TRY(launch_pdl(sums_r_kernel, dim3(static_cast<unsigned>((groups + 255) / 256)), dim3(256), 0, s, B.job[0].W, rows, nb,
-                            ldw, block, contig_vec(W, ldw, block), B.job[0].S, B.job[0].head));
+                            ldw, block, contig_vec(W, ldw, block), B.job[0].S, B.job[0].head,
+                            B.job[0].replicas));
   }
   return launch_select(B, sms, s);
 }
@@ -451,15 +684,13 @@ extern "C" int bsp_percentile_threshold_batched(const bsp_layer_job* jobs, int n
   for (int j0 = 0; j0 < n_jobs; j0 += kSelectBatch) {
     B.n_jobs = n_jobs - j0 < kSelectBatch ? n_jobs - j0 : kSelectBatch;
     B.block = block;
-    int blocks = 0;
     for (int i = 0; i < B.n_jobs; ++i) {
       const bsp_layer_job& u = jobs[j0 + i];
       B.job[i] = select_job(u.W, u.cols, u.ldw, u.rows / block, u.cols, rates[j0 + i], u.ws, const_cast<float*>(u.threshold_dev));
-      B.first_block[i] = blocks;
-      blocks += B.job[i].n_blocks;
     }
     BSP_CUDA_TRY(launch_pdl(select_clear_kernel<kSelectBatch>, dim3(B.n_jobs), dim3(kSelThreads), 0, s, B));
-    BSP_CUDA_TRY(launch_pdl(sums_c_kernel<kSelectBatch>, dim3(blocks), dim3(kSumThreads), 0, s, B));
+    st = launch_sums_c(B, sms, s);
+    if (st != BSP_OK) return st;
     st = launch_select(B, sms, s);
     if (st != BSP_OK) return st;
   }
