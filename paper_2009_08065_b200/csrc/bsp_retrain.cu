@@ -31,23 +31,8 @@ struct AdamArgs {
   int ldb;
 };
 
-__global__ void __launch_bounds__(256)
-masked_adam_kernel(AdamArgs A) {
-  pdl_wait();
-  pdl_launch_dependents();
-  // (32-bit division where the item number allows it: a 64-bit one is a third of the kernel's instructions)
-  const unsigned quads = static_cast<unsigned>(A.cols) >> 2;
-  const long long item = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (item >= static_cast<long long>(A.rows) * quads) return;
-  int r, c;
-  if (item <= 0xffffffffLL) {
-    const unsigned it = static_cast<unsigned>(item);
-    r = static_cast<int>(it / quads);
-    c = static_cast<int>(it - static_cast<unsigned>(r) * quads) << 2;
-  } else {
-    r = static_cast<int>(item / quads);
-    c = static_cast<int>(item - static_cast<long long>(r) * quads) << 2;
-  }
+// One 4-weight item; `keep` decides per weight.
+__device__ __forceinline__ void adam_item(const AdamArgs& A, int r, int c) {
   const size_t iw = static_cast<size_t>(r) * A.ldw + c, ig = static_cast<size_t>(r) * A.ldg + c;
   const float4 w4 = *reinterpret_cast<const float4*>(A.W + iw);
   const float4 g4 = __ldg(reinterpret_cast<const float4*>(A.G + ig));
@@ -94,12 +79,26 @@ masked_adam_kernel(AdamArgs A) {
   }
 }
 
+// One item per thread.  (A single wave of CTAs that loop over the items was 8 % slower; 32-bit item numbers where
+// they suffice: the 64-bit division to row and column is a third of the kernel's instructions.)
+template <typename Index>
+__global__ void __launch_bounds__(256)
+masked_adam_kernel(AdamArgs A) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const Index quads = static_cast<Index>(A.cols >> 2);
+  const Index item = static_cast<Index>(blockIdx.x) * 256u + threadIdx.x;
+  if (item >= static_cast<Index>(A.rows) * quads) return;
+  const Index r = item / quads;
+  adam_item(A, static_cast<int>(r), static_cast<int>(item - r * quads) << 2);
+}
+
 // Rows of one row-block: tile[r][p] = W[b*d + r][idx[lo + p]].  The vectorised form stages kRepackRows rows and
 // the block's index list (2 bytes per entry) in shared memory, 16 bytes per load with all of a thread's loads
 // in flight (at the usual rates every 32-byte sector of a row holds a kept column, so whole rows are read
 // anyway), and gathers from there, two positions per 4-byte store.  HBM-bound in total, latency-bound per
 // matrix: four rows per CTA give a 768 x 768 matrix 192 CTAs.  12 layers of four matrices: 5.3 -> 2.4 us each.
-constexpr int kRepackRows = 4, kRepackThreads = 128;
+constexpr int kRepackRows = 4, kRepackThreads = 256, kRepackLoads = 6;
 __global__ void __launch_bounds__(kRepackThreads)
 repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, const int32_t* __restrict__ blk_ptr,
                   const int32_t* __restrict__ idx, uint16_t* __restrict__ vals) {
@@ -112,15 +111,15 @@ repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, 
   const int lo = __ldg(blk_ptr + b), kc = __ldg(blk_ptr + b + 1) - lo;
   const uint16_t* src = W + (static_cast<size_t>(b) * block + r_lo) * ldw;
   const int total = n_rows * chunks;
-  for (int e0 = threadIdx.x; e0 < total; e0 += 4 * kRepackThreads) {
-    uint4 v[4];
+  for (int e0 = threadIdx.x; e0 < total; e0 += kRepackLoads * kRepackThreads) {
+    uint4 v[kRepackLoads];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kRepackLoads; ++u) {
       const int e = e0 + u * kRepackThreads, r = e / chunks;
       if (e < total) v[u] = __ldg(reinterpret_cast<const uint4*>(src + static_cast<size_t>(r) * ldw + ((e - r * chunks) << 3)));
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kRepackLoads; ++u) {
       const int e = e0 + u * kRepackThreads;
       if (e < total) reinterpret_cast<uint4*>(s_rows)[e] = v[u];   // rows are packed: chunk e of the pass
     }
@@ -222,7 +221,10 @@ extern "C" int bsp_masked_adam_step(float* W, const float* grad, float* m, float
   const long long items = static_cast<long long>(rows) * (cols >> 2);
   const long long blocks = (items + 255) / 256;
   if (blocks > 0x7fffffffLL) return BSP_ERR_UNSUPPORTED;
-  BSP_CUDA_TRY(launch_pdl(masked_adam_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, static_cast<cudaStream_t>(stream), A));
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const dim3 grid(static_cast<unsigned>(blocks));
+  if (blocks * 256 < (1LL << 32)) BSP_CUDA_TRY(launch_pdl(masked_adam_kernel<unsigned>, grid, dim3(256), 0, s, A));
+  else BSP_CUDA_TRY(launch_pdl(masked_adam_kernel<unsigned long long>, grid, dim3(256), 0, s, A));
   return BSP_OK;
 }
 
