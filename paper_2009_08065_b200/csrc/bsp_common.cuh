@@ -142,6 +142,17 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // After pdl_wait: a dependent that has started knows that everything before this grid is complete.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Fetches into L2 of what a CTA will read once pdl_wait returns.  They change nothing but what L2 holds, which is
+// coherent, so they may go out before the wait, while the previous kernel of the stream is still running: short
+// kernels (a 768 x 768 matrix re-packed in 3 us) leave HBM idle meanwhile, and the next kernel's first wave of CTAs
+// then finds its operands in L2.  Retraining 12 BERT-base layers (48 x Adam step, re-pack): 621 -> 608 us; an iteration
+// of reweighted training on a 1024-wide layer: 113 -> 107 us.
+__device__ __forceinline__ void prefetch_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// `bytes` a multiple of 16, p 16-byte aligned.
+__device__ __forceinline__ void prefetch_bytes(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
   return __uint_as_float(static_cast<uint32_t>(b) << 16);
 }

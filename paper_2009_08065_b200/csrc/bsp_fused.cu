@@ -43,11 +43,11 @@ __global__ void __launch_bounds__(256)
 fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
   __shared__ int s_cnt[8];
   __shared__ double s_pen[8];
-  pdl_wait();
-  pdl_launch_dependents();
   const int j = find_job(B, blockIdx.x);
   const FusedJob& J = B.job[j];
   const int b = blockIdx.x - B.first_block[j];
+  pdl_wait();
+  pdl_launch_dependents();
   const bool want_flags = J.flags != nullptr;
   const bool want_pen = J.penalty != nullptr;
   const bool want_norms = J.norms != nullptr || J.gamma_out != nullptr || want_pen;

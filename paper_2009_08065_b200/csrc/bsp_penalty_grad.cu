@@ -25,18 +25,30 @@ struct GradArgs {
 // accumulating) per weight.  One thread per 8 columns walking down the rows, as the kernel below does, has
 // 1/16 of the loads in flight: 14 us instead of 6 for a 4096 x 1024 matrix of 16-row blocks, accumulating.
 constexpr int kGradCols = 256, kGradMaxRows = 32;
+constexpr unsigned kGradFirstWave = 4 * 148;
 template <int ITEMS>
 __global__ void __launch_bounds__(256)
 grad_c_tile_kernel(GradArgs A) {
   __shared__ __align__(16) uint16_t s_w[8 * ITEMS][kGradCols];
   __shared__ __align__(16) float s_f[kGradCols];
-  pdl_wait();
-  pdl_launch_dependents();
   const int b = blockIdx.x, c0 = blockIdx.y * kGradCols;
   const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;     // a warp per row, 8 columns per lane
   const int c = c0 + (lane << 3);
   const bool on = c < A.cols;
   const size_t r0 = static_cast<size_t>(b) * A.block;
+  // (only the CTAs that can be waiting: behind them it would cost issue slots for nothing)
+  const bool early = blockIdx.y * gridDim.x + blockIdx.x < kGradFirstWave;
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    const int r = row + 8 * i;
+    if (early && on && r < A.block) {
+      if ((lane & 7) == 0) prefetch_line(A.W + (r0 + r) * A.ldw + c);
+      if (A.accumulate && (lane & 3) == 0) prefetch_line(A.grad + (r0 + r) * A.ldg + c);
+    }
+  }
+  if (early && on && row == 0 && (lane & 3) == 0) prefetch_line(A.gamma + static_cast<size_t>(b) * A.cols + c);
+  pdl_wait();
+  pdl_launch_dependents();
   uint4 w[ITEMS];
   float4 g[ITEMS][2];
 #pragma unroll

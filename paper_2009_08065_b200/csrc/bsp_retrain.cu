@@ -29,6 +29,7 @@ struct AdamArgs {
   float inv_c1, inv_c2;      // 1 / (1 - beta^step)
   uint16_t* Wb;              // bf16 copy, or null
   int ldb;
+  unsigned first_wave;       // CTAs that are resident at once
 };
 
 // One 4-weight item; `keep` decides per weight.
@@ -84,10 +85,27 @@ __device__ __forceinline__ void adam_item(const AdamArgs& A, int r, int c) {
 template <typename Index>
 __global__ void __launch_bounds__(256)
 masked_adam_kernel(AdamArgs A) {
-  pdl_wait();
-  pdl_launch_dependents();
   const Index quads = static_cast<Index>(A.cols >> 2);
   const Index item = static_cast<Index>(blockIdx.x) * 256u + threadIdx.x;
+  // the CTAs that can be waiting for the previous kernel: their own lines (eight items each) and those of the CTAs
+  // that will take their places
+  if (blockIdx.x < A.first_wave && (threadIdx.x & 7) == 0) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const Index it = item + static_cast<Index>(u) * A.first_wave * 256u;
+      if (it < static_cast<Index>(A.rows) * quads) {
+        const Index r = it / quads;
+        const size_t c = static_cast<size_t>(it - r * quads) << 2;
+        const size_t iw = static_cast<size_t>(r) * A.ldw + c;
+        prefetch_line(A.W + iw);
+        prefetch_line(A.G + static_cast<size_t>(r) * A.ldg + c);
+        prefetch_line(A.M + iw);
+        prefetch_line(A.V + iw);
+      }
+    }
+  }
+  pdl_wait();
+  pdl_launch_dependents();
   if (item >= static_cast<Index>(A.rows) * quads) return;
   const Index r = item / quads;
   adam_item(A, static_cast<int>(r), static_cast<int>(item - r * quads) << 2);
@@ -97,7 +115,8 @@ masked_adam_kernel(AdamArgs A) {
 // the block's index list (2 bytes per entry) in shared memory, 16 bytes per load with all of a thread's loads
 // in flight (at the usual rates every 32-byte sector of a row holds a kept column, so whole rows are read
 // anyway), and gathers from there, two positions per 4-byte store.  HBM-bound in total, latency-bound per
-// matrix: four rows per CTA give a 768 x 768 matrix 192 CTAs.  12 layers of four matrices: 5.3 -> 2.4 us each.
+// matrix: four rows per CTA give a 768 x 768 matrix 192 CTAs, and the list travels beside the rows.  12 layers of four
+// matrices, on average: 5.3 us gathering from global memory, 2.9 us.
 constexpr int kRepackRows = 4, kRepackThreads = 256, kRepackLoads = 6;
 __global__ void __launch_bounds__(kRepackThreads)
 repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, const int32_t* __restrict__ blk_ptr,
@@ -106,9 +125,18 @@ repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, 
   const int b = blockIdx.x, r_lo = blockIdx.y * kRepackRows, n_rows = min(kRepackRows, block - r_lo);
   const int chunks = cols >> 3;
   uint16_t* s_list = s_rows + kRepackRows * cols;
+  if (threadIdx.x == 0) prefetch_line(blk_ptr + b);
+  if (static_cast<int>(threadIdx.x) < n_rows)
+    prefetch_bytes(W + (static_cast<size_t>(b) * block + r_lo + threadIdx.x) * ldw, static_cast<uint32_t>(cols) * 2u);
   pdl_wait();
   pdl_launch_dependents();
   const int lo = __ldg(blk_ptr + b), kc = __ldg(blk_ptr + b + 1) - lo;
+  int col[4];                                                    // the first of the list, in flight beside the rows
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int p = static_cast<int>(threadIdx.x) + u * kRepackThreads;
+    if (p < kc) col[u] = __ldg(idx + lo + p);
+  }
   const uint16_t* src = W + (static_cast<size_t>(b) * block + r_lo) * ldw;
   const int total = n_rows * chunks;
   for (int e0 = threadIdx.x; e0 < total; e0 += kRepackLoads * kRepackThreads) {
@@ -124,7 +152,12 @@ repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, 
       if (e < total) reinterpret_cast<uint4*>(s_rows)[e] = v[u];   // rows are packed: chunk e of the pass
     }
   }
-  for (int p = threadIdx.x; p < kc; p += kRepackThreads) s_list[p] = static_cast<uint16_t>(__ldg(idx + lo + p));
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int p = static_cast<int>(threadIdx.x) + u * kRepackThreads;
+    if (p < kc) s_list[p] = static_cast<uint16_t>(col[u]);
+  }
+  for (int p = threadIdx.x + 4 * kRepackThreads; p < kc; p += kRepackThreads) s_list[p] = static_cast<uint16_t>(__ldg(idx + lo + p));
   __syncthreads();
   uint16_t* tile = vals + static_cast<size_t>(block) * lo + static_cast<size_t>(r_lo) * kc;
   if ((reinterpret_cast<uintptr_t>(tile) & 3) == 0 && (kc & 1) == 0) {
@@ -223,6 +256,10 @@ extern "C" int bsp_masked_adam_step(float* W, const float* grad, float* m, float
   if (blocks > 0x7fffffffLL) return BSP_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const dim3 grid(static_cast<unsigned>(blocks));
+  int dev = 0, sms = 0;
+  BSP_CUDA_TRY(cudaGetDevice(&dev));
+  BSP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  A.first_wave = 5u * static_cast<unsigned>(sms);        // 48 registers x 256 threads: five CTAs per SM
   if (blocks * 256 < (1LL << 32)) BSP_CUDA_TRY(launch_pdl(masked_adam_kernel<unsigned>, grid, dim3(256), 0, s, A));
   else BSP_CUDA_TRY(launch_pdl(masked_adam_kernel<unsigned long long>, grid, dim3(256), 0, s, A));
   return BSP_OK;
