@@ -80,12 +80,6 @@ __device__ __forceinline__ void tmem_load_cols(uint32_t taddr, uint32_t (&v)[N])
                  : "memory");
   }
 }
-// The registers of a TMEM load pass through an empty statement behind the wait, so that no use of them moves above it.
-template <int N>
-__device__ __forceinline__ void tmem_loaded(uint32_t (&v)[N]) {
-#pragma unroll
-  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(v[i]));
-}
 // MN-major operand tile with the 128-byte swizzle: 8-row atoms 1024 bytes apart along the contraction,
 // 64-element groups 8 KB apart along M / N.
 __device__ __forceinline__ uint64_t split_desc_mn(uint32_t smem_addr) {
@@ -267,7 +261,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   if (mine && ok) {
     const uint32_t out_base = smem_base + (C - 1) * kSlot + static_cast<uint32_t>(group) * 2u * kEpiStage;
 #pragma unroll 1
-    for (int p = 0; p < UW / PC; ++p) {
+    for (int p = 0; p < UW / PC && n_own + p * PC < P.cols; ++p) {
       const int c0 = group * UW + p * PC;
       uint32_t own[PC];
       tmem_load_cols<PC>(taddr + rank * W + c0, own);
@@ -335,11 +329,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                        o[4 * j + 2], o[4 * j + 3]);
         fence_async_smem();
         group_sync(group);
-        if (issuer) {
-          const int n = n0 + static_cast<int>(rank) * W + c0;
-          if (n < P.cols) tma_store_2d(&map_y, n, m0, buf);
-          tma_store_commit();
-        }
+        if (issuer) tma_store_2d(&map_y, n_own + p * PC, m0, buf);
       } else if (m < P.rows) {
         uint16_t* out = P.Y + static_cast<size_t>(m) * P.ldy + n0 + static_cast<int>(rank) * W + c0;
 #pragma unroll

@@ -206,7 +206,6 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
         group_sync(group);
         if (issuer) {
           tma_store_2d(&map_dw, n0 + c0, m0, buf);
-          tma_store_commit();
         }
       }
       if (!released) {

@@ -279,7 +279,6 @@ linear_chain_kernel(const __grid_constant__ ChainMaps M, const __grid_constant__
         group_sync(group);
         if (issuer) {
           tma_store_2d(&M.y[T.g], n0 + c0, m0, buf);
-          tma_store_commit();
         }
       }
       if (!released) {

@@ -21,14 +21,14 @@
 //   warps 0-3 : producers, warp w filling every fourth stage; lane = (64-token half, four rows): one
 //               gather4 per lane per stage, completion bytes counted on the stage's mbarrier;
 //               lane 0 also issues the bulk copy of the weight tile and hands the stage's byte on;
-//   warp 4    : one lane issues tcgen05.mma (M=128, N=d, K=16) into one of two TMEM accumulators,
+//   warp 4    : one lane issues tcgen05.mma (M=128, N=d, K=16) into one of the TMEM accumulators,
 //               commits stage release and, at the end of a row-block, accumulator ready;
-//   warps 5-12: epilogue, two groups of four warps that take the row-blocks in turn (group = accumulator);
-//               each warp reads its 32 TMEM lanes (tokens), adds bias, optional GELU, rounds to bf16, and the
-//               group's 128 x 32 pieces leave through staging buffers as TMA stores (blocks of 16 rows:
-//               straight from registers).  With one group storing from registers a row-block of 128 outputs
-//               with GELU, written transposed, took longer than its two stages of 64 columns: 54 us for
-//               4096 x 1024 at 8 times compression and 8192 tokens, 27 us for the same work without either.
+//   warps 5.. : epilogue, two or four groups of four warps that take the row-blocks in turn (group =
+//               accumulator); each warp reads its 32 TMEM lanes (tokens), adds bias, optional GELU, rounds to
+//               bf16, and the group's 128 x 32 pieces leave through staging buffers as TMA stores (blocks of 16
+//               rows: straight from registers).  A piece takes 1000 cycles, 1700 with GELU, nearly all of it
+//               latency: one group storing from registers took 54 us for 4096 x 1024 with GELU at 8 times
+//               compression and 8192 tokens, two groups 35, four 30; the gathering alone needs 19.
 // Every wait is bounded; on expiry the role records BSP_ERR_TIMEOUT and leaves its loop.
 //
 // What bounds it: every gathered element crosses L2 -> shared memory once per row-block and feeds
@@ -46,22 +46,22 @@ using namespace tc;
 
 namespace {
 
-constexpr int kGThreads = 416;              // 4 producer warps, MMA warp, 2 x 4 epilogue warps
+constexpr int gather_threads(int groups) { return 160 + 128 * groups; }   // 4 producer warps, MMA warp, epilogue groups
 constexpr int kGStageK = 64;                // kept columns per pipeline stage
 constexpr int kGStageA = kGStageK * kBlockM * 2;   // 16 KB: 64 rows of 128 tokens
 constexpr int kGQueue = 12;                 // a producer warp loads its column numbers up to this many stages ahead
 constexpr int kGPrefetch = kGQueue;         // the plan's column array is padded by this many stages
 
-template <int D>
+template <int D, int GROUPS>     // GROUPS epilogue groups of four warps, as many TMEM accumulators
 struct GatherCfg {
   static constexpr int kStageB = D * 128;                       // d rows of 64 bf16
   static constexpr int kStage = kGStageA + kStageB;
   static constexpr bool kStaged = D >= kEpiCols;                // outputs leave through staging buffers and TMA stores
-  static constexpr int kStaging = kStaged ? kEpiBytes : 0;
-  static constexpr int kFixed = 1024 /*alignment slack*/ + 512 /*barriers, stage bytes*/ + 2 * D * 2 /*bias, two blocks*/ + kStaging;
+  static constexpr int kStaging = kStaged ? kEpiBytes : 0;     // four buffers, shared out among the groups
+  static constexpr int kFixed = 1024 /*alignment slack*/ + 512 /*barriers, stage bytes*/ + GROUPS * D * 2 /*bias, a block per group*/ + kStaging;
   static constexpr int kStagesRaw = (kSmemLimit - kFixed) / kStage;
   static constexpr int kStages = kStagesRaw > 12 ? 12 : kStagesRaw;
-  static constexpr int kTmemCols = 2 * D < 32 ? 32 : 2 * D;     // 32, 64, 128, 256
+  static constexpr int kTmemCols = GROUPS * D;                  // a power of two, 32 ... 512
   static constexpr int kSmemBytes = kStages * kStage + kFixed;
 };
 
@@ -257,7 +257,9 @@ __device__ __forceinline__ void mma_gather_stage(uint32_t d_tmem, uint64_t a_des
       : "memory");
 }
 
-// The 128 threads of an epilogue group agree on whether all of their waits succeeded (named barrier 3 + group); also
+// Named barriers of the epilogue groups: 1 + g, and 5 + g with a vote.
+__device__ __forceinline__ void gather_group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory"); }
+// The 128 threads of an epilogue group agree on whether all of their waits succeeded; also
 // the barrier behind the group's bias writes.
 __device__ __forceinline__ bool group_all_ok(int group, bool ok) {
   uint32_t r;
@@ -267,24 +269,25 @@ __device__ __forceinline__ bool group_all_ok(int group, bool ok) {
       "barrier.cta.red.and.pred q, %2, 128, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"(ok ? 1u : 0u), "r"(3 + group)
+      : "r"(ok ? 1u : 0u), "r"(5 + group)
       : "memory");
   return r != 0u;
 }
 
-template <int D>
-__global__ void __launch_bounds__(kGThreads, 1)
+template <int D, int GROUPS>
+__global__ void __launch_bounds__(gather_threads(GROUPS), 1)
 linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_constant__ CUtensorMap map_y,
                      const __grid_constant__ GatherParams P) {
-  using Cfg = GatherCfg<D>;
+  using Cfg = GatherCfg<D, GROUPS>;
+  constexpr int kBuffers = kEpiBuffers / GROUPS;
   constexpr int S = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  // [S stages: A 16 KB, B D*128][output staging][bias of two row-blocks][mbarriers][stage bytes][TMEM base]
+  // [S stages: A 16 KB, B D*128][output staging][bias of a row-block per group][mbarriers][stage bytes][TMEM base]
   uint16_t* s_bias = reinterpret_cast<uint16_t*>(smem + S * Cfg::kStage + Cfg::kStaging);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_bias + 2 * D);
-  // bars[0..S) full, [S..2S) empty, [2S..2S+2) accumulator full, [2S+2..2S+4) accumulator empty
-  uint8_t* s_meta = reinterpret_cast<uint8_t*>(bars + 2 * S + 4);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_bias + GROUPS * D);
+  // bars[0..S) full, [S..2S) empty, then per accumulator full, empty
+  uint8_t* s_meta = reinterpret_cast<uint8_t*>(bars + 2 * S + 2 * GROUPS);
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(s_meta + 16);
   volatile uint32_t* timed_out = tmem_holder + 1;     // set by a role whose wait expired
 
@@ -294,13 +297,13 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (S + s); };
   auto acc_full_bar = [&](int a) { return bar_base + 8u * (2 * S + a); };
-  auto acc_empty_bar = [&](int a) { return bar_base + 8u * (2 * S + 2 + a); };
+  auto acc_empty_bar = [&](int a) { return bar_base + 8u * (2 * S + GROUPS + a); };
 
   if (threadIdx.x == 0) {
     *timed_out = 0u;
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_xt)) : "memory");
     for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), 4); }
+    for (int a = 0; a < GROUPS; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), 4); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -389,7 +392,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
       constexpr uint32_t idesc = gather_idesc(D);
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t acc_phase[2] = {0u, 0u};
+      uint32_t acc_phase = 0u;               // of every accumulator: they are used in turn
       int acc = 0;
       bool ok = true;
       for (int unit = blockIdx.x; unit < total_units && ok; unit += gridDim.x) {
@@ -403,7 +406,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
           const int groups = static_cast<int>(mt & 7u);
           const bool first = (mt & 0x10u) != 0, last = (mt & 0x20u) != 0;
           if (first) {
-            if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
+            if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase ^ 1u, P.status)) { ok = false; break; }
             tcgen05_fence_after();
           }
           const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * D);
@@ -413,8 +416,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
                            empty_bar(stage));
           if (last) {
             tcgen05_commit_elect(acc_full_bar(acc));
-            acc_phase[acc] ^= 1u;
-            acc ^= 1;
+            if (++acc == GROUPS) { acc = 0; acc_phase ^= 1u; }
           }
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
@@ -423,91 +425,111 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
     }
   } else {
     // ---------------------------------------------------------------- epilogue
-    const int group = (warp - 5) >> 2;       // takes accumulator `group`: every other row-block of this CTA's sequence
+    const int group = (warp - 5) >> 2;       // takes accumulator `group`: every GROUPS-th row-block of this CTA's sequence
     const int quad = warp & 3;               // TMEM lanes [32*quad, 32*quad+32) belong to this warp
     const int row = quad * 32 + lane;
     const int tid = static_cast<int>(threadIdx.x) - 160 - group * 128;
     const bool issuer = tid == 0;            // the thread that owns the group's TMA stores
     const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(group * D);
-    const uint32_t buf0 = smem_base + S * Cfg::kStage + static_cast<uint32_t>(group) * 2u * kEpiStage;
+    const uint32_t buf0 = smem_base + S * Cfg::kStage + static_cast<uint32_t>(group * kBuffers) * kEpiStage;
     uint16_t* my_bias = s_bias + group * D;
     uint32_t phase = 0u, piece_no = 0u;
-    int seq = 0;                             // row-blocks of this CTA so far
+    // position in this CTA's sequence of row-blocks
+    struct {
+      int unit, m, rb, rb1;
+    } at{static_cast<int>(blockIdx.x), 0, 0, 0};
+    auto enter = [&](auto& c) {
+      if (c.unit >= total_units) return;
+      const int ch = c.unit % P.n_chunks;
+      c.m = c.unit / P.n_chunks;
+      c.rb = ch * P.rb_per_chunk;
+      c.rb1 = min(P.n_blocks, c.rb + P.rb_per_chunk);
+    };
+    auto advance = [&](auto& c) {
+      if (c.unit < total_units && ++c.rb >= c.rb1) {
+        c.unit += gridDim.x;
+        enter(c);
+      }
+    };
+    auto bias_of = [&](const auto& c) -> uint16_t {
+      return tid < D && c.unit < total_units && P.bias != nullptr ? __ldg(P.bias + static_cast<size_t>(c.rb) * D + tid) : static_cast<uint16_t>(0);
+    };
+    enter(at);
+    for (int g = 0; g < group; ++g) advance(at);
+    uint16_t next_bias = bias_of(at);
     bool ok = true;
-    for (int unit = blockIdx.x; unit < total_units && ok; unit += gridDim.x) {
-      const int m = unit / P.n_chunks, ch = unit - m * P.n_chunks;
-      const int rb0 = ch * P.rb_per_chunk, rb1 = min(P.n_blocks, rb0 + P.rb_per_chunk);
-      for (int rb = rb0; rb < rb1; ++rb, ++seq) {
-        if ((seq & 1) != group) continue;
-        // the bias first, so that its latency overlaps the wait for the accumulator (its last readers are behind
-        // the group's last barrier)
-        if (tid < D) my_bias[tid] = P.bias != nullptr ? __ldg(P.bias + static_cast<size_t>(rb) * D + tid) : static_cast<uint16_t>(0);
-        // one decision for the group: nobody is left alone at its barriers
-        if (!group_all_ok(group, mbar_wait(acc_full_bar(group), phase, P.status))) { ok = false; break; }
-        phase ^= 1u;
-        tcgen05_fence_after();
-        if constexpr (Cfg::kStaged) {
+    while (at.unit < total_units) {
+      const int m = at.m, rb = at.rb;
+      // this block's bias was asked for a block ago (its slot's last readers are behind the group's last barrier)
+      if (tid < D) my_bias[tid] = next_bias;
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g) advance(at);
+      next_bias = bias_of(at);
+      // one decision for the group: nobody is left alone at its barriers
+      if (!group_all_ok(group, mbar_wait(acc_full_bar(group), phase, P.status))) { ok = false; break; }
+      phase ^= 1u;
+      tcgen05_fence_after();
+      if constexpr (Cfg::kStaged) {
 #pragma unroll 1
-          for (int c0 = 0; c0 < D; c0 += kEpiCols) {
-            const uint32_t buf = buf0 + (piece_no & 1u) * kEpiStage;
-            ++piece_no;
-            EpiloguePiece piece;
-            piece_load(taddr + c0, smem_u32(my_bias + c0), piece);
-            if (issuer) tma_store_wait_read<1>();   // the store issued two pieces ago has read this buffer
-            group_sync(group);
-            if (c0 + kEpiCols >= D) {               // this warp's last read of the accumulator
-              tcgen05_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(acc_empty_bar(group));
-            }
-            if (P.transposed) piece_store_transposed(piece, P.act, buf, row);
-            else piece_store(piece, P.act, buf + static_cast<uint32_t>(row) * 64u, static_cast<uint32_t>((row >> 1) & 3));
-            fence_async_smem();
-            group_sync(group);
-            if (issuer) {
-              if (P.transposed) tma_store_2d(&map_y, m * kBlockM, rb * D + c0, buf);
-              else tma_store_2d(&map_y, rb * D + c0, m * kBlockM, buf);
-              tma_store_commit();
-            }
+        for (int c0 = 0; c0 < D; c0 += kEpiCols) {
+          const uint32_t buf = buf0 + (piece_no % kBuffers) * kEpiStage;
+          ++piece_no;
+          EpiloguePiece piece;
+          piece_load(taddr + c0, smem_u32(my_bias + c0), piece);
+          if (issuer) tma_store_wait_read<kBuffers - 1>();   // the store that last used this buffer has read it
+          gather_group_sync(group);
+          if (c0 + kEpiCols >= D) {               // this warp's last read of the accumulator
+            tcgen05_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty_bar(group));
           }
-        } else {
-          uint32_t v[16];
-          tmem_load_16cols(taddr, v);
-          const uint4 b0 = ld_shared_v4(smem_u32(my_bias)), b1 = ld_shared_v4(smem_u32(my_bias) + 16u);
-          tmem_load_wait();
-          tcgen05_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acc_empty_bar(group));
-          const uint32_t bw[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-          float f[16];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            f[2 * i] = __uint_as_float(v[2 * i]) + __uint_as_float(bw[i] << 16);
-            f[2 * i + 1] = __uint_as_float(v[2 * i + 1]) + __uint_as_float(bw[i] & 0xffff0000u);
+          if (P.transposed) piece_store_transposed(piece, P.act, buf, row);
+          else piece_store(piece, P.act, buf + static_cast<uint32_t>(row) * 64u, static_cast<uint32_t>((row >> 1) & 3));
+          fence_async_smem();
+          gather_group_sync(group);
+          if (issuer) {
+            if (P.transposed) tma_store_2d(&map_y, m * kBlockM, rb * D + c0, buf);
+            else tma_store_2d(&map_y, rb * D + c0, m * kBlockM, buf);
           }
-          if (P.act == BSP_ACT_GELU) {
-#pragma unroll
-            for (int i = 0; i < 16; i += 2) gelu_erf_pair(f[i], f[i + 1]);
-          }
-          const int t = m * kBlockM + row;
-          if (t < P.tokens) {
-            uint32_t w[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) w[i] = pack_bf16x2(f[2 * i], f[2 * i + 1]);
-            if (P.transposed) {
-              // output row n = rb * D + i holds this thread's token in column t: the 32 lanes of a warp write 64
-              // contiguous bytes per output row
-              uint16_t* col = P.Y + static_cast<size_t>(rb) * D * P.ldy + t;
-#pragma unroll
-              for (int i = 0; i < 16; ++i) col[static_cast<size_t>(i) * P.ldy] = static_cast<uint16_t>(i & 1 ? w[i >> 1] >> 16 : w[i >> 1] & 0xffffu);
-            } else {
-              uint4* out = reinterpret_cast<uint4*>(P.Y + static_cast<size_t>(t) * P.ldy + static_cast<size_t>(rb) * D);
-              out[0] = make_uint4(w[0], w[1], w[2], w[3]);
-              out[1] = make_uint4(w[4], w[5], w[6], w[7]);
-            }
-          }
-          group_sync(group);                        // everyone has read the bias
         }
+      } else {
+        uint32_t v[16];
+        tmem_load_16cols(taddr, v);
+        const uint4 b0 = ld_shared_v4(smem_u32(my_bias)), b1 = ld_shared_v4(smem_u32(my_bias) + 16u);
+        tmem_load_wait();
+        tmem_loaded<16>(v);
+        tcgen05_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty_bar(group));
+        const uint32_t bw[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        float f[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          f[2 * i] = __uint_as_float(v[2 * i]) + __uint_as_float(bw[i] << 16);
+          f[2 * i + 1] = __uint_as_float(v[2 * i + 1]) + __uint_as_float(bw[i] & 0xffff0000u);
+        }
+        if (P.act == BSP_ACT_GELU) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) gelu_erf_pair(f[i], f[i + 1]);
+        }
+        const int t = m * kBlockM + row;
+        if (t < P.tokens) {
+          uint32_t w[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) w[i] = pack_bf16x2(f[2 * i], f[2 * i + 1]);
+          if (P.transposed) {
+            // output row n = rb * D + i holds this thread's token in column t: the 32 lanes of a warp write 64
+            // contiguous bytes per output row
+            uint16_t* col = P.Y + static_cast<size_t>(rb) * D * P.ldy + t;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) col[static_cast<size_t>(i) * P.ldy] = static_cast<uint16_t>(i & 1 ? w[i >> 1] >> 16 : w[i >> 1] & 0xffffu);
+          } else {
+            uint4* out = reinterpret_cast<uint4*>(P.Y + static_cast<size_t>(t) * P.ldy + static_cast<size_t>(rb) * D);
+            out[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            out[1] = make_uint4(w[4], w[5], w[6], w[7]);
+          }
+        }
+        gather_group_sync(group);                        // everyone has read the bias
       }
     }
     if (issuer) tma_store_wait_read<0>();
@@ -524,19 +546,18 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
   }
 }
 
-template <int D>
-int launch_gather(TcDevice* dev, int slot, const GatherParams& P, cudaStream_t s) {
-  using Cfg = GatherCfg<D>;
+template <int D, int GROUPS>
+int launch_gather_groups(TcDevice* dev, const GatherParams& P, cudaStream_t s) {
+  using Cfg = GatherCfg<D, GROUPS>;
   static_assert(Cfg::kStages >= 4, "pipeline too shallow");
   static bool attr_set[64] = {};
   int device = 0;
   BSP_CUDA_TRY(cudaGetDevice(&device));
   if (device < 0 || device >= 64) return BSP_ERR_CUDA;
   if (!attr_set[device]) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(linear_gather_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+    BSP_CUDA_TRY(cudaFuncSetAttribute(linear_gather_kernel<D, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
     attr_set[device] = true;
   }
-  (void)slot;
   CUtensorMap map_xt;      // XT as [k_in rows, tokens]; box = one row of 64 tokens, 128-byte swizzle, zeros out of range
   // (no L2 promotion: a gathered row is 128 bytes, and fetching 256 would read every line twice)
   if (!make_map(&map_xt, P.XT, P.tokens, P.k_in, P.ldxt, 1, 64, CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) return BSP_ERR_CUDA;
@@ -550,8 +571,18 @@ int launch_gather(TcDevice* dev, int slot, const GatherParams& P, cudaStream_t s
   }
   const int units = P.m_tiles * P.n_chunks;
   const int grid = units < dev->sms ? units : dev->sms;
-  BSP_CUDA_TRY(launch_pdl(linear_gather_kernel<D>, dim3(grid), dim3(kGThreads), Cfg::kSmemBytes, s, map_xt, map_y, P));
+  BSP_CUDA_TRY(launch_pdl(linear_gather_kernel<D, GROUPS>, dim3(grid), dim3(gather_threads(GROUPS)), Cfg::kSmemBytes, s, map_xt, map_y, P));
   return BSP_OK;
+}
+
+// Four epilogue groups where GELU makes a row-block's epilogue longer than its stages and a CTA has several
+// row-blocks to take turns with: 4096 x 1024 in 128-row blocks at 8x and 8192 tokens 35 us with two groups, 30 with
+// four; without GELU, or with a few row-blocks per CTA, the smaller CTA starts sooner (0.3 to 1 us).
+template <int D>
+int launch_gather(TcDevice* dev, const GatherParams& P, cudaStream_t s) {
+  const long long blocks = static_cast<long long>(P.m_tiles) * P.n_blocks;
+  return D >= 64 && P.act == BSP_ACT_GELU && blocks >= 8LL * dev->sms ? launch_gather_groups<D, 4>(dev, P, s)
+                                                                      : launch_gather_groups<D, 2>(dev, P, s);
 }
 
 bool gather_block_ok(int block) { return block == 16 || block == 32 || block == 64 || block == 128; }
@@ -654,9 +685,9 @@ extern "C" int bsp_linear_gathered_ex(const void* gplan, int n_out, int k_in, in
   P.status = dev->status;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   switch (block) {
-    case 16: return launch_gather<16>(dev, 0, P, s);
-    case 32: return launch_gather<32>(dev, 1, P, s);
-    case 64: return launch_gather<64>(dev, 2, P, s);
-    default: return launch_gather<128>(dev, 3, P, s);
+    case 16: return launch_gather<16>(dev, P, s);
+    case 32: return launch_gather<32>(dev, P, s);
+    case 64: return launch_gather<64>(dev, P, s);
+    default: return launch_gather<128>(dev, P, s);
   }
 }

@@ -260,7 +260,6 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
           // rows beyond `tokens` / columns beyond `n_out` are clipped by the tensor map
           if (P.transposed) tma_store_2d(&map_y, m0, n0 + c0, buf);
           else tma_store_2d(&map_y, n0 + c0, m0, buf);
-          tma_store_commit();
         }
       }
       if (!released) {                       // a group without a piece in this tile still releases the accumulator

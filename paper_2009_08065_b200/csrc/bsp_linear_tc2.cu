@@ -236,7 +236,6 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
         group_sync(group);
         if (issuer) {
           tma_store_2d(&map_y, n0 + c0, m0, buf);
-          tma_store_commit();
         }
       }
       if (!released) {

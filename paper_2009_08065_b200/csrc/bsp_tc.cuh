@@ -224,12 +224,14 @@ __device__ __forceinline__ void tmem_load_32cols(uint32_t taddr, uint32_t (&v)[3
       : "r"(taddr)
       : "memory");
 }
+// A TMA store of one staged piece as a bulk group of its own, and the wait until all but the N last groups of the
+// calling thread have read their source.
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, uint32_t src) {
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
                ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(src)
                : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
-__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void tma_store_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
@@ -265,6 +267,12 @@ __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   return v;
 }
 __device__ __forceinline__ void tmem_load_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The registers of a TMEM load pass through an empty statement behind the wait, so that no use of them moves above it.
+template <int N>
+__device__ __forceinline__ void tmem_loaded(uint32_t (&v)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(v[i]));
+}
 
 // Shared-memory matrix descriptor of a K-major bf16 tile stored as 128-byte swizzled rows
 // (what a TMA load with the 128-byte swizzle mode writes): 8-row groups 1024 bytes apart.
@@ -289,21 +297,8 @@ __host__ __device__ constexpr uint32_t instr_desc_bf16(int n) {
 // float32 is 3.2e-7 (below 1e-9 beyond a = 6), so x Phi(x) is off by at most 2e-6 in absolute terms,
 // far under the bf16 rounding of the output except deep in the lower tail.  One
 // special-function operation (ex2) per element, no branch, no select: with q = Phi(-|x|),
-// x Phi(x) = max(x, 0) - |x| q for either sign of x.
-__device__ __forceinline__ float gelu_erf(float x) {
-  const float a = fminf(fabsf(x), 6.0f);
-  float p = fmaf(-0.000518865308f, a, 0.00738722592f);
-  p = fmaf(p, a, -0.0525380379f);
-  p = fmaf(p, a, -0.459276694f);
-  p = fmaf(p, a, -1.15108313f);
-  p = fmaf(p, a, -1.00000084f);
-  float q;                                   // q = Phi(-|x|); the argument is in [-28, -1], far from any special case
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(p));
-  // x Phi(x) = max(x, 0) - |x| q for either sign of x: no compare, no select, and no cancellation
-  // in the lower tail (for x < 0 the result is -|x| q, rounded once)
-  return fmaf(-fabsf(x), q, fmaxf(x, 0.0f));
-}
-
+// x Phi(x) = max(x, 0) - |x| q for either sign of x, rounded once and without cancellation in the lower tail
+// (a stands for |x| in the product: beyond 6, where q is below 1e-9, the difference is too).
 // Two float32 values as one 64-bit register pair, and the packed float32 FMA of this architecture
 // (fma.rn.f32x2: two independent correctly rounded FMAs in one instruction, so a result is bit for
 // bit what fmaf gives).
@@ -320,21 +315,25 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-// gelu_erf for two values at once: the same operations in the same order per value, with the five
-// polynomial steps issued as packed FMAs (the epilogue of a GELU layer is bound by instruction issue).
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// GELU of two values, everything but the clamps and the two ex2 as packed operations (the epilogue of a GELU layer is
+// bound by instruction issue and latency).  b = -a; the odd coefficients of P change sign with it.
 __device__ __forceinline__ void gelu_erf_pair(float& x0, float& x1) {
-  const unsigned long long a = pack_f32x2(fminf(fabsf(x0), 6.0f), fminf(fabsf(x1), 6.0f));
-  unsigned long long p = fma_f32x2(pack_f32x2(-0.000518865308f, -0.000518865308f), a, pack_f32x2(0.00738722592f, 0.00738722592f));
-  p = fma_f32x2(p, a, pack_f32x2(-0.0525380379f, -0.0525380379f));
-  p = fma_f32x2(p, a, pack_f32x2(-0.459276694f, -0.459276694f));
-  p = fma_f32x2(p, a, pack_f32x2(-1.15108313f, -1.15108313f));
-  p = fma_f32x2(p, a, pack_f32x2(-1.00000084f, -1.00000084f));
-  float p0, p1, q0, q1;
+  const unsigned long long b = pack_f32x2(fmaxf(-fabsf(x0), -6.0f), fmaxf(-fabsf(x1), -6.0f));
+  unsigned long long p = fma_f32x2(pack_f32x2(0.000518865308f, 0.000518865308f), b, pack_f32x2(0.00738722592f, 0.00738722592f));
+  p = fma_f32x2(p, b, pack_f32x2(0.0525380379f, 0.0525380379f));
+  p = fma_f32x2(p, b, pack_f32x2(-0.459276694f, -0.459276694f));
+  p = fma_f32x2(p, b, pack_f32x2(1.15108313f, 1.15108313f));
+  p = fma_f32x2(p, b, pack_f32x2(-1.00000084f, -1.00000084f));
+  float p0, p1, q0, q1;                      // q = Phi(-|x|); the argument of ex2 is in [-28, -1], far from any special case
   unpack_f32x2(p, p0, p1);
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q0) : "f"(p0));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q1) : "f"(p1));
-  x0 = fmaf(-fabsf(x0), q0, fmaxf(x0, 0.0f));
-  x1 = fmaf(-fabsf(x1), q1, fmaxf(x1, 0.0f));
+  unpack_f32x2(fma_f32x2(b, pack_f32x2(q0, q1), pack_f32x2(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f))), x0, x1);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
@@ -357,6 +356,7 @@ __device__ __forceinline__ void piece_load(uint32_t taddr, uint32_t bias_smem, E
 #pragma unroll
   for (int j = 0; j < 4; ++j) p.bias[j] = ld_shared_v4(bias_smem + 16u * j);
   tmem_load_wait();
+  tmem_loaded<32>(p.v);
 }
 // bias + optional GELU + bf16 rounding, into this thread's 64-byte row of a staging buffer laid out
 // as a TMA store with the 64-byte swizzle expects it (16-byte chunk c of row r at chunk c ^ ((r >> 1) & 3)).
@@ -367,10 +367,10 @@ __device__ __forceinline__ void piece_store(const EpiloguePiece& p, int act, uin
     const uint32_t bw[4] = {p.bias[j].x, p.bias[j].y, p.bias[j].z, p.bias[j].w};
     float f[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      f[2 * i] = __uint_as_float(v[2 * i]) + __uint_as_float(bw[i] << 16);
-      f[2 * i + 1] = __uint_as_float(v[2 * i + 1]) + __uint_as_float(bw[i] & 0xffff0000u);
-    }
+    for (int i = 0; i < 4; ++i)
+      unpack_f32x2(add_f32x2(pack_f32x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])),
+                             pack_f32x2(__uint_as_float(bw[i] << 16), __uint_as_float(bw[i] & 0xffff0000u))),
+                   f[2 * i], f[2 * i + 1]);
     if (act == BSP_ACT_GELU) {
 #pragma unroll
       for (int i = 0; i < 8; i += 2) gelu_erf_pair(f[i], f[i + 1]);
@@ -389,10 +389,10 @@ __device__ __forceinline__ void piece_store_transposed(const EpiloguePiece& p, i
     const uint32_t bw[4] = {p.bias[j].x, p.bias[j].y, p.bias[j].z, p.bias[j].w};
     float f[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      f[2 * i] = __uint_as_float(v[2 * i]) + __uint_as_float(bw[i] << 16);
-      f[2 * i + 1] = __uint_as_float(v[2 * i + 1]) + __uint_as_float(bw[i] & 0xffff0000u);
-    }
+    for (int i = 0; i < 4; ++i)
+      unpack_f32x2(add_f32x2(pack_f32x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])),
+                             pack_f32x2(__uint_as_float(bw[i] << 16), __uint_as_float(bw[i] & 0xffff0000u))),
+                   f[2 * i], f[2 * i + 1]);
     if (act == BSP_ACT_GELU) {
 #pragma unroll
       for (int i = 0; i < 8; i += 2) gelu_erf_pair(f[i], f[i + 1]);
