@@ -8,15 +8,18 @@
 //            of 128 x 256 of a BERT-base weight left half to seven eighths of the SMs idle.
 // A CTA: warps 0 and 10 TMA producers of the two operands, warp 1 MMA issuer, warps
 // 2-9 the exchange and epilogue, in two groups of four warps (a warp per quarter of the TMEM lanes).  Each CTA owns
-// BN / C columns of the tile: once every CTA of the cluster has finished multiplying (first cluster barrier: the
-// operand stages are free) each sends the others their columns as float32 straight from tensor memory into their
-// stages (16 bytes per lane, 512 contiguous bytes per warp), and after the second barrier each adds its columns in
-// rank order (the result does not depend on timing), applies bias, GELU or mask, and stores bf16 rows: by TMA where
-// a warp group has 32 columns, from registers otherwise.  (Bulk copies between the CTAs' shared memories instead of
-// the stores, with an mbarrier instead of the second cluster barrier, were 0.6 us slower on the small tiles.)
+// BN / C columns of the tile.  Once a CTA's accumulator is complete it sends the others their columns as float32
+// straight from tensor memory (st.async, 16 bytes per lane, 512 contiguous bytes per warp; only the warps whose rows
+// exist), the owner counts the bytes on an mbarrier, adds them in rank order (the result does not depend on timing),
+// applies bias, GELU or mask, and stores bf16 rows: by TMA where a warp group has 32 columns, from registers otherwise.
+// The linear form has room for the receive buffers beside the stages, so nobody waits for the whole cluster; the
+// weight-gradient form receives over its stages and therefore first meets the others at a cluster barrier.
+// (Cluster barriers before and after plain remote stores: 1600 cycles of the 5600 of a 768 x 768 launch at 8 tokens.
+// Bulk copies between the CTAs' shared memories instead of the stores: 0.6 us slower on the small tiles.)
 // A CTA asks for more than half of an SM's shared memory even where a few stages would do: two CTAs of a cluster
 // on one SM share its path to L2 (768 outputs x 768 inputs, C = 4: 4.2 us against 3.7).
-// All waits are bounded; a CTA whose wait ran out still takes part in the cluster barriers.
+// All waits are bounded.  A CTA whose wait ran out stays until the rest of its cluster has left: what they were still
+// going to send arrives in memory that exists.
 #include <atomic>
 
 #include "bsp_tc.cuh"
@@ -33,7 +36,7 @@ struct SplitParams {
   int rows, cols;            // output matrix
   int n_tiles, k_blocks, stages;
   int a_bytes;               // bytes of one A copy: fewer than 128 rows where the matrix has fewer
-  int bars_off;              // offset of the mbarriers behind the operand stages
+  int recv_off, bars_off;    // offsets of the receive buffers and of the mbarriers
   int plan_stable, act;
   int transposed;            // linear: the output is written as [cols, rows]
   const uint16_t* bias;      // linear
@@ -49,17 +52,17 @@ __device__ __forceinline__ uint32_t split_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void split_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void split_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void split_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint32_t split_map(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d));
+// 16 bytes into another CTA's shared memory, counted on its mbarrier (both addresses from split_map).
+__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr), "r"(bar), "r"(a),
+               "r"(b), "r"(c), "r"(d));
 }
 template <int N>
 __device__ __forceinline__ void tmem_load_cols(uint32_t taddr, uint32_t (&v)[N]) {
@@ -107,17 +110,20 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   constexpr uint32_t kIdesc = kTn ? (instr_desc_bf16(BN) | (1u << 15) | (1u << 16)) : instr_desc_bf16(BN);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P.bars_off);       // [8] full, [8] empty, accumulator
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 17);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P.bars_off);       // [8] full, [8] empty, accumulator, received
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 18);
   float* s_bias = reinterpret_cast<float*>(bars + 20);                   // [W]
   volatile uint32_t* timed_out = tmem_holder + 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t smem_base = smem_u32(smem), bar_base = smem_u32(bars);
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (8 + s); };
-  const uint32_t acc_bar = bar_base + 8u * 16;
+  const uint32_t acc_bar = bar_base + 8u * 16, recv_bar = bar_base + 8u * 17;
   const int S = P.stages;
   const uint32_t rank = split_rank();
+  const int tile = static_cast<int>(blockIdx.x) / C;
+  const int m0 = (tile / P.n_tiles) * kBlockM, n0 = (tile % P.n_tiles) * BN;
+  const int quads = (min(kBlockM, P.rows - m0) + 31) >> 5;   // quarters of the tile with rows that exist
 
   if (threadIdx.x == 0) {
     *timed_out = 0u;
@@ -125,6 +131,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
     for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1); }
     mbar_init(acc_bar, 1);
+    mbar_init(recv_bar, 1);
+    mbar_arrive_expect_tx(recv_bar, static_cast<uint32_t>((C - 1) * quads * 32 * W * 4));   // what the others will send
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -136,13 +144,12 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_holder;
+  split_cluster_arrive();                              // this CTA runs and its mbarriers exist
 
   // The weights of a stable plan are older than the kernel before this one: their producer does not wait.
   if (!(P.plan_stable && warp == 10)) pdl_wait();
   pdl_launch_dependents();
 
-  const int tile = static_cast<int>(blockIdx.x) / C;
-  const int m0 = (tile / P.n_tiles) * kBlockM, n0 = (tile % P.n_tiles) * BN;
   const int kb0 = static_cast<int>(static_cast<long long>(P.k_blocks) * rank / C);
   const int kb1 = static_cast<int>(static_cast<long long>(P.k_blocks) * (rank + 1) / C);
 
@@ -207,9 +214,9 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   const bool epilogue = warp >= 2 && warp < 10;
   const int group = (warp - 2) >> 2, quad = warp & 3;
   const int row = quad * 32 + lane, m = m0 + row;
-  const bool mine = epilogue && group * UW < W;        // this warp has columns
+  const bool mine = epilogue && group * UW < W;        // this warp's group has columns
+  const bool live = quad < quads;                      // this warp's rows exist
   const int n_own = n0 + static_cast<int>(rank) * W + group * UW;   // its first output column
-  // the accumulator is complete: every MMA has read its operands, the stages are free
   bool ok = true;
   uint2 flags[kTn ? UW / 8 : 1];
   if (epilogue) {
@@ -224,17 +231,22 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           flags[i] = __ldg(reinterpret_cast<const uint2*>(P.keep + static_cast<size_t>(m / P.block) * P.cols + n_own + 8 * i));
       }
     }
-    ok = mbar_wait(acc_bar, 0u, P.status);
+    ok = __all_sync(0xffffffffu, mbar_wait(acc_bar, 0u, P.status));
     if (!ok && lane == 0) record_timeout(P.status, timed_out);
     tcgen05_fence_after();
   }
   __syncwarp();
-  split_cluster_sync();
+  split_cluster_wait();                                // the others run
+  if constexpr (kTn) {                                 // and no longer need their stages
+    split_cluster_arrive();
+    split_cluster_wait();
+  }
 
   const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-  // receive buffer of a CTA: [source, own rank left out][4-column group][row][4 floats], then the output staging
+  // receive buffer of a CTA: [source, own rank left out][4-column group][row][4 floats]
+  const uint32_t recv_base = smem_base + static_cast<uint32_t>(P.recv_off);
   const uint32_t row_at = static_cast<uint32_t>(row) * 16u;
-  if (mine) {
+  if (mine && live && ok) {
     // ---------------------------------------------------------------- partial columns to their owners
 #pragma unroll 1
     for (int c0 = group * UW; c0 < (group + 1) * UW; c0 += PC) {
@@ -246,20 +258,30 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       for (int o = 1; o < C; ++o) {
         tmem_loaded<PC>(v[o - 1]);
         const uint32_t q = (rank + o) % C, slot = rank < q ? rank : rank - 1;
-        const uint32_t dst = split_map(smem_base + slot * kSlot + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at, q);
+        const uint32_t dst = split_map(recv_base + slot * kSlot + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at, q);
+        const uint32_t bar = split_map(recv_bar, q);
 #pragma unroll
         for (int j = 0; j < PC / 4; ++j)
-          st_cluster_v4(dst + j * (kBlockM * 16u), v[o - 1][4 * j], v[o - 1][4 * j + 1], v[o - 1][4 * j + 2], v[o - 1][4 * j + 3]);
+          st_async_v4(dst + j * (kBlockM * 16u), bar, v[o - 1][4 * j], v[o - 1][4 * j + 1], v[o - 1][4 * j + 2], v[o - 1][4 * j + 3]);
       }
     }
   }
   __syncwarp();
-  split_cluster_sync();
 
   // ---------------------------------------------------------------- this CTA's columns
-  if (epilogue) ok = epilogue_all_ok(ok);              // one decision: nobody is left alone at a named barrier
+  if (epilogue) {
+    if constexpr (!kTmaStore) epilogue_sync_all();     // s_bias is complete (with TMA stores: the vote below)
+    if (!mbar_wait(recv_bar, 0u, P.status)) {
+      if (lane == 0) record_timeout(P.status, timed_out);
+      ok = false;
+    }
+    // one decision where a group shares barriers below: nobody is left alone at them
+    if constexpr (kTmaStore) ok = epilogue_all_ok(ok);
+    else ok = __all_sync(0xffffffffu, ok) && live;
+  }
   if (mine && ok) {
-    const uint32_t out_base = smem_base + (C - 1) * kSlot + static_cast<uint32_t>(group) * 2u * kEpiStage;
+    // output staging: over the stages, which only this CTA has used, or behind the receive buffers
+    const uint32_t out_base = smem_base + (kTn ? (C - 1) * kSlot : 0u) + static_cast<uint32_t>(group) * 2u * kEpiStage;
 #pragma unroll 1
     for (int p = 0; p < UW / PC && n_own + p * PC < P.cols; ++p) {
       const int c0 = group * UW + p * PC;
@@ -270,7 +292,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       float f[PC];
 #pragma unroll
       for (int i = 0; i < PC; ++i) f[i] = __uint_as_float(own[i]);
-      const uint32_t at = smem_base + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at;
+      const uint32_t at = recv_base + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at;
 #pragma unroll
       for (int src = 0; src < C - 1; ++src) {          // own part first, then the others in rank order
         uint4 a[PC / 4];
@@ -344,6 +366,10 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   tcgen05_fence_before();
   __syncthreads();
   quiet_period(timed_out);
+  if (*timed_out != 0u) {                              // (the same for every thread) until every other CTA has left, or waits here too
+    split_cluster_arrive();
+    split_cluster_wait();
+  }
   if (warp == 1) {
     tcgen05_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
@@ -357,15 +383,17 @@ int launch_split(TcDevice* dev, const CUtensorMap& map_a, const CUtensorMap& map
   else if (!make_map(&map_y, P.Y, P.cols, P.rows, P.ldy, kBlockM, kEpiCols)) return BSP_ERR_CUDA;
   constexpr int kStage = (kBlockM + BN) * kBlockK * 2;
   constexpr int kTail = 1024 + 160 + BN / C * 4 + 32;                // alignment slack, barriers, bias
-  constexpr int kFit = (kSmemLimit - kTail) / kStage;
   constexpr bool kTmaStore = BN / C >= 64;
-  constexpr int kExchange = (C - 1) * kBlockM * (BN / C) * 4 + (kTmaStore ? kEpiBytes : 0);
+  constexpr int kReceive = (C - 1) * kBlockM * (BN / C) * 4;
+  constexpr int kExchange = kReceive + (kTmaStore ? kEpiBytes : 0);  // over the stages (weight gradient)
+  constexpr int kFit = (kSmemLimit - kTail - (kTn ? 0 : kReceive)) / kStage;
   constexpr int kAlone = kSmemLimit / 2 + 1024;                      // one CTA per SM
-  static_assert(kExchange + kTail <= kSmemLimit, "exchange areas");
+  static_assert(kExchange + kTail <= kSmemLimit && kFit >= 3 && (kTn || !kTmaStore || kStage >= kEpiBytes), "shared memory");
   const int per_cta = (P.k_blocks + C - 1) / C;
   P.stages = per_cta < kFit ? per_cta : kFit;
   if (P.stages > 8) P.stages = 8;
-  P.bars_off = P.stages * kStage > kExchange ? P.stages * kStage : kExchange;
+  P.recv_off = kTn ? 0 : P.stages * kStage;
+  P.bars_off = kTn ? (P.stages * kStage > kExchange ? P.stages * kStage : kExchange) : P.recv_off + kReceive;
   if (P.bars_off < kAlone) P.bars_off = kAlone;
   P.status = dev->status;
   static std::atomic<bool> attr_set[64];
@@ -426,19 +454,24 @@ bool query_split_ctas(int (&ctas)[3]) {
 }
 
 // The choices below compare times in nanoseconds fitted to single launches on B200 (graphs of one launch, operands in
-// L2): a fixed part per kernel and a part per 64-deep stage.  They hold for grids of one wave only; a split is
-// considered where its clusters all run at once.
-//   whole tile, 64 / 128 / 192 / 256 wide: 2850 / 3200 / 3750 / 4400 + 158 / 168 / 250 / 320 per stage
-//   64-wide tile split 2 / 4 / 8:          3350 / 3450 / 3750       + 165
-//   128-wide tile split 2 / 4 / 8:         4600 / 4600 / 4600       + 170
-// (768 outputs x 3072 inputs at 128 tokens: 10.1 us whole, 4.8 us as 64-wide tiles split 8; 1024 x 4096 at 1003
-// tokens: 13.4 us whole, 128-wide tiles split 2; 768 x 768: 4.6 and 3.9; 304 inputs: not split.)
+// L2): a part per kernel, for a split also per quarter of a tile that has rows (1 to 4: what is exchanged) and per CTA,
+// and a part per 64-deep stage.  They hold for grids of one wave only; a split is considered where its clusters all
+// run at once.
+//   whole tile, 64 / 128 / 192 / 256 wide: 2830 / 3200 / 3750 / 4400 + 158 / 168 / 250 / 320 per stage
+//   64-wide tile split 2 / 4 / 8:          1950 / 2050 / 2400 + 300 / 270 / 250 per quarter + 165 / 165 / 185 per stage
+//   128-wide tile split 2 / 4 / 8:         2700 / 2100 / 2200 + 320 / 520 / 500 per quarter + 170 / 165 / 180 per stage
+//   and 2 per CTA
+// (768 outputs x 3072 inputs: 10.0 us whole, split 8 ways 3.8 us at 8 tokens and 4.6 us at 128; 768 x 768: 4.5 whole, 2.8
+// split 4 ways at 8 tokens; 1024 x 4096 at 1003 tokens: 13.4 whole, 10.6 as 128-wide tiles split 2; 304 x 304: 3.2 and
+// 2.6 at 8 tokens, not split at 1003.)
 int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, int bn_whole, int* bn) {
   const long long m_tiles = (tokens + kBlockM - 1) / kBlockM;
   const int kb = (k_in + kBlockK - 1) / kBlockK;
   if (m_tiles * ((n_out + bn_whole - 1) / bn_whole) > dev.sms) return -1;
-  static const int fixed_whole[4] = {2850, 3200, 3750, 4400}, stage_whole[4] = {158, 168, 250, 320};
-  static const int fixed_split[2][3] = {{3350, 3450, 3750}, {4600, 4600, 4600}}, stage_split[2] = {165, 170};
+  const int quads = tokens >= kBlockM ? 4 : (tokens + 31) / 32;
+  static const int fixed_whole[4] = {2830, 3200, 3750, 4400}, stage_whole[4] = {158, 168, 250, 320};
+  static const int fixed[2][3] = {{1950, 2050, 2400}, {2700, 2100, 2200}}, per_quad[2][3] = {{300, 270, 250}, {320, 520, 500}};
+  static const int per_stage[2][3] = {{165, 165, 185}, {170, 165, 180}};
   const int w = bn_whole / 64 - 1;
   int best = fixed_whole[w] + kb * stage_whole[w] - 100, choice = -1;      // a split has to win by more than noise
   for (int b = 0; b < 2; ++b) {
@@ -446,7 +479,7 @@ int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, in
     for (int i = 0; i < 3; ++i) {
       const int c = 2 << i;
       if (c > kb || tiles * c > dev.split_ctas[i]) continue;
-      const int t = fixed_split[b][i] + (kb + c - 1) / c * stage_split[b];
+      const int t = fixed[b][i] + quads * per_quad[b][i] + (kb + c - 1) / c * per_stage[b][i] + 2 * static_cast<int>(tiles) * c;
       if (t < best) { best = t; choice = i; *bn = 64 * (b + 1); }
     }
   }
