@@ -485,18 +485,33 @@ int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, in
   }
   return choice;
 }
-// dW, 128 x 256 tiles: 4600 + 360 per stage and wave whole, 6500 / 6300 / 6300 + 310 split 2 / 4 / 8.
-int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in) {
-  const long long tiles = static_cast<long long>((n_out + kBlockM - 1) / kBlockM) * ((k_in + 255) / 256);
+// dW: tiles 128 / 192 / 256 wide, whole (persistent kernel: per wave) or, 128 and 256 wide, split 2 / 4 / 8.  Rows of dY
+// or X that are no multiple of 128 bytes make the operand boxes straddle lines: a set of stage times of their own.
+// (4096 tokens: 768 x 768 24.6 us whole 256 wide, 12.4 split 4, 9.8 as 128-wide tiles split 2; 3072 x 768 17.0 as 256-wide
+// tiles split 2, 16.2 whole 128 wide; 3072 x 1024 26.2 whole 256 wide, 20.6 192 wide.  173 tokens: 7.3 and 5.0.)
+int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in, int* bn) {
+  const long long m_tiles = (n_out + kBlockM - 1) / kBlockM;
   const int kb = (tokens + kBlockK - 1) / kBlockK;
-  if (tiles > dev.sms) return -1;
-  static const int fixed_split[3] = {6500, 6300, 6300};
-  int best = 4600 + 360 * kb, choice = -1;
-  for (int i = 0; i < 3; ++i) {
-    const int c = 2 << i;
-    if (c > kb || tiles * c > dev.split_ctas[i]) continue;
-    const int t = fixed_split[i] + (kb + c - 1) / c * 310;
-    if (t < best) { best = t; choice = i; }
+  const int ragged = n_out % 64 || k_in % 64 ? 1 : 0;
+  static const int widths[3] = {128, 192, 256}, fixed_whole[3] = {4450, 5400, 6400};
+  static const int stage_whole[2][3] = {{175, 225, 283}, {250, 310, 366}};
+  static const int fixed_split[2][3] = {{4000, 4100, 4500}, {6700, 6700, 6600}};
+  static const int stage_split[2][2][3] = {{{178, 178, 200}, {265, 265, 265}}, {{270, 334, 373}, {365, 380, 400}}};
+  long long best = -1;
+  int choice = -1;
+  for (int w = 0; w < 3; ++w) {
+    const long long waves = (m_tiles * ((k_in + widths[w] - 1) / widths[w]) + dev.sms - 1) / dev.sms;
+    const long long t = fixed_whole[w] + 1500 * (waves - 1) + waves * kb * stage_whole[ragged][w];
+    if (best < 0 || t < best) { best = t; *bn = widths[w]; }
+  }
+  for (int b = 0; b < 2; ++b) {
+    const long long tiles = m_tiles * ((k_in + 128 * (b + 1) - 1) / (128 * (b + 1)));
+    for (int i = 0; i < 3; ++i) {
+      const int c = 2 << i;
+      if (c > kb || tiles * c > dev.split_ctas[i]) continue;
+      const long long t = fixed_split[b][i] + 4 * tiles * c + (kb + c - 1) / c * stage_split[b][ragged][i];
+      if (t < best) { best = t; choice = i; *bn = 128 * (b + 1); }
+    }
   }
   return choice;
 }
@@ -523,9 +538,9 @@ int launch_linear_split(TcDevice* dev, int bn, int c, const void* plan, const vo
   return bn == 64 ? launch_split_c<64, false>(dev, c, map_x, map_w, P, s) : launch_split_c<128, false>(dev, c, map_x, map_w, P, s);
 }
 
-// dW = (dY^T X) * Mask with a cluster of c = 2, 4 or 8 CTAs per 128 x 256 tile (arguments already validated; keep
+// dW = (dY^T X) * Mask with a cluster of c = 2, 4 or 8 CTAs per 128 x bn tile (arguments already validated; keep
 // 8-byte aligned or null).
-int launch_tn_split(TcDevice* dev, int c, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
+int launch_tn_split(TcDevice* dev, int bn, int c, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
                     int block, const uint8_t* keep, void* dW, int lddw, cudaStream_t s) {
   CUtensorMap map_dy, map_x;
   if (!make_map(&map_dy, dY, n_out, tokens, ldy, kBlockK)) return BSP_ERR_CUDA;
@@ -533,14 +548,14 @@ int launch_tn_split(TcDevice* dev, int c, const void* dY, int ldy, const void* X
   SplitParams P{};
   P.rows = n_out;
   P.cols = k_in;
-  P.n_tiles = (k_in + 255) / 256;
+  P.n_tiles = (k_in + bn - 1) / bn;
   P.k_blocks = (tokens + kBlockK - 1) / kBlockK;
   P.a_bytes = kBlockM * kBlockK * 2;
   P.keep = keep;
   P.block = block;
   P.Y = static_cast<uint16_t*>(dW);
   P.ldy = lddw;
-  return launch_split_c<256, true>(dev, c, map_dy, map_x, P, s);
+  return bn == 128 ? launch_split_c<128, true>(dev, c, map_dy, map_x, P, s) : launch_split_c<256, true>(dev, c, map_dy, map_x, P, s);
 }
 
 }  // namespace bsp

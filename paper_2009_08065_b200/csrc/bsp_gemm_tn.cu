@@ -3,15 +3,17 @@
 //
 // The contraction runs over tokens, the slow dimension of both operands, so the tensor-core tiles
 // are "MN-major": a pipeline stage holds 64 token rows of dY (128 output-row elements wide) and of
-// X (256 columns wide), each loaded as boxes of 64 elements x 64 token rows with the 128-byte
+// X (128, 192 or 256 columns wide), each loaded as boxes of 64 elements x 64 token rows with the 128-byte
 // swizzle; in shared memory that is a stack of 1024-byte atoms (8 token rows x 64 elements), 8 KB
 // from one 64-element column group to the next, which is what the MN-major form of the tcgen05
 // shared-memory descriptor describes (leading byte offset = distance between 64-element groups,
 // stride byte offset = distance between 8-row groups).  Everything else (persistent CTAs, TMA
 // producers, one MMA-issuing thread, two TMEM accumulators, two epilogue groups, TMA stores,
-// bounded waits) is the pipeline of bsp_linear_tc.cu with a 128 x 256 output tile.
+// bounded waits) is the pipeline of bsp_linear_tc.cu with a 128 x BN output tile.
 // The epilogue applies the mask (pruned groups of dW are written as zero).  A weight of fewer tiles than SMs goes
 // to the split contraction of bsp_gemm_split.cu instead where that is faster.
+#include <atomic>
+
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -19,9 +21,7 @@ using namespace tc;
 
 namespace {
 
-constexpr int kTnBN = 256;
 constexpr int kTnThreads = kThreads + 32;          // producer A, MMA, 8 epilogue warps, producer B
-using Cfg = TileCfg<kTnBN>;
 constexpr int kAtomGroup = 64 * kBlockK * 2;       // 64 elements x 64 token rows = 8 KB
 
 // MN-major operand tile with the 128-byte swizzle: 8-row atoms 1024 bytes apart along the
@@ -35,9 +35,8 @@ __device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t smem_addr) {
   d |= static_cast<uint64_t>(2) << 61;
   return d;
 }
-// bf16 x bf16 -> float32, both operands MN-major (bits 15 and 16), M = 128, N = 256.
-constexpr uint32_t kTnIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                              (static_cast<uint32_t>(kTnBN >> 3) << 17) | (static_cast<uint32_t>(kBlockM >> 4) << 24);
+// bf16 x bf16 -> float32, both operands MN-major (bits 15 and 16), M = 128, N = BN.
+__host__ __device__ constexpr uint32_t tn_idesc(int bn) { return instr_desc_bf16(bn) | (1u << 15) | (1u << 16); }
 
 struct TnParams {
   int tokens, n_out, k_in;
@@ -46,14 +45,16 @@ struct TnParams {
   int* status;
 };
 
+template <int BN>
 __global__ void __launch_bounds__(kTnThreads, 1)
 gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_x,
                const __grid_constant__ CUtensorMap map_dw, TnParams P) {
+  using Cfg = TileCfg<BN>;
   constexpr int S = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint16_t* s_zero = reinterpret_cast<uint16_t*>(smem + S * Cfg::kStage + kEpiBytes);       // zero "bias"
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * Cfg::kStage + kEpiBytes + 2 * kTnBN * 2);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * Cfg::kStage + kEpiBytes + 2 * BN * 2);
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 2 * S + 4);
   volatile uint32_t* timed_out = tmem_holder + 1;     // set by a role whose wait expired
 
@@ -72,7 +73,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  for (int c = threadIdx.x; c < 2 * kTnBN; c += blockDim.x) s_zero[c] = 0;
+  for (int c = threadIdx.x; c < 2 * BN; c += blockDim.x) s_zero[c] = 0;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
                  "r"(static_cast<uint32_t>(Cfg::kTmemCols)) : "memory");
@@ -87,7 +88,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
 
   // output tile (mt, nt): rows [128 mt, +128) of dW (output features), columns [256 nt, +256) (input features)
   const int m_tiles = (P.n_out + kBlockM - 1) / kBlockM;
-  const int n_tiles = (P.k_in + kTnBN - 1) / kTnBN;
+  const int n_tiles = (P.k_in + BN - 1) / BN;
   const int total_tiles = m_tiles * n_tiles;
   const int k_blocks = (P.tokens + kBlockK - 1) / kBlockK;
 
@@ -113,13 +114,13 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     uint32_t phase = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      const int n0 = (tile % n_tiles) * kTnBN;
+      const int n0 = (tile % n_tiles) * BN;
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
         const uint32_t b_dst = smem_base + stage * Cfg::kStage + Cfg::kStageA;
         tma_stage_load(b_dst, &map_x, n0, kb * kBlockK, full_bar(stage), Cfg::kStageB);
 #pragma unroll
-        for (int g = 1; g < kTnBN / 64; ++g)
+        for (int g = 1; g < BN / 64; ++g)
           tma_load_2d_elect(b_dst + g * kAtomGroup, &map_x, n0 + 64 * g, kb * kBlockK, full_bar(stage));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
@@ -135,14 +136,14 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
       if (!mbar_wait_warp(acc_empty_bar(acc), acc_phase[acc] ^ 1u, P.status)) { ok = false; break; }
       tcgen05_fence_after();
-      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * kTnBN);
+      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * BN);
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (!mbar_wait_warp(full_bar(stage), phase, P.status)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t a_addr = smem_base + stage * Cfg::kStage;
         const uint32_t b_addr = a_addr + Cfg::kStageA;
         // 16 token rows = two 8-row atoms = 2048 bytes per step
-        mma_stage<128, 128>(d_tmem, smem_desc_mn_sw128(a_addr), smem_desc_mn_sw128(b_addr), kTnIdesc, kb != 0 ? 1u : 0u, empty_bar(stage));
+        mma_stage<128, 128>(d_tmem, smem_desc_mn_sw128(a_addr), smem_desc_mn_sw128(b_addr), tn_idesc(BN), kb != 0 ? 1u : 0u, empty_bar(stage));
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
       if (!ok) break;
@@ -166,12 +167,12 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     int acc = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      const int m0 = (tile / n_tiles) * kBlockM, n0 = (tile % n_tiles) * kTnBN;
+      const int m0 = (tile / n_tiles) * kBlockM, n0 = (tile % n_tiles) * BN;
       // all 256 threads take the same decision, so nobody is left alone at a named barrier below
       if (!epilogue_all_ok(mbar_wait(acc_full_bar(acc), acc_phase[acc], P.status))) { ok = false; break; }
       tcgen05_fence_after();
-      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(acc * kTnBN);
-      const int pieces = (min(kTnBN, P.k_in - n0) + kEpiCols - 1) / kEpiCols;
+      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(acc * BN);
+      const int pieces = (min(BN, P.k_in - n0) + kEpiCols - 1) / kEpiCols;
       bool released = false;
 #pragma unroll 1
       for (int pc = group; pc < pieces; pc += 2) {
@@ -230,6 +231,24 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
   }
 }
 
+template <int BN>
+int launch_tn(TcDevice* dev, const CUtensorMap& map_dy, const CUtensorMap& map_x, const CUtensorMap& map_dw, const TnParams& P,
+              cudaStream_t s) {
+  using Cfg = TileCfg<BN>;
+  static std::atomic<bool> attr_set[64];
+  int device = 0;
+  BSP_CUDA_TRY(cudaGetDevice(&device));
+  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
+  if (!attr_set[device].load(std::memory_order_acquire)) {
+    BSP_CUDA_TRY(cudaFuncSetAttribute(gemm_tn_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+    attr_set[device].store(true, std::memory_order_release);
+  }
+  const int tiles = ((P.n_out + kBlockM - 1) / kBlockM) * ((P.k_in + BN - 1) / BN);
+  BSP_CUDA_TRY(launch_pdl(gemm_tn_kernel<BN>, dim3(tiles < dev->sms ? tiles : dev->sms), dim3(kTnThreads), Cfg::kSmemBytes, s, map_dy,
+                          map_x, map_dw, P));
+  return BSP_OK;
+}
+
 }  // namespace
 }  // namespace bsp
 
@@ -248,9 +267,10 @@ extern "C" int bsp_linear_backward_weight(const void* dY, int ldy, const void* X
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // (flags that are not 8-byte aligned are applied by the mask kernel afterwards)
   const uint8_t* flags = keep != nullptr && aligned_to(keep, 8) ? keep : nullptr;
-  const int split = choose_tn_split(*dev, tokens, n_out, k_in);
+  int bn = 256;
+  const int split = choose_tn_split(*dev, tokens, n_out, k_in, &bn);
   if (split >= 0) {
-    const int st = launch_tn_split(dev, 2 << split, dY, ldy, X, ldx, tokens, n_out, k_in, block, flags, dW, lddw, s);
+    const int st = launch_tn_split(dev, bn, 2 << split, dY, ldy, X, ldx, tokens, n_out, k_in, block, flags, dW, lddw, s);
     if (st != BSP_OK || keep == flags) return st;
     return bsp_apply_mask(dW, n_out, k_in, lddw, block, BSP_ORIENT_C, keep, stream);
   }
@@ -259,23 +279,11 @@ extern "C" int bsp_linear_backward_weight(const void* dY, int ldy, const void* X
   if (!make_map(&map_dy, dY, n_out, tokens, ldy, kBlockK)) return BSP_ERR_CUDA;
   if (!make_map(&map_x, X, k_in, tokens, ldx, kBlockK)) return BSP_ERR_CUDA;
   if (!make_map(&map_dw, dW, k_in, n_out, lddw, kBlockM, kEpiCols)) return BSP_ERR_CUDA;
-  if (!dev->attr_set[6]) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(gemm_tn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    dev->attr_set[6] = true;
-  }
-  TnParams P{tokens, n_out, k_in, flags, block, dev->status};
-  const int tiles = ((n_out + kBlockM - 1) / kBlockM) * ((k_in + kTnBN - 1) / kTnBN);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(tiles < dev->sms ? tiles : dev->sms);
-  cfg.blockDim = dim3(kTnThreads);
-  cfg.dynamicSmemBytes = Cfg::kSmemBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  BSP_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_tn_kernel, map_dy, map_x, map_dw, P));
+  const TnParams P{tokens, n_out, k_in, flags, block, dev->status};
+  const int st = bn == 128   ? launch_tn<128>(dev, map_dy, map_x, map_dw, P, s)
+                 : bn == 192 ? launch_tn<192>(dev, map_dy, map_x, map_dw, P, s)
+                             : launch_tn<256>(dev, map_dy, map_x, map_dw, P, s);
+  if (st != BSP_OK) return st;
   if (keep != flags) return bsp_apply_mask(dW, n_out, k_in, lddw, block, BSP_ORIENT_C, keep, stream);
   return BSP_OK;
 }

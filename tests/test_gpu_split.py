@@ -44,9 +44,9 @@ def test_linear_with_split_contraction(tokens, n_out, k_in, act, with_bias):
     assert torch.equal(yt[:, :tokens], y.t())
 
 
-# clusters of 8, 4 and 2, ragged tiles both ways, a contraction shorter than a stage; flags 8-byte aligned (mask in
-# the epilogue) and not (mask kernel)
-@pytest.mark.parametrize("tokens,n_out,k_in,block", [(4000, 136, 264, 8), (2500, 392, 400, 8), (1300, 1200, 520, 16), (700, 264, 1032, 12), (40, 96, 72, 96)])
+# clusters of 8, 4 and 2, ragged tiles both ways, a contraction shorter than a stage; whole tiles 128, 192 and 256
+# wide, one CTA with several of them; flags 8-byte aligned (mask in the epilogue) and not (mask kernel)
+@pytest.mark.parametrize("tokens,n_out,k_in,block", [(200, 2312, 776, 8), (170, 3072, 1000, 16), (130, 4104, 1032, 8), (4000, 136, 264, 8), (2500, 392, 400, 8), (1300, 1200, 520, 16), (700, 264, 1032, 12), (40, 96, 72, 96)])
 @pytest.mark.parametrize("aligned", [True, False])
 def test_weight_gradient_with_split_contraction(tokens, n_out, k_in, block, aligned):
     dy = si.normal_bf16(82, f"dy{tokens}", (tokens, n_out), 1.0)
