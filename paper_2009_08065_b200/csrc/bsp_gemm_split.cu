@@ -455,31 +455,29 @@ bool query_split_ctas(int (&ctas)[3]) {
 
 // The choices below compare times in nanoseconds fitted to single launches on B200 (graphs of one launch, operands in
 // L2): a part per kernel, for a split also per quarter of a tile that has rows (1 to 4: what is exchanged) and per CTA,
-// and a part per 64-deep stage.  They hold for grids of one wave only; a split is considered where its clusters all
-// run at once.
-//   whole tile, 64 / 128 / 192 / 256 wide: 2830 / 3200 / 3750 / 4400 + 158 / 168 / 250 / 320 per stage
+// and a part per 64-deep stage, against choose_dense's estimate for whole tiles.  They hold for grids of one wave only; a
+// split is considered where its clusters all run at once.
 //   64-wide tile split 2 / 4 / 8:          1950 / 2050 / 2400 + 300 / 270 / 250 per quarter + 165 / 165 / 185 per stage
 //   128-wide tile split 2 / 4 / 8:         2700 / 2100 / 2200 + 320 / 520 / 500 per quarter + 170 / 165 / 180 per stage
 //   and 2 per CTA
 // (768 outputs x 3072 inputs: 10.0 us whole, split 8 ways 3.8 us at 8 tokens and 4.6 us at 128; 768 x 768: 4.5 whole, 2.8
 // split 4 ways at 8 tokens; 1024 x 4096 at 1003 tokens: 13.4 whole, 10.6 as 128-wide tiles split 2; 304 x 304: 3.2 and
 // 2.6 at 8 tokens, not split at 1003.)
-int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, int bn_whole, int* bn) {
+int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn) {
   const long long m_tiles = (tokens + kBlockM - 1) / kBlockM;
   const int kb = (k_in + kBlockK - 1) / kBlockK;
-  if (m_tiles * ((n_out + bn_whole - 1) / bn_whole) > dev.sms) return -1;
   const int quads = tokens >= kBlockM ? 4 : (tokens + 31) / 32;
-  static const int fixed_whole[4] = {2830, 3200, 3750, 4400}, stage_whole[4] = {158, 168, 250, 320};
   static const int fixed[2][3] = {{1950, 2050, 2400}, {2700, 2100, 2200}}, per_quad[2][3] = {{300, 270, 250}, {320, 520, 500}};
   static const int per_stage[2][3] = {{165, 165, 185}, {170, 165, 180}};
-  const int w = bn_whole / 64 - 1;
-  int best = fixed_whole[w] + kb * stage_whole[w] - 100, choice = -1;      // a split has to win by more than noise
+  long long best = whole_ns - 100;                     // a split has to win by more than noise
+  int choice = -1;
   for (int b = 0; b < 2; ++b) {
     const long long tiles = m_tiles * ((n_out + 64 * (b + 1) - 1) / (64 * (b + 1)));
     for (int i = 0; i < 3; ++i) {
       const int c = 2 << i;
       if (c > kb || tiles * c > dev.split_ctas[i]) continue;
-      const int t = fixed[b][i] + quads * per_quad[b][i] + (kb + c - 1) / c * per_stage[b][i] + 2 * static_cast<int>(tiles) * c;
+      const long long stages = (kb + c - 1) / c * per_stage[b][i] * (k_in % 64 ? 115 : 100) / 100;   // ragged rows, as in choose_dense
+      const long long t = fixed[b][i] + quads * per_quad[b][i] + stages + 2 * tiles * c;
       if (t < best) { best = t; choice = i; *bn = 64 * (b + 1); }
     }
   }

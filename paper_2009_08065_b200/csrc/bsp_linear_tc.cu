@@ -526,22 +526,42 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
 // host side
 // ------------------------------------------------------------------------------------------
 }  // namespace
-// Output-tile width: fewest (waves x per-tile cost) over the candidates.  A 64-deep stage of the main
-// loop was measured at about 460 / 515 / 545 / 640 cycles for tiles 64 / 128 / 192 / 256 outputs wide (the
-// activation tile and the latencies are the same whatever the width), which 440 + width models.
-int choose_bn(int tokens, int n_out, int sms) {
-  const int cands[4] = {256, 192, 128, 64};
-  long long best = -1;
-  int best_bn = 128;
-  const long long m_tiles = (tokens + kBlockM - 1) / kBlockM;
-  for (int c = 0; c < 4; ++c) {
-    const int bn = cands[c];
-    const long long tiles = m_tiles * ((n_out + bn - 1) / bn);
-    const long long waves = (tiles + sms - 1) / sms;
-    const long long cost = waves * (bn + 440);
-    if (best < 0 || cost < best) { best = cost; best_bn = bn; }
+// Tile width, or the CTA-pair kernel, for a product of whole tiles: the least estimated time.  A launch costs a fixed
+// part (start-up, first operands, the last tile's epilogue), per wave of tiles the larger of its main loop and its
+// epilogue (with GELU also a part of the smaller one: they contend for issue slots), and something per wave after the
+// first.  A 64-deep stage takes longer the more SMs are drawing operands from L2 (two times per width, for a few CTAs
+// and for all of them), and where rows of X and the plan are no multiple of 128 bytes.  Fitted to launches of 8 to
+// 32768 tokens (nanoseconds; widths 64 / 128 / 192 / 256, pair): over 28 random layers and ten of 768 and 1024 features
+// the choice is about 1 % behind the best of the five on average.  Against the earlier rule (waves x (width + 440), pairs
+// from 1.25 x #SM tiles without GELU): 8192 tokens x 1024 outputs x 4096 inputs 52.7 -> 48.3 us, 4096 outputs with GELU
+// 55.5 -> 52.3.
+DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, int act, bool allow_pair) {
+  static const int width[5] = {64, 128, 192, 256, 256}, rows[5] = {128, 128, 128, 128, 256};
+  static const int fixed[5] = {2830, 3200, 3750, 4400, 5400}, extra_wave[5] = {500, 700, 300, 800, 800};
+  static const int stage_few[5] = {158, 168, 250, 320, 330}, stage_all[5] = {176, 210, 335, 370, 330};
+  static const int ragged_percent[5] = {114, 130, 103, 110, 117};
+  static const int epilogue[2][5] = {{500, 950, 1500, 1750, 2600}, {900, 1600, 2600, 2950, 3900}};
+  static const int gelu_tail[5] = {150, 500, 450, 600, 600}, gelu_overlap[5] = {8, 8, 8, 8, 5};
+  const long long kb = (k_in + kBlockK - 1) / kBlockK;
+  const bool gelu = act == BSP_ACT_GELU;
+  DenseChoice best{128, false, -1};
+  for (int c = 0; c < (allow_pair ? 5 : 4); ++c) {
+    const long long tiles = ((tokens + rows[c] - 1) / rows[c]) * static_cast<long long>((n_out + width[c] - 1) / width[c]);
+    const long long seats = c == 4 ? dev.sms / 2 : dev.sms;
+    const long long waves = (tiles + seats - 1) / seats;
+    const long long busy = tiles < seats ? tiles : seats;
+    long long main_ns = kb * (stage_few[c] + (stage_all[c] - stage_few[c]) * busy / seats);
+    if (k_in % 64) main_ns = main_ns * ragged_percent[c] / 100;
+    const long long epi_ns = epilogue[gelu][c];
+    long long tile_ns = main_ns > epi_ns ? main_ns : epi_ns;
+    if (gelu) {
+      const long long less = main_ns > epi_ns ? epi_ns : main_ns;
+      tile_ns += less * less / tile_ns / gelu_overlap[c];
+    }
+    const long long ns = fixed[c] + waves * tile_ns + (waves - 1) * extra_wave[c] + (gelu ? gelu_tail[c] : 0);
+    if (best.ns < 0 || ns < best.ns) best = DenseChoice{width[c], c == 4, ns};
   }
-  return best_bn;
+  return best;
 }
 namespace {
 
@@ -700,29 +720,21 @@ extern "C" int bsp_linear_planned_ex(const void* plan, int n_out, int k_in, int 
   TcDevice* dev = tc_device();
   if (dev == nullptr) return BSP_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // Measured on B200, single launches after an L2 flush: without GELU the CTA-pair kernel is level or ahead
-  // from about 1.25 x #SM pair-tiles on (8192 tokens x 2304 outputs: 3 %; 16384 x 768: 3-9 %; 32768 tokens: 4-11 %;
-  // a 1024 x 4096 weight at 16384 tokens: 30 %, the one-CTA kernel's last wave being half empty there) and behind
-  // below that (one encoder layer at 4096 tokens: +0 to +4 us per launch; 8192 x 768 x 768: +13 %), where its
-  // longer start-up shows.  With GELU the epilogue is the longer side of a tile and the two are level on average
-  // (0.92-1.05 over six shapes), so those launches stay with the one-CTA kernel.
-  const long long pair_tiles = static_cast<long long>((tokens + 255) / 256) * ((n_out + 255) / 256);
-  const bool pair = algo == BSP_LINEAR_CTA_PAIR ||
-                    (algo == BSP_LINEAR_AUTO && 4 * pair_tiles >= 5LL * dev->sms && act == BSP_ACT_NONE && !transposed);
-  if (pair) return launch_tc_pair(dev, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy, s);
-  LinearParams P{tokens, n_out, k_in, act, (algo_flags & BSP_LINEAR_PLAN_STABLE) ? 1 : 0, copy_rows(tokens) * kBlockK * 2,
-                 transposed ? 1 : 0,
-                 static_cast<const uint16_t*>(bias), dev->status};
-  const int bn = choose_bn(tokens, n_out, dev->sms);
+  DenseChoice choice = choose_dense(*dev, tokens, n_out, k_in, act, algo == BSP_LINEAR_AUTO && !transposed);
+  if (algo == BSP_LINEAR_CTA_PAIR) choice.pair = true;
   if (algo == BSP_LINEAR_AUTO) {
     // few output tiles: a cluster of CTAs per tile, each with a part of the contraction
     int bn_split = 0;
-    const int c = choose_linear_split(*dev, tokens, n_out, k_in, bn, &bn_split);
+    const int c = choose_linear_split(*dev, tokens, n_out, k_in, choice.ns, &bn_split);
     if (c >= 0)
       return launch_linear_split(dev, bn_split, 2 << c, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy,
                                  (algo_flags & BSP_LINEAR_PLAN_STABLE) != 0, transposed, s);
   }
-  switch (bn) {
+  if (choice.pair) return launch_tc_pair(dev, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy, s);
+  LinearParams P{tokens, n_out, k_in, act, (algo_flags & BSP_LINEAR_PLAN_STABLE) ? 1 : 0, copy_rows(tokens) * kBlockK * 2,
+                 transposed ? 1 : 0,
+                 static_cast<const uint16_t*>(bias), dev->status};
+  switch (choice.bn) {
     case 256: return launch_tc<256>(dev, 0, plan, X, Y, P, ldx, ldy, s);
     case 192: return launch_tc<192>(dev, 1, plan, X, Y, P, ldx, ldy, s);
     case 128: return launch_tc<128>(dev, 2, plan, X, Y, P, ldx, ldy, s);

@@ -470,8 +470,15 @@ bool query_split_ctas(int (&ctas)[3]);
 // Cluster size (2, 4, 8) index of dW's split contraction, or -1: the persistent kernel (bsp_gemm_split.cu); *bn = tile
 // width of either.
 int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in, int* bn);
-// The same for the linear layer; *bn = tile width.  bn_whole is the tile width of the one-CTA kernel.
-int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, int bn_whole, int* bn);
+// Kernel for a linear layer on whole tiles, with its estimated time (bsp_linear_tc.cu).
+struct DenseChoice {
+  int bn;
+  bool pair;
+  long long ns;
+};
+DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, int act, bool allow_pair);
+// Cluster size index for the same layer with its contraction split, or -1 where whole tiles (whole_ns) are as fast.
+int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn);
 int launch_linear_split(TcDevice* dev, int bn, int c, const void* plan, const void* X, void* Y, int tokens, int n_out, int k_in,
                         int act, const void* bias, int ldx, int ldy, bool plan_stable, bool transposed, cudaStream_t s);
 int launch_tn_split(TcDevice* dev, int bn, int c, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
