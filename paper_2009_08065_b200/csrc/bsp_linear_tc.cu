@@ -440,15 +440,19 @@ plan_expand_r_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
 // position; the values are read along k, where neighbours in the packed tile are neighbours in memory, turned
 // in shared memory (33-word rows: no bank conflicts either way) and written along n, 128 contiguous bytes a
 // plan row, zeros included.  Bound by a chain of four trips to memory (block pointers, index list, values,
-// stores), so all of a thread's values are asked for at once.  It replaces a clearing pass and 2-byte
-// scattered stores: 19 -> 4 us for a 3072 x 768 matrix of 16-row blocks.
-constexpr int kPlanTK = 64, kPlanTN = 64, kPlanTMaxBlocks = 32;
+// stores) and, with four CTAs per SM, by issue slots: all of a thread's values are asked for at once, the unit's
+// values are fetched into L2 while the lists are read, and a warp takes adjacent rows so that the table and the
+// block's place are looked up once per row-block.  (Looked up per element, with a division each, the values took 4 us
+// even from L2.)  Between the products of a backward pass (768 features, 16-row blocks, cold operands) a 3072 x 768
+// matrix takes 4 us from the wait on; it took 6.5, and 19 with a clearing pass and scattered 2-byte stores; the
+// pass over four matrices at 4096 tokens 165 -> 151 us.
+constexpr int kPlanTK = 64, kPlanTN = 64, kPlanTMaxBlocks = 32, kPlanTThreads = 512;
 struct PlanTGeometry {
   int n_out, k_in, block;
   int blocks_per_unit;      // whole row-blocks of a unit, 1 where a block is cut into segments
   int segments;             // 64-row segments of a row-block taller than 64 rows, else 1
 };
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kPlanTThreads, 4)
 plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restrict__ idx,
                      const uint16_t* __restrict__ vals, PlanTGeometry G, uint16_t* __restrict__ PT) {
   __shared__ int32_t s_col_pos[kPlanTMaxBlocks][kPlanTK];
@@ -461,23 +465,31 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
   const int rows_per_block = G.segments > 1 ? min(kPlanTN, G.block - seg * kPlanTN) : G.block;
   const int n0 = b0 * G.block + seg * kPlanTN;
   const int n_rows = nb * rows_per_block;
-  for (int e = threadIdx.x; e < nb * kPlanTK; e += 256) s_col_pos[0][e] = -1;
+  for (int e = threadIdx.x; e < nb * kPlanTK; e += kPlanTThreads) s_col_pos[0][e] = -1;
+  if (threadIdx.x == 0) prefetch_line(blk_ptr + b0);
   pdl_wait();
   pdl_launch_dependents();
   if (static_cast<int>(threadIdx.x) <= nb) s_ptr[threadIdx.x] = __ldg(blk_ptr + b0 + threadIdx.x);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  {
+    // the unit's values are one run too: its CTAs fetch a share of it each into L2 while the lists are read
+    const int lo = s_ptr[0], kept = s_ptr[nb] - lo;
+    const char* run = reinterpret_cast<const char*>(vals + static_cast<size_t>(G.block) * lo + static_cast<size_t>(seg) * kPlanTN * kept);
+    const long long bytes = 2LL * rows_per_block * kept, step = 128LL * kPlanTThreads * gridDim.y;
+    for (long long at = 128LL * threadIdx.x * gridDim.y + 128LL * blockIdx.y; at < bytes; at += step) prefetch_line(run + at);
+  }
   // the index lists of the unit's row-blocks are one run of the index array
   {
     const int lo = s_ptr[0], n_idx = s_ptr[nb] - lo;
-    for (int j0 = threadIdx.x; j0 < n_idx; j0 += 8 * 256) {
-      int k[8];
+    for (int j0 = threadIdx.x; j0 < n_idx; j0 += 4 * kPlanTThreads) {
+      int k[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) k[u] = j0 + u * 256 < n_idx ? __ldg(idx + lo + j0 + u * 256) - k0 : -1;
+      for (int u = 0; u < 4; ++u) k[u] = j0 + u * kPlanTThreads < n_idx ? __ldg(idx + lo + j0 + u * kPlanTThreads) - k0 : -1;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
+      for (int u = 0; u < 4; ++u) {
         if (k[u] < 0 || k[u] >= nk) continue;
-        const int j = lo + j0 + u * 256;
+        const int j = lo + j0 + u * kPlanTThreads;
         int q = 0;
         while (q + 1 < nb && s_ptr[q + 1] <= j) ++q;
         s_col_pos[q][k[u]] = j - s_ptr[q];
@@ -485,37 +497,46 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
     }
   }
   __syncthreads();
-  uint16_t v[kPlanTN / 8][2];
+  // a warp takes adjacent rows, a lane two columns: their places in the packed tile change only with the row-block
+  constexpr int kRows = kPlanTN / (kPlanTThreads / 32);
+  const int n_first = warp * kRows;
+  int q = n_first / rows_per_block, r = n_first - q * rows_per_block, kc = 0, p0 = -1, p1 = -1;
+  const uint16_t* row = vals;
+  auto enter = [&]() {
+    if (q >= nb) return;
+    const int lo = s_ptr[q];
+    kc = s_ptr[q + 1] - lo;
+    row = vals + static_cast<size_t>(G.block) * lo + static_cast<size_t>(r + seg * kPlanTN) * kc;
+    p0 = s_col_pos[q][lane];
+    p1 = s_col_pos[q][lane + 32];
+  };
+  enter();
+  uint32_t v[kRows][2];
 #pragma unroll
-  for (int i = 0; i < kPlanTN / 8; ++i) {
-    const int n = warp + 8 * i;
-    const int q = n / rows_per_block, r = n - q * rows_per_block + seg * kPlanTN;
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      v[i][u] = 0;
-      if (n < n_rows) {
-        const int p = s_col_pos[q][u * 32 + lane];
-        const int lo = s_ptr[q], kc = s_ptr[q + 1] - lo;
-        if (p >= 0) v[i][u] = __ldg(vals + static_cast<size_t>(G.block) * lo + static_cast<size_t>(r) * kc + p);
-      }
-    }
+  for (int i = 0; i < kRows; ++i) {
+    v[i][0] = v[i][1] = 0u;
+    if (n_first + i >= n_rows) continue;
+    if (p0 >= 0) v[i][0] = __ldg(row + p0);
+    if (p1 >= 0) v[i][1] = __ldg(row + p1);
+    row += kc;
+    if (++r == rows_per_block) { r = 0; ++q; enter(); }
   }
 #pragma unroll
-  for (int i = 0; i < kPlanTN / 8; ++i) {
-    s_t[lane][warp + 8 * i] = v[i][0];
-    s_t[lane + 32][warp + 8 * i] = v[i][1];
+  for (int i = 0; i < kRows; ++i) {
+    s_t[lane][n_first + i] = static_cast<uint16_t>(v[i][0]);
+    s_t[lane + 32][n_first + i] = static_cast<uint16_t>(v[i][1]);
   }
   __syncthreads();
   uint16_t* out = PT + static_cast<size_t>(k0) * G.n_out + n0;
   if (n_rows % 8 == 0 && n0 % 8 == 0 && G.n_out % 8 == 0) {
     const int per_row = n_rows >> 3;
-    for (int e = threadIdx.x; e < nk * per_row; e += 256) {
+    for (int e = threadIdx.x; e < nk * per_row; e += kPlanTThreads) {
       const int k = e / per_row, c = (e - k * per_row) << 3;
       const uint32_t* w = reinterpret_cast<const uint32_t*>(&s_t[k][c]);
       *reinterpret_cast<uint4*>(out + static_cast<size_t>(k) * G.n_out + c) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   } else {
-    for (int e = threadIdx.x; e < nk * n_rows; e += 256) {
+    for (int e = threadIdx.x; e < nk * n_rows; e += kPlanTThreads) {
       const int k = e / n_rows, c = e - k * n_rows;
       out[static_cast<size_t>(k) * G.n_out + c] = s_t[k][c];
     }
@@ -697,7 +718,7 @@ extern "C" int bsp_linear_plan_t(const int32_t* blk_ptr, const int32_t* idx, con
   const int units = (nb + G.blocks_per_unit - 1) / G.blocks_per_unit * G.segments;
   const dim3 grid(units, (k_in + kPlanTK - 1) / kPlanTK);
   if (grid.y > 65535) return BSP_ERR_UNSUPPORTED;
-  BSP_CUDA_TRY(launch_pdl(plan_expand_t_kernel, grid, dim3(256), 0, static_cast<cudaStream_t>(stream), blk_ptr, idx,
+  BSP_CUDA_TRY(launch_pdl(plan_expand_t_kernel, grid, dim3(kPlanTThreads), 0, static_cast<cudaStream_t>(stream), blk_ptr, idx,
                           static_cast<const uint16_t*>(vals), G, static_cast<uint16_t*>(plan_t)));
   return BSP_OK;
 }
