@@ -7,12 +7,17 @@
 //            per CTA, then one global addition per bin that was hit (a hundred or so);
 //   select   one thread-block cluster per matrix: every CTA looks the answer's bin up in the histogram and
 //            lists its keys of that bin (a few per cent) in shared memory; CTA 0 gathers the lists through
-//            distributed shared memory and finds the answer among them in two more digits (10 and 9 bits).
+//            distributed shared memory and finds the answer among them: a digit of 10 bits more, then a warp ranks
+//            the few keys that are left (or a last digit of 9 bits, where many are alike).
 // Matrices whose flag region is too small for the histogram are selected by one CTA straight from the sums, and
 // so is what overflows a list (a matrix of equal groups).  Latency bounds all of this.  Measured on 147456
 // groups: one CTA with four 8-bit digits over all keys 197 us; a cluster that also made the histogram 12 us;
 // many CTAs with their lists in global memory, the last one finishing, 9 us (fences and atomics through L2
-// instead of cluster barriers).
+// instead of cluster barriers); one launch for everything, a cluster of 16 CTAs that sums its matrix itself, 16 us (W
+// through 16 SMs, histograms through distributed shared memory).  The three launches: 15.0 -> 11.6 us for 3072 x 768 in
+// 16-row blocks, 54.6 -> 48.3 for 72 matrices of a BERT-base stack, when the sums no longer waited for the clearing, the
+// list was stored with predicated stores, all keys of a thread were asked for in one round, the gather kept four remote
+// loads in flight and the last digit became a ranking.
 #include <atomic>
 
 #include "bsp_tc.cuh"
@@ -26,6 +31,7 @@ constexpr int kBins1 = 1 << kBits1, kBins2 = 1 << kBits2, kBins3 = 1 << kBits3;
 constexpr int kList = 4096, kCandidates = 12288;              // keys on a CTA's list, and that CTA 0 gathers
 constexpr int kSelSmem = (kList + kCandidates) * 4;
 constexpr int kSelMaxCluster = 8;
+constexpr int kSelLoads = 6;                                 // 16-byte loads of a thread in flight: a round of the list
 // Copies of a histogram: a CTA of the sums adds to one of them (its number modulo the copies).  A sum of squares
 // falls into a hundred bins or so, and 192 CTAs adding to the same words kept the next launch waiting for 1 us.
 constexpr int kReplicas = 4;
@@ -47,6 +53,7 @@ struct SelectJob {
 template <int N>
 struct SelectBatchT {
   int n_jobs, block;
+  int cleared;                      // the kernel before the sums is the clearing one
   int max_part_cols, total_items;   // streaming sums kernel
   int* status;
   int first_block[N];        // apart from the wide records: a search stays within a few lines of the constant cache
@@ -88,9 +95,12 @@ __device__ __forceinline__ void add_bins(const uint32_t* hist, uint32_t* head) {
   }
 }
 
+// Behind the clearing kernel the sums have started only because everything before that one is complete
+// (pdl_launch_dependents comes after pdl_wait in every kernel): W may be read and the sums written at once, and only
+// the additions to the histogram wait for the zeros.  A warp of its own waits early and lets the select take its seats.
 // Orientation C, one CTA per row-block of every matrix.
 template <int N>
-__global__ void __launch_bounds__(kSumThreads)
+__global__ void __launch_bounds__(kSumThreads + 32)
 sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
   __shared__ __align__(16) uint32_t hist[kBins1];
   const int jn = owner(B.first_block, B.n_jobs, static_cast<int>(blockIdx.x));
@@ -100,10 +110,12 @@ sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
   float* out = J.S + static_cast<size_t>(b) * J.cols;
   const bool count = J.head != nullptr;
   if (count) clear_bins(hist);
-  pdl_wait();
-  pdl_launch_dependents();
+  if (!B.cleared) pdl_wait();
   __syncthreads();
-  if (J.vec) {
+  if (threadIdx.x >= kSumThreads) {
+    pdl_wait();
+    pdl_launch_dependents();
+  } else if (J.vec) {
     for (int q = threadIdx.x; q < (J.cols >> 3); q += kSumThreads) {
       float acc[8];
       sumsq8(wblk + (q << 3), B.block, J.ldw, acc);
@@ -124,6 +136,7 @@ sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
   }
   if (!count) return;
   __syncthreads();
+  pdl_wait();
   add_bins(hist, J.head + (blockIdx.x % J.replicas) * kBins1);
 }
 
@@ -173,11 +186,12 @@ sums_stream_kernel(const __grid_constant__ SelectBatchT<N> B) {
                    : "memory");
   };
   int jn = owner(B.first_block, B.n_jobs, i0), b, c0, pc;
-  pdl_wait();
-  pdl_launch_dependents();
+  if (!B.cleared) pdl_wait();
   __syncthreads();
   locate(i0, jn, b, c0, pc);
   if (warp == 0 && i0 < i1) fetch(jn, b, c0, pc, 0);
+  pdl_wait();
+  pdl_launch_dependents();
   uint32_t parity[2] = {0u, 0u};
   for (int item = i0; item < i1; ++item) {
     const int slot = (item - i0) & 1;
@@ -235,16 +249,19 @@ sums_stream_kernel(const __grid_constant__ SelectBatchT<N> B) {
 }
 
 // Orientation R: one thread per group, neighbouring threads on neighbouring groups of a row.
-__global__ void __launch_bounds__(256)
+constexpr int kSumRThreads = 256;
+__global__ void __launch_bounds__(kSumRThreads + 32)
 sums_r_kernel(const uint16_t* __restrict__ W, int rows, int per_row, int ldw, int block, int vec, float* __restrict__ S,
               uint32_t* head, int replicas) {
   __shared__ __align__(16) uint32_t hist[kBins1];
   if (head != nullptr) clear_bins(hist);
-  pdl_wait();
-  pdl_launch_dependents();
+  else pdl_wait();                                           // (no clearing kernel)
   __syncthreads();
-  const long long g = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (g < static_cast<long long>(rows) * per_row) {
+  const long long g = static_cast<long long>(blockIdx.x) * kSumRThreads + threadIdx.x;
+  if (threadIdx.x >= kSumRThreads) {
+    pdl_wait();
+    pdl_launch_dependents();
+  } else if (g < static_cast<long long>(rows) * per_row) {
     const long long i = g / per_row;
     const int a = static_cast<int>(g - i * per_row);
     const float v = group_sumsq_contig(W + static_cast<size_t>(i) * ldw + static_cast<size_t>(a) * block, block, vec);
@@ -253,13 +270,14 @@ sums_r_kernel(const uint16_t* __restrict__ W, int rows, int per_row, int ldw, in
   }
   if (head == nullptr) return;
   __syncthreads();
+  pdl_wait();
   add_bins(hist, head + (blockIdx.x % replicas) * kBins1);
 }
 
 // ---------------------------------------------------------------------------------------- select
 // The bin of a histogram that holds the want-th smallest key (1-based) and the rank inside that bin; the whole
-// CTA takes part and gets the answer.  A warp adds up a 32nd of the bins, every warp scans the 32 sums, and the
-// one that holds the answer scans its bins.
+// CTA takes part and gets the answer.  A warp adds up a 32nd of the bins, every warp adds up the sums before its own,
+// and the one that holds the answer scans its bins.
 struct Pick {
   uint32_t bin, want;
 };
@@ -277,14 +295,7 @@ __device__ __forceinline__ Pick pick_bin(const uint32_t* hist, uint32_t want, ui
   }
   if (lane == 0) s_sum[warp] = sum;
   __syncthreads();
-  const uint32_t w = s_sum[lane];
-  uint32_t incl = w;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += up;
-  }
-  uint32_t before = __shfl_sync(0xffffffffu, incl - w, warp);
+  uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? s_sum[lane] : 0u);
   if (before < want && want <= before + sum) {               // all lanes of a warp agree; exactly one warp goes on
     uint32_t mine = c[0];
     int round = 0;
@@ -358,13 +369,24 @@ __device__ __forceinline__ uint32_t ld_cluster(uint32_t addr) {
   return v;
 }
 
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// The least float whose square, rounded, reaches the sum of squares with these bits.
+__device__ __forceinline__ float threshold_of(uint32_t bits) {
+  const float s_r = __uint_as_float(bits);
+  float t = __fsqrt_rn(s_r);
+  while (__fmul_rn(t, t) < s_r) t = __uint_as_float(__float_as_uint(t) + 1u);  // next float up (t >= 0)
+  return t;
+}
+
 template <int N>
 __global__ void __launch_bounds__(kSelThreads)
 select_kernel(const __grid_constant__ SelectBatchT<N> B) {
   __shared__ __align__(16) uint32_t hist[kBins1];
   __shared__ uint32_t s_sum[32];
   __shared__ uint32_t s_pick[2];
-  __shared__ uint32_t s_n;
+  __shared__ uint32_t s_n, s_last_n, s_last[32], s_len[kSelMaxCluster];
   extern __shared__ uint32_t s_list[];                       // [kList], then in CTA 0 [kCandidates]
   uint32_t* s_cand = s_list + kList;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -372,9 +394,11 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
   const SelectJob& J = B.job[blockIdx.x / n_cta];
   const uint32_t* keys = reinterpret_cast<const uint32_t*>(J.S);
   const long long n = J.n;
-  if (threadIdx.x == 0) s_n = 0u;
+  if (threadIdx.x == 0) s_n = s_last_n = 0u;
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   pdl_wait();
   pdl_launch_dependents();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");   // every CTA of the cluster has started
   if (J.r <= 0) {                                            // the same for the whole cluster
     if (rank == 0 && threadIdx.x == 0) *J.out = -1.0f;
     return;
@@ -387,16 +411,13 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
     const uint4* v4 = reinterpret_cast<const uint4*>(keys);
     const long long n4 = n >> 2, step = static_cast<long long>(n_cta) * kSelThreads;
     long long i0 = static_cast<long long>(rank) * kSelThreads;
-    uint32_t k[16], valid = 0u;
+    uint32_t k[4 * kSelLoads];
     auto load = [&]() {
-      valid = 0u;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (i0 + u * step + threadIdx.x < n4) {
-          const uint4 v = __ldcg(v4 + i0 + u * step + threadIdx.x);
-          k[4 * u] = v.x; k[4 * u + 1] = v.y; k[4 * u + 2] = v.z; k[4 * u + 3] = v.w;
-          valid |= 0xfu << (4 * u);
-        }
+      for (int u = 0; u < kSelLoads; ++u) {
+        uint4 v = make_uint4(~0u, ~0u, ~0u, ~0u);             // (no key: the sign bit is set)
+        if (i0 + u * step + threadIdx.x < n4) v = __ldcg(v4 + i0 + u * step + threadIdx.x);
+        k[4 * u] = v.x; k[4 * u + 1] = v.y; k[4 * u + 2] = v.z; k[4 * u + 3] = v.w;
       }
     };
     load();
@@ -411,28 +432,43 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
     __syncthreads();
     p = pick_bin<kBins1>(hist, p.want, s_sum, s_pick);
     prefix = p.bin;
+    if (rank == 0) {                                         // the bins of the digits to come
+      hist[threadIdx.x] = 0u;
+      if (threadIdx.x < kBins3) hist[kBins2 + threadIdx.x] = 0u;
+    }
+    const uint32_t in_bin = prefix << (kBits2 + kBits3);
     for (;;) {
+      // (32 warps share the issue slots, so instructions count: a warp's places on the list come from one addition)
       uint32_t hit = 0u;
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
-        if ((valid >> i & 1u) && (k[i] >> (kBits2 + kBits3)) == prefix) hit |= 1u << i;
-      const uint32_t mine = __popc(hit);
-      uint32_t incl = mine;
+      for (int u = 0; u < kSelLoads; ++u) {
+        if (u > 0 && i0 + u * step + (threadIdx.x & ~31u) >= n4) break;   // none of the warp's lanes has a key here
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
+        for (int i = 4 * u; i < 4 * u + 4; ++i)
+          if ((k[i] ^ in_bin) < (1u << (kBits2 + kBits3))) hit |= 1u << i;
       }
-      uint32_t at = 0u;
-      if (lane == 31 && incl) at = atomicAdd(&s_n, incl);
-      at = __shfl_sync(0xffffffffu, at, 31) + incl - mine;
+      if (__any_sync(0xffffffffu, hit != 0u)) {
+        const uint32_t mine = __popc(hit);
+        uint32_t incl = mine;
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
-        if (hit >> i & 1u) {
-          if (at < kList) s_list[at] = k[i];
-          ++at;
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += up;
         }
-      i0 += 4 * step;
+        uint32_t at = 0u;
+        if (lane == 31) at = atomicAdd(&s_n, incl);
+        const uint32_t end = __shfl_sync(0xffffffffu, at + incl, 31);
+        at = __shfl_sync(0xffffffffu, at, 31) + incl - mine;
+        if (end <= kList) {                                  // (a list that overflows is not used)
+          // predicated by hand: as branches, the 24 stores of a warp that keeps ten keys took 0.8 us
+          uint32_t to = tc::smem_u32(s_list + at);
+#pragma unroll
+          for (int i = 0; i < 4 * kSelLoads; ++i)
+            asm volatile("{\n.reg .pred p;\n.reg .b32 t;\nand.b32 t, %2, %3;\nsetp.ne.u32 p, t, 0;\n@p st.shared.u32 [%0], %1;\n@p add.u32 %0, %0, 4;\n}"
+                         : "+r"(to) : "r"(k[i]), "r"(hit), "r"(1u << i) : "memory");
+        }
+      }
+      i0 += kSelLoads * step;
       if (i0 >= n4) break;
       load();
     }
@@ -443,22 +479,28 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
         if (at < kList) s_list[at] = tail;
       }
     }
-    cluster_sync();                                          // the lists are complete
+    __syncthreads();
+    if (threadIdx.x == 0) st_cluster(map_to_cta(&s_len[rank], 0u), s_n);
+    cluster_sync();                                          // the lists and their lengths are complete
     if (rank == 0) {
-      const uint32_t length = lane < static_cast<int>(n_cta) ? ld_cluster(map_to_cta(&s_n, lane)) : 0u;
+      const uint32_t length = lane < static_cast<int>(n_cta) ? s_len[lane] : 0u;
       found = __reduce_add_sync(0xffffffffu, length);
       if (__any_sync(0xffffffffu, length > kList) || found > kCandidates) {
         found = 0xffffffffu;
       } else {
-        // four lists at a time, eight warps each; a list's keys go behind those of the lists before it
-        uint32_t at = 0u;
-        for (uint32_t q = 0; q < n_cta; ++q) {
+        // eight warps a list, four lists at a time; a list's keys go behind those of the lists before it
+        for (uint32_t q = warp & 3u; q < n_cta; q += 4u) {
           const uint32_t len = __shfl_sync(0xffffffffu, length, static_cast<int>(q));
-          if ((q & 3u) == static_cast<uint32_t>(warp & 3)) {
-            const uint32_t src = map_to_cta(s_list, q);
-            for (uint32_t i = static_cast<uint32_t>((warp >> 2) * 32 + lane); i < len; i += kSelThreads / 4) s_cand[at + i] = ld_cluster(src + 4u * i);
+          const uint32_t at = __reduce_add_sync(0xffffffffu, lane < static_cast<int>(q) ? length : 0u);
+          const uint32_t src = map_to_cta(s_list, q);
+          for (uint32_t i0 = static_cast<uint32_t>((warp >> 2) * 32 + lane); i0 < len; i0 += 4 * (kSelThreads / 4)) {
+            uint32_t c[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4u; ++u) c[u] = i0 + u * (kSelThreads / 4) < len ? ld_cluster(src + 4u * (i0 + u * (kSelThreads / 4))) : 0u;
+#pragma unroll
+            for (uint32_t u = 0; u < 4u; ++u)
+              if (i0 + u * (kSelThreads / 4) < len) s_cand[at + i0 + u * (kSelThreads / 4)] = c[u];
           }
-          at += len;
         }
       }
     }
@@ -470,6 +512,8 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
       __syncthreads();
       p = pick_bin<kBins1>(hist, p.want, s_sum, s_pick);
       prefix = p.bin;
+      hist[threadIdx.x] = 0u;
+      if (threadIdx.x < kBins3) hist[kBins2 + threadIdx.x] = 0u;
     }
     cluster_sync();
   }
@@ -477,10 +521,8 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
     cluster_sync();                                          // CTA 0 has read this CTA's list
     return;
   }
-  // two digits more, each with bins of its own, over the listed keys or all of them
-  __syncthreads();
-  hist[threadIdx.x] = 0u;
-  if (threadIdx.x < kBins3) hist[kBins2 + threadIdx.x] = 0u;
+  // the next digit over the listed keys or all of them; then a warp ranks the few keys that are left, or the last
+  // digit has bins of its own
   __syncthreads();
   auto over_keys = [&](int above, uint32_t upper, auto f) {
     if (found != 0xffffffffu) {
@@ -494,14 +536,28 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
   __syncthreads();
   p = pick_bin<kBins2>(hist, p.want, s_sum, s_pick);
   prefix = (prefix << kBits2) | p.bin;
-  over_keys(kBits3, prefix, [&](uint32_t k) { atomicAdd(&hist[kBins2 + (k & (kBins3 - 1))], 1u); });
+  over_keys(kBits3, prefix, [&](uint32_t k) {
+    const uint32_t at = atomicAdd(&s_last_n, 1u);
+    if (at < 32u) s_last[at] = k;
+  });
   __syncthreads();
-  p = pick_bin<kBins3>(hist + kBins2, p.want, s_sum, s_pick);
-  if (threadIdx.x == 0) {
-    const float s_r = __uint_as_float((prefix << kBits3) | p.bin);
-    float t = __fsqrt_rn(s_r);
-    while (__fmul_rn(t, t) < s_r) t = __uint_as_float(__float_as_uint(t) + 1u);  // next float up (t >= 0)
-    *J.out = t;
+  const uint32_t left = s_last_n;
+  if (left <= 32u) {
+    if (warp == 0) {
+      const uint32_t k = lane < static_cast<int>(left) ? s_last[lane] : ~0u;
+      uint32_t less = 0u, upto = 0u;
+      for (uint32_t j = 0; j < left; ++j) {
+        const uint32_t o = __shfl_sync(0xffffffffu, k, static_cast<int>(j));
+        less += o < k ? 1u : 0u;
+        upto += o <= k ? 1u : 0u;
+      }
+      if (lane < static_cast<int>(left) && less < p.want && p.want <= upto) *J.out = threshold_of(k);   // (equal keys agree)
+    }
+  } else {
+    over_keys(kBits3, prefix, [&](uint32_t k) { atomicAdd(&hist[kBins2 + (k & (kBins3 - 1))], 1u); });
+    __syncthreads();
+    p = pick_bin<kBins3>(hist + kBins2, p.want, s_sum, s_pick);
+    if (threadIdx.x == 0) *J.out = threshold_of((prefix << kBits3) | p.bin);
   }
   cluster_sync();
 }
@@ -614,7 +670,7 @@ int launch_sums_c(SelectBatchT<N>& B, int sms, cudaStream_t s) {
   }
   int at = 0;
   for (int i = 0; i < B.n_jobs; ++i) { B.first_block[i] = at; at += B.job[i].n_blocks; }
-  BSP_CUDA_TRY(launch_pdl(sums_c_kernel<N>, dim3(blocks), dim3(kSumThreads), 0, s, B));
+  BSP_CUDA_TRY(launch_pdl(sums_c_kernel<N>, dim3(blocks), dim3(kSumThreads + 32), 0, s, B));
   return BSP_OK;
 }
 
@@ -650,12 +706,14 @@ extern "C" int bsp_percentile_threshold(const void* W, int rows, int cols, int l
   B.n_jobs = 1;
   B.block = block;
   B.job[0] = select_job(W, cols, ldw, nb, ng, rate, ws, threshold_out);
-  if (B.job[0].head != nullptr) BSP_CUDA_TRY(launch_pdl(select_clear_kernel<1>, dim3(1), dim3(kSelThreads), 0, s, B));
+  B.cleared = B.job[0].head != nullptr ? 1 : 0;
+  if (B.cleared) BSP_CUDA_TRY(launch_pdl(select_clear_kernel<1>, dim3(1), dim3(kSelThreads), 0, s, B));
   if (orient == BSP_ORIENT_C) {
     st = launch_sums_c(B, sms, s);
     if (st != BSP_OK) return st;
   } else {
-    BSP_CUDA_TRY(launch_pdl(sums_r_kernel, dim3(static_cast<unsigned>((groups + 255) / 256)), dim3(256), 0, s, B.job[0].W, rows, nb,
+    BSP_CUDA_TRY(launch_pdl(sums_r_kernel, dim3(static_cast<unsigned>((groups + kSumRThreads - 1) / kSumRThreads)),
+                            dim3(kSumRThreads + 32), 0, s, B.job[0].W, rows, nb,
                             ldw, block, contig_vec(W, ldw, block), B.job[0].S, B.job[0].head,
                             B.job[0].replicas));
   }
@@ -688,6 +746,7 @@ extern "C" int bsp_percentile_threshold_batched(const bsp_layer_job* jobs, int n
       const bsp_layer_job& u = jobs[j0 + i];
       B.job[i] = select_job(u.W, u.cols, u.ldw, u.rows / block, u.cols, rates[j0 + i], u.ws, const_cast<float*>(u.threshold_dev));
     }
+    B.cleared = 1;
     BSP_CUDA_TRY(launch_pdl(select_clear_kernel<kSelectBatch>, dim3(B.n_jobs), dim3(kSelThreads), 0, s, B));
     st = launch_sums_c(B, sms, s);
     if (st != BSP_OK) return st;
