@@ -229,10 +229,15 @@ __device__ __forceinline__ void sumsq8_rows(const uint16_t* __restrict__ p, int 
     }
   }
 }
+// kTall: 32 rows in flight instead of 16, for blocks of 32 rows and more (such a matrix has few of them, and a thread's
+// rows are a chain of trips to memory; not for the others, since it takes 128 registers).
+template <bool kTall = false>
 __device__ __forceinline__ void sumsq8(const uint16_t* __restrict__ p, int d, int ldw, float (&acc)[8]) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
   int r = 0;
+  if (kTall)
+    for (; r + 32 <= d; r += 32) sumsq8_rows<32>(p + static_cast<size_t>(r) * ldw, ldw, acc);   // 512 bytes in flight
   for (; r + 16 <= d; r += 16) sumsq8_rows<16>(p + static_cast<size_t>(r) * ldw, ldw, acc);   // 256 bytes in flight
   for (; r + 4 <= d; r += 4) sumsq8_rows<4>(p + static_cast<size_t>(r) * ldw, ldw, acc);
   for (; r < d; ++r) sumsq8_rows<1>(p + static_cast<size_t>(r) * ldw, ldw, acc);

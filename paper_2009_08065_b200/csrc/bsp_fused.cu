@@ -15,6 +15,7 @@
 namespace bsp {
 namespace {
 
+constexpr int kStage1Ctas = 148;  // stage 1: below it some SMs have no row-block
 constexpr int kRowsPerPass = 4;   // rows staged in shared memory at a time
 
 // The job table travels as a kernel parameter; a single-matrix call gets a table of one job (0.2 KB instead
@@ -23,6 +24,8 @@ template <int N>
 struct BatchT {
   int n_jobs, block, squared;
   float eps;
+  int parts;                // stage 1 without flags: CTAs per row-block, each with part_chunks of its 8-column pieces
+  int part_chunks;
   int first_block[N + 1];   // CTA index of each job's first row-block
   FusedJob job[N];
 };
@@ -38,14 +41,18 @@ __device__ __forceinline__ int find_job(const BatchT<N>& B, int cta) {
   return lo;
 }
 
-template <int N>
+// (kParts as a template parameter: with the ranges as run-time values whole row-blocks took up to 2 us longer)
+template <int N, bool kParts, bool kTall>
 __global__ void __launch_bounds__(256)
 fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
   __shared__ int s_cnt[8];
   __shared__ double s_pen[8];
-  const int j = find_job(B, blockIdx.x);
+  const int cta = kParts ? static_cast<int>(blockIdx.x) / B.parts : static_cast<int>(blockIdx.x);
+  const int q0 = kParts ? (static_cast<int>(blockIdx.x) - cta * B.parts) * B.part_chunks : 0;
+  const int j = find_job(B, cta);
   const FusedJob& J = B.job[j];
-  const int b = blockIdx.x - B.first_block[j];
+  const int b = cta - B.first_block[j];
+  const int q_end = kParts ? min(J.cols >> 3, q0 + B.part_chunks) : J.cols >> 3;
   pdl_wait();
   pdl_launch_dependents();
   const bool want_flags = J.flags != nullptr;
@@ -60,9 +67,9 @@ fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
   }
   int count = 0;
   float pen = 0.0f;
-  for (int q = threadIdx.x; q < (J.cols >> 3); q += blockDim.x) {
+  for (int q = q0 + threadIdx.x; q < q_end; q += blockDim.x) {
     float acc[8];
-    sumsq8(J.W + static_cast<size_t>(b) * B.block * J.ldw + (q << 3), B.block, J.ldw, acc);
+    sumsq8<kTall>(J.W + static_cast<size_t>(b) * B.block * J.ldw + (q << 3), B.block, J.ldw, acc);
     const size_t g0 = static_cast<size_t>(b) * J.cols + (q << 3);
     if (want_flags) {
       uint32_t lo = 0, hi = 0;
@@ -329,9 +336,22 @@ int launch_stage1(const FusedJob* jobs, int n_jobs, int block, float eps, int sq
   fill_batch(B, jobs, n_jobs, block, &total, &max_cols);
   B.eps = eps;
   B.squared = squared;
-  int threads = ((max_cols >> 3) + 31) / 32 * 32;
+  const int chunks = max_cols >> 3;
+  int threads = (chunks + 31) / 32 * 32;
   threads = threads > 256 ? 256 : threads;
-  BSP_CUDA_TRY(launch_pdl(fused_stage1_kernel<N>, dim3(total), dim3(threads), 0, s, B));
+  B.parts = 1;
+  B.part_chunks = chunks;
+  if (N == 1 && jobs[0].flags == nullptr && jobs[0].partial == nullptr && total < kStage1Ctas && chunks > 128) {
+    // A matrix of few wide row-blocks leaves SMs idle: they are cut into column ranges of a piece per thread (11 blocks of
+    // 96 x 3072: 13.7 -> 8.9 us; ranges of 64 or 32 pieces cost 0.7 us more than whole blocks of 1024 columns).  Not where
+    // a row-block is counted as a whole.
+    threads = 128;
+    B.parts = (chunks + 127) / 128;
+    B.part_chunks = 128;
+  }
+  auto* kernel = block >= 32 && N == 1 ? (B.parts > 1 ? fused_stage1_kernel<N, N == 1, N == 1> : fused_stage1_kernel<N, false, N == 1>)
+                                       : (B.parts > 1 ? fused_stage1_kernel<N, N == 1, false> : fused_stage1_kernel<N, false, false>);
+  BSP_CUDA_TRY(launch_pdl(kernel, dim3(total * B.parts), dim3(threads), 0, s, B));
   return BSP_OK;
 }
 
@@ -342,6 +362,8 @@ int launch_stage2(const FusedJob* jobs, int n_jobs, int block, cudaStream_t s) {
   fill_batch(B, jobs, n_jobs, block, &total, &max_cols);
   B.eps = 0.0f;
   B.squared = 0;
+  B.parts = 1;
+  B.part_chunks = 0;
   int splits = 1;
   size_t smem = 0;
   for (int i = 0; i < n_jobs; ++i) {

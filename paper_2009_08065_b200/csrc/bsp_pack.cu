@@ -78,34 +78,39 @@ flags_threshold_kernel(const uint16_t* __restrict__ W, Geometry G, float thresho
 // select of three digits finds the smallest kept one, and a scan in index order decides which of its equals
 // are kept.  O(groups) work per digit; ranking every sum against every other one (O(groups^2)) took
 // 0.5-1 ms on the larger matrices.
+// Blocks of 1024 groups or more get 1024 threads: the digits are passes over the keys, and a GPU that is still busy with
+// the launch before puts several of the smaller CTAs on one SM, where they share its issue slots (16 strips of 3072
+// groups, packed behind their norms: 101 -> 55 us; 192 strips of 1024 groups 30 -> 21).  With more blocks than two per
+// SM the smaller CTAs are level or ahead.
 constexpr int kTopkDigit = 11;                       // 31 bits = 11 + 10 + 10
 constexpr int kTopkBins = 1 << kTopkDigit;
-__global__ void __launch_bounds__(kPackThreads)
+template <int T>
+__global__ void __launch_bounds__(T)
 flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
                   uint8_t* __restrict__ keep, int32_t* __restrict__ counts) {
   extern __shared__ uint32_t s_key[];                // [n_groups]
   __shared__ uint32_t hist[kTopkBins];
   __shared__ int s_warp[32];
   __shared__ uint32_t s_pick[2];
-  constexpr int kPer = kTopkBins / kPackThreads;
+  constexpr int kPer = kTopkBins / T;
   const int b = blockIdx.x, n = G.n_groups;
   pdl_wait();
   pdl_launch_dependents();
   if (keep_count <= 0 || keep_count >= n) {
     const uint8_t all = keep_count > 0 ? 1 : 0;
-    for (int g = threadIdx.x; g < n; g += kPackThreads) keep[group_slot(G, b, g)] = all;
+    for (int g = threadIdx.x; g < n; g += T) keep[group_slot(G, b, g)] = all;
     if (threadIdx.x == 0) counts[b] = all ? n : 0;
     return;
   }
   if (G.orient == BSP_ORIENT_C && G.vec == 8) {
-    for (int q = threadIdx.x; q < (n >> 3); q += kPackThreads) {
+    for (int q = threadIdx.x; q < (n >> 3); q += T) {
       float acc[8];
       sumsq8(W + static_cast<size_t>(b) * G.block * G.ldw + (q << 3), G.block, G.ldw, acc);
 #pragma unroll
       for (int i = 0; i < 8; ++i) s_key[(q << 3) + i] = __float_as_uint(acc[i]);
     }
   } else {
-    for (int g = threadIdx.x; g < n; g += kPackThreads) s_key[g] = __float_as_uint(group_sum(W, G, b, g));
+    for (int g = threadIdx.x; g < n; g += T) s_key[g] = __float_as_uint(group_sum(W, G, b, g));
   }
   uint32_t want = static_cast<uint32_t>(n - keep_count + 1);   // the smallest kept sum is the want-th smallest
   uint32_t prefix = 0u;
@@ -116,10 +121,10 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
     const int above = shift;                         // bits above `above` are decided
     shift -= bits;
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) hist[threadIdx.x + i * kPackThreads] = 0u;
+    for (int i = 0; i < kPer; ++i) hist[threadIdx.x + i * T] = 0u;
     __syncthreads();
     const uint32_t mask = (1u << bits) - 1u;
-    for (int g = threadIdx.x; g < n; g += kPackThreads) {
+    for (int g = threadIdx.x; g < n; g += T) {
       const uint32_t u = s_key[g];
       if (above >= 31 || (u >> above) == prefix) atomicAdd(&hist[(u >> shift) & mask], 1u);
     }
@@ -144,12 +149,12 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
   // groups above the smallest kept sum stay; of the e groups equal to it the first e - want + 1 do
   // (the select counted want - 1 of them as smaller)
   int larger = 0;
-  for (int g = threadIdx.x; g < n; g += kPackThreads) larger += s_key[g] > prefix ? 1 : 0;
+  for (int g = threadIdx.x; g < n; g += T) larger += s_key[g] > prefix ? 1 : 0;
   int total;
   block_exclusive_scan(larger, s_warp, &total);
   const int equals_kept = keep_count - total;
   int seen = 0;
-  for (int g0 = 0; g0 < n; g0 += kPackThreads) {
+  for (int g0 = 0; g0 < n; g0 += T) {
     const int g = g0 + threadIdx.x;
     const uint32_t u = g < n ? s_key[g] : 0u;
     const int eq = g < n && u == prefix ? 1 : 0;
@@ -159,6 +164,12 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
     if (g < n) keep[group_slot(G, b, g)] = u > prefix || (eq && rank < equals_kept) ? 1 : 0;
   }
   if (threadIdx.x == 0) counts[b] = keep_count;
+}
+
+cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, uint8_t* flags, int32_t* counts, cudaStream_t s) {
+  const size_t smem = sizeof(uint32_t) * G.n_groups;
+  return G.n_groups >= 1024 && G.n_blocks <= 296 ? launch_pdl(flags_topk_kernel<1024>, dim3(G.n_blocks), dim3(1024), smem, s, w, G, keep_count, flags, counts)
+                            : launch_pdl(flags_topk_kernel<kPackThreads>, dim3(G.n_blocks), dim3(kPackThreads), smem, s, w, G, keep_count, flags, counts);
 }
 
 // (2) counts -> blk_ptr (exclusive scan) and the kept-weight total: matrices with more blocks than the
@@ -338,8 +349,7 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
     FusedJob j{w, rows, cols, ldw, G.n_blocks, threshold, threshold_dev, nullptr, nullptr, nullptr, nullptr, nullptr,
                flags, counts, blk_ptr, idx, static_cast<uint16_t*>(vals), kept_weights, nullptr};
     if (keep_per_block >= 0) {
-      BSP_CUDA_TRY(launch_pdl(flags_topk_kernel, dim3(G.n_blocks), dim3(kPackThreads), sizeof(uint32_t) * G.n_groups, s, w, G,
-                              keep_per_block, flags, counts));
+      BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, s));
     } else {
       st = fused_stage1(&j, 1, block, 0.0f, 0, s);
       if (st != BSP_OK) return st;
@@ -349,8 +359,7 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
   // a CTA per block, threads for its groups: up to 1024 of them, since a matrix of few tall blocks has few CTAs
   const int threads = G.n_groups >= 1024 ? 1024 : G.n_groups <= 128 ? 128 : (G.n_groups + 31) / 32 * 32;
   if (keep_per_block >= 0) {
-    BSP_CUDA_TRY(launch_pdl(flags_topk_kernel, dim3(G.n_blocks), dim3(kPackThreads), sizeof(uint32_t) * G.n_groups, s, w, G,
-                            keep_per_block, flags, counts));
+    BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, s));
   } else {
     BSP_CUDA_TRY(launch_pdl(flags_threshold_kernel, dim3(G.n_blocks), dim3(threads), 0, s, w, G, threshold, threshold_dev, flags, counts));
   }

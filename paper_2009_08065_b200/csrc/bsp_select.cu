@@ -43,7 +43,7 @@ constexpr int kSumPerSm = 3;                                 // its CTAs per SM:
 struct SelectJob {
   const uint16_t* W;
   int cols, ldw, n_blocks, vec;
-  int parts, part_cols;      // streaming sums kernel: column ranges of a row-block
+  int parts, part_cols;      // sums in orientation C: column ranges of a row-block
   float* S;
   float* out;
   long long n, r;
@@ -56,7 +56,7 @@ struct SelectBatchT {
   int cleared;                      // the kernel before the sums is the clearing one
   int max_part_cols, total_items;   // streaming sums kernel
   int* status;
-  int first_block[N];        // apart from the wide records: a search stays within a few lines of the constant cache
+  int first_block[N];        // (row-blocks x parts before the job's own) apart from the wide records: a search stays within a few lines of the constant cache
   SelectJob job[N];
 };
 template <int N>
@@ -98,14 +98,17 @@ __device__ __forceinline__ void add_bins(const uint32_t* hist, uint32_t* head) {
 // Behind the clearing kernel the sums have started only because everything before that one is complete
 // (pdl_launch_dependents comes after pdl_wait in every kernel): W may be read and the sums written at once, and only
 // the additions to the histogram wait for the zeros.  A warp of its own waits early and lets the select take its seats.
-// Orientation C, one CTA per row-block of every matrix.
-template <int N>
+// Orientation C, one CTA per row-block of every matrix, or per column range of one.
+// (kParts as a template parameter: with the ranges as run-time values whole row-blocks took up to 2 us longer)
+template <int N, bool kParts, bool kTall>
 __global__ void __launch_bounds__(kSumThreads + 32)
 sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
   __shared__ __align__(16) uint32_t hist[kBins1];
   const int jn = owner(B.first_block, B.n_jobs, static_cast<int>(blockIdx.x));
   const SelectJob& J = B.job[jn];
-  const int b = static_cast<int>(blockIdx.x) - B.first_block[jn];
+  const int at = static_cast<int>(blockIdx.x) - B.first_block[jn];
+  const int b = kParts ? at / J.parts : at;
+  const int c0 = kParts ? (at - b * J.parts) * J.part_cols : 0, c_end = kParts ? min(J.cols, c0 + J.part_cols) : J.cols;
   const uint16_t* wblk = J.W + static_cast<size_t>(b) * B.block * J.ldw;
   float* out = J.S + static_cast<size_t>(b) * J.cols;
   const bool count = J.head != nullptr;
@@ -116,9 +119,9 @@ sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
     pdl_wait();
     pdl_launch_dependents();
   } else if (J.vec) {
-    for (int q = threadIdx.x; q < (J.cols >> 3); q += kSumThreads) {
+    for (int q = (c0 >> 3) + threadIdx.x; q < (c_end >> 3); q += kSumThreads) {
       float acc[8];
-      sumsq8(wblk + (q << 3), B.block, J.ldw, acc);
+      sumsq8<kTall>(wblk + (q << 3), B.block, J.ldw, acc);
       float4* dst = reinterpret_cast<float4*>(out + (q << 3));
       dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
       dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
@@ -128,7 +131,7 @@ sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
       }
     }
   } else {
-    for (int g = threadIdx.x; g < J.cols; g += kSumThreads) {
+    for (int g = c0 + threadIdx.x; g < c_end; g += kSumThreads) {
       const float S = group_sumsq_strided(wblk + g, B.block, J.ldw);
       out[g] = S;
       if (count) count_key(hist, S);
@@ -668,9 +671,22 @@ int launch_sums_c(SelectBatchT<N>& B, int sms, cudaStream_t s) {
     BSP_CUDA_TRY(launch_pdl(sums_stream_kernel<N>, dim3(kSumPerSm * sms), dim3(kSumThreads), smem, s, B));
     return BSP_OK;
   }
+  // few row-blocks: cut into ranges of a piece per thread (narrower ones cost more in histograms than they gain: 9.6 ->
+  // 11.6 us for 768 x 768)
   int at = 0;
-  for (int i = 0; i < B.n_jobs; ++i) { B.first_block[i] = at; at += B.job[i].n_blocks; }
-  BSP_CUDA_TRY(launch_pdl(sums_c_kernel<N>, dim3(blocks), dim3(kSumThreads + 32), 0, s, B));
+  bool parts = false;
+  for (int i = 0; i < B.n_jobs; ++i) {
+    SelectJob& J = B.job[i];
+    const int width = kSumThreads * (J.vec ? 8 : 1);
+    J.part_cols = blocks < sms && width < J.cols ? width : J.cols;
+    J.parts = (J.cols + J.part_cols - 1) / J.part_cols;
+    parts = parts || J.parts > 1;
+    B.first_block[i] = at;
+    at += J.n_blocks * J.parts;
+  }
+  auto* kernel = B.block >= 32 ? (parts ? sums_c_kernel<N, true, true> : sums_c_kernel<N, false, true>)
+                               : (parts ? sums_c_kernel<N, true, false> : sums_c_kernel<N, false, false>);
+  BSP_CUDA_TRY(launch_pdl(kernel, dim3(at), dim3(kSumThreads + 32), 0, s, B));
   return BSP_OK;
 }
 
