@@ -48,7 +48,7 @@ struct SelectJob {
   float* out;
   long long n, r;
   uint32_t* head;            // histograms, or null: one CTA selects straight from the sums
-  int replicas;              // 1 or kReplicas histograms
+  int replicas;              // histograms: as many as fit, up to kReplicas
 };
 template <int N>
 struct SelectBatchT {
@@ -260,16 +260,18 @@ sums_r_kernel(const uint16_t* __restrict__ W, int rows, int per_row, int ldw, in
   if (head != nullptr) clear_bins(hist);
   else pdl_wait();                                           // (no clearing kernel)
   __syncthreads();
-  const long long g = static_cast<long long>(blockIdx.x) * kSumRThreads + threadIdx.x;
   if (threadIdx.x >= kSumRThreads) {
     pdl_wait();
     pdl_launch_dependents();
-  } else if (g < static_cast<long long>(rows) * per_row) {
-    const long long i = g / per_row;
-    const int a = static_cast<int>(g - i * per_row);
-    const float v = group_sumsq_contig(W + static_cast<size_t>(i) * ldw + static_cast<size_t>(a) * block, block, vec);
-    S[g] = v;
-    if (head != nullptr) count_key(hist, v);
+  } else {
+    const long long n = static_cast<long long>(rows) * per_row, step = static_cast<long long>(gridDim.x) * kSumRThreads;
+    for (long long g = static_cast<long long>(blockIdx.x) * kSumRThreads + threadIdx.x; g < n; g += step) {
+      const long long i = g / per_row;
+      const int a = static_cast<int>(g - i * per_row);
+      const float v = group_sumsq_contig(W + static_cast<size_t>(i) * ldw + static_cast<size_t>(a) * block, block, vec);
+      S[g] = v;
+      if (head != nullptr) count_key(hist, v);
+    }
   }
   if (head == nullptr) return;
   __syncthreads();
@@ -586,8 +588,9 @@ SelectJob select_job(const void* W, int cols, int ldw, int n_blocks, int n_group
   J.n = groups;
   J.r = groups_to_remove(groups, rate);
   // the region of the flags: one byte per group
-  J.replicas = L.sumsq_off - L.keep_off >= kReplicas * kBins1 * sizeof(uint32_t) ? kReplicas : 1;
-  if (L.sumsq_off - L.keep_off >= kBins1 * sizeof(uint32_t)) J.head = reinterpret_cast<uint32_t*>(base + L.keep_off);
+  const size_t fit = (L.sumsq_off - L.keep_off) / (kBins1 * sizeof(uint32_t));
+  J.replicas = fit < kReplicas ? static_cast<int>(fit) : kReplicas;
+  if (fit > 0) J.head = reinterpret_cast<uint32_t*>(base + L.keep_off);
   return J;
 }
 
@@ -728,8 +731,9 @@ extern "C" int bsp_percentile_threshold(const void* W, int rows, int cols, int l
     st = launch_sums_c(B, sms, s);
     if (st != BSP_OK) return st;
   } else {
-    BSP_CUDA_TRY(launch_pdl(sums_r_kernel, dim3(static_cast<unsigned>((groups + kSumRThreads - 1) / kSumRThreads)),
-                            dim3(kSumRThreads + 32), 0, s, B.job[0].W, rows, nb,
+    // (at most four CTAs per SM, since every one adds a histogram of its own in the end)
+    const long long ctas = (groups + kSumRThreads - 1) / kSumRThreads;
+    BSP_CUDA_TRY(launch_pdl(sums_r_kernel, dim3(static_cast<unsigned>(ctas < 4 * sms ? ctas : 4 * sms)), dim3(kSumRThreads + 32), 0, s, B.job[0].W, rows, nb,
                             ldw, block, contig_vec(W, ldw, block), B.job[0].S, B.job[0].head,
                             B.job[0].replicas));
   }
