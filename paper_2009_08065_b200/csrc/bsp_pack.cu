@@ -6,8 +6,8 @@
 // (2) CTAs per block turn the counts before theirs into blk_ptr, list the kept indices in
 // ascending order and gather the dense tile of kept values.  W is read from HBM once by (1);
 // (2) re-reads it from L2.  Orientation C with 8-element alignment runs the vectorised
-// two-stage kernels of bsp_fused.cu; this file holds the generic kernels (any alignment,
-// orientation R), the keep-count kernel and the entry points.
+// two-stage kernels of bsp_fused.cu, orientation R goes by segments of a strip; this file holds
+// the latter, the generic kernels, the keep-count kernel and the entry points.
 #include <mutex>
 
 #include "bsp_common.cuh"
@@ -16,6 +16,8 @@ namespace bsp {
 namespace {
 
 constexpr int kPackThreads = 256;
+constexpr int kSegment = 256;          // groups of a strip that one CTA packs (orientation R)
+constexpr int kMaxSegments = 16384;    // segments of a matrix: every CTA adds up the counts before its own
 
 struct Geometry {
   int rows, cols, ldw, block, orient, n_blocks, n_groups;
@@ -87,8 +89,9 @@ constexpr int kTopkBins = 1 << kTopkDigit;
 template <int T>
 __global__ void __launch_bounds__(T)
 flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
-                  uint8_t* __restrict__ keep, int32_t* __restrict__ counts) {
+                  uint8_t* __restrict__ keep, int32_t* __restrict__ counts, int32_t* __restrict__ seg_counts) {
   extern __shared__ uint32_t s_key[];                // [n_groups]
+  __shared__ int s_seg[BSP_TOPK_MAX_GROUPS / kSegment];
   __shared__ uint32_t hist[kTopkBins];
   __shared__ int s_warp[32];
   __shared__ uint32_t s_pick[2];
@@ -100,8 +103,12 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
     const uint8_t all = keep_count > 0 ? 1 : 0;
     for (int g = threadIdx.x; g < n; g += T) keep[group_slot(G, b, g)] = all;
     if (threadIdx.x == 0) counts[b] = all ? n : 0;
+    const int segments = (n + kSegment - 1) / kSegment;
+    if (seg_counts != nullptr && static_cast<int>(threadIdx.x) < segments)
+      seg_counts[b * segments + threadIdx.x] = all ? min(kSegment, n - static_cast<int>(threadIdx.x) * kSegment) : 0;
     return;
   }
+  if (threadIdx.x < BSP_TOPK_MAX_GROUPS / kSegment) s_seg[threadIdx.x] = 0;
   if (G.orient == BSP_ORIENT_C && G.vec == 8) {
     for (int q = threadIdx.x; q < (n >> 3); q += T) {
       float acc[8];
@@ -161,15 +168,26 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
     int round;
     const int rank = seen + block_exclusive_scan(eq, s_warp, &round);
     seen += round;
-    if (g < n) keep[group_slot(G, b, g)] = u > prefix || (eq && rank < equals_kept) ? 1 : 0;
+    const bool k = g < n && (u > prefix || (eq && rank < equals_kept));
+    if (g < n) keep[group_slot(G, b, g)] = k ? 1 : 0;
+    if (seg_counts != nullptr) {                     // (a warp's groups are in one segment)
+      const unsigned kept = __ballot_sync(0xffffffffu, k);
+      if ((threadIdx.x & 31) == 0 && kept != 0u) atomicAdd(&s_seg[g / kSegment], __popc(kept));
+    }
   }
   if (threadIdx.x == 0) counts[b] = keep_count;
+  if (seg_counts != nullptr) {
+    __syncthreads();
+    const int segments = (n + kSegment - 1) / kSegment;
+    if (static_cast<int>(threadIdx.x) < segments) seg_counts[b * segments + threadIdx.x] = s_seg[threadIdx.x];
+  }
 }
 
-cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, uint8_t* flags, int32_t* counts, cudaStream_t s) {
+cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, uint8_t* flags, int32_t* counts, int32_t* seg_counts,
+                        cudaStream_t s) {
   const size_t smem = sizeof(uint32_t) * G.n_groups;
-  return G.n_groups >= 1024 && G.n_blocks <= 296 ? launch_pdl(flags_topk_kernel<1024>, dim3(G.n_blocks), dim3(1024), smem, s, w, G, keep_count, flags, counts)
-                            : launch_pdl(flags_topk_kernel<kPackThreads>, dim3(G.n_blocks), dim3(kPackThreads), smem, s, w, G, keep_count, flags, counts);
+  return G.n_groups >= 1024 && G.n_blocks <= 296 ? launch_pdl(flags_topk_kernel<1024>, dim3(G.n_blocks), dim3(1024), smem, s, w, G, keep_count, flags, counts, seg_counts)
+                            : launch_pdl(flags_topk_kernel<kPackThreads>, dim3(G.n_blocks), dim3(kPackThreads), smem, s, w, G, keep_count, flags, counts, seg_counts);
 }
 
 // (2) counts -> blk_ptr (exclusive scan) and the kept-weight total: matrices with more blocks than the
@@ -253,6 +271,88 @@ compact_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __rest
         for (int c = 0; c < G.block; ++c) dst[c] = src[c];
       }
     }
+  }
+}
+
+// Orientation R by segments of 256 groups (rows) of a strip, a CTA each: a few wide strips are only a few CTAs
+// otherwise.  A segment's kept count goes to a list of its own, from which the compaction takes blk_ptr and the place of
+// its part of the tile; there a CTA moves the kept groups as one run of vectors, coalesced on the packed side.
+// Latency-bound.  3072 x 1024, the two launches: 64-column strips 30.8 -> 7.5 us, 16-column 15.7 -> 9.4; 768 x 768 in
+// 12-column strips 8.2 -> 6.2.
+__global__ void __launch_bounds__(kSegment)
+flags_segment_kernel(const uint16_t* __restrict__ W, Geometry G, float threshold, const float* __restrict__ threshold_dev,
+                     uint8_t* __restrict__ keep, int32_t* __restrict__ seg_counts) {
+  __shared__ int s_warp[kSegment / 32];
+  const int b = blockIdx.x, g = blockIdx.y * kSegment + threadIdx.x;
+  pdl_wait();
+  pdl_launch_dependents();
+  const float t = threshold_dev ? *threshold_dev : threshold;
+  bool k = false;
+  if (g < G.n_groups) {
+    k = group_sum(W, G, b, g) > __fmul_rn(t, t) || t < 0.0f;
+    keep[group_slot(G, b, g)] = k ? 1 : 0;
+  }
+  const unsigned kept = __ballot_sync(0xffffffffu, k);
+  if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = __popc(kept);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int c = 0;
+#pragma unroll
+    for (int w = 0; w < kSegment / 32; ++w) c += s_warp[w];
+    seg_counts[b * gridDim.y + blockIdx.y] = c;
+  }
+}
+
+template <int VEC>
+__global__ void __launch_bounds__(kSegment)
+compact_segment_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep,
+                       const int32_t* __restrict__ seg_counts, int32_t* __restrict__ blk_ptr, int32_t* __restrict__ idx,
+                       uint16_t* __restrict__ vals, int64_t* __restrict__ kept_weights) {
+  __shared__ int s_base[kSegment / 32], s_warp[kSegment / 32];
+  __shared__ int s_group[kSegment];
+  const int b = blockIdx.x, segments = gridDim.y, seg = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = seg * kSegment + threadIdx.x;
+  pdl_wait();
+  pdl_launch_dependents();
+  const bool k = g < G.n_groups && keep[group_slot(G, b, g)] != 0;
+  int part = 0;                                              // kept groups before this segment, in the order of the strips
+  const int before = b * segments + seg;
+  for (int i = threadIdx.x; i < before; i += kSegment) part += seg_counts[i];
+  part = warp_sum(part);
+  const unsigned kept = __ballot_sync(0xffffffffu, k);
+  if (lane == 0) { s_base[warp] = part; s_warp[warp] = __popc(kept); }
+  __syncthreads();
+  int base = 0, p = 0, m = 0;
+#pragma unroll
+  for (int w = 0; w < kSegment / 32; ++w) {
+    base += s_base[w];
+    if (w < warp) p += s_warp[w];
+    m += s_warp[w];
+  }
+  p += __popc(kept & ((1u << lane) - 1u));
+  if (k) {
+    idx[base + p] = g;
+    s_group[p] = g;
+  }
+  if (threadIdx.x == 0) {
+    if (seg == 0) blk_ptr[b] = base;
+    if (before + 1 == G.n_blocks * segments) {               // the matrix's last segment
+      blk_ptr[G.n_blocks] = base + m;
+      if (kept_weights) *kept_weights = static_cast<int64_t>(base + m) * G.block;
+    }
+  }
+  __syncthreads();
+  const int per = G.block / VEC;
+  const uint16_t* strip = W + static_cast<size_t>(b) * G.block;
+  uint16_t* out = vals + static_cast<size_t>(G.block) * base;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < m * per; e += kSegment) {
+    const int q = e / per, c = (e - q * per) * VEC;
+    const uint16_t* src = strip + static_cast<size_t>(s_group[q]) * G.ldw + c;
+    uint16_t* dst = out + static_cast<size_t>(e) * VEC;
+    if (VEC == 8) *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(src));
+    else if (VEC == 4) *reinterpret_cast<uint2*>(dst) = __ldg(reinterpret_cast<const uint2*>(src));
+    else *dst = __ldg(src);
   }
 }
 
@@ -349,17 +449,31 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
     FusedJob j{w, rows, cols, ldw, G.n_blocks, threshold, threshold_dev, nullptr, nullptr, nullptr, nullptr, nullptr,
                flags, counts, blk_ptr, idx, static_cast<uint16_t*>(vals), kept_weights, nullptr};
     if (keep_per_block >= 0) {
-      BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, s));
+      BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, nullptr, s));
     } else {
       st = fused_stage1(&j, 1, block, 0.0f, 0, s);
       if (st != BSP_OK) return st;
     }
     return fused_stage2(&j, 1, block, s);
   }
+  const long long segments = (G.n_groups + kSegment - 1) / kSegment;
+  const bool keep_in_ws = keep >= reinterpret_cast<uint8_t*>(wsb) && keep < reinterpret_cast<uint8_t*>(wsb) + ws_bytes;
+  if (orient == BSP_ORIENT_R && keep != nullptr && !keep_in_ws && G.n_blocks * segments <= kMaxSegments &&
+      G.n_blocks * segments * sizeof(int32_t) <= L.sumsq_off - L.keep_off) {
+    // (the flags go to the caller's array, so the workspace's flags are free for the segments' counts)
+    int32_t* seg_counts = reinterpret_cast<int32_t*>(wsb + L.keep_off);
+    const dim3 grid(G.n_blocks, static_cast<unsigned>(segments));
+    if (keep_per_block >= 0) BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, seg_counts, s));
+    else BSP_CUDA_TRY(launch_pdl(flags_segment_kernel, grid, dim3(kSegment), 0, s, w, G, threshold, threshold_dev, flags, seg_counts));
+    const int vec = (reinterpret_cast<uintptr_t>(vals) & 15) == 0 ? G.vec : 1;
+    BSP_CUDA_TRY(launch_pdl(vec == 8 ? compact_segment_kernel<8> : vec == 4 ? compact_segment_kernel<4> : compact_segment_kernel<1>, grid,
+                            dim3(kSegment), 0, s, w, G, flags, seg_counts, blk_ptr, idx, static_cast<uint16_t*>(vals), kept_weights));
+    return BSP_OK;
+  }
   // a CTA per block, threads for its groups: up to 1024 of them, since a matrix of few tall blocks has few CTAs
   const int threads = G.n_groups >= 1024 ? 1024 : G.n_groups <= 128 ? 128 : (G.n_groups + 31) / 32 * 32;
   if (keep_per_block >= 0) {
-    BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, s));
+    BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, nullptr, s));
   } else {
     BSP_CUDA_TRY(launch_pdl(flags_threshold_kernel, dim3(G.n_blocks), dim3(threads), 0, s, w, G, threshold, threshold_dev, flags, counts));
   }

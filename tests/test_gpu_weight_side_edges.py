@@ -73,6 +73,26 @@ def test_pack_and_layout_of_row_pruned_strips(rows, cols, block):
     assert np.array_equal(bits_of(plan.view(torch.int16)[: rows * cols]).reshape(rows, cols), O.prune(w, block, "R", t))
 
 
+# segments of 256 rows: a whole one, one row short, one row more, a single strip of many; 16400 strips are packed
+# without segments
+@pytest.mark.parametrize("rows,cols,block", [(256, 24, 12), (255, 16, 8), (257, 64, 64), (8192, 8, 8), (5, 16400, 1)])
+def test_row_pruned_segments(rows, cols, block):
+    w = weights(f"s{rows}x{cols}", rows, cols)
+    t = float(np.median(O.group_norms(w, block, "R")))
+    for keep_n in (-1, max(1, rows // 3), rows):
+        pk = bsp.PackedMatrix.allocate(rows, cols, block, bsp.ORIENT_R)
+        if keep_n < 0:
+            keep_ref = O.keep_flags(w, block, "R", t)
+            bsp.bsp_prune_pack(to_dev(w), pk, t)
+        else:
+            keep_ref = O.keep_topk_per_block(w, block, "R", keep_n)
+            bsp.bsp_prune_pack(to_dev(w), pk, keep_per_block=keep_n)
+        ref = O.pack(w, keep_ref, block, "R")
+        blk_ptr, idx, vals, keep, kept = packed_to_host(pk)
+        assert np.array_equal(keep, keep_ref) and kept == block * int(keep_ref.sum())
+        assert np.array_equal(blk_ptr, ref[0]) and np.array_equal(idx, ref[1]) and np.array_equal(vals, ref[2])
+
+
 @pytest.mark.parametrize("rows,cols,block", [(33, 72, 1), (63, 64, 3), (96, 136, 12), (144, 1024, 16), (128, 8, 64), (192, 200, 96), (200, 72, 100)])
 def test_column_pruned_layouts_mask_and_repack(rows, cols, block):
     w = weights(f"c{rows}x{cols}", rows, cols)
