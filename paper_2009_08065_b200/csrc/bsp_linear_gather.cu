@@ -153,35 +153,42 @@ gather_plan_fill_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __re
 
 // ---- transposed copy ---------------------------------------------------------------------
 // XT[c, r] = X[r, c] for a row-major bf16 matrix; 64 x 64 tiles through shared memory, 16-byte
-// global accesses on both sides (rows and cols multiples of 8).
+// global accesses on both sides (rows and cols multiples of 8).  Bound by memory (2 bytes in and out) once the shared
+// memory side is cheap: a tile row is 32 words, turned by 4 words for every 8 rows, so that rows go in as 16-byte stores
+// and a thread reads the words of two columns in 8 rows, both without bank conflicts, and sorts the halves into the
+// two columns' 16-byte stores.  (By single elements, 16 stores and 16 loads a thread, 8192 x 1024 took 8.2 us, 6.9 now.)
 __global__ void __launch_bounds__(256)
 transpose_kernel(const uint16_t* __restrict__ X, int rows, int cols, int ldx, uint16_t* __restrict__ XT, int ldxt) {
-  __shared__ uint16_t s_t[64][66];
+  __shared__ __align__(16) uint32_t s_t[64][32];
+  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   pdl_wait();
   pdl_launch_dependents();
-  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
-  for (int e = threadIdx.x; e < 512; e += 256) {
-    const int r = e >> 3, q = e & 7;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r0 + r < rows && c0 + q * 8 < cols) v = __ldg(reinterpret_cast<const uint4*>(X + static_cast<size_t>(r0 + r) * ldx + c0 + q * 8));
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint4 v[2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      s_t[r][q * 8 + 2 * i] = static_cast<uint16_t>(w[i] & 0xffffu);
-      s_t[r][q * 8 + 2 * i + 1] = static_cast<uint16_t>(w[i] >> 16);
-    }
+  for (int u = 0; u < 2; ++u) {
+    const int r = (threadIdx.x >> 3) + 32 * u, q = threadIdx.x & 7;
+    v[u] = make_uint4(0u, 0u, 0u, 0u);
+    if (r0 + r < rows && c0 + q * 8 < cols) v[u] = __ldg(reinterpret_cast<const uint4*>(X + static_cast<size_t>(r0 + r) * ldx + c0 + q * 8));
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int r = (threadIdx.x >> 3) + 32 * u, q = threadIdx.x & 7;
+    *reinterpret_cast<uint4*>(&s_t[r][(4 * q + 4 * (r >> 3)) & 31]) = v[u];
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < 512; e += 256) {
-    const int c = e >> 3, q = e & 7;             // output row c (a column of X), 8 source rows q*8..q*8+7
-    if (c0 + c < cols && r0 + q * 8 < rows) {
-      uint32_t w[4];
+  const int q = threadIdx.x & 7, pair = threadIdx.x >> 3;      // source rows 8q..8q+7 of columns 2 pair, 2 pair + 1
+  if (c0 + 2 * pair >= cols || r0 + 8 * q >= rows) return;
+  uint32_t w[8], a[4], b[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        w[i] = static_cast<uint32_t>(s_t[q * 8 + 2 * i][c]) | (static_cast<uint32_t>(s_t[q * 8 + 2 * i + 1][c]) << 16);
-      *reinterpret_cast<uint4*>(XT + static_cast<size_t>(c0 + c) * ldxt + r0 + q * 8) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
+  for (int i = 0; i < 8; ++i) w[i] = s_t[8 * q + i][(pair + 4 * q) & 31];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    a[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410);        // the low halves: the even column
+    b[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632);
   }
+  uint16_t* out = XT + static_cast<size_t>(c0 + 2 * pair) * ldxt + r0 + 8 * q;
+  *reinterpret_cast<uint4*>(out) = make_uint4(a[0], a[1], a[2], a[3]);
+  *reinterpret_cast<uint4*>(out + ldxt) = make_uint4(b[0], b[1], b[2], b[3]);
 }
 
 // ---- the kernel --------------------------------------------------------------------------
