@@ -94,7 +94,7 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
   __shared__ int s_seg[BSP_TOPK_MAX_GROUPS / kSegment];
   __shared__ uint32_t hist[kTopkBins];
   __shared__ int s_warp[32];
-  __shared__ uint32_t s_pick[2];
+  __shared__ uint32_t s_pick[3];
   constexpr int kPer = kTopkBins / T;
   const int b = blockIdx.x, n = G.n_groups;
   pdl_wait();
@@ -144,7 +144,7 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
     if (before < want && want <= before + mine) {    // exactly one thread
 #pragma unroll
       for (int i = 0; i < kPer; ++i) {
-        if (before < want && want <= before + c[i]) { s_pick[0] = threadIdx.x * kPer + i; s_pick[1] = want - before; }
+        if (before < want && want <= before + c[i]) { s_pick[0] = threadIdx.x * kPer + i; s_pick[1] = want - before; s_pick[2] = c[i]; }
         before += c[i];
       }
     }
@@ -154,20 +154,20 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
     __syncthreads();
   }
   // groups above the smallest kept sum stay; of the e groups equal to it the first e - want + 1 do
-  // (the select counted want - 1 of them as smaller)
-  int larger = 0;
-  for (int g = threadIdx.x; g < n; g += T) larger += s_key[g] > prefix ? 1 : 0;
-  int total;
-  block_exclusive_scan(larger, s_warp, &total);
-  const int equals_kept = keep_count - total;
+  // (the select counted want - 1 of them as smaller): all of them in most cases, which takes no ranking
+  const bool all_equals = want == 1u;
+  const int equals_kept = static_cast<int>(s_pick[2] - want) + 1;
   int seen = 0;
   for (int g0 = 0; g0 < n; g0 += T) {
     const int g = g0 + threadIdx.x;
     const uint32_t u = g < n ? s_key[g] : 0u;
     const int eq = g < n && u == prefix ? 1 : 0;
-    int round;
-    const int rank = seen + block_exclusive_scan(eq, s_warp, &round);
-    seen += round;
+    int rank = 0;
+    if (!all_equals) {
+      int round;
+      rank = seen + block_exclusive_scan(eq, s_warp, &round);
+      seen += round;
+    }
     const bool k = g < n && (u > prefix || (eq && rank < equals_kept));
     if (g < n) keep[group_slot(G, b, g)] = k ? 1 : 0;
     if (seg_counts != nullptr) {                     // (a warp's groups are in one segment)
