@@ -80,10 +80,10 @@ flags_threshold_kernel(const uint16_t* __restrict__ W, Geometry G, float thresho
 // select of three digits finds the smallest kept one, and a scan in index order decides which of its equals
 // are kept.  O(groups) work per digit; ranking every sum against every other one (O(groups^2)) took
 // 0.5-1 ms on the larger matrices.
-// Blocks of 1024 groups or more get 1024 threads: the digits are passes over the keys, and a GPU that is still busy with
-// the launch before puts several of the smaller CTAs on one SM, where they share its issue slots (16 strips of 3072
-// groups, packed behind their norms: 101 -> 55 us; 192 strips of 1024 groups 30 -> 21).  With more blocks than two per
-// SM the smaller CTAs are level or ahead.
+// Blocks of 512 groups or more get 512 threads (orientation C, whose rows in flight take 64 registers) or 1024 (R): the
+// digits are passes over the keys, and a GPU that is still busy with the launch before puts several of the smaller CTAs on
+// one SM, where they share its issue slots.  Norms, packing and layout together, against 256 threads: 16 strips of 3072
+// groups 105 -> 46 us, 64 strips of 768 28 -> 16, 11 row-blocks of 3072 44 -> 33, 192 of 768 22.6 -> 18.5.
 constexpr int kTopkDigit = 11;                       // 31 bits = 11 + 10 + 10
 constexpr int kTopkBins = 1 << kTopkDigit;
 template <int T>
@@ -186,8 +186,12 @@ flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
 cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, uint8_t* flags, int32_t* counts, int32_t* seg_counts,
                         cudaStream_t s) {
   const size_t smem = sizeof(uint32_t) * G.n_groups;
-  return G.n_groups >= 1024 && G.n_blocks <= 296 ? launch_pdl(flags_topk_kernel<1024>, dim3(G.n_blocks), dim3(1024), smem, s, w, G, keep_count, flags, counts, seg_counts)
-                            : launch_pdl(flags_topk_kernel<kPackThreads>, dim3(G.n_blocks), dim3(kPackThreads), smem, s, w, G, keep_count, flags, counts, seg_counts);
+  auto launch = [&](auto kernel, int threads) {
+    return launch_pdl(kernel, dim3(G.n_blocks), dim3(threads), smem, s, w, G, keep_count, flags, counts, seg_counts);
+  };
+  if (G.n_groups < 512) return launch(flags_topk_kernel<kPackThreads>, kPackThreads);
+  if (G.orient == BSP_ORIENT_C) return launch(flags_topk_kernel<512>, 512);
+  return G.n_blocks <= 296 ? launch(flags_topk_kernel<1024>, 1024) : launch(flags_topk_kernel<kPackThreads>, kPackThreads);
 }
 
 // (2) counts -> blk_ptr (exclusive scan) and the kept-weight total: matrices with more blocks than the
