@@ -479,21 +479,25 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
     const long long bytes = 2LL * rows_per_block * kept, step = 128LL * kPlanTThreads * gridDim.y;
     for (long long at = 128LL * threadIdx.x * gridDim.y + 128LL * blockIdx.y; at < bytes; at += step) prefetch_line(run + at);
   }
-  // the index lists of the unit's row-blocks are one run of the index array
-  {
-    const int lo = s_ptr[0], n_idx = s_ptr[nb] - lo;
-    for (int j0 = threadIdx.x; j0 < n_idx; j0 += 4 * kPlanTThreads) {
-      int k[4];
+  // A warp lists a row-block's columns of the tile.  A longer list is narrowed down by 32 samples first: one trip to
+  // memory more, but every CTA reading its blocks' whole lists took as many instructions as moving the values (a backward
+  // pass of 944 features, 8-row blocks, 4508 tokens: 242 -> 236 us).
+  for (int q = warp; q < nb; q += kPlanTThreads / 32) {
+    const int lo = s_ptr[q], kc = s_ptr[q + 1] - lo;
+    int first = 0, last = kc;                                  // where columns of the tile can stand
+    if (kc > 256) {
+      const int col = __ldg(idx + lo + static_cast<int>(static_cast<long long>(kc) * lane >> 5));
+      const int below = __popc(__ballot_sync(0xffffffffu, col < k0)), upto = __popc(__ballot_sync(0xffffffffu, col < k0 + nk));
+      if (below > 0) first = static_cast<int>(static_cast<long long>(kc) * (below - 1) >> 5);
+      if (upto < 32) last = static_cast<int>(static_cast<long long>(kc) * upto >> 5);
+    }
+    for (int j0 = first + lane; j0 < last; j0 += 8 * 32) {
+      int k[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) k[u] = j0 + u * kPlanTThreads < n_idx ? __ldg(idx + lo + j0 + u * kPlanTThreads) - k0 : -1;
+      for (int u = 0; u < 8; ++u) k[u] = j0 + u * 32 < last ? __ldg(idx + lo + j0 + u * 32) - k0 : -1;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (k[u] < 0 || k[u] >= nk) continue;
-        const int j = lo + j0 + u * kPlanTThreads;
-        int q = 0;
-        while (q + 1 < nb && s_ptr[q + 1] <= j) ++q;
-        s_col_pos[q][k[u]] = j - s_ptr[q];
-      }
+      for (int u = 0; u < 8; ++u)
+        if (static_cast<unsigned>(k[u]) < static_cast<unsigned>(nk)) s_col_pos[q][k[u]] = j0 + u * 32;
     }
   }
   __syncthreads();
