@@ -320,6 +320,13 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+// max(x, 0), NaN for NaN.  (fmaxf returns its other operand there, and so does the clamp below: of a NaN nothing else
+// would be left, and a diverged activation would leave the layer as an ordinary -6e-9.)
+__device__ __forceinline__ float positive_part(float x) {
+  float r;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(x));
+  return r;
+}
 // GELU of two values, everything but the clamps and the two ex2 as packed operations (the epilogue of a GELU layer is
 // bound by instruction issue and latency).  b = -a; the odd coefficients of P change sign with it.
 __device__ __forceinline__ void gelu_erf_pair(float& x0, float& x1) {
@@ -333,7 +340,7 @@ __device__ __forceinline__ void gelu_erf_pair(float& x0, float& x1) {
   unpack_f32x2(p, p0, p1);
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q0) : "f"(p0));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q1) : "f"(p1));
-  unpack_f32x2(fma_f32x2(b, pack_f32x2(q0, q1), pack_f32x2(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f))), x0, x1);
+  unpack_f32x2(fma_f32x2(b, pack_f32x2(q0, q1), pack_f32x2(positive_part(x0), positive_part(x1))), x0, x1);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
