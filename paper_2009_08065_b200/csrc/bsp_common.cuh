@@ -121,9 +121,15 @@ inline int contig_vec(const void* W, int ldw, int block) {
 
 #ifdef __CUDACC__
 // Launch with programmatic stream serialization: the grid may take its seats while the previous kernel of
-// the stream drains.  Every kernel launched this way calls pdl_wait before it touches global memory, so
-// what it reads is complete and the order of the stream is kept; it saves about 1 us between two of this
-// library's short kernels.
+// the stream drains; it saves about 1 us between two of this library's short kernels.
+// The rule that keeps the order of the stream: a thread signals (pdl_launch_dependents) only after its own
+// pdl_wait.  A grid starts once every CTA of its direct predecessor has signalled or ended, so a grid that has
+// started knows that everything BEFORE that predecessor is complete, though not the predecessor itself; and once
+// its own pdl_wait returns, that too.  Hence global memory is touched after pdl_wait, except for
+//   - data older than the direct predecessor, where the library itself launched that predecessor: W and the sums
+//     behind the percentile's clearing kernel (bsp_select.cu), W in the second packing stage (bsp_fused.cu);
+//   - the weights of a plan that the caller vouches for (BSP_LINEAR_PLAN_STABLE): the weight warp of
+//     linear_tc_kernel and gemm_split_kernel, which does not wait and therefore does not signal either.
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -139,7 +145,7 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// After pdl_wait: a dependent that has started knows that everything before this grid is complete.
+// Only after the same thread's pdl_wait (see launch_pdl).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Fetches into L2 of what a CTA will read once pdl_wait returns.  They change nothing but what L2 holds, which is

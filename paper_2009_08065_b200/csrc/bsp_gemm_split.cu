@@ -146,9 +146,12 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   const uint32_t tmem_base = *tmem_holder;
   split_cluster_arrive();                              // this CTA runs and its mbarriers exist
 
-  // The weights of a stable plan are older than the kernel before this one: their producer does not wait.
-  if (!(P.plan_stable && warp == 10)) pdl_wait();
-  pdl_launch_dependents();
+  // The weights of a stable plan are older than the kernel before this one: their producer does not wait, and
+  // leaves the signal to the warps that do (see launch_pdl).
+  if (!(P.plan_stable && warp == 10)) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
 
   const int kb0 = static_cast<int>(static_cast<long long>(P.k_blocks) * rank / C);
   const int kb1 = static_cast<int>(static_cast<long long>(P.k_blocks) * (rank + 1) / C);

@@ -136,9 +136,13 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
   // reads memory that kernel may have written (X, the plan), so wait for it to finish; and let
   // the next kernel in the stream start its own prologue as soon as SMs become free.  When the
   // caller vouches that the plan is older than the previous kernel, the weight producer does not
-  // wait: its first tiles are on their way while the previous kernel finishes writing X.
-  if (!(P.plan_stable && warp == kWeightWarp)) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // wait: its first tiles are on their way while the previous kernel finishes writing X.  It leaves
+  // the signal to the warps that have waited: one thread's signal counts for its CTA, and the kernel
+  // that it lets in may read weights at once in the same way (see launch_pdl).
+  if (!(P.plan_stable && warp == kWeightWarp)) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
 
   const int m_tiles = (P.tokens + kBlockM - 1) / kBlockM;
   const int n_tiles = (P.n_out + BN - 1) / BN;

@@ -95,9 +95,9 @@ __device__ __forceinline__ void add_bins(const uint32_t* hist, uint32_t* head) {
   }
 }
 
-// Behind the clearing kernel the sums have started only because everything before that one is complete
-// (pdl_launch_dependents comes after pdl_wait in every kernel): W may be read and the sums written at once, and only
-// the additions to the histogram wait for the zeros.  A warp of its own waits early and lets the select take its seats.
+// Behind the clearing kernel the sums have started only because everything before that one is complete (it signals
+// after its wait, see launch_pdl): W may be read and the sums written at once, and only the additions to the histogram
+// wait for the zeros.  A warp of its own waits early and lets the select take its seats.
 // Orientation C, one CTA per row-block of every matrix, or per column range of one.
 // (kParts as a template parameter: with the ranges as run-time values whole row-blocks took up to 2 us longer)
 template <int N, bool kParts, bool kTall>
