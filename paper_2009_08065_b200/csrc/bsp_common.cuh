@@ -159,6 +159,32 @@ __device__ __forceinline__ void prefetch_bytes(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// A load of what an earlier launch may have written, for kernels that are resident while that launch still runs (every
+// kernel that calls pdl_wait): an ordinary coherent load, which the wait's memory clobber keeps behind it.  Such data
+// does change while the kernel lives, so the read-only path (__ldg, or const __restrict__ parameters, which a compiler
+// may send there and may read ahead of the wait) is not defined for it.  Without __restrict__ a load does not move
+// ahead of a store either: loops that copy ask for several elements before they store the first.
+template <class T>
+__device__ __forceinline__ T ld_global(const T* p) {
+  return *p;
+}
+
+// The type that moves N 16-bit elements at once.
+template <int N>
+struct VectorOf {
+  using type = uint16_t;
+};
+template <>
+struct VectorOf<4> {
+  using type = uint2;
+};
+template <>
+struct VectorOf<8> {
+  using type = uint4;
+};
+template <int N>
+using vector_of = typename VectorOf<N>::type;
+
 __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
   return __uint_as_float(static_cast<uint32_t>(b) << 16);
 }
@@ -166,22 +192,22 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
 // Sum of squares of one group in float32, elements taken in increasing index order starting
 // from +0.  The square of a bf16 value is exact in float32, so the fused multiply-add rounds
 // exactly once per element, the same as a separate multiply and add would.
-__device__ __forceinline__ float group_sumsq_strided(const uint16_t* __restrict__ p, int n, size_t stride) {
+__device__ __forceinline__ float group_sumsq_strided(const uint16_t* p, int n, size_t stride) {
   float acc = 0.0f;
   for (int e = 0; e < n; ++e) {
-    const float w = bf16_bits_to_float(p[static_cast<size_t>(e) * stride]);
+    const float w = bf16_bits_to_float(ld_global(p + static_cast<size_t>(e) * stride));
     acc = __fmaf_rn(w, w, acc);
   }
   return acc;
 }
 
 // The same for a group of contiguous elements (orientation R), by vectors of `vec` elements (contig_vec).
-__device__ __forceinline__ float group_sumsq_contig(const uint16_t* __restrict__ p, int n, int vec) {
+__device__ __forceinline__ float group_sumsq_contig(const uint16_t* p, int n, int vec) {
   float acc = 0.0f;
   if (vec == 8) {
 #pragma unroll 4
     for (int e = 0; e < n; e += 8) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(p + e));
+      const uint4 v = ld_global(reinterpret_cast<const uint4*>(p + e));
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -192,7 +218,7 @@ __device__ __forceinline__ float group_sumsq_contig(const uint16_t* __restrict__
   } else if (vec == 4) {
 #pragma unroll 4
     for (int e = 0; e < n; e += 4) {
-      const uint2 v = __ldg(reinterpret_cast<const uint2*>(p + e));
+      const uint2 v = ld_global(reinterpret_cast<const uint2*>(p + e));
       const uint32_t w[2] = {v.x, v.y};
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -220,10 +246,10 @@ __device__ __forceinline__ int warp_sum(int v) {
 // Float32 sums of squares of 8 adjacent columns over the d rows of a row-block: eight independent
 // sequential chains, each the defined decision quantity of its group.
 template <int ROWS>
-__device__ __forceinline__ void sumsq8_rows(const uint16_t* __restrict__ p, int ldw, float (&acc)[8]) {
+__device__ __forceinline__ void sumsq8_rows(const uint16_t* p, int ldw, float (&acc)[8]) {
   uint4 v[ROWS];
 #pragma unroll
-  for (int u = 0; u < ROWS; ++u) v[u] = __ldg(reinterpret_cast<const uint4*>(p + static_cast<size_t>(u) * ldw));
+  for (int u = 0; u < ROWS; ++u) v[u] = ld_global(reinterpret_cast<const uint4*>(p + static_cast<size_t>(u) * ldw));
 #pragma unroll
   for (int u = 0; u < ROWS; ++u) {     // rows in increasing order: the chains stay sequential
     const uint32_t w32[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
@@ -238,7 +264,7 @@ __device__ __forceinline__ void sumsq8_rows(const uint16_t* __restrict__ p, int 
 // kTall: 32 rows in flight instead of 16, for blocks of 32 rows and more (such a matrix has few of them, and a thread's
 // rows are a chain of trips to memory; not for the others, since it takes 128 registers).
 template <bool kTall = false>
-__device__ __forceinline__ void sumsq8(const uint16_t* __restrict__ p, int d, int ldw, float (&acc)[8]) {
+__device__ __forceinline__ void sumsq8(const uint16_t* p, int d, int ldw, float (&acc)[8]) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
   int r = 0;

@@ -101,8 +101,8 @@ fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
       }
       if (want_pen) {
         if (J.gamma_in) {
-          const float4 a = __ldg(reinterpret_cast<const float4*>(J.gamma_in + g0));
-          const float4 c = __ldg(reinterpret_cast<const float4*>(J.gamma_in + g0 + 4));
+          const float4 a = ld_global(reinterpret_cast<const float4*>(J.gamma_in + g0));
+          const float4 c = ld_global(reinterpret_cast<const float4*>(J.gamma_in + g0 + 4));
           const float w[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
 #pragma unroll
           for (int i = 0; i < 8; ++i) pen = fmaf(w[i], base[i], pen);

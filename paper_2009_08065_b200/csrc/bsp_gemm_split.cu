@@ -225,13 +225,13 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   if (epilogue) {
     if constexpr (!kTn) {
       const int c = static_cast<int>(threadIdx.x) - 64, n = n0 + static_cast<int>(rank) * W + c;
-      if (c < W) s_bias[c] = P.bias != nullptr && n < P.cols ? bf16_bits_to_float(__ldg(P.bias + n)) : 0.0f;
+      if (c < W) s_bias[c] = P.bias != nullptr && n < P.cols ? bf16_bits_to_float(ld_global(P.bias + n)) : 0.0f;
     } else {
 #pragma unroll
       for (int i = 0; i < UW / 8; ++i) {               // (cols is a multiple of 8: eight columns are inside or outside)
         flags[i] = make_uint2(0x01010101u, 0x01010101u);
         if (P.keep != nullptr && mine && m < P.rows && n_own + 8 * i < P.cols)
-          flags[i] = __ldg(reinterpret_cast<const uint2*>(P.keep + static_cast<size_t>(m / P.block) * P.cols + n_own + 8 * i));
+          flags[i] = ld_global(reinterpret_cast<const uint2*>(P.keep + static_cast<size_t>(m / P.block) * P.cols + n_own + 8 * i));
       }
     }
     ok = __all_sync(0xffffffffu, mbar_wait(acc_bar, 0u, P.status));

@@ -188,7 +188,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
           flags[j] = make_uint2(0x01010101u, 0x01010101u);
           const int n = n0 + c0 + 8 * j;
           if (P.keep != nullptr && m0 + row < P.n_out && n < P.k_in)
-            flags[j] = __ldg(reinterpret_cast<const uint2*>(P.keep + static_cast<size_t>((m0 + row) / P.block) * P.k_in + n));
+            flags[j] = ld_global(reinterpret_cast<const uint2*>(P.keep + static_cast<size_t>((m0 + row) / P.block) * P.k_in + n));
         }
         piece_load(taddr + c0, smem_u32(s_zero), piece);
         if (P.keep != nullptr) {

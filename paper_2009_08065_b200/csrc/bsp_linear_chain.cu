@@ -250,7 +250,7 @@ linear_chain_kernel(const __grid_constant__ ChainMaps M, const __grid_constant__
       const int bn = op.bn;
       const int m0 = T.m * kBlockM, n0 = T.n * bn;
       for (int c = epi_tid; c < bn; c += 256)
-        s_bias[acc * kMaxBN + c] = (op.bias != nullptr && n0 + c < op.n_out) ? __ldg(op.bias + n0 + c) : static_cast<uint16_t>(0);
+        s_bias[acc * kMaxBN + c] = (op.bias != nullptr && n0 + c < op.n_out) ? ld_global(op.bias + n0 + c) : static_cast<uint16_t>(0);
       epilogue_sync_all();                   // (every thread has read the slot: it may be reused)
       if (epi_tid == 0) mbar_arrive(taken_bar(seq % kRing));
       if (!epilogue_all_ok(mbar_wait(acc_full_bar(acc), acc_phase[acc], P.status))) { ok = false; break; }

@@ -158,7 +158,7 @@ gather_plan_fill_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __re
 // and a thread reads the words of two columns in 8 rows, both without bank conflicts, and sorts the halves into the
 // two columns' 16-byte stores.  (By single elements, 16 stores and 16 loads a thread, 8192 x 1024 took 8.2 us, 6.9 now.)
 __global__ void __launch_bounds__(256)
-transpose_kernel(const uint16_t* __restrict__ X, int rows, int cols, int ldx, uint16_t* __restrict__ XT, int ldxt) {
+transpose_kernel(const uint16_t* X, int rows, int cols, int ldx, uint16_t* XT, int ldxt) {
   __shared__ __align__(16) uint32_t s_t[64][32];
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   pdl_wait();
@@ -168,7 +168,7 @@ transpose_kernel(const uint16_t* __restrict__ X, int rows, int cols, int ldx, ui
   for (int u = 0; u < 2; ++u) {
     const int r = (threadIdx.x >> 3) + 32 * u, q = threadIdx.x & 7;
     v[u] = make_uint4(0u, 0u, 0u, 0u);
-    if (r0 + r < rows && c0 + q * 8 < cols) v[u] = __ldg(reinterpret_cast<const uint4*>(X + static_cast<size_t>(r0 + r) * ldx + c0 + q * 8));
+    if (r0 + r < rows && c0 + q * 8 < cols) v[u] = ld_global(reinterpret_cast<const uint4*>(X + static_cast<size_t>(r0 + r) * ldx + c0 + q * 8));
   }
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
@@ -340,7 +340,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
     for (int unit = blockIdx.x; unit < total_units && ok; unit += gridDim.x) {
       const int m = unit / P.n_chunks, ch = unit - m * P.n_chunks;
       const int rb0 = ch * P.rb_per_chunk, rb1 = min(P.n_blocks, rb0 + P.rb_per_chunk);
-      const int g_begin = __ldg(P.soff + rb0), g_end = __ldg(P.soff + rb1);
+      const int g_begin = ld_global(P.soff + rb0), g_end = ld_global(P.soff + rb1);
       const int x = m * kBlockM;
       const int first = g_begin + static_cast<int>(((warp - n0) % 4 + 4) % 4);   // this warp's first stage of the unit
       // column numbers and stage bytes are loaded two of the warp's stages (eight stages) ahead
@@ -348,8 +348,8 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
       uint32_t mq[2];
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        cq[q] = __ldg(reinterpret_cast<const uint2*>(P.cols + static_cast<size_t>(first + 4 * q) * kGStageK + quad4 * 4));
-        mq[q] = __ldg(P.meta + first + 4 * q);
+        cq[q] = ld_global(reinterpret_cast<const uint2*>(P.cols + static_cast<size_t>(first + 4 * q) * kGStageK + quad4 * 4));
+        mq[q] = ld_global(P.meta + first + 4 * q);
       }
       for (int g0 = first; g0 < g_end && ok; g0 += 8) {
 #pragma unroll
@@ -363,8 +363,8 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
             if (ok) {
               const uint2 cv = cq[q];
               const uint32_t mt = mq[q];
-              cq[q] = __ldg(reinterpret_cast<const uint2*>(P.cols + static_cast<size_t>(g + 8) * kGStageK + quad4 * 4));
-              mq[q] = __ldg(P.meta + g + 8);
+              cq[q] = ld_global(reinterpret_cast<const uint2*>(P.cols + static_cast<size_t>(g + 8) * kGStageK + quad4 * 4));
+              mq[q] = ld_global(P.meta + g + 8);
               const uint32_t a_dst = smem_base + stage * Cfg::kStage;
               const int groups = static_cast<int>(mt & 7u);
               if (lane == 0) {
@@ -405,7 +405,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
       for (int unit = blockIdx.x; unit < total_units && ok; unit += gridDim.x) {
         const int m = unit / P.n_chunks, ch = unit - m * P.n_chunks;
         const int rb0 = ch * P.rb_per_chunk, rb1 = min(P.n_blocks, rb0 + P.rb_per_chunk);
-        const int g_begin = __ldg(P.soff + rb0), g_end = __ldg(P.soff + rb1);
+        const int g_begin = ld_global(P.soff + rb0), g_end = ld_global(P.soff + rb1);
         for (int g = g_begin; g < g_end; ++g) {
           if (!mbar_wait_warp(full_bar(stage), phase, P.status)) { ok = false; break; }
           tcgen05_fence_after();
@@ -459,7 +459,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
       }
     };
     auto bias_of = [&](const auto& c) -> uint16_t {
-      return tid < D && c.unit < total_units && P.bias != nullptr ? __ldg(P.bias + static_cast<size_t>(c.rb) * D + tid) : static_cast<uint16_t>(0);
+      return tid < D && c.unit < total_units && P.bias != nullptr ? ld_global(P.bias + static_cast<size_t>(c.rb) * D + tid) : static_cast<uint16_t>(0);
     };
     enter(at);
     for (int g = 0; g < group; ++g) advance(at);

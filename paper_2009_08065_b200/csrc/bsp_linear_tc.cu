@@ -233,7 +233,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
       // other group can lag by at most one tile (it has to reach the barrier below for this tile),
       // so the values it may still be reading are in the other half.
       for (int c = epi_tid; c < BN; c += kEpiThreads)
-        s_bias[acc * BN + c] = (P.bias != nullptr && n0 + c < P.n_out) ? __ldg(P.bias + n0 + c) : static_cast<uint16_t>(0);
+        s_bias[acc * BN + c] = (P.bias != nullptr && n0 + c < P.n_out) ? ld_global(P.bias + n0 + c) : static_cast<uint16_t>(0);
       tc_epilogue_sync_all();
       // all epilogue threads take the same decision, so nobody is left alone at a named barrier below
       if (!tc_epilogue_all_ok(mbar_wait(acc_full_bar(acc), acc_phase[acc], P.status))) { ok = false; break; }
@@ -346,8 +346,8 @@ __host__ __device__ inline int plan_rows_per_cta(int k_in) {
   return r > 4 ? 4 : r < 1 ? 1 : r;
 }
 __global__ void __launch_bounds__(256)
-plan_expand_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restrict__ idx,
-                   const uint16_t* __restrict__ vals, int k_in, int block, uint16_t* __restrict__ Wx) {
+plan_expand_kernel(const int32_t* blk_ptr, const int32_t* idx,
+                   const uint16_t* vals, int k_in, int block, uint16_t* Wx) {
   extern __shared__ __align__(16) int16_t s_pos[];   // [k_in] column -> position in the kept list, or -1 (k_in < 32768)
   const int b = blockIdx.x;
   const int rows_per = plan_rows_per_cta(k_in);
@@ -357,17 +357,17 @@ plan_expand_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restric
   for (int k = threadIdx.x; k < chunks; k += 256) reinterpret_cast<uint4*>(s_pos)[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
   pdl_wait();
   pdl_launch_dependents();
-  const int lo = __ldg(blk_ptr + b), kc = __ldg(blk_ptr + b + 1) - lo;
+  const int lo = ld_global(blk_ptr + b), kc = ld_global(blk_ptr + b + 1) - lo;
   const uint16_t* run = vals + static_cast<size_t>(block) * lo + static_cast<size_t>(r_lo) * kc;
   int col[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) col[u] = static_cast<int>(threadIdx.x) + u * 256 < kc ? __ldg(idx + lo + threadIdx.x + u * 256) : -1;
+  for (int u = 0; u < 4; ++u) col[u] = static_cast<int>(threadIdx.x) + u * 256 < kc ? ld_global(idx + lo + threadIdx.x + u * 256) : -1;
   const int n_val = n_rows * kc;
   for (int e0 = threadIdx.x; e0 < n_val; e0 += 8 * 256) {
     uint16_t v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u)
-      if (e0 + u * 256 < n_val) v[u] = __ldg(run + e0 + u * 256);
+      if (e0 + u * 256 < n_val) v[u] = ld_global(run + e0 + u * 256);
 #pragma unroll
     for (int u = 0; u < 8; ++u)
       if (e0 + u * 256 < n_val) s_val[e0 + u * 256] = v[u];
@@ -376,7 +376,7 @@ plan_expand_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restric
 #pragma unroll
   for (int u = 0; u < 4; ++u)
     if (col[u] >= 0) s_pos[col[u]] = static_cast<int16_t>(threadIdx.x + u * 256);
-  for (int j = threadIdx.x + 1024; j < kc; j += 256) s_pos[__ldg(idx + lo + j)] = static_cast<int16_t>(j);
+  for (int j = threadIdx.x + 1024; j < kc; j += 256) s_pos[ld_global(idx + lo + j)] = static_cast<int16_t>(j);
   __syncthreads();
   for (int e = threadIdx.x; e < n_rows * chunks; e += 256) {
     const int r = e / chunks, q = e - r * chunks;
@@ -404,8 +404,8 @@ plan_expand_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restric
 constexpr int kPlanRRows = 256;
 template <int VEC>
 __global__ void __launch_bounds__(256)
-plan_expand_r_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restrict__ row_idx,
-                     const uint16_t* __restrict__ vals, int n_out, int k_in, int h, uint16_t* __restrict__ Wx) {
+plan_expand_r_kernel(const int32_t* blk_ptr, const int32_t* row_idx,
+                     const uint16_t* vals, int n_out, int k_in, int h, uint16_t* Wx) {
   __shared__ int s_pos[kPlanRRows];
   const int a = blockIdx.x, r0 = blockIdx.y * kPlanRRows;
   const int n_rows = min(kPlanRRows, n_out - r0);
@@ -422,6 +422,8 @@ plan_expand_r_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
   const uint16_t* tile = vals + static_cast<size_t>(h) * lo;
   uint16_t* out = Wx + static_cast<size_t>(r0) * k_in + static_cast<size_t>(a) * h;
   const int per_row = h / VEC;
+  // (the places come from this kernel's own loads, so these are behind the wait; unlike ordinary loads they may pass the
+  // stores of the element before)
 #pragma unroll 4
   for (int e = threadIdx.x; e < n_rows * per_row; e += 256) {
     const int r = e / per_row, c = (e - r * per_row) * VEC;
@@ -429,11 +431,11 @@ plan_expand_r_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
     uint16_t* dst = out + static_cast<size_t>(r) * k_in + c;
     const uint16_t* src = tile + static_cast<size_t>(p) * h + c;
     if (VEC == 8) {
-      *reinterpret_cast<uint4*>(dst) = p >= 0 ? __ldg(reinterpret_cast<const uint4*>(src)) : make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(dst) = p >= 0 ? __ldcg(reinterpret_cast<const uint4*>(src)) : make_uint4(0u, 0u, 0u, 0u);
     } else if (VEC == 4) {
-      *reinterpret_cast<uint2*>(dst) = p >= 0 ? __ldg(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
+      *reinterpret_cast<uint2*>(dst) = p >= 0 ? __ldcg(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
     } else {
-      *dst = p >= 0 ? *src : static_cast<uint16_t>(0);
+      *dst = p >= 0 ? __ldcg(src) : static_cast<uint16_t>(0);
     }
   }
 }
@@ -457,8 +459,8 @@ struct PlanTGeometry {
   int segments;             // 64-row segments of a row-block taller than 64 rows, else 1
 };
 __global__ void __launch_bounds__(kPlanTThreads, 4)
-plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restrict__ idx,
-                     const uint16_t* __restrict__ vals, PlanTGeometry G, uint16_t* __restrict__ PT) {
+plan_expand_t_kernel(const int32_t* blk_ptr, const int32_t* idx,
+                     const uint16_t* vals, PlanTGeometry G, uint16_t* PT) {
   __shared__ int32_t s_col_pos[kPlanTMaxBlocks][kPlanTK];
   __shared__ uint16_t s_t[kPlanTK][kPlanTN + 2];
   __shared__ int32_t s_ptr[kPlanTMaxBlocks + 1];
@@ -473,7 +475,7 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
   if (threadIdx.x == 0) prefetch_line(blk_ptr + b0);
   pdl_wait();
   pdl_launch_dependents();
-  if (static_cast<int>(threadIdx.x) <= nb) s_ptr[threadIdx.x] = __ldg(blk_ptr + b0 + threadIdx.x);
+  if (static_cast<int>(threadIdx.x) <= nb) s_ptr[threadIdx.x] = ld_global(blk_ptr + b0 + threadIdx.x);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   {
@@ -490,7 +492,7 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
     const int lo = s_ptr[q], kc = s_ptr[q + 1] - lo;
     int first = 0, last = kc;                                  // where columns of the tile can stand
     if (kc > 256) {
-      const int col = __ldg(idx + lo + static_cast<int>(static_cast<long long>(kc) * lane >> 5));
+      const int col = ld_global(idx + lo + static_cast<int>(static_cast<long long>(kc) * lane >> 5));
       const int below = __popc(__ballot_sync(0xffffffffu, col < k0)), upto = __popc(__ballot_sync(0xffffffffu, col < k0 + nk));
       if (below > 0) first = static_cast<int>(static_cast<long long>(kc) * (below - 1) >> 5);
       if (upto < 32) last = static_cast<int>(static_cast<long long>(kc) * upto >> 5);
@@ -498,7 +500,7 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
     for (int j0 = first + lane; j0 < last; j0 += 8 * 32) {
       int k[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) k[u] = j0 + u * 32 < last ? __ldg(idx + lo + j0 + u * 32) - k0 : -1;
+      for (int u = 0; u < 8; ++u) k[u] = j0 + u * 32 < last ? ld_global(idx + lo + j0 + u * 32) - k0 : -1;
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (static_cast<unsigned>(k[u]) < static_cast<unsigned>(nk)) s_col_pos[q][k[u]] = j0 + u * 32;
@@ -524,8 +526,8 @@ plan_expand_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restr
   for (int i = 0; i < kRows; ++i) {
     v[i][0] = v[i][1] = 0u;
     if (n_first + i >= n_rows) continue;
-    if (p0 >= 0) v[i][0] = __ldg(row + p0);
-    if (p1 >= 0) v[i][1] = __ldg(row + p1);
+    if (p0 >= 0) v[i][0] = ld_global(row + p0);
+    if (p1 >= 0) v[i][1] = ld_global(row + p1);
     row += kc;
     if (++r == rows_per_block) { r = 0; ++q; enter(); }
   }

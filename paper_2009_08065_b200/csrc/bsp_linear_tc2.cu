@@ -207,7 +207,7 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     for (int tile = pair; tile < total_tiles && ok; tile += n_pairs) {
       const int m0 = (tile / n_tiles) * 256 + static_cast<int>(rank) * kBlockM, n0 = (tile % n_tiles) * kPairBN;
       for (int c = epi_tid; c < kPairBN; c += 256)
-        s_bias[acc * kPairBN + c] = (P.bias != nullptr && n0 + c < P.n_out) ? __ldg(P.bias + n0 + c) : static_cast<uint16_t>(0);
+        s_bias[acc * kPairBN + c] = (P.bias != nullptr && n0 + c < P.n_out) ? ld_global(P.bias + n0 + c) : static_cast<uint16_t>(0);
       epilogue_sync_all();
       // all 256 threads take the same decision, so nobody is left alone at a named barrier below
       if (!epilogue_all_ok(mbar_wait(acc_full_bar(acc), acc_phase[acc], P.status))) { ok = false; break; }

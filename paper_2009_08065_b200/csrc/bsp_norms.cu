@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(32) clear_penalty_kernel(double* penalty) {
 // contiguously by the warp).  R: lanes run along the strips of one row (adjacent groups are
 // adjacent in memory).
 __global__ void __launch_bounds__(256)
-norms_generic_kernel(const uint16_t* __restrict__ W, int rows, int cols, int ldw, int block, int orient, int vec,
+norms_generic_kernel(const uint16_t* W, int rows, int cols, int ldw, int block, int orient, int vec,
                      NormOut o) {
   pdl_wait();
   pdl_launch_dependents();

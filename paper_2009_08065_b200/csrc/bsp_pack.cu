@@ -42,17 +42,33 @@ __device__ __forceinline__ size_t group_slot(const Geometry& G, int b, int g) {
 }
 
 // Float32 sum of squares of group g of block b.
-__device__ __forceinline__ float group_sum(const uint16_t* __restrict__ W, const Geometry& G, int b, int g) {
+__device__ __forceinline__ float group_sum(const uint16_t* W, const Geometry& G, int b, int g) {
   size_t stride;
   const uint16_t* p = group_ptr(W, G, b, g, &stride);
   return G.orient == BSP_ORIENT_C ? group_sumsq_strided(p, G.block, stride) : group_sumsq_contig(p, G.block, G.vec);
 }
 
+// n elements from stride to stride, four loads in flight.
+template <class T>
+__device__ __forceinline__ void copy_strided(T* dst, size_t dst_stride, const T* src, size_t src_stride, int n) {
+  int left = n;
+#pragma unroll 1
+  for (; left >= 4; left -= 4) {
+    T v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u, src += src_stride) v[u] = ld_global(src);
+#pragma unroll
+    for (int u = 0; u < 4; ++u, dst += dst_stride) *dst = v[u];
+  }
+#pragma unroll 1
+  for (; left > 0; --left, src += src_stride, dst += dst_stride) *dst = ld_global(src);
+}
+
 // (1a) threshold mode, one CTA per block.
 __global__ void __launch_bounds__(1024)
-flags_threshold_kernel(const uint16_t* __restrict__ W, Geometry G, float threshold,
-                       const float* __restrict__ threshold_dev, uint8_t* __restrict__ keep,
-                       int32_t* __restrict__ counts) {
+flags_threshold_kernel(const uint16_t* W, Geometry G, float threshold,
+                       const float* threshold_dev, uint8_t* keep,
+                       int32_t* counts) {
   __shared__ int s_count;
   if (threadIdx.x == 0) s_count = 0;
   pdl_wait();
@@ -86,10 +102,12 @@ flags_threshold_kernel(const uint16_t* __restrict__ W, Geometry G, float thresho
 // groups 105 -> 46 us, 64 strips of 768 28 -> 16, 11 row-blocks of 3072 44 -> 33, 192 of 768 22.6 -> 18.5.
 constexpr int kTopkDigit = 11;                       // 31 bits = 11 + 10 + 10
 constexpr int kTopkBins = 1 << kTopkDigit;
+// (CTAs per SM that leave the registers for ten rows of eight columns in flight; left alone the compiler takes 32 and
+// spills, and a block of 256 rows 2 x as long.)
 template <int T>
-__global__ void __launch_bounds__(T)
-flags_topk_kernel(const uint16_t* __restrict__ W, Geometry G, int keep_count,
-                  uint8_t* __restrict__ keep, int32_t* __restrict__ counts, int32_t* __restrict__ seg_counts) {
+__global__ void __launch_bounds__(T, T == 1024 ? 2 : T == 512 ? 3 : 6)
+flags_topk_kernel(const uint16_t* W, Geometry G, int keep_count,
+                  uint8_t* keep, int32_t* counts, int32_t* seg_counts) {
   extern __shared__ uint32_t s_key[];                // [n_groups]
   __shared__ int s_seg[BSP_TOPK_MAX_GROUPS / kSegment];
   __shared__ uint32_t hist[kTopkBins];
@@ -197,8 +215,8 @@ cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, ui
 // (2) counts -> blk_ptr (exclusive scan) and the kept-weight total: matrices with more blocks than the
 // compaction kernel adds up by itself.
 __global__ void __launch_bounds__(1024)
-scan_counts_kernel(const int32_t* __restrict__ counts, int n_blocks, int block,
-                   int32_t* __restrict__ blk_ptr, int64_t* __restrict__ kept_weights) {
+scan_counts_kernel(const int32_t* counts, int n_blocks, int block,
+                   int32_t* blk_ptr, int64_t* kept_weights) {
   __shared__ int s_warp[32];
   pdl_wait();
   pdl_launch_dependents();
@@ -222,9 +240,9 @@ scan_counts_kernel(const int32_t* __restrict__ counts, int n_blocks, int block,
 // CTA from L2), without it blk_ptr is there already.  Orientation R: a thread moves its whole group, by
 // vectors of G.vec elements; the kept groups of a warp are neighbours in the tile.
 __global__ void __launch_bounds__(1024)
-compact_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep, const int32_t* __restrict__ counts,
-               int32_t* __restrict__ blk_ptr, int32_t* __restrict__ idx, uint16_t* __restrict__ vals,
-               int64_t* __restrict__ kept_weights) {
+compact_kernel(const uint16_t* W, Geometry G, const uint8_t* keep, const int32_t* counts,
+               int32_t* blk_ptr, int32_t* idx, uint16_t* vals,
+               int64_t* kept_weights) {
   __shared__ int s_warp[32];
   const int b = blockIdx.x;
   pdl_wait();
@@ -262,18 +280,10 @@ compact_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __rest
       size_t stride;
       const uint16_t* src = group_ptr(W, G, b, g, &stride);
       uint16_t* dst = tile + static_cast<size_t>(p) * G.block;
-      if (G.orient == BSP_ORIENT_C) {
-        // tile [d, kc]: element r of the group goes to row r, position p
-        for (int r = 0; r < G.block; ++r) tile[static_cast<size_t>(r) * kc + p] = src[static_cast<size_t>(r) * stride];
-      } else if (vec == 8) {
-#pragma unroll 4
-        for (int c = 0; c < G.block; c += 8) *reinterpret_cast<uint4*>(dst + c) = __ldg(reinterpret_cast<const uint4*>(src + c));
-      } else if (vec == 4) {
-#pragma unroll 4
-        for (int c = 0; c < G.block; c += 4) *reinterpret_cast<uint2*>(dst + c) = __ldg(reinterpret_cast<const uint2*>(src + c));
-      } else {
-        for (int c = 0; c < G.block; ++c) dst[c] = src[c];
-      }
+      if (G.orient == BSP_ORIENT_C) copy_strided(tile + p, kc, src, stride, G.block);   // tile [d, kc]: element r goes to row r
+      else if (vec == 8) copy_strided(reinterpret_cast<uint4*>(dst), 1, reinterpret_cast<const uint4*>(src), 1, G.block >> 3);
+      else if (vec == 4) copy_strided(reinterpret_cast<uint2*>(dst), 1, reinterpret_cast<const uint2*>(src), 1, G.block >> 2);
+      else copy_strided(dst, 1, src, 1, G.block);
     }
   }
 }
@@ -284,8 +294,8 @@ compact_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __rest
 // Latency-bound.  3072 x 1024, the two launches: 64-column strips 30.8 -> 7.5 us, 16-column 15.7 -> 9.4; 768 x 768 in
 // 12-column strips 8.2 -> 6.2.
 __global__ void __launch_bounds__(kSegment)
-flags_segment_kernel(const uint16_t* __restrict__ W, Geometry G, float threshold, const float* __restrict__ threshold_dev,
-                     uint8_t* __restrict__ keep, int32_t* __restrict__ seg_counts) {
+flags_segment_kernel(const uint16_t* W, Geometry G, float threshold, const float* threshold_dev,
+                     uint8_t* keep, int32_t* seg_counts) {
   __shared__ int s_warp[kSegment / 32];
   const int b = blockIdx.x, g = blockIdx.y * kSegment + threadIdx.x;
   pdl_wait();
@@ -309,9 +319,9 @@ flags_segment_kernel(const uint16_t* __restrict__ W, Geometry G, float threshold
 
 template <int VEC>
 __global__ void __launch_bounds__(kSegment)
-compact_segment_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep,
-                       const int32_t* __restrict__ seg_counts, int32_t* __restrict__ blk_ptr, int32_t* __restrict__ idx,
-                       uint16_t* __restrict__ vals, int64_t* __restrict__ kept_weights) {
+compact_segment_kernel(const uint16_t* W, Geometry G, const uint8_t* keep,
+                       const int32_t* seg_counts, int32_t* blk_ptr, int32_t* idx,
+                       uint16_t* vals, int64_t* kept_weights) {
   __shared__ int s_base[kSegment / 32], s_warp[kSegment / 32];
   __shared__ int s_group[kSegment];
   const int b = blockIdx.x, segments = gridDim.y, seg = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -349,27 +359,33 @@ compact_segment_kernel(const uint16_t* __restrict__ W, Geometry G, const uint8_t
   const int per = G.block / VEC;
   const uint16_t* strip = W + static_cast<size_t>(b) * G.block;
   uint16_t* out = vals + static_cast<size_t>(G.block) * base;
-#pragma unroll 4
-  for (int e = threadIdx.x; e < m * per; e += kSegment) {
-    const int q = e / per, c = (e - q * per) * VEC;
-    const uint16_t* src = strip + static_cast<size_t>(s_group[q]) * G.ldw + c;
-    uint16_t* dst = out + static_cast<size_t>(e) * VEC;
-    if (VEC == 8) *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(src));
-    else if (VEC == 4) *reinterpret_cast<uint2*>(dst) = __ldg(reinterpret_cast<const uint2*>(src));
-    else *dst = __ldg(src);
+  using Vec = vector_of<VEC>;
+  for (int e0 = threadIdx.x; e0 < m * per; e0 += 4 * kSegment) {
+    Vec v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = min(e0 + u * kSegment, m * per - 1);
+      const int q = e / per, c = (e - q * per) * VEC;
+      v[u] = ld_global(reinterpret_cast<const Vec*>(strip + static_cast<size_t>(s_group[q]) * G.ldw + c));
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * kSegment;
+      if (e < m * per) *reinterpret_cast<Vec*>(out + static_cast<size_t>(e) * VEC) = v[u];
+    }
   }
 }
 
 // Orientation C, 8 adjacent columns per thread: nothing is read but the flags, and only pieces with a
 // pruned group are written.
 __global__ void __launch_bounds__(256)
-apply_mask_c_kernel(uint16_t* __restrict__ W, int rows, int cols, int ldw, int block, const uint8_t* __restrict__ keep) {
+apply_mask_c_kernel(uint16_t* W, int rows, int cols, int ldw, int block, const uint8_t* keep) {
   pdl_wait();
   pdl_launch_dependents();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= (cols >> 3)) return;
   for (int i = blockIdx.y; i < rows; i += gridDim.y) {
-    const uint2 f = __ldg(reinterpret_cast<const uint2*>(keep + static_cast<size_t>(i / block) * cols + (q << 3)));
+    const uint2 f = ld_global(reinterpret_cast<const uint2*>(keep + static_cast<size_t>(i / block) * cols + (q << 3)));
     if (((f.x - 0x01010101u) & ~f.x & 0x80808080u) == 0u && ((f.y - 0x01010101u) & ~f.y & 0x80808080u) == 0u) continue;   // no zero byte
     uint16_t* w = W + static_cast<size_t>(i) * ldw + (q << 3);
     if ((f.x | f.y) == 0u) {
@@ -382,7 +398,7 @@ apply_mask_c_kernel(uint16_t* __restrict__ W, int rows, int cols, int ldw, int b
   }
 }
 __global__ void __launch_bounds__(256)
-apply_mask_kernel(uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep) {
+apply_mask_kernel(uint16_t* W, Geometry G, const uint8_t* keep) {
   pdl_wait();
   pdl_launch_dependents();
   const long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;

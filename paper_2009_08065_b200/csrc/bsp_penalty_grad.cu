@@ -54,9 +54,9 @@ grad_c_tile_kernel(GradArgs A) {
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     const int r = row + 8 * i;
-    if (on && r < A.block) w[i] = __ldg(reinterpret_cast<const uint4*>(A.W + (r0 + r) * A.ldw + c));
+    if (on && r < A.block) w[i] = ld_global(reinterpret_cast<const uint4*>(A.W + (r0 + r) * A.ldw + c));
   }
-  const float gamma = c0 + static_cast<int>(threadIdx.x) < A.cols ? __ldg(A.gamma + static_cast<size_t>(b) * A.cols + c0 + threadIdx.x) : 0.0f;
+  const float gamma = c0 + static_cast<int>(threadIdx.x) < A.cols ? ld_global(A.gamma + static_cast<size_t>(b) * A.cols + c0 + threadIdx.x) : 0.0f;
   if (A.accumulate) {
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
@@ -114,8 +114,8 @@ grad_c_vec8_kernel(GradArgs A) {
   const int b = static_cast<int>(item / chunks), q = static_cast<int>(item - static_cast<long long>(b) * chunks);
   const uint16_t* p = A.W + static_cast<size_t>(b) * A.block * A.ldw + (q << 3);
   float factor[8];
-  const float4 g0 = __ldg(reinterpret_cast<const float4*>(A.gamma + static_cast<size_t>(b) * A.cols + (q << 3)));
-  const float4 g1 = __ldg(reinterpret_cast<const float4*>(A.gamma + static_cast<size_t>(b) * A.cols + (q << 3) + 4));
+  const float4 g0 = ld_global(reinterpret_cast<const float4*>(A.gamma + static_cast<size_t>(b) * A.cols + (q << 3)));
+  const float4 g1 = ld_global(reinterpret_cast<const float4*>(A.gamma + static_cast<size_t>(b) * A.cols + (q << 3) + 4));
   const float gam[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
   if (A.squared) {
 #pragma unroll
@@ -129,8 +129,11 @@ grad_c_vec8_kernel(GradArgs A) {
       factor[i] = n > 0.0f ? __fdiv_rn(A.scale * gam[i], n) : 0.0f;
     }
   }
+  uint4 next = ld_global(reinterpret_cast<const uint4*>(p));     // a row ahead of the stores
   for (int r = 0; r < A.block; ++r) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p + static_cast<size_t>(r) * A.ldw));
+    const uint4 v = next;
+    p += A.ldw;
+    if (r + 1 < A.block) next = ld_global(reinterpret_cast<const uint4*>(p));
     const uint32_t w32[4] = {v.x, v.y, v.z, v.w};
     float o[8];
 #pragma unroll

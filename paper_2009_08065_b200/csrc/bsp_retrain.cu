@@ -36,7 +36,7 @@ struct AdamArgs {
 __device__ __forceinline__ void adam_item(const AdamArgs& A, int r, int c) {
   const size_t iw = static_cast<size_t>(r) * A.ldw + c, ig = static_cast<size_t>(r) * A.ldg + c;
   const float4 w4 = *reinterpret_cast<const float4*>(A.W + iw);
-  const float4 g4 = __ldg(reinterpret_cast<const float4*>(A.G + ig));
+  const float4 g4 = ld_global(reinterpret_cast<const float4*>(A.G + ig));
   const float4 m4 = *reinterpret_cast<const float4*>(A.M + iw);
   const float4 v4 = *reinterpret_cast<const float4*>(A.V + iw);
   float w[4] = {w4.x, w4.y, w4.z, w4.w};
@@ -48,7 +48,7 @@ __device__ __forceinline__ void adam_item(const AdamArgs& A, int r, int c) {
     if (A.orient == BSP_ORIENT_C) {
       const uint8_t* f = A.keep + static_cast<size_t>(r / A.block) * A.cols + c;
       if (A.keep_vec) {
-        const uint32_t f4 = __ldg(reinterpret_cast<const uint32_t*>(f));
+        const uint32_t f4 = ld_global(reinterpret_cast<const uint32_t*>(f));
 #pragma unroll
         for (int i = 0; i < 4; ++i) keep[i] = (f4 >> (8 * i)) & 0xffu;
       } else {
@@ -119,8 +119,8 @@ masked_adam_kernel(AdamArgs A) {
 // matrices, on average: 5.3 us gathering from global memory, 2.9 us.
 constexpr int kRepackRows = 4, kRepackThreads = 256, kRepackLoads = 6;
 __global__ void __launch_bounds__(kRepackThreads)
-repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, const int32_t* __restrict__ blk_ptr,
-                  const int32_t* __restrict__ idx, uint16_t* __restrict__ vals) {
+repack_vec_kernel(const uint16_t* W, int cols, int ldw, int block, const int32_t* blk_ptr,
+                  const int32_t* idx, uint16_t* vals) {
   extern __shared__ __align__(16) uint16_t s_rows[];             // [kRepackRows][cols], then the list [cols]
   const int b = blockIdx.x, r_lo = blockIdx.y * kRepackRows, n_rows = min(kRepackRows, block - r_lo);
   const int chunks = cols >> 3;
@@ -130,12 +130,12 @@ repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, 
     prefetch_bytes(W + (static_cast<size_t>(b) * block + r_lo + threadIdx.x) * ldw, static_cast<uint32_t>(cols) * 2u);
   pdl_wait();
   pdl_launch_dependents();
-  const int lo = __ldg(blk_ptr + b), kc = __ldg(blk_ptr + b + 1) - lo;
+  const int lo = ld_global(blk_ptr + b), kc = ld_global(blk_ptr + b + 1) - lo;
   int col[4];                                                    // the first of the list, in flight beside the rows
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int p = static_cast<int>(threadIdx.x) + u * kRepackThreads;
-    if (p < kc) col[u] = __ldg(idx + lo + p);
+    if (p < kc) col[u] = ld_global(idx + lo + p);
   }
   const uint16_t* src = W + (static_cast<size_t>(b) * block + r_lo) * ldw;
   const int total = n_rows * chunks;
@@ -144,7 +144,7 @@ repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, 
 #pragma unroll
     for (int u = 0; u < kRepackLoads; ++u) {
       const int e = e0 + u * kRepackThreads, r = e / chunks;
-      if (e < total) v[u] = __ldg(reinterpret_cast<const uint4*>(src + static_cast<size_t>(r) * ldw + ((e - r * chunks) << 3)));
+      if (e < total) v[u] = ld_global(reinterpret_cast<const uint4*>(src + static_cast<size_t>(r) * ldw + ((e - r * chunks) << 3)));
     }
 #pragma unroll
     for (int u = 0; u < kRepackLoads; ++u) {
@@ -157,7 +157,7 @@ repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, 
     const int p = static_cast<int>(threadIdx.x) + u * kRepackThreads;
     if (p < kc) s_list[p] = static_cast<uint16_t>(col[u]);
   }
-  for (int p = threadIdx.x + 4 * kRepackThreads; p < kc; p += kRepackThreads) s_list[p] = static_cast<uint16_t>(__ldg(idx + lo + p));
+  for (int p = threadIdx.x + 4 * kRepackThreads; p < kc; p += kRepackThreads) s_list[p] = static_cast<uint16_t>(ld_global(idx + lo + p));
   __syncthreads();
   uint16_t* tile = vals + static_cast<size_t>(block) * lo + static_cast<size_t>(r_lo) * kc;
   if ((reinterpret_cast<uintptr_t>(tile) & 3) == 0 && (kc & 1) == 0) {
@@ -182,8 +182,8 @@ repack_vec_kernel(const uint16_t* __restrict__ W, int cols, int ldw, int block, 
 
 // Any alignment or width.
 __global__ void __launch_bounds__(256)
-repack_kernel(const uint16_t* __restrict__ W, int ldw, int block, const int32_t* __restrict__ blk_ptr,
-              const int32_t* __restrict__ idx, uint16_t* __restrict__ vals) {
+repack_kernel(const uint16_t* W, int ldw, int block, const int32_t* blk_ptr,
+              const int32_t* idx, uint16_t* vals) {
   const int b = blockIdx.x;
   pdl_wait();
   pdl_launch_dependents();
@@ -191,9 +191,19 @@ repack_kernel(const uint16_t* __restrict__ W, int ldw, int block, const int32_t*
   const uint16_t* wblk = W + static_cast<size_t>(b) * block * ldw;
   uint16_t* tile = vals + static_cast<size_t>(block) * lo;
   const int r_lo = blockIdx.y * kRepackRows, r_hi = min(block, r_lo + kRepackRows);
-  for (int r = r_lo; r < r_hi; ++r)
-    for (int p = threadIdx.x; p < kc; p += blockDim.x)
-      tile[static_cast<size_t>(r) * kc + p] = wblk[static_cast<size_t>(r) * ldw + __ldg(idx + lo + p)];
+  for (int p0 = threadIdx.x; p0 < kc; p0 += 4 * 256) {
+    int col[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) col[u] = ld_global(idx + lo + min(p0 + u * 256, kc - 1));
+    for (int r = r_lo; r < r_hi; ++r) {
+      uint16_t v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = ld_global(wblk + static_cast<size_t>(r) * ldw + col[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (p0 + u * 256 < kc) tile[static_cast<size_t>(r) * kc + p0 + u * 256] = v[u];
+    }
+  }
 }
 
 // Algorithm 2's mask loop: Mask_ij = 0 if W_ij == 0 else 1 (either sign of zero is zero).

@@ -254,7 +254,7 @@ sums_stream_kernel(const __grid_constant__ SelectBatchT<N> B) {
 // Orientation R: one thread per group, neighbouring threads on neighbouring groups of a row.
 constexpr int kSumRThreads = 256;
 __global__ void __launch_bounds__(kSumRThreads + 32)
-sums_r_kernel(const uint16_t* __restrict__ W, int rows, int per_row, int ldw, int block, int vec, float* __restrict__ S,
+sums_r_kernel(const uint16_t* W, int rows, int per_row, int ldw, int block, int vec, float* S,
               uint32_t* head, int replicas) {
   __shared__ __align__(16) uint32_t hist[kBins1];
   if (head != nullptr) clear_bins(hist);
@@ -325,7 +325,7 @@ __device__ __forceinline__ Pick pick_bin(const uint32_t* hist, uint32_t want, ui
 // Calls f(key) for every key whose upper bits (from bit `above` on) are `prefix`: one CTA, all of the keys
 // (read from L2: a list was written by other CTAs of the same launch).
 template <class F>
-__device__ __forceinline__ void for_matching(const uint32_t* __restrict__ keys, long long n, int above, uint32_t prefix, F f) {
+__device__ __forceinline__ void for_matching(const uint32_t* keys, long long n, int above, uint32_t prefix, F f) {
   const uint4* v4 = reinterpret_cast<const uint4*>(keys);
   const long long n4 = n >> 2;
   for (long long i = threadIdx.x; i < n4; i += 4 * kSelThreads) {
