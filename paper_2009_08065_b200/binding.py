@@ -277,15 +277,24 @@ def make_job_array(jobs):
     return arr
 
 
+def _job_array(jobs):
+    """The address of a descriptor array goes to C++ as a number, so its type is checked here."""
+    if not isinstance(jobs, ctypes.Array):
+        return make_job_array(jobs)
+    if jobs._type_ is not _LayerJob:
+        raise ctypes.ArgumentError(f"expected an array made by make_job_array, got {type(jobs).__name__}")
+    return jobs
+
+
 def bsp_prepare_batched(jobs, block: int, eps: float = 1e-3, pen: int = PEN_L2, stream=None) -> None:
     """jobs: a list of LayerJob, or an array made by make_job_array."""
-    arr = jobs if isinstance(jobs, ctypes.Array) else make_job_array(jobs)
+    arr = _job_array(jobs)
     _check(_native.prepare_batched(ctypes.addressof(arr), len(arr), block, eps, pen, stream), "bsp_prepare_batched")
 
 
 def bsp_percentile_threshold_batched(jobs, block: int, rates, stream=None) -> None:
     """Per-matrix percentile thresholds for a job array (each job's threshold_dev tensor receives its threshold)."""
-    arr = jobs if isinstance(jobs, ctypes.Array) else make_job_array(jobs)
+    arr = _job_array(jobs)
     r = (_d * len(arr))(*[float(v) for v in rates])
     _check(_native.percentile_threshold_batched(ctypes.addressof(arr), len(arr), block, ctypes.addressof(r), stream),
            "bsp_percentile_threshold_batched")
@@ -478,6 +487,8 @@ def bsp_linear_route(call) -> int:
 
 def bsp_linear_run(call, route: int = ROUTE_AUTO, stream=None) -> int:
     """Runs the layer; returns the route taken (ROUTE_ZERO_EXPANDED or ROUTE_GATHERED)."""
+    if not isinstance(call, _LinearCall):
+        raise ctypes.ArgumentError(f"expected a descriptor made by make_linear_call, got {type(call).__name__}")
     r = _native.linear_run(ctypes.addressof(call), route, stream)     # the route, or a negative status
     if r < 0:
         _check(r, "bsp_linear_run")
