@@ -10,6 +10,7 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 #include <algorithm>
 
@@ -58,24 +59,27 @@ class Args {
     return v;
   }
   float f32(int i) const { return static_cast<float>(real(i)); }
-  // None = torch's current stream; otherwise a stream object or a raw handle.
+  // None = torch's current stream; otherwise a stream object, a raw handle, or a ctypes object that holds one.
   void* stream(int i) const {
     if (a_[i] == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-    if (PyLong_Check(a_[i])) return PyLong_AsVoidPtr(a_[i]);
+    if (PyLong_Check(a_[i])) return handle(a_[i]);
     PyObject* h = PyObject_GetAttrString(a_[i], "cuda_stream");
+    if (h == nullptr && PyErr_ExceptionMatches(PyExc_AttributeError)) {
+      PyErr_Clear();
+      h = PyObject_GetAttrString(a_[i], "value");
+    }
     if (h == nullptr) throw python_error();
-    void* s = PyLong_AsVoidPtr(h);
-    Py_DECREF(h);
-    if (s == nullptr && PyErr_Occurred()) throw python_error();
-    return s;
+    const THPObjectPtr owner(h);
+    return h == Py_None ? nullptr : handle(h);              // (the value of a null pointer is None)
   }
-  void* address(int i) const {
-    void* p = PyLong_AsVoidPtr(a_[i]);
+  void* address(int i) const { return handle(a_[i]); }
+
+ private:
+  static void* handle(PyObject* number) {
+    void* p = PyLong_AsVoidPtr(number);
     if (p == nullptr && PyErr_Occurred()) throw python_error();
     return p;
   }
-
- private:
   PyObject* const* a_;
 };
 
