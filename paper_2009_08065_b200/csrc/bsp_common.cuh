@@ -12,7 +12,10 @@ namespace bsp {
 // Last CUDA error seen by this host thread inside the library.
 int& last_cuda_error_ref();
 
+// (The runtime keeps the error of a failed call until it is asked for it: left there, the check behind the next plain
+// launch would report it again.)
 inline int cuda_fail(cudaError_t e) {
+  cudaGetLastError();
   last_cuda_error_ref() = static_cast<int>(e);
   return BSP_ERR_CUDA;
 }
