@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "bsp.h"
 
 namespace bsp {
@@ -121,6 +123,28 @@ inline int contig_vec(const void* W, int ldw, int block) {
   if (block % 4 == 0 && ldw % 4 == 0 && aligned_to(W, 8)) return 4;
   return 1;
 }
+
+// Set-up that a kernel needs once on every device before its first launch.  First calls may come from several host
+// threads at once (the binding runs them without the interpreter lock); doing it twice does no harm.
+struct OncePerDevice {
+  std::atomic<bool> done[64];
+};
+template <class K>
+inline int allow_dynamic_smem(OncePerDevice& once, K* kernel, int bytes) {
+  int device = 0;
+  BSP_CUDA_TRY(cudaGetDevice(&device));
+  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
+  if (!once.done[device].load(std::memory_order_acquire)) {
+    BSP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    once.done[device].store(true, std::memory_order_release);
+  }
+  return BSP_OK;
+}
+#define BSP_TRY(expr)                \
+  do {                               \
+    const int _st = (expr);          \
+    if (_st != BSP_OK) return _st;   \
+  } while (0)
 
 #ifdef __CUDACC__
 // Launch with programmatic stream serialization: the grid may take its seats while the previous kernel of

@@ -688,17 +688,12 @@ int fused_stream(const FusedJob* jobs, int n_jobs, int block, float eps, int squ
   int per_sm = 0;
   int st = BSP_OK;
   if (ok) {
-    if (!td->attr_set[7]) {
-      cudaError_t e = cudaFuncSetAttribute(fused_stream_kernel<kStreamMaxJobs, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fused_stream_kernel<kStreamMaxJobs, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fused_stream_kernel<kStreamFewJobs, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fused_stream_kernel<kStreamFewJobs, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap);
-      if (e != cudaSuccess) { delete B; return cuda_fail(e); }
-      td->attr_set[7] = true;
-    }
+    static OncePerDevice once[4];
+    st = allow_dynamic_smem(once[0], fused_stream_kernel<kStreamMaxJobs, false>, kSmemCap);
+    if (st == BSP_OK) st = allow_dynamic_smem(once[1], fused_stream_kernel<kStreamMaxJobs, true>, kSmemCap);
+    if (st == BSP_OK) st = allow_dynamic_smem(once[2], fused_stream_kernel<kStreamFewJobs, false>, kSmemCap);
+    if (st == BSP_OK) st = allow_dynamic_smem(once[3], fused_stream_kernel<kStreamFewJobs, true>, kSmemCap);
+    if (st != BSP_OK) { delete B; return st; }
     int per_sm_one_wave = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_stream_kernel<kStreamMaxJobs, false>, kStreamThreads, smem_max);
     if (e == cudaSuccess)

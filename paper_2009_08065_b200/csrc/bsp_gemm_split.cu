@@ -20,8 +20,6 @@
 // on one SM share its path to L2 (768 outputs x 768 inputs, C = 4: 4.2 us against 3.7).
 // All waits are bounded.  A CTA whose wait ran out stays until the rest of its cluster has left: what they were still
 // going to send arrives in memory that exists.
-#include <atomic>
-
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -399,14 +397,8 @@ int launch_split(TcDevice* dev, const CUtensorMap& map_a, const CUtensorMap& map
   P.bars_off = kTn ? (P.stages * kStage > kExchange ? P.stages * kStage : kExchange) : P.recv_off + kReceive;
   if (P.bars_off < kAlone) P.bars_off = kAlone;
   P.status = dev->status;
-  static std::atomic<bool> attr_set[64];
-  int device = 0;
-  BSP_CUDA_TRY(cudaGetDevice(&device));
-  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
-  if (!attr_set[device].load(std::memory_order_acquire)) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(gemm_split_kernel<BN, C, kTn>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
-    attr_set[device].store(true, std::memory_order_release);
-  }
+  static OncePerDevice once;
+  BSP_TRY(allow_dynamic_smem(once, gemm_split_kernel<BN, C, kTn>, kSmemLimit));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((P.rows + kBlockM - 1) / kBlockM * P.n_tiles * C);
   cfg.blockDim = dim3(kSplitThreads);

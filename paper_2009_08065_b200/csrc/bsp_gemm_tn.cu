@@ -12,8 +12,6 @@
 // bounded waits) is the pipeline of bsp_linear_tc.cu with a 128 x BN output tile.
 // The epilogue applies the mask (pruned groups of dW are written as zero).  A weight of fewer tiles than SMs goes
 // to the split contraction of bsp_gemm_split.cu instead where that is faster.
-#include <atomic>
-
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -235,14 +233,8 @@ template <int BN>
 int launch_tn(TcDevice* dev, const CUtensorMap& map_dy, const CUtensorMap& map_x, const CUtensorMap& map_dw, const TnParams& P,
               cudaStream_t s) {
   using Cfg = TileCfg<BN>;
-  static std::atomic<bool> attr_set[64];
-  int device = 0;
-  BSP_CUDA_TRY(cudaGetDevice(&device));
-  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
-  if (!attr_set[device].load(std::memory_order_acquire)) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(gemm_tn_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    attr_set[device].store(true, std::memory_order_release);
-  }
+  static OncePerDevice once;
+  BSP_TRY(allow_dynamic_smem(once, gemm_tn_kernel<BN>, Cfg::kSmemBytes));
   const int tiles = ((P.n_out + kBlockM - 1) / kBlockM) * ((P.k_in + BN - 1) / BN);
   BSP_CUDA_TRY(launch_pdl(gemm_tn_kernel<BN>, dim3(tiles < dev->sms ? tiles : dev->sms), dim3(kTnThreads), Cfg::kSmemBytes, s, map_dy,
                           map_x, map_dw, P));

@@ -392,10 +392,8 @@ extern "C" int bsp_linear_chain(const bsp_chain_op* ops, int n_ops, const void* 
   P.ticket = P.done + n_ops * m_tiles;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   BSP_CUDA_TRY(cudaMemsetAsync(ws, 0, need, s));
-  if (!dev->attr_set[4]) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(linear_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    dev->attr_set[4] = true;
-  }
+  static OncePerDevice once;
+  BSP_TRY(allow_dynamic_smem(once, linear_chain_kernel, Cfg::kSmemBytes));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P.total_tiles < dev->sms ? P.total_tiles : dev->sms);
   cfg.blockDim = dim3(kChainThreads);

@@ -557,14 +557,8 @@ template <int D, int GROUPS>
 int launch_gather_groups(TcDevice* dev, const GatherParams& P, cudaStream_t s) {
   using Cfg = GatherCfg<D, GROUPS>;
   static_assert(Cfg::kStages >= 4, "pipeline too shallow");
-  static bool attr_set[64] = {};
-  int device = 0;
-  BSP_CUDA_TRY(cudaGetDevice(&device));
-  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
-  if (!attr_set[device]) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(linear_gather_kernel<D, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    attr_set[device] = true;
-  }
+  static OncePerDevice once;
+  BSP_TRY(allow_dynamic_smem(once, linear_gather_kernel<D, GROUPS>, Cfg::kSmemBytes));
   CUtensorMap map_xt;      // XT as [k_in rows, tokens]; box = one row of 64 tokens, 128-byte swizzle, zeros out of range
   // (no L2 promotion: a gathered row is 128 bytes, and fetching 256 would read every line twice)
   if (!make_map(&map_xt, P.XT, P.tokens, P.k_in, P.ldxt, 1, 64, CU_TENSOR_MAP_L2_PROMOTION_L2_128B)) return BSP_ERR_CUDA;

@@ -597,7 +597,7 @@ DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, i
 namespace {
 
 template <int BN>
-int launch_tc(TcDevice* dev, int slot, const void* plan, const void* X, void* Y, const LinearParams& P, int ldx,
+int launch_tc(TcDevice* dev, const void* plan, const void* X, void* Y, const LinearParams& P, int ldx,
               int ldy, cudaStream_t s) {
   using Cfg = TileCfg<BN>;
   static_assert(Cfg::kStages >= 3, "pipeline too shallow");
@@ -610,10 +610,8 @@ int launch_tc(TcDevice* dev, int slot, const void* plan, const void* X, void* Y,
   } else if (!make_map(&map_y, Y, P.n_out, P.tokens, ldy, kBlockM, kEpiCols)) {
     return BSP_ERR_CUDA;
   }
-  if (!dev->attr_set[slot]) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(linear_tc_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    dev->attr_set[slot] = true;
-  }
+  static OncePerDevice once;
+  BSP_TRY(allow_dynamic_smem(once, linear_tc_kernel<BN>, Cfg::kSmemBytes));
   const int m_tiles = (P.tokens + kBlockM - 1) / kBlockM;
   const int n_tiles = (P.n_out + BN - 1) / BN;
   const int tiles = m_tiles * n_tiles;
@@ -766,10 +764,10 @@ extern "C" int bsp_linear_planned_ex(const void* plan, int n_out, int k_in, int 
                  transposed ? 1 : 0,
                  static_cast<const uint16_t*>(bias), dev->status};
   switch (choice.bn) {
-    case 256: return launch_tc<256>(dev, 0, plan, X, Y, P, ldx, ldy, s);
-    case 192: return launch_tc<192>(dev, 1, plan, X, Y, P, ldx, ldy, s);
-    case 128: return launch_tc<128>(dev, 2, plan, X, Y, P, ldx, ldy, s);
-    default: return launch_tc<64>(dev, 3, plan, X, Y, P, ldx, ldy, s);
+    case 256: return launch_tc<256>(dev, plan, X, Y, P, ldx, ldy, s);
+    case 192: return launch_tc<192>(dev, plan, X, Y, P, ldx, ldy, s);
+    case 128: return launch_tc<128>(dev, plan, X, Y, P, ldx, ldy, s);
+    default: return launch_tc<64>(dev, plan, X, Y, P, ldx, ldy, s);
   }
 }
 

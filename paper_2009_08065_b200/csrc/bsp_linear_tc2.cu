@@ -270,10 +270,8 @@ int launch_tc_pair(TcDevice* dev, const void* plan, const void* X, void* Y, int 
   if (!make_map(&map_x, X, k_in, tokens, ldx, kBlockM)) return BSP_ERR_CUDA;
   if (!make_map(&map_w, plan, k_in, n_out, k_in, kPairBN / 2)) return BSP_ERR_CUDA;
   if (!make_map(&map_y, Y, n_out, tokens, ldy, kBlockM, kEpiCols)) return BSP_ERR_CUDA;
-  if (!dev->attr_set[5]) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(linear_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes));
-    dev->attr_set[5] = true;
-  }
+  static OncePerDevice once;
+  BSP_TRY(allow_dynamic_smem(once, linear_tc_pair_kernel, kPairSmemBytes));
   PairParams P{tokens, n_out, k_in, act, static_cast<const uint16_t*>(bias), dev->status};
   const int tiles = ((tokens + 255) / 256) * ((n_out + kPairBN - 1) / kPairBN);
   const int pairs = tiles < dev->sms / 2 ? tiles : dev->sms / 2;

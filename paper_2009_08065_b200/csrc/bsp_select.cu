@@ -18,8 +18,6 @@
 // 16-row blocks, 54.6 -> 48.3 for 72 matrices of a BERT-base stack, when the sums no longer waited for the clearing, the
 // list was stored with predicated stores, all keys of a thread were asked for in one round, the gather kept four remote
 // loads in flight and the last digit became a ranking.
-#include <atomic>
-
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -610,14 +608,8 @@ int launch_select(const SelectBatchT<N>& B, int sms, cudaStream_t s) {
   for (int i = 0; i < B.n_jobs; ++i)
     if (B.job[i].n > largest) largest = B.job[i].n;
   const int c = select_cluster(B.n_jobs, largest, sms);
-  static std::atomic<bool> attr_set[64];            // per device; setting the attribute twice does no harm
-  int device = 0;
-  BSP_CUDA_TRY(cudaGetDevice(&device));
-  if (device < 0 || device >= 64) return BSP_ERR_CUDA;
-  if (!attr_set[device].load(std::memory_order_acquire)) {
-    BSP_CUDA_TRY(cudaFuncSetAttribute(select_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmem));
-    attr_set[device].store(true, std::memory_order_release);
-  }
+  static OncePerDevice once;
+  BSP_TRY(allow_dynamic_smem(once, select_kernel<N>, kSelSmem));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(B.n_jobs * c));
   cfg.blockDim = dim3(kSelThreads);
@@ -663,14 +655,8 @@ int launch_sums_c(SelectBatchT<N>& B, int sms, cudaStream_t s) {
     int at = 0;
     for (int i = 0; i < B.n_jobs; ++i) { B.first_block[i] = at; at += B.job[i].n_blocks * B.job[i].parts; }
     const size_t smem = 2 * round_up(static_cast<size_t>(B.block) * B.max_part_cols * 2, 128) + kBins1 * 4;
-    static std::atomic<bool> attr_set[64];
-    int device = 0;
-    BSP_CUDA_TRY(cudaGetDevice(&device));
-    if (device < 0 || device >= 64) return BSP_ERR_CUDA;
-    if (!attr_set[device].load(std::memory_order_acquire)) {
-      BSP_CUDA_TRY(cudaFuncSetAttribute(sums_stream_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSumRowBytes + 256 + kBins1 * 4));
-      attr_set[device].store(true, std::memory_order_release);
-    }
+    static OncePerDevice once;
+    BSP_TRY(allow_dynamic_smem(once, sums_stream_kernel<N>, 2 * kSumRowBytes + 256 + kBins1 * 4));
     BSP_CUDA_TRY(launch_pdl(sums_stream_kernel<N>, dim3(kSumPerSm * sms), dim3(kSumThreads), smem, s, B));
     return BSP_OK;
   }

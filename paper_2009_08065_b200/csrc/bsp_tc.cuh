@@ -423,16 +423,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 inline EncodeTiledFn encode_tiled_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  // (initialised by the first caller, while others wait for it)
+  static const EncodeTiledFn fn = [] {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
+    const bool ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return ok ? reinterpret_cast<EncodeTiledFn>(p) : nullptr;
+  }();
   return fn;
 }
 
@@ -468,7 +466,6 @@ inline int copy_rows(int tokens) { return tokens >= kBlockM ? kBlockM : (tokens 
 struct TcDevice {
   int sms = 0;
   int* status = nullptr;
-  bool attr_set[8] = {false, false, false, false, false, false, false, false};
   int split_ctas[3] = {0, 0, 0};     // CTAs of bsp_gemm_split.cu's kernel that run at once in clusters of 2, 4, 8
 };
 TcDevice* tc_device();
