@@ -379,8 +379,15 @@ extern "C" int bsp_linear_chain(const bsp_chain_op* ops, int n_ops, const void* 
     for (int i = 0; i < n_ops; ++i) {
       const bsp_chain_op& u = ops[i];
       const uint16_t* src = static_cast<const uint16_t*>(u.src >= 0 ? ops[u.src].Y : X) + u.src_col;
-      st = bsp_linear_planned(u.plan, u.n_out, u.k_in, u.block, src, tokens, u.src >= 0 ? ops[u.src].ldy : ldx, u.bias, u.act, u.Y,
-                              u.ldy, stream);
+      const int src_ld = u.src >= 0 ? ops[u.src].ldy : ldx;
+      if (u.k_in <= 12288) {
+        st = bsp_linear_planned(u.plan, u.n_out, u.k_in, u.block, src, tokens, src_ld, u.bias, u.act, u.Y, u.ldy, stream);
+      } else {               // wider than the single launches take: a chain of its own
+        bsp_chain_op alone = u;
+        alone.src = -1;
+        alone.src_col = 0;
+        st = bsp_linear_chain(&alone, 1, src, tokens, src_ld, ws, ws_bytes, stream);
+      }
       if (st != BSP_OK) return st;
     }
     return BSP_OK;

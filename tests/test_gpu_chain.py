@@ -99,3 +99,25 @@ def test_chain_argument_errors():
     with pytest.raises(bsp.BspError) as e:
         bsp.bsp_linear_chain(ops, x, ws[:16])
     assert e.value.status == -3
+
+
+def test_chain_with_an_op_wider_than_the_single_launches_take():
+    """At 8 tokens the last op is split over a cluster, which sends the chain through single launches; the second has
+    more input features than those accept."""
+    tokens, wide = 8, 12296
+    x = to_dev(si.normal_bf16(91, "widechain.x", (tokens, 256), 1.0))
+    weights = [si.normal_bf16(91, f"widechain.w{i}", s, 0.02) for i, s in enumerate([(wide, 256), (64, wide)])]
+    ys = [torch.full((tokens, w.shape[0]), 0x7FC0, dtype=torch.int16, device=DEV) for w in weights]
+    ops = [bsp.ChainOp(plan=to_dev(w), n_out=w.shape[0], k_in=w.shape[1], block=8, bias=None, act=0, Y=y, src=i - 1)
+           for i, (w, y) in enumerate(zip(weights, ys))]
+    narrow = bsp.ChainOp(plan=ops[1].plan, n_out=64, k_in=256, block=8, bias=None, act=0, src=-1,
+                         Y=torch.full((tokens, 64), 0x7FC0, dtype=torch.int16, device=DEV))
+    ops.append(narrow)
+    ws = torch.empty(bsp.bsp_linear_chain_ws_bytes(3, tokens), dtype=torch.uint8, device=DEV)
+    bsp.bsp_linear_chain(ops, x, ws)
+    bsp.bsp_linear_status()
+    xs = bits_of(x)
+    for op, w in zip(ops, [weights[0], weights[1], weights[1].reshape(-1)[: 64 * 256].reshape(64, 256)]):
+        src = xs if op.src < 0 else bits_of(ops[op.src].Y)
+        m, b = O.mask_of(w), np.zeros(w.shape[0], np.uint16)
+        assert_linear_close(bits_of(op.Y), O.linear_masked_dense(src, w, m, b, 0), O.row_scales(src, w, m, b), f"{w.shape}")
