@@ -340,6 +340,7 @@ __global__ void __launch_bounds__(128, 1) wait_selftest_kernel(int* status) {
 // adjacent columns of a row (one 16-byte store).  Latency-bound: block pointers, then values and list, then stores.
 // Looking the values up in global memory instead, eight dependent 2-byte loads per store, took 4.2 us for a
 // 3072 x 768 matrix of 16-row blocks.
+__device__ __forceinline__ long long grid_piece() { return static_cast<long long>(blockIdx.z) * gridDim.y + blockIdx.y; }   // see grid_of
 constexpr int kPlanSmem = 48 * 1024;
 __host__ __device__ inline int plan_rows_per_cta(int k_in) {
   const int r = kPlanSmem / (2 * k_in) - 1;     // rows of at most k_in values, and the table
@@ -351,7 +352,9 @@ plan_expand_kernel(const int32_t* blk_ptr, const int32_t* idx,
   extern __shared__ __align__(16) int16_t s_pos[];   // [k_in] column -> position in the kept list, or -1 (k_in < 32768)
   const int b = blockIdx.x;
   const int rows_per = plan_rows_per_cta(k_in);
-  const int r_lo = blockIdx.y * rows_per, n_rows = min(rows_per, block - r_lo);
+  const long long at = grid_piece() * rows_per;
+  if (at >= block) return;
+  const int r_lo = static_cast<int>(at), n_rows = min(rows_per, block - r_lo);
   uint16_t* s_val = reinterpret_cast<uint16_t*>(s_pos + k_in);   // [n_rows][kc]
   const int chunks = k_in >> 3;
   for (int k = threadIdx.x; k < chunks; k += 256) reinterpret_cast<uint4*>(s_pos)[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
@@ -407,7 +410,9 @@ __global__ void __launch_bounds__(256)
 plan_expand_r_kernel(const int32_t* blk_ptr, const int32_t* row_idx,
                      const uint16_t* vals, int n_out, int k_in, int h, uint16_t* Wx) {
   __shared__ int s_pos[kPlanRRows];
-  const int a = blockIdx.x, r0 = blockIdx.y * kPlanRRows;
+  const long long at = grid_piece() * kPlanRRows;
+  if (at >= n_out) return;
+  const int a = blockIdx.x, r0 = static_cast<int>(at);
   const int n_rows = min(kPlanRRows, n_out - r0);
   s_pos[threadIdx.x] = -1;
   pdl_wait();
@@ -464,7 +469,9 @@ plan_expand_t_kernel(const int32_t* blk_ptr, const int32_t* idx,
   __shared__ int32_t s_col_pos[kPlanTMaxBlocks][kPlanTK];
   __shared__ uint16_t s_t[kPlanTK][kPlanTN + 2];
   __shared__ int32_t s_ptr[kPlanTMaxBlocks + 1];
-  const int k0 = blockIdx.y * kPlanTK, nk = min(kPlanTK, G.k_in - k0);
+  const long long piece = grid_piece(), pieces = static_cast<long long>(gridDim.y) * gridDim.z;
+  if (piece * kPlanTK >= G.k_in) return;
+  const int k0 = static_cast<int>(piece) * kPlanTK, nk = min(kPlanTK, G.k_in - k0);
   const int b0 = static_cast<int>(blockIdx.x) / G.segments * G.blocks_per_unit;
   const int seg = static_cast<int>(blockIdx.x) % G.segments;
   const int nb = min(G.blocks_per_unit, G.n_out / G.block - b0);
@@ -482,8 +489,8 @@ plan_expand_t_kernel(const int32_t* blk_ptr, const int32_t* idx,
     // the unit's values are one run too: its CTAs fetch a share of it each into L2 while the lists are read
     const int lo = s_ptr[0], kept = s_ptr[nb] - lo;
     const char* run = reinterpret_cast<const char*>(vals + static_cast<size_t>(G.block) * lo + static_cast<size_t>(seg) * kPlanTN * kept);
-    const long long bytes = 2LL * rows_per_block * kept, step = 128LL * kPlanTThreads * gridDim.y;
-    for (long long at = 128LL * threadIdx.x * gridDim.y + 128LL * blockIdx.y; at < bytes; at += step) prefetch_line(run + at);
+    const long long bytes = 2LL * rows_per_block * kept, step = 128LL * kPlanTThreads * pieces;
+    for (long long at = 128LL * (threadIdx.x * pieces + piece); at < bytes; at += step) prefetch_line(run + at);
   }
   // A warp lists a row-block's columns of the tile.  A longer list is narrowed down by 32 samples first: one trip to
   // memory more, but every CTA reading its blocks' whole lists took as many instructions as moving the values (a backward
@@ -556,6 +563,11 @@ plan_expand_t_kernel(const int32_t* blk_ptr, const int32_t* idx,
 // ------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------
+// A grid of x by `pieces`, the pieces spread over y and z where y alone (65535) does not hold them.
+dim3 grid_of(int x, long long pieces) {
+  const long long z = (pieces + 65534) / 65535;
+  return dim3(x, static_cast<unsigned>((pieces + z - 1) / z), static_cast<unsigned>(z));
+}
 }  // namespace
 // Tile width, or the CTA-pair kernel, for a product of whole tiles: the least estimated time.  A launch costs a fixed
 // part (start-up, first operands, the last tile's epilogue), per wave of tiles the larger of its main loop and its
@@ -677,8 +689,7 @@ extern "C" int bsp_linear_plan(const int32_t* blk_ptr, const int32_t* idx, const
   if (k_in > 12288) return BSP_ERR_UNSUPPORTED;
   if (k_in % 8) return BSP_ERR_UNSUPPORTED;
   const int rows_per = plan_rows_per_cta(k_in);
-  const dim3 grid(n_out / block, (block + rows_per - 1) / rows_per);
-  if (grid.y > 65535) return BSP_ERR_UNSUPPORTED;
+  const dim3 grid = grid_of(n_out / block, (static_cast<long long>(block) + rows_per - 1) / rows_per);
   BSP_CUDA_TRY(launch_pdl(plan_expand_kernel, grid, dim3(256), static_cast<size_t>(k_in) * 2 * (1 + rows_per),
                           static_cast<cudaStream_t>(stream), blk_ptr, idx, static_cast<const uint16_t*>(vals), k_in, block,
                           static_cast<uint16_t*>(plan)));
@@ -694,11 +705,10 @@ extern "C" int bsp_linear_plan_r(const int32_t* blk_ptr, const int32_t* row_idx,
   if (!aligned_to(plan, 256)) return BSP_ERR_ARG;
   const size_t need = round_up(static_cast<size_t>(n_out) * k_in * 2, 256);
   if (plan_bytes < need) return BSP_ERR_WORKSPACE;
-  if ((n_out + kPlanRRows - 1) / kPlanRRows > 65535) return BSP_ERR_UNSUPPORTED;
   // widest vector: every segment starts at a multiple of `block` in rows of k_in elements (a multiple of it too)
   const int vec = block % 8 == 0 && aligned_to(vals, 16) ? 8 : block % 4 == 0 && aligned_to(vals, 8) ? 4 : 1;
   BSP_CUDA_TRY(launch_pdl(vec == 8 ? plan_expand_r_kernel<8> : vec == 4 ? plan_expand_r_kernel<4> : plan_expand_r_kernel<1>,
-                          dim3(k_in / block, (n_out + kPlanRRows - 1) / kPlanRRows), dim3(256), 0,
+                          grid_of(k_in / block, (static_cast<long long>(n_out) + kPlanRRows - 1) / kPlanRRows), dim3(256), 0,
                           static_cast<cudaStream_t>(stream), blk_ptr, row_idx, static_cast<const uint16_t*>(vals), n_out, k_in,
                           block, static_cast<uint16_t*>(plan)));
   return BSP_OK;
@@ -724,8 +734,7 @@ extern "C" int bsp_linear_plan_t(const int32_t* blk_ptr, const int32_t* idx, con
   }
   const int nb = n_out / block;
   const int units = (nb + G.blocks_per_unit - 1) / G.blocks_per_unit * G.segments;
-  const dim3 grid(units, (k_in + kPlanTK - 1) / kPlanTK);
-  if (grid.y > 65535) return BSP_ERR_UNSUPPORTED;
+  const dim3 grid = grid_of(units, (static_cast<long long>(k_in) + kPlanTK - 1) / kPlanTK);
   BSP_CUDA_TRY(launch_pdl(plan_expand_t_kernel, grid, dim3(kPlanTThreads), 0, static_cast<cudaStream_t>(stream), blk_ptr, idx,
                           static_cast<const uint16_t*>(vals), G, static_cast<uint16_t*>(plan_t)));
   return BSP_OK;
