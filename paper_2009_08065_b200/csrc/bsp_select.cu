@@ -565,10 +565,83 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
   cluster_sync();
 }
 
+// ------------------------------------------------------------ select where counts do not fit 32 bits (select_large)
+// A launch counts one digit over all keys (in shared memory per CTA, whose keys do fit 32 bits), a launch of one CTA
+// picks the digit that holds the answer.  Bound by the passes over the sums.
+struct LargeState {                                          // in the part of the workspace that holds flags elsewhere
+  unsigned long long want, hist[kBins1];
+  uint32_t prefix;
+};
+__global__ void __launch_bounds__(kSelThreads)
+large_start_kernel(LargeState* state, long long r) {
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int i = threadIdx.x; i < kBins1; i += kSelThreads) state->hist[i] = 0ull;
+  if (threadIdx.x == 0) {
+    state->want = static_cast<unsigned long long>(r);
+    state->prefix = 0u;
+  }
+}
+__global__ void __launch_bounds__(256)
+large_count_kernel(const uint32_t* keys, long long n, int above, int bits, LargeState* state) {
+  __shared__ __align__(16) uint32_t hist[kBins1];
+  clear_bins(hist);
+  pdl_wait();
+  pdl_launch_dependents();
+  __syncthreads();
+  const uint32_t prefix = state->prefix, mask = (1u << bits) - 1u;
+  const int shift = above - bits;
+  const long long n4 = n >> 2, step = static_cast<long long>(gridDim.x) * 256;
+  auto count = [&](uint32_t k) {
+    if ((k >> above) == prefix) atomicAdd(&hist[(k >> shift) & mask], 1u);
+  };
+  for (long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x; i < n4; i += step) {
+    const uint4 v = ld_global(reinterpret_cast<const uint4*>(keys) + i);
+    count(v.x); count(v.y); count(v.z); count(v.w);
+  }
+  if (blockIdx.x == 0 && threadIdx.x < static_cast<unsigned>(n & 3)) count(ld_global(keys + (n4 << 2) + threadIdx.x));
+  __syncthreads();
+  for (int i = threadIdx.x; i < kBins1; i += 256)
+    if (hist[i] != 0u) atomicAdd(&state->hist[i], static_cast<unsigned long long>(hist[i]));
+}
+__global__ void __launch_bounds__(kSelThreads)
+large_pick_kernel(LargeState* state, int bits, long long r, float* out) {
+  __shared__ unsigned long long hist[kBins1];
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int i = threadIdx.x; i < kBins1; i += kSelThreads) {
+    hist[i] = state->hist[i];
+    state->hist[i] = 0ull;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  unsigned long long want = state->want;
+  uint32_t bin = 0u;
+  if (r > 0)
+    for (; want > hist[bin]; ++bin) want -= hist[bin];
+  state->want = want;
+  state->prefix = (state->prefix << bits) | bin;
+  if (out != nullptr) *out = r > 0 ? threshold_of(state->prefix) : -1.0f;
+}
+int launch_select_large(const SelectJob& J, void* state_bytes, int sms, cudaStream_t s) {
+  LargeState* state = static_cast<LargeState*>(state_bytes);
+  BSP_CUDA_TRY(launch_pdl(large_start_kernel, dim3(1), dim3(kSelThreads), 0, s, state, J.r));
+  int above = kBits1 + kBits2 + kBits3;
+  for (const int bits : {kBits1, kBits2, kBits3}) {
+    BSP_CUDA_TRY(launch_pdl(large_count_kernel, dim3(4 * sms), dim3(256), 0, s, reinterpret_cast<const uint32_t*>(J.S), J.n, above, bits, state));
+    above -= bits;
+    BSP_CUDA_TRY(launch_pdl(large_pick_kernel, dim3(1), dim3(kSelThreads), 0, s, state, bits, J.r, above == 0 ? J.out : nullptr));
+  }
+  return BSP_OK;
+}
+
 // r = floor(G * (1 - 1/c)) in float64, as the definition states it
 long long groups_to_remove(long long groups, double rate) {
   return static_cast<long long>(static_cast<double>(groups) * (1.0 - 1.0 / rate));
 }
+
+// The histograms and lists of the select count in 32 bits.
+bool select_large(long long groups) { return groups >= (1LL << 32); }
 
 // A matrix's entry of the table; n_blocks x n_groups is its geometry in either orientation.
 SelectJob select_job(const void* W, int cols, int ldw, int n_blocks, int n_groups, double rate, void* ws, float* out) {
@@ -588,12 +661,9 @@ SelectJob select_job(const void* W, int cols, int ldw, int n_blocks, int n_group
   // the region of the flags: one byte per group
   const size_t fit = (L.sumsq_off - L.keep_off) / (kBins1 * sizeof(uint32_t));
   J.replicas = fit < kReplicas ? static_cast<int>(fit) : kReplicas;
-  if (fit > 0) J.head = reinterpret_cast<uint32_t*>(base + L.keep_off);
+  if (fit > 0 && !select_large(groups)) J.head = reinterpret_cast<uint32_t*>(base + L.keep_off);
   return J;
 }
-
-// The select counts in 32 bits.
-bool too_many_groups(long long groups) { return groups >= (1LL << 32); }
 
 // CTAs per matrix: as many as fit the GPU at once (one per SM: 1024 threads of 48 registers), up to the portable
 // cluster size, but not so many that a CTA has fewer than 2048 keys.
@@ -702,7 +772,6 @@ extern "C" int bsp_percentile_threshold(const void* W, int rows, int cols, int l
   const WsLayout L = ws_layout(nb, ng);
   if (ws_bytes < L.total) return BSP_ERR_WORKSPACE;
   const long long groups = static_cast<long long>(nb) * ng;
-  if (too_many_groups(groups)) return BSP_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int sms;
   st = sm_count(&sms);
@@ -723,6 +792,7 @@ extern "C" int bsp_percentile_threshold(const void* W, int rows, int cols, int l
                             ldw, block, contig_vec(W, ldw, block), B.job[0].S, B.job[0].head,
                             B.job[0].replicas));
   }
+  if (select_large(groups)) return launch_select_large(B.job[0], static_cast<char*>(ws) + L.keep_off, sms, s);
   return launch_select(B, sms, s);
 }
 
@@ -731,6 +801,7 @@ extern "C" int bsp_percentile_threshold_batched(const bsp_layer_job* jobs, int n
   using namespace bsp;
   if (jobs == nullptr || rates == nullptr || n_jobs <= 0 || block <= 0) return BSP_ERR_ARG;
   if (n_jobs > 4096) return BSP_ERR_UNSUPPORTED;
+  bool large = false;
   for (int i = 0; i < n_jobs; ++i) {                       // everything is checked before the first launch
     const bsp_layer_job& u = jobs[i];
     int st = check_matrix_args(u.W, u.rows, u.cols, u.ldw, block, BSP_ORIENT_C);
@@ -738,7 +809,15 @@ extern "C" int bsp_percentile_threshold_batched(const bsp_layer_job* jobs, int n
     if (u.threshold_dev == nullptr || u.ws == nullptr || !aligned_to(u.ws, 256)) return BSP_ERR_ARG;
     if (!(rates[i] >= 1.0)) return BSP_ERR_ARG;
     if (u.ws_bytes < ws_layout(u.rows / block, u.cols).total) return BSP_ERR_WORKSPACE;
-    if (too_many_groups(static_cast<long long>(u.rows / block) * u.cols)) return BSP_ERR_UNSUPPORTED;
+    large = large || select_large(static_cast<long long>(u.rows / block) * u.cols);
+  }
+  if (large) {                                             // (a workspace of 20 GB each: one after the other)
+    for (int i = 0; i < n_jobs; ++i) {
+      const bsp_layer_job& u = jobs[i];
+      BSP_TRY(bsp_percentile_threshold(u.W, u.rows, u.cols, u.ldw, block, BSP_ORIENT_C, rates[i], const_cast<float*>(u.threshold_dev),
+                                       u.ws, u.ws_bytes, stream));
+    }
+    return BSP_OK;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int sms;

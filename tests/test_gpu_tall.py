@@ -47,3 +47,24 @@ def test_layout_of_16777472_rows_in_strips():
     want = torch.zeros_like(w)
     want[::3] = w[::3]
     assert torch.equal(plan.view(torch.int16).view(rows, cols), want)
+
+
+def test_percentile_of_2_to_the_32_groups():
+    """Single weights as groups, more than 32-bit counts hold.  Row i repeats one value, the values grow with i, and
+    every 1024th row starts a new one: the r-th smallest square follows from r."""
+    n = 65536
+    values = 0x3C00 + np.arange(n // 1024)                    # bf16 bit patterns, ascending
+    rows = torch.from_numpy(np.repeat(values, 1024).astype(np.int16)).to(DEV)
+    w = torch.empty(n, n, dtype=torch.int16, device=DEV)
+    w.copy_(rows.view(n, 1).expand(n, n))
+    ws = torch.empty(bsp.bsp_pack_bound(n, n, 1, bsp.ORIENT_C)[2], dtype=torch.uint8, device=DEV)
+    t = torch.zeros(1, device=DEV)
+    for rate in (1.5, 16.0):
+        bsp.bsp_percentile_threshold(w, 1, bsp.ORIENT_C, rate, t, ws)
+        r = int(float(n) * n * (1.0 - 1.0 / rate))
+        v = np.uint32(int(values[(r - 1) // (1024 * n)]) << 16).view(np.float32)
+        s = np.float32(v * v)
+        want = np.sqrt(s)
+        while np.float32(want * want) < s:
+            want = np.nextafter(want, np.float32(np.inf))
+        assert np.float32(t.item()) == want, rate
