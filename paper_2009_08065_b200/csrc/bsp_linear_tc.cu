@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(128, 1) wait_selftest_kernel(int* status) {
 // adjacent columns of a row (one 16-byte store).  Latency-bound: block pointers, then values and list, then stores.
 // Looking the values up in global memory instead, eight dependent 2-byte loads per store, took 4.2 us for a
 // 3072 x 768 matrix of 16-row blocks.
-__device__ __forceinline__ long long grid_piece() { return static_cast<long long>(blockIdx.z) * gridDim.y + blockIdx.y; }   // see grid_of
+__device__ __forceinline__ unsigned grid_piece() { return blockIdx.z * gridDim.y + blockIdx.y; }   // see grid_of
 constexpr int kPlanSmem = 48 * 1024;
 __host__ __device__ inline int plan_rows_per_cta(int k_in) {
   const int r = kPlanSmem / (2 * k_in) - 1;     // rows of at most k_in values, and the table
@@ -352,8 +352,8 @@ plan_expand_kernel(const int32_t* blk_ptr, const int32_t* idx,
   extern __shared__ __align__(16) int16_t s_pos[];   // [k_in] column -> position in the kept list, or -1 (k_in < 32768)
   const int b = blockIdx.x;
   const int rows_per = plan_rows_per_cta(k_in);
-  const long long at = grid_piece() * rows_per;
-  if (at >= block) return;
+  const unsigned at = grid_piece() * static_cast<unsigned>(rows_per);
+  if (at >= static_cast<unsigned>(block)) return;
   const int r_lo = static_cast<int>(at), n_rows = min(rows_per, block - r_lo);
   uint16_t* s_val = reinterpret_cast<uint16_t*>(s_pos + k_in);   // [n_rows][kc]
   const int chunks = k_in >> 3;
@@ -410,8 +410,8 @@ __global__ void __launch_bounds__(256)
 plan_expand_r_kernel(const int32_t* blk_ptr, const int32_t* row_idx,
                      const uint16_t* vals, int n_out, int k_in, int h, uint16_t* Wx) {
   __shared__ int s_pos[kPlanRRows];
-  const long long at = grid_piece() * kPlanRRows;
-  if (at >= n_out) return;
+  const unsigned at = grid_piece() * kPlanRRows;
+  if (at >= static_cast<unsigned>(n_out)) return;
   const int a = blockIdx.x, r0 = static_cast<int>(at);
   const int n_rows = min(kPlanRRows, n_out - r0);
   s_pos[threadIdx.x] = -1;
@@ -445,6 +445,20 @@ plan_expand_r_kernel(const int32_t* blk_ptr, const int32_t* row_idx,
   }
 }
 
+// The same for strips of a few columns, by scattering the kept segments over a cleared plan: a CTA of the kernel above has
+// 256 short segments there and little else, and there are as many CTAs as strips.
+__global__ void __launch_bounds__(256)
+plan_scatter_r_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restrict__ row_idx,
+                      const uint16_t* __restrict__ vals, int k_in, int h, uint16_t* __restrict__ Wx) {
+  const int a = blockIdx.x;                       // strip
+  const int lo = blk_ptr[a], kc = blk_ptr[a + 1] - lo;
+  const uint16_t* tile = vals + static_cast<size_t>(h) * lo;
+  for (int e = threadIdx.x; e < kc * h; e += 256) {
+    const int p = e / h, c = e - p * h;
+    Wx[static_cast<size_t>(row_idx[lo + p]) * k_in + static_cast<size_t>(a) * h + c] = tile[e];
+  }
+}
+
 // Transposed plan from the orientation-C packed form: PT[k, n] = (W * Mask)[n, k], for the product
 // dX = dY (W * Mask).  A CTA makes the piece of 64 plan rows (columns k of W) x up to 64 plan columns (rows
 // n of W: as many whole row-blocks as fit, or 64 rows of a taller one).  Per row-block a table column -> kept
@@ -469,8 +483,8 @@ plan_expand_t_kernel(const int32_t* blk_ptr, const int32_t* idx,
   __shared__ int32_t s_col_pos[kPlanTMaxBlocks][kPlanTK];
   __shared__ uint16_t s_t[kPlanTK][kPlanTN + 2];
   __shared__ int32_t s_ptr[kPlanTMaxBlocks + 1];
-  const long long piece = grid_piece(), pieces = static_cast<long long>(gridDim.y) * gridDim.z;
-  if (piece * kPlanTK >= G.k_in) return;
+  const unsigned piece = grid_piece(), pieces = gridDim.y * gridDim.z;
+  if (piece * kPlanTK >= static_cast<unsigned>(G.k_in)) return;
   const int k0 = static_cast<int>(piece) * kPlanTK, nk = min(kPlanTK, G.k_in - k0);
   const int b0 = static_cast<int>(blockIdx.x) / G.segments * G.blocks_per_unit;
   const int seg = static_cast<int>(blockIdx.x) % G.segments;
@@ -490,7 +504,7 @@ plan_expand_t_kernel(const int32_t* blk_ptr, const int32_t* idx,
     const int lo = s_ptr[0], kept = s_ptr[nb] - lo;
     const char* run = reinterpret_cast<const char*>(vals + static_cast<size_t>(G.block) * lo + static_cast<size_t>(seg) * kPlanTN * kept);
     const long long bytes = 2LL * rows_per_block * kept, step = 128LL * kPlanTThreads * pieces;
-    for (long long at = 128LL * (threadIdx.x * pieces + piece); at < bytes; at += step) prefetch_line(run + at);
+    for (long long at = 128LL * (static_cast<long long>(threadIdx.x) * pieces + piece); at < bytes; at += step) prefetch_line(run + at);
   }
   // A warp lists a row-block's columns of the tile.  A longer list is narrowed down by 32 samples first: one trip to
   // memory more, but every CTA reading its blocks' whole lists took as many instructions as moving the values (a backward
@@ -705,11 +719,24 @@ extern "C" int bsp_linear_plan_r(const int32_t* blk_ptr, const int32_t* row_idx,
   if (!aligned_to(plan, 256)) return BSP_ERR_ARG;
   const size_t need = round_up(static_cast<size_t>(n_out) * k_in * 2, 256);
   if (plan_bytes < need) return BSP_ERR_WORKSPACE;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const dim3 grid = grid_of(k_in / block, (static_cast<long long>(n_out) + kPlanRRows - 1) / kPlanRRows);
+  TcDevice* dev = tc_device();
+  if (dev == nullptr) return BSP_ERR_CUDA;
+  // Strips narrower than 8 columns in more CTAs than the GPU holds at once (eight per SM) are scattered, a clearing pass
+  // more: 1216 x 6264 in single columns 15 us against 75, 1168 x 2152 in fours 5.0 against 6.8.  Not below that (536 x 1964
+  // in fours 4.9 against 4.7) and not in eights (5328 x 1648 14.8 against 10.9).
+  if (block < 8 && static_cast<long long>(grid.x) * grid.y * grid.z > 8LL * dev->sms) {
+    BSP_CUDA_TRY(cudaMemsetAsync(plan, 0, static_cast<size_t>(n_out) * k_in * 2, s));
+    plan_scatter_r_kernel<<<k_in / block, 256, 0, s>>>(blk_ptr, row_idx, static_cast<const uint16_t*>(vals), k_in, block,
+                                                       static_cast<uint16_t*>(plan));
+    BSP_LAUNCH_CHECK();
+    return BSP_OK;
+  }
   // widest vector: every segment starts at a multiple of `block` in rows of k_in elements (a multiple of it too)
   const int vec = block % 8 == 0 && aligned_to(vals, 16) ? 8 : block % 4 == 0 && aligned_to(vals, 8) ? 4 : 1;
   BSP_CUDA_TRY(launch_pdl(vec == 8 ? plan_expand_r_kernel<8> : vec == 4 ? plan_expand_r_kernel<4> : plan_expand_r_kernel<1>,
-                          grid_of(k_in / block, (static_cast<long long>(n_out) + kPlanRRows - 1) / kPlanRRows), dim3(256), 0,
-                          static_cast<cudaStream_t>(stream), blk_ptr, row_idx, static_cast<const uint16_t*>(vals), n_out, k_in,
+                          grid, dim3(256), 0, s, blk_ptr, row_idx, static_cast<const uint16_t*>(vals), n_out, k_in,
                           block, static_cast<uint16_t*>(plan)));
   return BSP_OK;
 }

@@ -73,6 +73,19 @@ def test_pack_and_layout_of_row_pruned_strips(rows, cols, block):
     assert np.array_equal(bits_of(plan.view(torch.int16)[: rows * cols]).reshape(rows, cols), O.prune(w, block, "R", t))
 
 
+# strips of 1 to 7 columns on both sides of the scattering rule (more than eight CTAs per SM), 8 columns beyond it
+@pytest.mark.parametrize("rows,cols,block", [(300, 1200, 1), (300, 580, 1), (1100, 1204, 4), (260, 4200, 7), (280, 9600, 8)])
+def test_layout_of_narrow_strips(rows, cols, block):
+    w = weights(f"n{rows}x{cols}", rows, cols)
+    keep = si.random_keep_sets(72, f"n{rows}x{cols}", cols // block, rows, rows // 3).T.copy()
+    keep[:, 1] = False                                        # an empty strip
+    blk_ptr, idx, vals = O.pack(w, keep, block, "R")
+    pk = upload_packed(blk_ptr, idx, vals, rows, cols, block, bsp.ORIENT_R)
+    plan = torch.full(((rows * cols * 2 + 255) // 256 * 256,), 0x33, dtype=torch.uint8, device=DEV)
+    bsp.bsp_linear_plan(pk, plan)
+    assert np.array_equal(bits_of(plan.view(torch.int16)[: rows * cols]).reshape(rows, cols), si.zero_groups(w, keep, block, "R"))
+
+
 # segments of 256 rows: a whole one, one row short, one row more, a single strip of many; 16400 strips are packed
 # without segments
 @pytest.mark.parametrize("rows,cols,block", [(256, 24, 12), (255, 16, 8), (257, 64, 64), (8192, 8, 8), (5, 16400, 1)])
