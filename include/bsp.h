@@ -269,11 +269,12 @@ typedef struct bsp_layer_job {
 } bsp_layer_job;
 int bsp_prepare_batched(const bsp_layer_job* jobs, int n_jobs, int block, float eps, int pen, void* stream);
 /* bsp_percentile_threshold_batched — bsp_percentile_threshold (Section 3.1's percentile) for the
- * matrices of a job array in two launches (orientation C): job i's threshold for the target rate
+ * matrices of a job array in three launches per 96 matrices (orientation C): job i's threshold for the target rate
  * rates[i] (HOST array of n_jobs doubles, each >= 1) is written to the device float that the job
  * names as threshold_dev, where a following bsp_prepare_batched on the same array reads it.
  * Uses each job's ws (as bsp_percentile_threshold does); only W, rows, cols, ldw, threshold_dev,
  * ws and ws_bytes of a job are read.  Results are those of the single-matrix call, bit for bit.
+ * Bounded waits report through bsp_linear_status (also in the single-matrix call, for large matrices).
  * Errors: BSP_ERR_ARG (NULL threshold_dev or ws, rate < 1), BSP_ERR_SHAPE, BSP_ERR_WORKSPACE. */
 int bsp_percentile_threshold_batched(const bsp_layer_job* jobs, int n_jobs, int block, const double* rates,
                                      void* stream);
@@ -335,18 +336,24 @@ int bsp_linear_planned(const void* plan, int n_out, int k_in, int block,
 /* bsp_linear_planned with the kernel variant chosen by the caller: BSP_LINEAR_AUTO (what
  * bsp_linear_planned does), BSP_LINEAR_ONE_CTA (128 x BN tiles, one CTA each) or
  * BSP_LINEAR_CTA_PAIR (256 x 256 tiles shared by a cluster of two CTAs, one third less operand
- * traffic from L2).  Results are identical up to float32 summation order (the same in both). */
+ * traffic from L2).  The two named variants sum in the same order and give the same bits.
+ * BSP_LINEAR_AUTO takes the fastest by estimate and has a third choice: where a layer has few output
+ * tiles (few tokens, or few outputs) a cluster of 2, 4 or 8 CTAs splits the contraction and adds the
+ * float32 partial sums in a fixed order.  Its results are reproducible and as accurate, but their last
+ * bits differ from the named variants', and as the choice depends on `tokens`, a row's last bits may
+ * differ between batch sizes; name a variant where they must not. */
 typedef enum { BSP_LINEAR_AUTO = 0, BSP_LINEAR_ONE_CTA = 1, BSP_LINEAR_CTA_PAIR = 2 } bsp_linear_algo;
-/* May be OR-ed into `algo`: the caller vouches that the plan was complete before the work that
- * immediately precedes this call in the stream was launched (the usual case in a chain of layers:
- * the weights are old, only X is fresh).  The one-CTA kernel then starts fetching weight tiles
- * while that work is still finishing.  Never set it when the preceding kernel writes the plan. */
+/* May be OR-ed into `algo`: the caller vouches that the plan is older than the work that immediately
+ * precedes this call in the stream (the usual case in a chain of layers: the weights are old, only X is
+ * fresh): whatever wrote the plan stands at least one kernel further ahead.  The one-CTA and the split
+ * kernel then start fetching weight tiles while that work is still finishing; the pair kernel ignores
+ * the flag.  Never set it when the preceding kernel writes the plan. */
 #define BSP_LINEAR_PLAN_STABLE 0x100
 /* May be OR-ed into `algo`: write the output TRANSPOSED, Y := YT [n_out, tokens] row-major with
  * leading dimension ldy >= tokens (a multiple of 8), bit for bit the transpose of what the call
  * writes otherwise.  It is the form bsp_linear_gathered reads its activations in, so a chain of
- * layers can hand them on without a separate transposing pass.  One-CTA kernel only
- * (BSP_LINEAR_CTA_PAIR with this flag is BSP_ERR_UNSUPPORTED). */
+ * layers can hand them on without a separate transposing pass.  Written by the one-CTA and the split
+ * kernel (BSP_LINEAR_CTA_PAIR with this flag is BSP_ERR_UNSUPPORTED). */
 #define BSP_LINEAR_OUT_TRANSPOSED 0x200
 int bsp_linear_planned_ex(const void* plan, int n_out, int k_in, int block,
                           const void* X, int tokens, int ldx, const void* bias, int act,
@@ -382,7 +389,8 @@ int bsp_wait_selftest(int* expired, long long* waited_ns, void* stream);
  * Row-tile m of an op needs only row-tile m of its source, so no grid-wide barrier separates the
  * layers: the CTAs take output tiles of all ops from one list through a ticket counter, and a tile
  * waits (bounded) until the source rows it reads have been stored; see csrc/bsp_linear_chain.cu.
- * Outputs are bit-identical to calling bsp_linear_planned op by op.
+ * Outputs are bit-identical to calling bsp_linear_planned op by op.  (Where that would split an op's
+ * contraction, few tokens, the chain is served by single launches, which are faster there.)
  *
  * ops: HOST array of n_ops (1..8) descriptors; plan / bias / Y are device pointers as in
  * bsp_linear_planned (plan from bsp_linear_plan or bsp_prepare_batched).  ws: device scratch of
