@@ -574,10 +574,32 @@ plan_expand_t_kernel(const int32_t* blk_ptr, const int32_t* idx,
   }
 }
 
+// The same by scattering the kept columns over a cleared plan, one CTA per row-block: consecutive threads take consecutive
+// rows of a kept column.
+__global__ void __launch_bounds__(256)
+plan_scatter_t_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __restrict__ idx,
+                      const uint16_t* __restrict__ vals, int n_out, int block, uint16_t* __restrict__ PT) {
+  const int b = blockIdx.x;
+  const int lo = blk_ptr[b], kc = blk_ptr[b + 1] - lo;
+  const uint16_t* tile = vals + static_cast<size_t>(block) * lo;
+  for (int e = threadIdx.x; e < kc * block; e += 256) {
+    const int j = e / block, r = e - j * block;
+    PT[static_cast<size_t>(idx[lo + j]) * n_out + static_cast<size_t>(b) * block + r] = tile[static_cast<size_t>(r) * kc + j];
+  }
+}
+
 // ------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------
 // A grid of x by `pieces`, the pieces spread over y and z where y alone (65535) does not hold them.
+// Which transposed layouts are scattered: rows whose number is no multiple of 8 would be stored one element at a time by
+// the one-pass kernel (1126 x 1320, 2-row blocks 8.7 us against 4.6; 4668 x 3288, 12-row 59 against 50; not tall blocks,
+// of which there are too few to scatter), and past a thousand row-blocks the scattering has its CTAs
+// (7048 x 2160, 4-row 36 against 15).  Otherwise the one pass wins between the products of a backward step (3072 x 768,
+// 16-row 5.4 against 7.3, 768 x 3072 5.4 against 33, 6360 x 432, 8-row 7.6 against 8.5).
+bool transposed_by_scatter(int n_out, int block) {
+  return (n_out % 8 != 0 && block < 16) || n_out / block > 1024;
+}
 dim3 grid_of(int x, long long pieces) {
   const long long z = (pieces + 65534) / 65535;
   return dim3(x, static_cast<unsigned>((pieces + z - 1) / z), static_cast<unsigned>(z));
@@ -750,6 +772,14 @@ extern "C" int bsp_linear_plan_t(const int32_t* blk_ptr, const int32_t* idx, con
   if (st != BSP_OK) return st;
   if (!aligned_to(plan_t, 256)) return BSP_ERR_ARG;
   if (plan_bytes < need) return BSP_ERR_WORKSPACE;
+  if (transposed_by_scatter(n_out, block)) {
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    BSP_CUDA_TRY(cudaMemsetAsync(plan_t, 0, static_cast<size_t>(n_out) * k_in * 2, s));
+    plan_scatter_t_kernel<<<n_out / block, 256, 0, s>>>(blk_ptr, idx, static_cast<const uint16_t*>(vals), n_out, block,
+                                                        static_cast<uint16_t*>(plan_t));
+    BSP_LAUNCH_CHECK();
+    return BSP_OK;
+  }
   PlanTGeometry G{n_out, k_in, block, 1, 1};
   if (block > kPlanTN) {
     G.segments = (block + kPlanTN - 1) / kPlanTN;

@@ -39,6 +39,30 @@ def test_percentile_select(rows, cols, block, orient, ties):
         assert np.float32(t.item()) == np.float32(O.percentile_threshold(w, block, "CR"[orient], rate)), rate
 
 
+def test_percentile_of_a_streamed_batch():
+    """More items than the streaming sums need (six per SM) and more matrices than one launch takes: matrices with a
+    histogram (16384 groups and more) among ones without, so that a CTA crosses from either kind to either; one cut into
+    three column ranges of which the last is shorter; ties; rates of their own.  Bit for bit the single call's threshold."""
+    block = 16
+    shapes = []
+    for i in range(104):
+        shapes.append((1024, 264) if i % 3 == 0 else (160 + 16 * (i % 5), 8 * (1 + i % 31)))
+    shapes[7], shapes[8], shapes[100] = (480, 2000), (1024, 776), (496, 2000)
+    jobs, refs, rates = [], [], []
+    for i, (rows, cols) in enumerate(shapes):
+        w = weights(f"stream{i}", rows, cols, ties=i % 13 == 5)
+        pk = bsp.PackedMatrix.allocate(rows, cols, block, bsp.ORIENT_C)
+        pk.ws.fill_(0x5A)
+        rates.append(1.0 + 0.37 * (i % 17))
+        jobs.append(bsp.LayerJob(to_dev(w), pk, 0.0, torch.zeros(1, dtype=torch.float32, device=DEV)))
+        refs.append(np.float32(O.percentile_threshold(w, block, "C", rates[-1])))
+    items = sum(r // block * -(-c // 768) for r, c in shapes[:96])
+    assert items >= 6 * torch.cuda.get_device_properties(0).multi_processor_count
+    bsp.bsp_percentile_threshold_batched(jobs, block, rates)
+    bsp.bsp_linear_status()
+    assert [np.float32(j.threshold_dev.item()) for j in jobs] == refs
+
+
 @pytest.mark.parametrize("rows,cols,block,orient,ties", [
     (16, 8192, 8, 0, False), (16, 8192, 8, 0, True), (24, 264, 12, 0, True), (10, 77, 5, 0, True),
     (2100, 24, 12, 1, True), (257, 16, 8, 1, False)])
@@ -125,6 +149,19 @@ def test_column_pruned_layouts_mask_and_repack(rows, cols, block):
     bsp.bsp_repack_values(to_dev(w2), pk)
     n = int(blk_ptr[-1]) * block
     assert np.array_equal(bits_of(pk.vals)[:n], O.repack_values(w2, blk_ptr, idx, block))
+
+
+# rows that are no multiple of 8 and more than 1024 row-blocks are scattered; blocks of 16 rows, and 1024 row-blocks, not
+@pytest.mark.parametrize("rows,cols,block", [(1025, 72, 1), (2056, 40, 2), (1024, 72, 1), (60, 136, 12), (102, 264, 3), (100, 72, 20)])
+def test_transposed_layout_on_both_sides_of_the_scattering_rule(rows, cols, block):
+    w = weights(f"t{rows}x{cols}", rows, cols)
+    keep = si.random_keep_sets(73, f"t{rows}x{cols}", rows // block, cols, cols // 3)
+    keep[1, :] = False
+    pk = upload_packed(*O.pack(w, keep, block, "C"), rows, cols, block)
+    plan_t = torch.full((bsp.bsp_linear_plan_bytes(rows, cols, block),), 0x33, dtype=torch.uint8, device=DEV)
+    bsp.bsp_linear_plan_t(pk, plan_t)
+    want = si.zero_groups(w, keep, block, "C").T
+    assert np.array_equal(bits_of(plan_t.view(torch.int16)[: rows * cols]).reshape(cols, rows), np.ascontiguousarray(want))
 
 
 def test_repack_of_a_wide_matrix():
