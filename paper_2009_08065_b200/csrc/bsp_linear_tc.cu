@@ -344,7 +344,8 @@ __device__ __forceinline__ unsigned grid_piece() { return blockIdx.z * gridDim.y
 constexpr int kPlanSmem = 48 * 1024;
 __host__ __device__ inline int plan_rows_per_cta(int k_in) {
   const int r = kPlanSmem / (2 * k_in) - 1;     // rows of at most k_in values, and the table
-  return r > 4 ? 4 : r < 1 ? 1 : r;
+  const int want = k_in >= 512 ? 4 : 2048 / k_in;   // four rows, or a piece of 8 columns for every thread
+  return r > want ? want : r < 1 ? 1 : r;
 }
 __global__ void __launch_bounds__(256)
 plan_expand_kernel(const int32_t* blk_ptr, const int32_t* idx,
