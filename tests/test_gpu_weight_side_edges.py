@@ -65,7 +65,8 @@ def test_percentile_of_a_streamed_batch():
 
 @pytest.mark.parametrize("rows,cols,block,orient,ties", [
     (16, 8192, 8, 0, False), (16, 8192, 8, 0, True), (24, 264, 12, 0, True), (10, 77, 5, 0, True),
-    (2100, 24, 12, 1, True), (257, 16, 8, 1, False)])
+    (2100, 24, 12, 1, True), (257, 16, 8, 1, False),
+    (16, 192, 8, 0, True), (16, 200, 8, 0, False), (191, 24, 12, 1, True), (193, 16, 8, 1, False), (3, 24, 12, 1, True)])
 def test_keep_count_select(rows, cols, block, orient, ties):
     w = weights(f"topk{rows}x{cols}", rows, cols, ties)
     o = "CR"[orient]
