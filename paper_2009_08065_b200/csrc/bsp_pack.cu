@@ -21,7 +21,10 @@ constexpr int kPackThreads = 256;
 constexpr int kRankGroups = 192;
 static_assert(kRankGroups <= 256, "a block of few groups is one segment");
 constexpr int kSegment = 256;          // groups of a strip that one CTA packs (orientation R)
-constexpr int kMaxSegments = 16384;    // segments of a matrix: every CTA adds up the counts before its own
+// Segments of a matrix: every CTA adds up the counts before its own.  4000 of them (1000 x 1000 in single columns) 26 us, 30
+// without; 8192 equal; 13870 (280 x 6935) 67, 51 without.
+constexpr int kMaxSegments = 4096;
+constexpr int kTallBlocks = 296;       // blocks up to which a CTA of 1024 threads per block fits the GPU at once (two per SM)
 
 struct Geometry {
   int rows, cols, ldw, block, orient, n_blocks, n_groups;
@@ -69,7 +72,8 @@ __device__ __forceinline__ void copy_strided(T* dst, size_t dst_stride, const T*
 }
 
 // (1a) threshold mode, one CTA per block.
-__global__ void __launch_bounds__(1024)
+template <int T>
+__global__ void __launch_bounds__(T)
 flags_threshold_kernel(const uint16_t* W, Geometry G, float threshold,
                        const float* threshold_dev, uint8_t* keep,
                        int32_t* counts) {
@@ -240,7 +244,10 @@ cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, ui
   };
   if (G.n_groups < 512) return launch(flags_topk_kernel<kPackThreads>, kPackThreads);
   if (G.orient == BSP_ORIENT_C) return launch(flags_topk_kernel<512>, 512);
-  return G.n_blocks <= 296 ? launch(flags_topk_kernel<1024>, 1024) : launch(flags_topk_kernel<kPackThreads>, kPackThreads);
+  // 1024 threads where all strips run at once, and where a strip has so many groups that its passes count more than the
+  // waves (512 strips of 8192 groups 136 us, 215 with 256 threads; 600 of 768 groups 25 against 22)
+  return G.n_blocks <= kTallBlocks || G.n_groups >= 4096 ? launch(flags_topk_kernel<1024>, 1024)
+                                                         : launch(flags_topk_kernel<kPackThreads>, kPackThreads);
 }
 
 // (2) counts -> blk_ptr (exclusive scan) and the kept-weight total: matrices with more blocks than the
@@ -270,7 +277,8 @@ scan_counts_kernel(const int32_t* counts, int n_blocks, int block,
 // CTA adds up the counts before its block itself and writes blk_ptr (one launch less; 4 bytes per block and
 // CTA from L2), without it blk_ptr is there already.  Orientation R: a thread moves its whole group, by
 // vectors of G.vec elements; the kept groups of a warp are neighbours in the tile.
-__global__ void __launch_bounds__(1024)
+template <int T>
+__global__ void __launch_bounds__(T)
 compact_kernel(const uint16_t* W, Geometry G, const uint8_t* keep, const int32_t* counts,
                int32_t* blk_ptr, int32_t* idx, uint16_t* vals,
                int64_t* kept_weights) {
@@ -524,19 +532,23 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
                             dim3(kSegment), 0, s, w, G, flags, seg_counts, blk_ptr, idx, static_cast<uint16_t*>(vals), kept_weights));
     return BSP_OK;
   }
-  // a CTA per block, threads for its groups: up to 1024 of them, since a matrix of few tall blocks has few CTAs
-  const int threads = G.n_groups >= 1024 ? 1024 : G.n_groups <= 128 ? 128 : (G.n_groups + 31) / 32 * 32;
+  // A CTA per block, threads for its groups: up to 1024 of them, since a matrix of few wide blocks has few CTAs (768 x 5120
+  // in 16-row blocks 27 us, 83 with 256 threads).  Many row-blocks fill the GPU by themselves and want CTAs that come and
+  // go (5343 x 920 in single rows 47 us, 67 with 1024; 2204 x 1214 in fours 12.7 against 15).
+  const bool tall = orient == BSP_ORIENT_R || G.n_blocks <= kTallBlocks;
+  const int threads = !tall ? 256 : G.n_groups >= 1024 ? 1024 : G.n_groups <= 128 ? 128 : (G.n_groups + 31) / 32 * 32;
   if (keep_per_block >= 0) {
     BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, nullptr, s));
   } else {
-    BSP_CUDA_TRY(launch_pdl(flags_threshold_kernel, dim3(G.n_blocks), dim3(threads), 0, s, w, G, threshold, threshold_dev, flags, counts));
+    BSP_CUDA_TRY(launch_pdl(tall ? flags_threshold_kernel<1024> : flags_threshold_kernel<256>, dim3(G.n_blocks), dim3(threads), 0, s, w, G,
+                            threshold, threshold_dev, flags, counts));
   }
   // every CTA of the compaction adds up the counts before its block; past 4096 blocks that costs more than a
   // scan of its own (it grows with the square of the block count)
   const bool own_scan = G.n_blocks > 4096;
   if (own_scan) BSP_CUDA_TRY(launch_pdl(scan_counts_kernel, dim3(1), dim3(1024), 0, s, counts, G.n_blocks, block, blk_ptr, kept_weights));
-  BSP_CUDA_TRY(launch_pdl(compact_kernel, dim3(G.n_blocks), dim3(threads), 0, s, w, G, flags, own_scan ? nullptr : counts, blk_ptr, idx,
-                          static_cast<uint16_t*>(vals), kept_weights));
+  BSP_CUDA_TRY(launch_pdl(tall ? compact_kernel<1024> : compact_kernel<256>, dim3(G.n_blocks), dim3(threads), 0, s, w, G, flags,
+                          own_scan ? nullptr : counts, blk_ptr, idx, static_cast<uint16_t*>(vals), kept_weights));
   return BSP_OK;
 }
 

@@ -111,6 +111,24 @@ def test_layout_of_narrow_strips(rows, cols, block):
     assert np.array_equal(bits_of(plan.view(torch.int16)[: rows * cols]).reshape(rows, cols), si.zero_groups(w, keep, block, "R"))
 
 
+# row-blocks on both sides of the rule for 1024 threads each (296), of columns that are no multiple of 8, by threshold and by
+# keep count; segments on both sides of the 4096 up to which strips are packed by them; strips of 4096 groups and fewer
+@pytest.mark.parametrize("rows,cols,block,orient", [(592, 1037, 2, 0), (594, 1037, 2, 0), (300, 2100, 1, 1), (300, 2048, 1, 1),
+                                                    (4096, 300, 1, 1), (4090, 300, 1, 1)])
+def test_pack_of_any_geometry(rows, cols, block, orient):
+    w, o = weights(f"any{rows}x{cols}", rows, cols), "CR"[orient]
+    t = float(np.median(O.group_norms(w, block, o)))
+    groups = cols if orient == 0 else rows
+    for keep_n in (-1, groups // 3):
+        pk = bsp.PackedMatrix.allocate(rows, cols, block, orient)
+        keep_ref = O.keep_flags(w, block, o, t) if keep_n < 0 else O.keep_topk_per_block(w, block, o, keep_n)
+        bsp.bsp_prune_pack(to_dev(w), pk, t if keep_n < 0 else 0.0, keep_per_block=keep_n)
+        ref = O.pack(w, keep_ref, block, o)
+        blk_ptr, idx, vals, keep, kept = packed_to_host(pk)
+        assert np.array_equal(keep, keep_ref) and kept == block * int(keep_ref.sum())
+        assert np.array_equal(blk_ptr, ref[0]) and np.array_equal(idx, ref[1]) and np.array_equal(vals, ref[2])
+
+
 # segments of 256 rows: a whole one, one row short, one row more, a single strip of many; 16400 strips are packed
 # without segments
 @pytest.mark.parametrize("rows,cols,block", [(256, 24, 12), (255, 16, 8), (257, 64, 64), (8192, 8, 8), (5, 16400, 1)])
