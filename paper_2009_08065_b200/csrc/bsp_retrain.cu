@@ -117,7 +117,7 @@ masked_adam_kernel(AdamArgs A) {
 // anyway), and gathers from there, two positions per 4-byte store.  HBM-bound in total, latency-bound per
 // matrix: four rows per CTA give a 768 x 768 matrix 192 CTAs, and the list travels beside the rows.  12 layers of four
 // matrices, on average: 5.3 us gathering from global memory, 2.9 us.
-constexpr int kRepackRows = 4, kRepackThreads = 256, kRepackLoads = 6;
+constexpr int kRepackRows = 4, kRepackThreads = 256, kRepackLoads = 6, kRepackMaxCols = 3072;
 __global__ void __launch_bounds__(kRepackThreads)
 repack_vec_kernel(const uint16_t* W, int cols, int ldw, int block, const int32_t* blk_ptr,
                   const int32_t* idx, uint16_t* vals) {
@@ -180,7 +180,7 @@ repack_vec_kernel(const uint16_t* W, int cols, int ldw, int block, const int32_t
   }
 }
 
-// Any alignment or width.
+// Any alignment or width, four positions of a row in flight per thread.
 __global__ void __launch_bounds__(256)
 repack_kernel(const uint16_t* W, int ldw, int block, const int32_t* blk_ptr,
               const int32_t* idx, uint16_t* vals) {
@@ -287,7 +287,10 @@ extern "C" int bsp_repack_values(const void* W, int rows, int cols, int ldw, int
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint16_t* w = static_cast<const uint16_t*>(W);
   const size_t smem = static_cast<size_t>(cols) * (kRepackRows + 1) * 2;
-  if (cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && smem <= 48 * 1024) {
+  // Staged rows, where several CTAs fit an SM and have more than one row each.  Behind the Adam step, staged / gathered from
+  // global memory: 4096 x 1024 in 16-row blocks 4.0 / 5.7 us, 768 x 3072 5.5 / 5.2, 8192 x 4096 49 / 26, 5344 x 920 in single
+  // rows 11.2 / 10.2.
+  if (cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && cols <= kRepackMaxCols && block > 1) {
     BSP_CUDA_TRY(launch_pdl(repack_vec_kernel, grid, dim3(kRepackThreads), smem, s, w, cols, ldw, block, blk_ptr, idx,
                             static_cast<uint16_t*>(vals)));
   } else {

@@ -183,12 +183,13 @@ def test_transposed_layout_on_both_sides_of_the_scattering_rule(rows, cols, bloc
     assert np.array_equal(bits_of(plan_t.view(torch.int16)[: rows * cols]).reshape(cols, rows), np.ascontiguousarray(want))
 
 
-def test_repack_of_a_wide_matrix():
-    """5120 columns do not fit the staging buffer of the vectorised kernel."""
-    w = weights("wide", 8, 5120)
-    keep = si.random_keep_sets(5, "wide", 2, 5120, 1001)
-    blk_ptr, idx, vals = O.pack(w, keep, 4, "C")
-    pk = upload_packed(blk_ptr, idx, np.zeros_like(vals), 8, 5120, 4)
+# 3072 columns are staged, more are gathered from global memory, and so are single rows
+@pytest.mark.parametrize("rows,cols,block,kept", [(8, 5120, 4, 1001), (8, 3072, 4, 1100), (8, 3080, 4, 1027), (6, 264, 1, 100), (6, 264, 2, 100)])
+def test_repack_of_a_wide_matrix(rows, cols, block, kept):
+    w = weights(f"wide{cols}", rows, cols)
+    keep = si.random_keep_sets(5, "wide", rows // block, cols, kept)
+    blk_ptr, idx, vals = O.pack(w, keep, block, "C")
+    pk = upload_packed(blk_ptr, idx, np.zeros_like(vals), rows, cols, block)
     bsp.bsp_repack_values(to_dev(w), pk)
     assert np.array_equal(bits_of(pk.vals)[: vals.size], vals)
 
