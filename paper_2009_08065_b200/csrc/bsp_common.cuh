@@ -227,6 +227,26 @@ __device__ __forceinline__ float group_sumsq_strided(const uint16_t* p, int n, s
   }
   return acc;
 }
+// The same with eight loads in flight, for kernels that do little else.
+__device__ __forceinline__ float group_sumsq_strided8(const uint16_t* p, int n, size_t stride) {
+  float acc = 0.0f;
+  int e = 0;
+  for (; e + 8 <= n; e += 8, p += 8 * stride) {
+    uint16_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = ld_global(p + u * stride);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const float w = bf16_bits_to_float(v[u]);
+      acc = __fmaf_rn(w, w, acc);
+    }
+  }
+  for (; e < n; ++e, p += stride) {
+    const float w = bf16_bits_to_float(ld_global(p));
+    acc = __fmaf_rn(w, w, acc);
+  }
+  return acc;
+}
 
 // The same for a group of contiguous elements (orientation R), by vectors of `vec` elements (contig_vec).
 __device__ __forceinline__ float group_sumsq_contig(const uint16_t* p, int n, int vec) {

@@ -52,7 +52,7 @@ __device__ __forceinline__ size_t group_slot(const Geometry& G, int b, int g) {
 __device__ __forceinline__ float group_sum(const uint16_t* W, const Geometry& G, int b, int g) {
   size_t stride;
   const uint16_t* p = group_ptr(W, G, b, g, &stride);
-  return G.orient == BSP_ORIENT_C ? group_sumsq_strided(p, G.block, stride) : group_sumsq_contig(p, G.block, G.vec);
+  return G.orient == BSP_ORIENT_C ? group_sumsq_strided8(p, G.block, stride) : group_sumsq_contig(p, G.block, G.vec);
 }
 
 // n elements from stride to stride, four loads in flight.

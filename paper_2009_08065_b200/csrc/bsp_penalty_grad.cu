@@ -176,7 +176,7 @@ grad_generic_kernel(GradArgs A) {
   if (A.squared) {
     factor = 2.0f * A.scale * A.gamma[g];
   } else {
-    const float n = __fsqrt_rn(group_sumsq_strided(A.W + first, A.block, stride));
+    const float n = __fsqrt_rn(group_sumsq_strided8(A.W + first, A.block, stride));
     factor = n > 0.0f ? __fdiv_rn(A.scale * A.gamma[g], n) : 0.0f;
   }
   // the same element position in grad: row = first / ldw, col = first % ldw
