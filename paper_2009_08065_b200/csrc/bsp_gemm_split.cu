@@ -458,7 +458,7 @@ bool query_split_ctas(int (&ctas)[3]) {
 // (768 outputs x 3072 inputs: 10.0 us whole, split 8 ways 3.8 us at 8 tokens and 4.6 us at 128; 768 x 768: 4.5 whole, 2.8
 // split 4 ways at 8 tokens; 1024 x 4096 at 1003 tokens: 13.4 whole, 10.6 as 128-wide tiles split 2; 304 x 304: 3.2 and
 // 2.6 at 8 tokens, not split at 1003.)
-int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn) {
+int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn, long long* ns) {
   const long long m_tiles = (tokens + kBlockM - 1) / kBlockM;
   const int kb = (k_in + kBlockK - 1) / kBlockK;
   const int quads = tokens >= kBlockM ? 4 : (tokens + 31) / 32;
@@ -476,6 +476,7 @@ int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, lo
       if (t < best) { best = t; choice = i; *bn = 64 * (b + 1); }
     }
   }
+  if (ns != nullptr) *ns = choice < 0 ? whole_ns : best;
   return choice;
 }
 // dW: tiles 128 / 192 / 256 wide, whole (persistent kernel: per wave) or, 128 and 256 wide, split 2 / 4 / 8.  Rows of dY

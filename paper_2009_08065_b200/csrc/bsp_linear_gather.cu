@@ -676,13 +676,10 @@ extern "C" int bsp_linear_gathered_ex(const void* gplan, int n_out, int k_in, in
   P.cols = reinterpret_cast<const int16_t*>(base + L.cols_off);
   P.tiles = reinterpret_cast<const uint16_t*>(base + L.tiles_off);
   P.n_blocks = n_out / block;
-  P.m_tiles = (tokens + kBlockM - 1) / kBlockM;
-  // runs of consecutive row-blocks: enough units for about six per SM, runs as long as that allows
-  int n_chunks = (6 * dev->sms + P.m_tiles - 1) / P.m_tiles;
-  if (n_chunks < 1) n_chunks = 1;
-  if (n_chunks > P.n_blocks) n_chunks = P.n_blocks;
-  P.rb_per_chunk = (P.n_blocks + n_chunks - 1) / n_chunks;
-  P.n_chunks = (P.n_blocks + P.rb_per_chunk - 1) / P.rb_per_chunk;
+  const GatherUnits units = gather_units(tokens, P.n_blocks, dev->sms);
+  P.m_tiles = units.m_tiles;
+  P.rb_per_chunk = units.rb_per_chunk;
+  P.n_chunks = units.n_chunks;
   P.status = dev->status;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   switch (block) {

@@ -488,10 +488,26 @@ struct DenseChoice {
   long long ns;
 };
 DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, int act, bool allow_pair);
-// Cluster size index for the same layer with its contraction split, or -1 where whole tiles (whole_ns) are as fast.
-int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn);
+// Cluster size index for the same layer with its contraction split, or -1 where whole tiles (whole_ns) are as fast; *ns
+// (may be null) receives the estimated time of what is faster.
+int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn, long long* ns = nullptr);
 int launch_linear_split(TcDevice* dev, int bn, int c, const void* plan, const void* X, void* Y, int tokens, int n_out, int k_in,
                         int act, const void* bias, int ldx, int ldy, bool plan_stable, bool transposed, cudaStream_t s);
+// How bsp_linear_gathered cuts a layer: runs of rb_per_chunk consecutive row-blocks x 128-token tiles, enough of them for
+// about six per SM, runs as long as that allows.
+struct GatherUnits {
+  int m_tiles, n_chunks, rb_per_chunk;
+};
+inline GatherUnits gather_units(int tokens, int n_blocks, int sms) {
+  GatherUnits u;
+  u.m_tiles = (tokens + tc::kBlockM - 1) / tc::kBlockM;
+  int n_chunks = (6 * sms + u.m_tiles - 1) / u.m_tiles;
+  if (n_chunks < 1) n_chunks = 1;
+  if (n_chunks > n_blocks) n_chunks = n_blocks;
+  u.rb_per_chunk = (n_blocks + n_chunks - 1) / n_chunks;
+  u.n_chunks = (n_blocks + u.rb_per_chunk - 1) / u.rb_per_chunk;
+  return u;
+}
 int launch_tn_split(TcDevice* dev, int bn, int c, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
                     int block, const uint8_t* keep, void* dW, int lddw, cudaStream_t s);
 

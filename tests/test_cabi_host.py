@@ -195,12 +195,15 @@ def _fake_call(n, k, d, c, tokens=32768, act=0, z=True, g=True):
 
 def test_route_choice_follows_the_measured_crossovers():
     """bsp_linear_route is host-only: with both routes possible it takes the gathering kernel where it was measured
-    to win on B200 (64-row blocks at 8x on the FFN shapes) and the zero-expanded route elsewhere."""
+    to win on B200 (64-row blocks from 5x to 8x on, 128-row blocks earlier) and the zero-expanded route elsewhere."""
     lib = bsp.lib
     assert bsp.bsp_linear_route(_fake_call(1024, 4096, 64, 8.0)) == bsp.ROUTE_GATHERED             # FFN-down
     assert bsp.bsp_linear_route(_fake_call(4096, 1024, 64, 8.0, act=1)) == bsp.ROUTE_GATHERED      # FFN-up + GELU
-    assert bsp.bsp_linear_route(_fake_call(3072, 1024, 64, 8.0)) == bsp.ROUTE_ZERO_EXPANDED        # QKV
-    assert bsp.bsp_linear_route(_fake_call(1024, 4096, 64, 5.0)) == bsp.ROUTE_ZERO_EXPANDED
+    assert bsp.bsp_linear_route(_fake_call(3072, 1024, 64, 8.0)) == bsp.ROUTE_GATHERED             # QKV: 84 us against 118
+    assert bsp.bsp_linear_route(_fake_call(1024, 4096, 64, 5.0)) == bsp.ROUTE_GATHERED
+    assert bsp.bsp_linear_route(_fake_call(1024, 4096, 64, 3.0)) == bsp.ROUTE_ZERO_EXPANDED
+    assert bsp.bsp_linear_route(_fake_call(1024, 1024, 64, 8.0)) == bsp.ROUTE_GATHERED             # attention output
+    assert bsp.bsp_linear_route(_fake_call(768, 3072, 64, 8.0, tokens=128)) == bsp.ROUTE_ZERO_EXPANDED   # split contraction
     assert bsp.bsp_linear_route(_fake_call(1024, 4096, 32, 8.0)) == bsp.ROUTE_ZERO_EXPANDED
     assert bsp.bsp_linear_route(_fake_call(2304, 768, 16, 3.0, tokens=4096)) == bsp.ROUTE_ZERO_EXPANDED
     # only one route possible: that one, whatever the estimate says
