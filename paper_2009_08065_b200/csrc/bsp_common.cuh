@@ -140,6 +140,12 @@ inline int allow_dynamic_smem(OncePerDevice& once, K* kernel, int bytes) {
   }
   return BSP_OK;
 }
+inline int sm_count(int* sms) {
+  int dev = 0;
+  BSP_CUDA_TRY(cudaGetDevice(&dev));
+  BSP_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+  return BSP_OK;
+}
 #define BSP_TRY(expr)                \
   do {                               \
     const int _st = (expr);          \

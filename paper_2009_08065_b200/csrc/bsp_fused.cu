@@ -15,7 +15,6 @@
 namespace bsp {
 namespace {
 
-constexpr int kStage1Ctas = 148;  // stage 1: below it some SMs have no row-block
 constexpr int kRowsPerPass = 4;   // rows staged in shared memory at a time
 
 // The job table travels as a kernel parameter; a single-matrix call gets a table of one job (0.2 KB instead
@@ -341,7 +340,9 @@ int launch_stage1(const FusedJob* jobs, int n_jobs, int block, float eps, int sq
   threads = threads > 256 ? 256 : threads;
   B.parts = 1;
   B.part_chunks = chunks;
-  if (N == 1 && jobs[0].flags == nullptr && jobs[0].partial == nullptr && total < kStage1Ctas && chunks > 128) {
+  int sms = 0;
+  BSP_TRY(sm_count(&sms));
+  if (N == 1 && jobs[0].flags == nullptr && jobs[0].partial == nullptr && total < sms && chunks > 128) {
     // A matrix of few wide row-blocks leaves SMs idle: they are cut into column ranges of a piece per thread (11 blocks of
     // 96 x 3072: 13.7 -> 8.9 us; ranges of 64 or 32 pieces cost 0.7 us more than whole blocks of 1024 columns).  Not where
     // a row-block is counted as a whole.

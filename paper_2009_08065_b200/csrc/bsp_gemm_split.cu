@@ -28,7 +28,6 @@ using namespace tc;
 namespace {
 
 constexpr int kSplitThreads = 352;
-constexpr int kAtomBytes = 64 * kBlockK * 2;       // MN-major: 64 elements x 64 contraction rows = 8 KB
 
 struct SplitParams {
   int rows, cols;            // output matrix
@@ -45,19 +44,7 @@ struct SplitParams {
   int* status;
 };
 
-__device__ __forceinline__ uint32_t split_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void split_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void split_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t split_map(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-// 16 bytes into another CTA's shared memory, counted on its mbarrier (both addresses from split_map).
+// 16 bytes into another CTA's shared memory, counted on its mbarrier (both addresses from map_to_cta).
 __device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr), "r"(bar), "r"(a),
                "r"(b), "r"(c), "r"(d));
@@ -81,18 +68,6 @@ __device__ __forceinline__ void tmem_load_cols(uint32_t taddr, uint32_t (&v)[N])
                  : "memory");
   }
 }
-// MN-major operand tile with the 128-byte swizzle: 8-row atoms 1024 bytes apart along the contraction,
-// 64-element groups 8 KB apart along M / N.
-__device__ __forceinline__ uint64_t split_desc_mn(uint32_t smem_addr) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((smem_addr & 0x3ffff) >> 4);
-  d |= static_cast<uint64_t>(kAtomBytes >> 4) << 16;             // leading byte offset / 16
-  d |= static_cast<uint64_t>(1024 >> 4) << 32;                   // stride byte offset / 16
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(2) << 61;
-  return d;
-}
-
 template <int BN, int C, bool kTn>
 __global__ void __launch_bounds__(kSplitThreads, 1)
 gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
@@ -118,7 +93,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   auto empty_bar = [&](int s) { return bar_base + 8u * (8 + s); };
   const uint32_t acc_bar = bar_base + 8u * 16, recv_bar = bar_base + 8u * 17;
   const int S = P.stages;
-  const uint32_t rank = split_rank();
+  const uint32_t rank = cluster_rank();
   const int tile = static_cast<int>(blockIdx.x) / C;
   const int m0 = (tile / P.n_tiles) * kBlockM, n0 = (tile % P.n_tiles) * BN;
   const int quads = (min(kBlockM, P.rows - m0) + 31) >> 5;   // quarters of the tile with rows that exist
@@ -142,7 +117,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_holder;
-  split_cluster_arrive();                              // this CTA runs and its mbarriers exist
+  cluster_arrive();                              // this CTA runs and its mbarriers exist
 
   // The weights of a stable plan are older than the kernel before this one: their producer does not wait, and
   // leaves the signal to the warps that do (see launch_pdl).
@@ -164,7 +139,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       const uint32_t dst = smem_base + stage * kStage;
       if constexpr (kTn) {
         tma_stage_load(dst, &map_a, m0, kb * kBlockK, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
-        tma_load_2d_elect(dst + kAtomBytes, &map_a, m0 + 64, kb * kBlockK, full_bar(stage));
+        tma_load_2d_elect(dst + kAtomGroup, &map_a, m0 + 64, kb * kBlockK, full_bar(stage));
       } else {
         tma_stage_load(dst, &map_a, kb * kBlockK, m0, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
       }
@@ -182,7 +157,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       if constexpr (kTn) {
         tma_stage_load(dst, &map_b, n0, kb * kBlockK, full_bar(stage), kStageB);
 #pragma unroll
-        for (int g = 1; g < BN / 64; ++g) tma_load_2d_elect(dst + g * kAtomBytes, &map_b, n0 + 64 * g, kb * kBlockK, full_bar(stage));
+        for (int g = 1; g < BN / 64; ++g) tma_load_2d_elect(dst + g * kAtomGroup, &map_b, n0 + 64 * g, kb * kBlockK, full_bar(stage));
       } else {
         tma_stage_load(dst, &map_b, kb * kBlockK, n0, full_bar(stage), kStageB);
       }
@@ -202,7 +177,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       ready = kb + 1 < kb1 && mbar_try_wait(full_bar(next), next_phase);
       const uint32_t a_addr = smem_base + stage * kStage, b_addr = a_addr + kStageA;
       if constexpr (kTn)     // 16 contraction rows = two 8-row atoms = 2048 bytes per step
-        mma_stage<128, 128>(tmem_base, split_desc_mn(a_addr), split_desc_mn(b_addr), kIdesc, kb != kb0 ? 1u : 0u, empty_bar(stage));
+        mma_stage<128, 128>(tmem_base, smem_desc_mn_sw128(a_addr), smem_desc_mn_sw128(b_addr), kIdesc, kb != kb0 ? 1u : 0u, empty_bar(stage));
       else                   // 16 columns = 32 bytes
         mma_stage<2, 2>(tmem_base, smem_desc_sw128(a_addr), smem_desc_sw128(b_addr), kIdesc, kb != kb0 ? 1u : 0u, empty_bar(stage));
       stage = next;
@@ -237,10 +212,10 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     tcgen05_fence_after();
   }
   __syncwarp();
-  split_cluster_wait();                                // the others run
+  cluster_wait();                                // the others run
   if constexpr (kTn) {                                 // and no longer need their stages
-    split_cluster_arrive();
-    split_cluster_wait();
+    cluster_arrive();
+    cluster_wait();
   }
 
   const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
@@ -259,8 +234,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       for (int o = 1; o < C; ++o) {
         tmem_loaded<PC>(v[o - 1]);
         const uint32_t q = (rank + o) % C, slot = rank < q ? rank : rank - 1;
-        const uint32_t dst = split_map(recv_base + slot * kSlot + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at, q);
-        const uint32_t bar = split_map(recv_bar, q);
+        const uint32_t dst = map_to_cta(recv_base + slot * kSlot + static_cast<uint32_t>(c0 >> 2) * (kBlockM * 16u) + row_at, q);
+        const uint32_t bar = map_to_cta(recv_bar, q);
 #pragma unroll
         for (int j = 0; j < PC / 4; ++j)
           st_async_v4(dst + j * (kBlockM * 16u), bar, v[o - 1][4 * j], v[o - 1][4 * j + 1], v[o - 1][4 * j + 2], v[o - 1][4 * j + 3]);
@@ -368,8 +343,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   __syncthreads();
   quiet_period(timed_out);
   if (*timed_out != 0u) {                              // (the same for every thread) until every other CTA has left, or waits here too
-    split_cluster_arrive();
-    split_cluster_wait();
+    cluster_arrive();
+    cluster_wait();
   }
   if (warp == 1) {
     tcgen05_fence_after();

@@ -20,19 +20,7 @@ using namespace tc;
 namespace {
 
 constexpr int kTnThreads = kThreads + 32;          // producer A, MMA, 8 epilogue warps, producer B
-constexpr int kAtomGroup = 64 * kBlockK * 2;       // 64 elements x 64 token rows = 8 KB
 
-// MN-major operand tile with the 128-byte swizzle: 8-row atoms 1024 bytes apart along the
-// contraction, 64-element groups 8 KB apart along M / N.
-__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t smem_addr) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((smem_addr & 0x3ffff) >> 4);
-  d |= static_cast<uint64_t>(kAtomGroup >> 4) << 16;            // leading byte offset / 16
-  d |= static_cast<uint64_t>(1024 >> 4) << 32;                   // stride byte offset / 16
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(2) << 61;
-  return d;
-}
 // bf16 x bf16 -> float32, both operands MN-major (bits 15 and 16), M = 128, N = BN.
 __host__ __device__ constexpr uint32_t tn_idesc(int bn) { return instr_desc_bf16(bn) | (1u << 15) | (1u << 16); }
 

@@ -62,13 +62,9 @@ struct LinearParams {
 // Four groups with one buffer each (the same 32 KB; the exposed epilogue of a CTA's last tile then takes
 // two pieces per group instead of four) were measured 1.5 us slower per four-GEMM layer at 4096 tokens:
 // sixteen warps contend for the shared memory that the operand copies and the tensor core keep busy.
-#ifndef BSP_TC_GROUPS
-#define BSP_TC_GROUPS 2
-#endif
-constexpr int kGroups = BSP_TC_GROUPS;
+constexpr int kGroups = 2;
 constexpr int kEpiThreads = 128 * kGroups;
 constexpr int kBufPerGroup = kEpiBuffers / kGroups;
-static_assert(kGroups == 2 || kGroups == 4, "two or four epilogue groups");
 constexpr int kWeightWarp = 2 + 4 * kGroups;            // the second TMA producer warp, for the weight tiles
 constexpr int kThreadsTc = 32 * (kWeightWarp + 1);
 

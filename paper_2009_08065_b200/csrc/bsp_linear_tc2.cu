@@ -29,21 +29,6 @@ constexpr int kPairStages = (kSmemLimit - kPairFixed) / kPairStage > 8 ? 8 : (kS
 constexpr int kPairSmemBytes = kPairStages * kPairStage + kPairFixed;
 constexpr int kPairTmemCols = 512;
 
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// Address of the same shared-memory location in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // TMA load whose completion bytes are counted on an mbarrier that may live in the peer CTA.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar_cluster) {
   asm volatile(
@@ -103,7 +88,7 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   volatile uint32_t* timed_out = tmem_holder + 1;     // set by a role of this CTA whose wait expired
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
+  const uint32_t rank = cluster_rank();          // 0 = leader of the pair
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar_base = smem_u32(bars);
@@ -129,7 +114,7 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
   tcgen05_fence_before();
   __syncthreads();
-  cluster_sync_all();          // both CTAs' barriers exist before anything signals across the pair
+  cluster_sync();          // both CTAs' barriers exist before anything signals across the pair
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_holder;
 
@@ -253,7 +238,7 @@ linear_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   tcgen05_fence_before();
   __syncthreads();
   quiet_period(timed_out);
-  cluster_sync_all();          // neither CTA leaves while the other may still touch its memory or barriers
+  cluster_sync();          // neither CTA leaves while the other may still touch its memory or barriers
   if (warp == 1) {
     tcgen05_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),

@@ -24,7 +24,6 @@ constexpr int kSegment = 256;          // groups of a strip that one CTA packs (
 // Segments of a matrix: every CTA adds up the counts before its own.  4000 of them (1000 x 1000 in single columns) 26 us, 30
 // without; 8192 equal; 13870 (280 x 6935) 67, 51 without.
 constexpr int kMaxSegments = 4096;
-constexpr int kTallBlocks = 296;       // blocks up to which a CTA of 1024 threads per block fits the GPU at once (two per SM)
 
 struct Geometry {
   int rows, cols, ldw, block, orient, n_blocks, n_groups;
@@ -234,7 +233,7 @@ flags_rank_kernel(const uint16_t* W, Geometry G, int keep_count, uint8_t* keep, 
   }
 }
 
-cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, uint8_t* flags, int32_t* counts, int32_t* seg_counts,
+cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int sms, int keep_count, uint8_t* flags, int32_t* counts, int32_t* seg_counts,
                         cudaStream_t s) {
   if (G.n_groups <= kRankGroups)
     return launch_pdl(flags_rank_kernel, dim3(G.n_blocks), dim3((G.n_groups + 31) / 32 * 32), 0, s, w, G, keep_count, flags, counts, seg_counts);
@@ -246,7 +245,7 @@ cudaError_t launch_topk(const uint16_t* w, const Geometry& G, int keep_count, ui
   if (G.orient == BSP_ORIENT_C) return launch(flags_topk_kernel<512>, 512);
   // 1024 threads where all strips run at once, and where a strip has so many groups that its passes count more than the
   // waves (512 strips of 8192 groups 136 us, 215 with 256 threads; 600 of 768 groups 25 against 22)
-  return G.n_blocks <= kTallBlocks || G.n_groups >= 4096 ? launch(flags_topk_kernel<1024>, 1024)
+  return G.n_blocks <= 2 * sms || G.n_groups >= 4096 ? launch(flags_topk_kernel<1024>, 1024)
                                                          : launch(flags_topk_kernel<kPackThreads>, kPackThreads);
 }
 
@@ -505,13 +504,15 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
   uint8_t* flags = keep ? keep : reinterpret_cast<uint8_t*>(wsb + L.keep_off);
   const uint16_t* w = static_cast<const uint16_t*>(W);
 
+  int sms = 0;                          // (two CTAs of 1024 threads fit one)
+  BSP_TRY(sm_count(&sms));
   const bool fast = orient == BSP_ORIENT_C && fused_shape_ok(W, rows, cols, ldw, block) && aligned_to(flags, 8);
   if (fast) {
     // vectorised kernels of bsp_fused.cu: stage 1 for the flags (unless the keep-count kernel makes them), stage 2
     FusedJob j{w, rows, cols, ldw, G.n_blocks, threshold, threshold_dev, nullptr, nullptr, nullptr, nullptr, nullptr,
                flags, counts, blk_ptr, idx, static_cast<uint16_t*>(vals), kept_weights, nullptr};
     if (keep_per_block >= 0) {
-      BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, nullptr, s));
+      BSP_CUDA_TRY(launch_topk(w, G, sms, keep_per_block, flags, counts, nullptr, s));
     } else {
       st = fused_stage1(&j, 1, block, 0.0f, 0, s);
       if (st != BSP_OK) return st;
@@ -525,7 +526,7 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
     // (the flags go to the caller's array, so the workspace's flags are free for the segments' counts)
     int32_t* seg_counts = reinterpret_cast<int32_t*>(wsb + L.keep_off);
     const dim3 grid(G.n_blocks, static_cast<unsigned>(segments));
-    if (keep_per_block >= 0) BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, seg_counts, s));
+    if (keep_per_block >= 0) BSP_CUDA_TRY(launch_topk(w, G, sms, keep_per_block, flags, counts, seg_counts, s));
     else BSP_CUDA_TRY(launch_pdl(flags_segment_kernel, grid, dim3(kSegment), 0, s, w, G, threshold, threshold_dev, flags, seg_counts));
     const int vec = (reinterpret_cast<uintptr_t>(vals) & 15) == 0 ? G.vec : 1;
     BSP_CUDA_TRY(launch_pdl(vec == 8 ? compact_segment_kernel<8> : vec == 4 ? compact_segment_kernel<4> : compact_segment_kernel<1>, grid,
@@ -535,10 +536,10 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
   // A CTA per block, threads for its groups: up to 1024 of them, since a matrix of few wide blocks has few CTAs (768 x 5120
   // in 16-row blocks 27 us, 83 with 256 threads).  Many row-blocks fill the GPU by themselves and want CTAs that come and
   // go (5343 x 920 in single rows 47 us, 67 with 1024; 2204 x 1214 in fours 12.7 against 15).
-  const bool tall = orient == BSP_ORIENT_R || G.n_blocks <= kTallBlocks;
+  const bool tall = orient == BSP_ORIENT_R || G.n_blocks <= 2 * sms;
   const int threads = !tall ? 256 : G.n_groups >= 1024 ? 1024 : G.n_groups <= 128 ? 128 : (G.n_groups + 31) / 32 * 32;
   if (keep_per_block >= 0) {
-    BSP_CUDA_TRY(launch_topk(w, G, keep_per_block, flags, counts, nullptr, s));
+    BSP_CUDA_TRY(launch_topk(w, G, sms, keep_per_block, flags, counts, nullptr, s));
   } else {
     BSP_CUDA_TRY(launch_pdl(tall ? flags_threshold_kernel<1024> : flags_threshold_kernel<256>, dim3(G.n_blocks), dim3(threads), 0, s, w, G,
                             threshold, threshold_dev, flags, counts));

@@ -16,6 +16,7 @@ struct GradArgs {
   float scale;
   float* grad;
   int ldg;
+  unsigned first_wave;       // CTAs of the tiled kernel that are resident at once
 };
 
 // Orientation C, 8-element alignment, blocks of 8 to 32 rows: a CTA takes 256 columns of a row-block.  Its
@@ -25,7 +26,6 @@ struct GradArgs {
 // accumulating) per weight.  One thread per 8 columns walking down the rows, as the kernel below does, has
 // 1/16 of the loads in flight: 14 us instead of 6 for a 4096 x 1024 matrix of 16-row blocks, accumulating.
 constexpr int kGradCols = 256, kGradMinRows = 8, kGradMaxRows = 32;
-constexpr unsigned kGradFirstWave = 4 * 148;
 template <int ITEMS>
 __global__ void __launch_bounds__(256)
 grad_c_tile_kernel(GradArgs A) {
@@ -37,7 +37,7 @@ grad_c_tile_kernel(GradArgs A) {
   const bool on = c < A.cols;
   const size_t r0 = static_cast<size_t>(b) * A.block;
   // (only the CTAs that can be waiting: behind them it would cost issue slots for nothing)
-  const bool early = blockIdx.y * gridDim.x + blockIdx.x < kGradFirstWave;
+  const bool early = blockIdx.y * gridDim.x + blockIdx.x < A.first_wave;
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     const int r = row + 8 * i;
@@ -203,7 +203,7 @@ extern "C" int bsp_penalty_grad(const void* W, int rows, int cols, int ldw, int 
   if (scale != scale) return BSP_ERR_ARG;
   if (ldg < cols) return BSP_ERR_SHAPE;
   GradArgs A{static_cast<const uint16_t*>(W), rows, cols, ldw, block, orient, pen == BSP_PEN_L2SQ ? 1 : 0,
-             accumulate ? 1 : 0, gamma, scale, grad, ldg};
+             accumulate ? 1 : 0, gamma, scale, grad, ldg, 0u};
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool vec = orient == BSP_ORIENT_C && cols % 8 == 0 && ldw % 8 == 0 && ldg % 4 == 0 && aligned_to(W, 16) &&
                    aligned_to(grad, 16) && aligned_to(gamma, 16);
@@ -211,6 +211,9 @@ extern "C" int bsp_penalty_grad(const void* W, int rows, int cols, int ldw, int 
   // 7048 x 2160 in fours 28 against 21)
   if (vec && block >= kGradMinRows && block <= kGradMaxRows && (cols + kGradCols - 1) / kGradCols <= 65535) {
     const dim3 grid(rows / block, (cols + kGradCols - 1) / kGradCols);
+    int sms = 0;
+    BSP_TRY(sm_count(&sms));
+    A.first_wave = 4u * static_cast<unsigned>(sms);
     BSP_CUDA_TRY(launch_pdl(block <= 8 ? grad_c_tile_kernel<1> : block <= 16 ? grad_c_tile_kernel<2> : grad_c_tile_kernel<4>, grid,
                             dim3(256), 0, s, A));
   } else if (vec) {

@@ -266,9 +266,8 @@ extern "C" int bsp_masked_adam_step(float* W, const float* grad, float* m, float
   if (blocks > 0x7fffffffLL) return BSP_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const dim3 grid(static_cast<unsigned>(blocks));
-  int dev = 0, sms = 0;
-  BSP_CUDA_TRY(cudaGetDevice(&dev));
-  BSP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  int sms = 0;
+  BSP_TRY(sm_count(&sms));
   A.first_wave = 5u * static_cast<unsigned>(sms);        // 48 registers x 256 threads: five CTAs per SM
   if (blocks * 256 < (1LL << 32)) BSP_CUDA_TRY(launch_pdl(masked_adam_kernel<unsigned>, grid, dim3(256), 0, s, A));
   else BSP_CUDA_TRY(launch_pdl(masked_adam_kernel<unsigned long long>, grid, dim3(256), 0, s, A));

@@ -346,26 +346,6 @@ __device__ __forceinline__ void for_matching(const uint32_t* keys, long long n, 
   }
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_size() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Shared memory of CTA `rank` of the cluster, at the address that p has in this CTA.
-__device__ __forceinline__ uint32_t map_to_cta(const void* p, uint32_t rank) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(tc::smem_u32(p)), "r"(rank));
-  return remote;
-}
 __device__ __forceinline__ uint32_t ld_cluster(uint32_t addr) {
   uint32_t v;
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
@@ -393,7 +373,7 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
   extern __shared__ uint32_t s_list[];                       // [kList], then in CTA 0 [kCandidates]
   uint32_t* s_cand = s_list + kList;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_rank(), n_cta = cluster_size();
+  const uint32_t rank = tc::cluster_rank(), n_cta = tc::cluster_size();
   const SelectJob& J = B.job[blockIdx.x / n_cta];
   const uint32_t* keys = reinterpret_cast<const uint32_t*>(J.S);
   const long long n = J.n;
@@ -483,8 +463,8 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) st_cluster(map_to_cta(&s_len[rank], 0u), s_n);
-    cluster_sync();                                          // the lists and their lengths are complete
+    if (threadIdx.x == 0) st_cluster(tc::map_to_cta(tc::smem_u32(&s_len[rank]), 0u), s_n);
+    tc::cluster_sync();                                          // the lists and their lengths are complete
     if (rank == 0) {
       const uint32_t length = lane < static_cast<int>(n_cta) ? s_len[lane] : 0u;
       found = __reduce_add_sync(0xffffffffu, length);
@@ -495,7 +475,7 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
         for (uint32_t q = warp & 3u; q < n_cta; q += 4u) {
           const uint32_t len = __shfl_sync(0xffffffffu, length, static_cast<int>(q));
           const uint32_t at = __reduce_add_sync(0xffffffffu, lane < static_cast<int>(q) ? length : 0u);
-          const uint32_t src = map_to_cta(s_list, q);
+          const uint32_t src = tc::map_to_cta(tc::smem_u32(s_list), q);
           for (uint32_t i0 = static_cast<uint32_t>((warp >> 2) * 32 + lane); i0 < len; i0 += 4 * (kSelThreads / 4)) {
             uint32_t c[4];
 #pragma unroll
@@ -518,10 +498,10 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
       hist[threadIdx.x] = 0u;
       if (threadIdx.x < kBins3) hist[kBins2 + threadIdx.x] = 0u;
     }
-    cluster_sync();
+    tc::cluster_sync();
   }
   if (rank != 0) {
-    cluster_sync();                                          // CTA 0 has read this CTA's list
+    tc::cluster_sync();                                          // CTA 0 has read this CTA's list
     return;
   }
   // the next digit over the listed keys or all of them; then a warp ranks the few keys that are left, or the last
@@ -562,7 +542,7 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
     p = pick_bin<kBins3>(hist + kBins2, p.want, s_sum, s_pick);
     if (threadIdx.x == 0) *J.out = threshold_of((prefix << kBits3) | p.bin);
   }
-  cluster_sync();
+  tc::cluster_sync();
 }
 
 // ------------------------------------------------------------ select where counts do not fit 32 bits (select_large)
@@ -746,13 +726,6 @@ int launch_sums_c(SelectBatchT<N>& B, int sms, cudaStream_t s) {
   auto* kernel = B.block >= 32 ? (parts ? sums_c_kernel<N, true, true> : sums_c_kernel<N, false, true>)
                                : (parts ? sums_c_kernel<N, true, false> : sums_c_kernel<N, false, false>);
   BSP_CUDA_TRY(launch_pdl(kernel, dim3(at), dim3(kSumThreads + 32), 0, s, B));
-  return BSP_OK;
-}
-
-int sm_count(int* sms) {
-  int dev = 0;
-  BSP_CUDA_TRY(cudaGetDevice(&dev));
-  BSP_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
   return BSP_OK;
 }
 

@@ -164,6 +164,30 @@ __device__ __forceinline__ bool mbar_wait_probed(bool ready, uint32_t bar, uint3
   return __all_sync(0xffffffffu, ready) || mbar_wait_warp(bar, parity, status);
 }
 
+// ---- thread-block clusters
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
+}
+// Address of the same shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
 // ---- issue by an elected lane of a converged warp
 // The tensor core's and the copy engine's instructions take their operands from the warp-uniform registers.  Issued
 // inside `if (lane == 0)` every operand is first moved there as a per-thread value: 72 cycles per tcgen05.mma and
@@ -283,6 +307,18 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t smem_addr) {
   d |= static_cast<uint64_t>(1024 >> 4) << 32;                   // stride byte offset / 16
   d |= static_cast<uint64_t>(1) << 46;                           // descriptor version of this architecture
   d |= static_cast<uint64_t>(2) << 61;                           // 128-byte swizzle
+  return d;
+}
+// The same of an MN-major tile: 8-row atoms 1024 bytes apart along the contraction, 64-element groups (8 KB: 64
+// elements x 64 contraction rows) one after the other along M / N.
+constexpr int kAtomGroup = 64 * kBlockK * 2;
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t smem_addr) {
+  uint64_t d = 0;
+  d |= static_cast<uint64_t>((smem_addr & 0x3ffff) >> 4);
+  d |= static_cast<uint64_t>(kAtomGroup >> 4) << 16;             // leading byte offset / 16
+  d |= static_cast<uint64_t>(1024 >> 4) << 32;                   // stride byte offset / 16
+  d |= static_cast<uint64_t>(1) << 46;
+  d |= static_cast<uint64_t>(2) << 61;
   return d;
 }
 // Instruction descriptor: bf16 x bf16 -> float32, both operands K-major, M = 128, N = BN.
