@@ -405,11 +405,9 @@ constexpr int kPlanRRows = 256;
 template <int VEC>
 __global__ void __launch_bounds__(256)
 plan_expand_r_kernel(const int32_t* blk_ptr, const int32_t* row_idx,
-                     const uint16_t* vals, int n_out, int k_in, int h, uint16_t* Wx) {
+                     const uint16_t* vals, int first_row, int n_out, int k_in, int h, uint16_t* Wx) {
   __shared__ int s_pos[kPlanRRows];
-  const unsigned at = grid_piece() * kPlanRRows;
-  if (at >= static_cast<unsigned>(n_out)) return;
-  const int a = blockIdx.x, r0 = static_cast<int>(at);
+  const int a = blockIdx.x, r0 = first_row + blockIdx.y * kPlanRRows;
   const int n_rows = min(kPlanRRows, n_out - r0);
   s_pos[threadIdx.x] = -1;
   pdl_wait();
@@ -739,13 +737,13 @@ extern "C" int bsp_linear_plan_r(const int32_t* blk_ptr, const int32_t* row_idx,
   const size_t need = round_up(static_cast<size_t>(n_out) * k_in * 2, 256);
   if (plan_bytes < need) return BSP_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const dim3 grid = grid_of(k_in / block, (static_cast<long long>(n_out) + kPlanRRows - 1) / kPlanRRows);
-  TcDevice* dev = tc_device();
-  if (dev == nullptr) return BSP_ERR_CUDA;
+  const long long pieces = (static_cast<long long>(n_out) + kPlanRRows - 1) / kPlanRRows;
+  int sms = 0;
+  BSP_TRY(sm_count(&sms));
   // Strips narrower than 8 columns in more CTAs than the GPU holds at once (eight per SM) are scattered, a clearing pass
   // more: 1216 x 6264 in single columns 15 us against 75, 1168 x 2152 in fours 5.0 against 6.8.  Not below that (536 x 1964
   // in fours 4.9 against 4.7) and not in eights (5328 x 1648 14.8 against 10.9).
-  if (block < 8 && static_cast<long long>(grid.x) * grid.y * grid.z > 8LL * dev->sms) {
+  if (block < 8 && k_in / block * pieces > 8LL * sms) {
     BSP_CUDA_TRY(cudaMemsetAsync(plan, 0, static_cast<size_t>(n_out) * k_in * 2, s));
     plan_scatter_r_kernel<<<k_in / block, 256, 0, s>>>(blk_ptr, row_idx, static_cast<const uint16_t*>(vals), k_in, block,
                                                        static_cast<uint16_t*>(plan));
@@ -754,9 +752,13 @@ extern "C" int bsp_linear_plan_r(const int32_t* blk_ptr, const int32_t* row_idx,
   }
   // widest vector: every segment starts at a multiple of `block` in rows of k_in elements (a multiple of it too)
   const int vec = block % 8 == 0 && aligned_to(vals, 16) ? 8 : block % 4 == 0 && aligned_to(vals, 8) ? 4 : 1;
-  BSP_CUDA_TRY(launch_pdl(vec == 8 ? plan_expand_r_kernel<8> : vec == 4 ? plan_expand_r_kernel<4> : plan_expand_r_kernel<1>,
-                          grid, dim3(256), 0, s, blk_ptr, row_idx, static_cast<const uint16_t*>(vals), n_out, k_in,
-                          block, static_cast<uint16_t*>(plan)));
+  // (a launch takes 16.7 million rows; numbering the pieces over two grid dimensions cost the short launches 0.6 us)
+  for (long long done = 0; done < pieces; done += 65535) {
+    const dim3 grid(k_in / block, static_cast<unsigned>(pieces - done < 65535 ? pieces - done : 65535));
+    BSP_CUDA_TRY(launch_pdl(vec == 8 ? plan_expand_r_kernel<8> : vec == 4 ? plan_expand_r_kernel<4> : plan_expand_r_kernel<1>,
+                            grid, dim3(256), 0, s, blk_ptr, row_idx, static_cast<const uint16_t*>(vals),
+                            static_cast<int>(done * kPlanRRows), n_out, k_in, block, static_cast<uint16_t*>(plan)));
+  }
   return BSP_OK;
 }
 
