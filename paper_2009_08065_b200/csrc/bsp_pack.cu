@@ -534,9 +534,10 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
     return BSP_OK;
   }
   // A CTA per block, threads for its groups: up to 1024 of them, since a matrix of few wide blocks has few CTAs (768 x 5120
-  // in 16-row blocks 27 us, 83 with 256 threads).  Many row-blocks fill the GPU by themselves and want CTAs that come and
-  // go (5343 x 920 in single rows 47 us, 67 with 1024; 2204 x 1214 in fours 12.7 against 15).
-  const bool tall = orient == BSP_ORIENT_R || G.n_blocks <= 2 * sms;
+  // in 16-row blocks 27 us, 83 with 256 threads).  Many blocks fill the GPU by themselves and want CTAs that come and
+  // go (5343 x 920 in single rows 47 us, 67 with 1024; 2204 x 1214 in fours 12.7 against 15; 7826 x 4759 in single columns
+  // 650 against 730).
+  const bool tall = G.n_blocks <= 2 * sms;
   const int threads = !tall ? 256 : G.n_groups >= 1024 ? 1024 : G.n_groups <= 128 ? 128 : (G.n_groups + 31) / 32 * 32;
   if (keep_per_block >= 0) {
     BSP_CUDA_TRY(launch_topk(w, G, sms, keep_per_block, flags, counts, nullptr, s));
