@@ -286,10 +286,10 @@ extern "C" int bsp_repack_values(const void* W, int rows, int cols, int ldw, int
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint16_t* w = static_cast<const uint16_t*>(W);
   const size_t smem = static_cast<size_t>(cols) * (kRepackRows + 1) * 2;
-  // Staged rows, where several CTAs fit an SM and have more than one row each.  Behind the Adam step, staged / gathered from
+  // Staged rows, where several CTAs fit an SM and have all of their rows.  Behind the Adam step, staged / gathered from
   // global memory: 4096 x 1024 in 16-row blocks 4.0 / 5.7 us, 768 x 3072 5.5 / 5.2, 8192 x 4096 49 / 26, 5344 x 920 in single
-  // rows 11.2 / 10.2.
-  if (cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && cols <= kRepackMaxCols && block > 1) {
+  // rows 11.2 / 10.2; 6042 x 2128 in pairs, by itself, 10.7 / 7.5.
+  if (cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && cols <= kRepackMaxCols && block >= kRepackRows) {
     BSP_CUDA_TRY(launch_pdl(repack_vec_kernel, grid, dim3(kRepackThreads), smem, s, w, cols, ldw, block, blk_ptr, idx,
                             static_cast<uint16_t*>(vals)));
   } else {
