@@ -247,6 +247,18 @@ __device__ __forceinline__ float group_sumsq_strided8(const uint16_t* p, int n, 
       acc = __fmaf_rn(w, w, acc);
     }
   }
+  if (e + 4 <= n) {
+    uint16_t v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = ld_global(p + u * stride);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float w = bf16_bits_to_float(v[u]);
+      acc = __fmaf_rn(w, w, acc);
+    }
+    e += 4;
+    p += 4 * stride;
+  }
   for (; e < n; ++e, p += stride) {
     const float w = bf16_bits_to_float(ld_global(p));
     acc = __fmaf_rn(w, w, acc);
@@ -324,6 +336,7 @@ __device__ __forceinline__ void sumsq8(const uint16_t* p, int d, int ldw, float 
   if (kTall)
     for (; r + 32 <= d; r += 32) sumsq8_rows<32>(p + static_cast<size_t>(r) * ldw, ldw, acc);   // 512 bytes in flight
   for (; r + 16 <= d; r += 16) sumsq8_rows<16>(p + static_cast<size_t>(r) * ldw, ldw, acc);   // 256 bytes in flight
+  if (!kTall && r + 8 <= d) { sumsq8_rows<8>(p + static_cast<size_t>(r) * ldw, ldw, acc); r += 8; }
   for (; r + 4 <= d; r += 4) sumsq8_rows<4>(p + static_cast<size_t>(r) * ldw, ldw, acc);
   for (; r < d; ++r) sumsq8_rows<1>(p + static_cast<size_t>(r) * ldw, ldw, acc);
 }
