@@ -446,7 +446,7 @@ int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, lo
     for (int i = 0; i < 3; ++i) {
       const int c = 2 << i;
       if (c > kb || tiles * c > dev.split_ctas[i]) continue;
-      const long long stages = (kb + c - 1) / c * per_stage[b][i] * (k_in % 64 ? 115 : 100) / 100;   // ragged rows, as in choose_dense
+      const long long stages = (kb + c - 1) / c * per_stage[b][i] * (k_in % 16 ? 161 : k_in % 64 ? 115 : 100) / 100;   // ragged rows, as in choose_dense
       const long long t = fixed[b][i] + quads * per_quad[b][i] + stages + 2 * tiles * c;
       if (t < best) { best = t; choice = i; *bn = 64 * (b + 1); }
     }

@@ -604,7 +604,9 @@ dim3 grid_of(int x, long long pieces) {
 // part (start-up, first operands, the last tile's epilogue), per wave of tiles the larger of its main loop and its
 // epilogue (with GELU also a part of the smaller one: they contend for issue slots), and something per wave after the
 // first.  A 64-deep stage takes longer the more SMs are drawing operands from L2 (two times per width, for a few CTAs
-// and for all of them), and where rows of X and the plan are no multiple of 128 bytes.  Fitted to launches of 8 to
+// and for all of them), and where rows of X and the plan are no multiple of 128 bytes; more so where they are no multiple
+// of 32 either (every row then straddles sectors: 12891 x 3856 x 3080 one CTA 326 us, pair 259, 16650 x 1288 x 2136 130 and
+// 103; measured over estimated without that 1.4 to 1.5, pairs 1.16, over 17 such layers).  Fitted to launches of 8 to
 // 32768 tokens (nanoseconds; widths 64 / 128 / 192 / 256, pair): over 28 random layers and ten of 768 and 1024 features
 // the choice is about 1 % behind the best of the five on average.  Against the earlier rule (waves x (width + 440), pairs
 // from 1.25 x #SM tiles without GELU): 8192 tokens x 1024 outputs x 4096 inputs 52.7 -> 48.3 us, 4096 outputs with GELU
@@ -613,7 +615,7 @@ DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, i
   static const int width[5] = {64, 128, 192, 256, 256}, rows[5] = {128, 128, 128, 128, 256};
   static const int fixed[5] = {2830, 3200, 3750, 4400, 5400}, extra_wave[5] = {500, 700, 300, 800, 800};
   static const int stage_few[5] = {158, 168, 250, 320, 330}, stage_all[5] = {176, 210, 335, 370, 330};
-  static const int ragged_percent[5] = {114, 130, 103, 110, 117};
+  static const int ragged_percent[2][5] = {{114, 130, 103, 110, 117}, {160, 170, 155, 160, 136}};
   static const int epilogue[2][5] = {{500, 950, 1500, 1750, 2600}, {900, 1600, 2600, 2950, 3900}};
   static const int gelu_tail[5] = {150, 500, 450, 600, 600}, gelu_overlap[5] = {8, 8, 8, 8, 5};
   const long long kb = (k_in + kBlockK - 1) / kBlockK;
@@ -625,7 +627,7 @@ DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, i
     const long long waves = (tiles + seats - 1) / seats;
     const long long busy = tiles < seats ? tiles : seats;
     long long main_ns = kb * (stage_few[c] + (stage_all[c] - stage_few[c]) * busy / seats);
-    if (k_in % 64) main_ns = main_ns * ragged_percent[c] / 100;
+    if (k_in % 64) main_ns = main_ns * ragged_percent[k_in % 16 != 0][c] / 100;
     const long long epi_ns = epilogue[gelu][c];
     long long tile_ns = main_ns > epi_ns ? main_ns : epi_ns;
     if (gelu) {
