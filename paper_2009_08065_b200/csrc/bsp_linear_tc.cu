@@ -414,9 +414,13 @@ plan_expand_r_kernel(const int32_t* blk_ptr, const int32_t* row_idx,
   pdl_launch_dependents();
   const int lo = blk_ptr[a], kc = blk_ptr[a + 1] - lo;
   __syncthreads();
-  for (int j = threadIdx.x; j < kc; j += 256) {
-    const int r = row_idx[lo + j] - r0;
-    if (r >= 0 && r < n_rows) s_pos[r] = j;
+  for (int j0 = threadIdx.x; j0 < kc; j0 += 4 * 256) {
+    int r[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) r[u] = ld_global(row_idx + lo + min(j0 + u * 256, kc - 1)) - r0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + u * 256 < kc && r[u] >= 0 && r[u] < n_rows) s_pos[r[u]] = j0 + u * 256;
   }
   __syncthreads();
   const uint16_t* tile = vals + static_cast<size_t>(h) * lo;
