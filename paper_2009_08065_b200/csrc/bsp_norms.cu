@@ -51,7 +51,7 @@ norms_generic_kernel(const uint16_t* W, int rows, int cols, int ldw, int block, 
     if (orient == BSP_ORIENT_C) {
       const long long b = g / cols;
       const int j = static_cast<int>(g - b * cols);
-      S = group_sumsq_strided8(W + static_cast<size_t>(b) * block * ldw + j, block, ldw);
+      S = group_sumsq_strided(W + static_cast<size_t>(b) * block * ldw + j, block, ldw);
     } else {
       const int per_row = cols / block;
       const long long i = g / per_row;

@@ -152,10 +152,16 @@ grad_c_vec8_kernel(GradArgs A) {
   }
 }
 
-// Any geometry: one thread per group.  An ordinary launch: CTAs placed while the kernel before still holds seats spread
-// unevenly over the SMs, and 2848 x 2080 in strips of 32 took 78 us against 53.
+// Any geometry: one thread per group.  It overlaps the kernel before it only where it has a CTA per SM or fewer: CTAs
+// placed while that kernel still holds seats spread unevenly over the SMs, and 2848 x 2080 in strips of 32 took 78 us
+// against 53.
+template <bool kOverlap>
 __global__ void __launch_bounds__(256)
 grad_generic_kernel(GradArgs A) {
+  if (kOverlap) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
   const bool c_orient = A.orient == BSP_ORIENT_C;
   const long long n_groups = c_orient ? static_cast<long long>(A.rows / A.block) * A.cols
                                       : static_cast<long long>(A.rows) * (A.cols / A.block);
@@ -176,7 +182,7 @@ grad_generic_kernel(GradArgs A) {
   if (A.squared) {
     factor = 2.0f * A.scale * A.gamma[g];
   } else {
-    const float n = __fsqrt_rn(group_sumsq_strided8(A.W + first, A.block, stride));
+    const float n = __fsqrt_rn(group_sumsq_strided(A.W + first, A.block, stride));
     factor = n > 0.0f ? __fdiv_rn(A.scale * A.gamma[g], n) : 0.0f;
   }
   // the same element position in grad: row = first / ldw, col = first % ldw
@@ -207,14 +213,17 @@ extern "C" int bsp_penalty_grad(const void* W, int rows, int cols, int ldw, int 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool vec = orient == BSP_ORIENT_C && cols % 8 == 0 && ldw % 8 == 0 && ldg % 4 == 0 && aligned_to(W, 16) &&
                    aligned_to(grad, 16) && aligned_to(gamma, 16);
-  // (a warp per row: blocks of fewer than 8 rows leave warps without work, 5343 x 920 in single rows 27 us against 12 and
-  // 7048 x 2160 in fours 28 against 21)
-  if (vec && block >= kGradMinRows && block <= kGradMaxRows && (cols + kGradCols - 1) / kGradCols <= 65535) {
-    const dim3 grid(rows / block, (cols + kGradCols - 1) / kGradCols);
-    int sms = 0;
-    BSP_TRY(sm_count(&sms));
+  int sms = 0;
+  BSP_TRY(sm_count(&sms));
+  const dim3 tiles(rows / block, (cols + kGradCols - 1) / kGradCols);
+  // A warp per row: blocks of fewer than 8 rows leave warps without work, which counts once the CTAs are more than run at
+  // once (5343 x 920 in single rows 27 us, 12 by the other kernel, 7048 x 2160 in fours 28 and 21; but 117 x 544 in threes
+  // 2.1 and 4.0).
+  const bool tiled = tiles.y <= 65535 && block <= kGradMaxRows &&
+                     (block >= kGradMinRows || static_cast<long long>(tiles.x) * tiles.y <= 8LL * sms);
+  if (vec && tiled) {
     A.first_wave = 4u * static_cast<unsigned>(sms);
-    BSP_CUDA_TRY(launch_pdl(block <= 8 ? grad_c_tile_kernel<1> : block <= 16 ? grad_c_tile_kernel<2> : grad_c_tile_kernel<4>, grid,
+    BSP_CUDA_TRY(launch_pdl(block <= 8 ? grad_c_tile_kernel<1> : block <= 16 ? grad_c_tile_kernel<2> : grad_c_tile_kernel<4>, tiles,
                             dim3(256), 0, s, A));
   } else if (vec) {
     const long long items = static_cast<long long>(rows / block) * (cols / 8);
@@ -223,7 +232,9 @@ extern "C" int bsp_penalty_grad(const void* W, int rows, int cols, int ldw, int 
     int nb, ng;
     geometry(rows, cols, block, orient, &nb, &ng);
     const long long groups = static_cast<long long>(nb) * ng;
-    grad_generic_kernel<<<static_cast<unsigned>((groups + 255) / 256), 256, 0, s>>>(A);
+    const dim3 grid(static_cast<unsigned>((groups + 255) / 256));
+    if (grid.x <= static_cast<unsigned>(sms)) BSP_CUDA_TRY(launch_pdl(grad_generic_kernel<true>, grid, dim3(256), 0, s, A));
+    else grad_generic_kernel<false><<<grid, 256, 0, s>>>(A);
     BSP_LAUNCH_CHECK();
   }
   return BSP_OK;
