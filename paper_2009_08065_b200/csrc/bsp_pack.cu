@@ -21,9 +21,10 @@ constexpr int kPackThreads = 256;
 constexpr int kRankGroups = 192;
 static_assert(kRankGroups <= 256, "a block of few groups is one segment");
 constexpr int kSegment = 256;          // groups of a strip that one CTA packs (orientation R)
-// Segments of a matrix: every CTA adds up the counts before its own.  4000 of them (1000 x 1000 in single columns) 26 us, 30
-// without; 8192 equal; 13870 (280 x 6935) 67, 51 without.
-constexpr int kMaxSegments = 4096;
+// Segments of a matrix up to which strips are packed by them: every CTA adds up the counts before its own.  With many
+// strips, 4000 segments (1000 x 1000 in single columns) 26 us, 30 without; 8192 equal; 13870 (280 x 6935) 67, 51 without.
+// With few, a CTA per strip leaves more to lose: 5115 (7928 x 2640 in strips of 16) 37, 57 without.
+constexpr int kMaxSegments = 4096, kFewStrips = 512, kMaxSegmentsFew = 16384;
 
 struct Geometry {
   int rows, cols, ldw, block, orient, n_blocks, n_groups;
@@ -420,13 +421,13 @@ compact_segment_kernel(const uint16_t* W, Geometry G, const uint8_t* keep,
 template <typename Index>
 __global__ void __launch_bounds__(256)
 apply_mask_c_kernel(uint16_t* W, int rows, int cols, int ldw, int block, const uint8_t* keep) {
-  pdl_wait();
-  pdl_launch_dependents();
   const Index chunks = static_cast<Index>(cols >> 3), item = static_cast<Index>(blockIdx.x) * 256u + threadIdx.x;
   const Index i = item / chunks;
-  if (i >= static_cast<Index>(rows)) return;
   const size_t c = static_cast<size_t>(item - i * chunks) << 3;
   const size_t b = static_cast<unsigned>(i) / static_cast<unsigned>(block);
+  pdl_wait();
+  pdl_launch_dependents();
+  if (i >= static_cast<Index>(rows)) return;
   const uint2 f = ld_global(reinterpret_cast<const uint2*>(keep + b * cols + c));
   if (((f.x - 0x01010101u) & ~f.x & 0x80808080u) == 0u && ((f.y - 0x01010101u) & ~f.y & 0x80808080u) == 0u) return;   // no zero byte
   uint16_t* w = W + static_cast<size_t>(i) * ldw + c;
@@ -438,16 +439,22 @@ apply_mask_c_kernel(uint16_t* W, int rows, int cols, int ldw, int block, const u
       if ((((e < 4 ? f.x : f.y) >> (8 * (e & 3))) & 0xffu) == 0u) w[e] = 0;
   }
 }
-// Any geometry, a weight per thread.  An ordinary launch: there are many short CTAs, and taking seats among those of the
-// kernel before cost 13 % of a 7928 x 2640 matrix in orientation R (75.7 against 85.7 us).
+// Any geometry, a weight per thread.  It overlaps the kernel before it only where it has a CTA per SM or fewer: many short
+// CTAs that take seats among those of the kernel before cost 13 % of a 7928 x 2640 matrix in orientation R (75.7 against
+// 85.7 us), and a few save half a microsecond.
+template <bool kOverlap>
 __global__ void __launch_bounds__(256)
-apply_mask_kernel(uint16_t* __restrict__ W, Geometry G, const uint8_t* __restrict__ keep) {
+apply_mask_kernel(uint16_t* W, Geometry G, const uint8_t* keep) {
+  if (kOverlap) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
   const long long e = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= static_cast<long long>(G.rows) * G.cols) return;
   const int i = static_cast<int>(e / G.cols), j = static_cast<int>(e - static_cast<long long>(i) * G.cols);
   const size_t slot = G.orient == BSP_ORIENT_C ? static_cast<size_t>(i / G.block) * G.cols + j
                                                : static_cast<size_t>(i) * (G.cols / G.block) + j / G.block;
-  if (!keep[slot]) W[static_cast<size_t>(i) * G.ldw + j] = 0;
+  if (!ld_global(keep + slot)) W[static_cast<size_t>(i) * G.ldw + j] = 0;
 }
 
 // Fixed scratch for bsp_prune_pack_static: lives in the library's device image, so every GPU
@@ -521,7 +528,7 @@ extern "C" int bsp_prune_pack(const void* W, int rows, int cols, int ldw, int bl
   }
   const long long segments = (G.n_groups + kSegment - 1) / kSegment;
   const bool keep_in_ws = keep >= reinterpret_cast<uint8_t*>(wsb) && keep < reinterpret_cast<uint8_t*>(wsb) + ws_bytes;
-  if (orient == BSP_ORIENT_R && keep != nullptr && !keep_in_ws && G.n_blocks * segments <= kMaxSegments &&
+  if (orient == BSP_ORIENT_R && keep != nullptr && !keep_in_ws && G.n_blocks * segments <= (G.n_blocks <= kFewStrips ? kMaxSegmentsFew : kMaxSegments) &&
       G.n_blocks * segments * sizeof(int32_t) <= L.sumsq_off - L.keep_off) {
     // (the flags go to the caller's array, so the workspace's flags are free for the segments' counts)
     int32_t* seg_counts = reinterpret_cast<int32_t*>(wsb + L.keep_off);
@@ -572,7 +579,11 @@ extern "C" int bsp_apply_mask(void* W, int rows, int cols, int ldw, int block, i
   Geometry G{rows, cols, ldw, block, orient, 0, 0, 1};
   geometry(rows, cols, block, orient, &G.n_blocks, &G.n_groups);
   const long long elems = static_cast<long long>(rows) * cols;
-  apply_mask_kernel<<<static_cast<unsigned>((elems + 255) / 256), 256, 0, s>>>(w, G, keep);
+  const dim3 grid(static_cast<unsigned>((elems + 255) / 256));
+  int sms = 0;
+  BSP_TRY(sm_count(&sms));
+  if (grid.x <= static_cast<unsigned>(sms)) BSP_CUDA_TRY(launch_pdl(apply_mask_kernel<true>, grid, dim3(256), 0, s, w, G, keep));
+  else apply_mask_kernel<false><<<grid, 256, 0, s>>>(w, G, keep);
   BSP_LAUNCH_CHECK();
   return BSP_OK;
 }
