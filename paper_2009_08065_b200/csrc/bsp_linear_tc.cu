@@ -468,8 +468,7 @@ plan_scatter_r_kernel(const int32_t* __restrict__ blk_ptr, const int32_t* __rest
 // values are fetched into L2 while the lists are read, and a warp takes adjacent rows so that the table and the
 // block's place are looked up once per row-block.  (Looked up per element, with a division each, the values took 4 us
 // even from L2.)  Between the products of a backward pass (768 features, 16-row blocks, cold operands) a 3072 x 768
-// matrix takes 4 us from the wait on; it took 6.5, and 19 with a clearing pass and scattered 2-byte stores; the
-// pass over four matrices at 4096 tokens 165 -> 151 us.
+// matrix takes 5.4 us, 7.3 scattered over a cleared plan; a 768 x 3072 one 5.4 and 33.
 constexpr int kPlanTK = 64, kPlanTN = 64, kPlanTMaxBlocks = 32, kPlanTThreads = 512;
 struct PlanTGeometry {
   int n_out, k_in, block;
