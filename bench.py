@@ -977,7 +977,8 @@ def run_case(args):
     --case qkv|attn_out|ffn_up|ffn_down runs that linear's GEMM on the bench workload, --case prepare the batched
     weight-side call on its four matrices, --case prepare_stack the same call on the 72 matrices of a BERT-base
     stack (inputs larger than L2), --case gather the gathering linear kernel on a BERT-large FFN-up point
-    (16384 tokens, 1024 -> 4096, 64-row blocks, 5x)."""
+    (16384 tokens, 1024 -> 4096, 64-row blocks, 5x), --case split a linear of 8 tokens (3072 -> 768), whose contraction
+    is split over clusters, --case percentile the threshold of a 3072 x 768 matrix of 16-row blocks."""
     import torch
     torch.cuda.set_device(0)
     device = torch.device("cuda", 0)
@@ -1013,6 +1014,24 @@ def run_case(args):
         bsp.bsp_linear_status()
         print("case gather: 3 launches done")
         return
+    if args.case in ("split", "percentile"):
+        import paper_2009_08065_b200 as bsp
+        gen = torch.Generator(device=device)
+        gen.manual_seed(si.DEFAULT_SEED)
+        n, k = (768, 3072) if args.case == "split" else (3072, 768)
+        W = (torch.randn(n, k, device=device, generator=gen) * 0.02).to(torch.bfloat16)
+        X = torch.randn(8, k, device=device, generator=gen).to(torch.bfloat16)
+        Y = torch.empty(8, n, dtype=torch.bfloat16, device=device)
+        t = torch.zeros(1, device=device)
+        ws = torch.empty(bsp.bsp_pack_bound(n, k, 16)[2], dtype=torch.uint8, device=device)
+        for _ in range(4):
+            if args.case == "split":
+                bsp.bsp_linear_planned(W, n, k, 16, X, None, bsp.ACT_NONE, Y)
+            else:
+                bsp.bsp_percentile_threshold(W, 16, bsp.ORIENT_C, 3.0, t, ws)
+        bsp.bsp_linear_status()
+        print(f"case {args.case}: 4 calls done")
+        return
     layer = LayerOnDevice(workload(), si.DEFAULT_SEED, 0, device)
     layer.step()
     torch.cuda.synchronize()
@@ -1046,7 +1065,8 @@ def main():
     ap.add_argument("--steps", type=int, default=200)
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", choices=["cuda", "reference"], default="cuda")
-    ap.add_argument("--case", choices=["qkv", "attn_out", "ffn_up", "ffn_down", "prepare", "prepare_stack", "gather"], default=None,
+    ap.add_argument("--case", choices=["qkv", "attn_out", "ffn_up", "ffn_down", "prepare", "prepare_stack", "gather", "split", "percentile"],
+                    default=None,
                     help="run a few launches of one call for a profiler and exit")
     ap.add_argument("--sweep", choices=["bert_large"], default=None,
                     help="time the BERT-large compression x block-height grid and print one JSON line per point")
