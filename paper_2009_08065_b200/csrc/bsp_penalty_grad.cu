@@ -129,11 +129,13 @@ grad_c_vec8_kernel(GradArgs A) {
       factor[i] = n > 0.0f ? __fdiv_rn(A.scale * gam[i], n) : 0.0f;
     }
   }
-  uint4 next = ld_global(reinterpret_cast<const uint4*>(p));     // a row ahead of the stores
+  // (the address passes through an empty statement behind the wait, and so do these loads; unlike ordinary ones they may
+  // pass the stores of the rows before)
+  asm volatile("" : "+l"(p));
+#pragma unroll 4
   for (int r = 0; r < A.block; ++r) {
-    const uint4 v = next;
-    p += A.ldw;
-    if (r + 1 < A.block) next = ld_global(reinterpret_cast<const uint4*>(p));
+    uint4 v;
+    asm("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p + static_cast<size_t>(r) * A.ldw));
     const uint32_t w32[4] = {v.x, v.y, v.z, v.w};
     float o[8];
 #pragma unroll
