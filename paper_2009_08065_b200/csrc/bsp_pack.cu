@@ -416,18 +416,21 @@ compact_segment_kernel(const uint16_t* W, Geometry G, const uint8_t* keep,
 }
 
 // Orientation C, 8 adjacent columns of a row per thread: nothing is read but the flags, and only pieces with a
-// pruned group are written.  (A row per CTA left a narrow matrix with mostly idle warps: 6272 x 80 8.0 us, 3.7 by single
-// weights.)
-template <typename Index>
+// pruned group are written.  CTAs take pieces of one row, or of the matrix numbered through (kFlat) where a row has too
+// few for a warp and there are many rows: 6272 x 80 a row per CTA 8.0 us, flat 3.3; 256 x 88 1.8 and 2.5, 3240 x 1848 15.5
+// and 17.8 (two divisions a thread).
+template <bool kFlat, typename Index>
 __global__ void __launch_bounds__(256)
 apply_mask_c_kernel(uint16_t* W, int rows, int cols, int ldw, int block, const uint8_t* keep) {
-  const Index chunks = static_cast<Index>(cols >> 3), item = static_cast<Index>(blockIdx.x) * 256u + threadIdx.x;
-  const Index i = item / chunks;
-  const size_t c = static_cast<size_t>(item - i * chunks) << 3;
+  const Index chunks = static_cast<Index>(cols >> 3);
+  const Index item = static_cast<Index>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const Index i = kFlat ? item / chunks : static_cast<Index>(blockIdx.y);
+  const Index q = kFlat ? item - i * chunks : item;
+  const size_t c = static_cast<size_t>(q) << 3;
   const size_t b = static_cast<unsigned>(i) / static_cast<unsigned>(block);
   pdl_wait();
   pdl_launch_dependents();
-  if (i >= static_cast<Index>(rows)) return;
+  if (i >= static_cast<Index>(rows) || q >= chunks) return;
   const uint2 f = ld_global(reinterpret_cast<const uint2*>(keep + b * cols + c));
   if (((f.x - 0x01010101u) & ~f.x & 0x80808080u) == 0u && ((f.y - 0x01010101u) & ~f.y & 0x80808080u) == 0u) return;   // no zero byte
   uint16_t* w = W + static_cast<size_t>(i) * ldw + c;
@@ -570,10 +573,16 @@ extern "C" int bsp_apply_mask(void* W, int rows, int cols, int ldw, int block, i
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint16_t* w = static_cast<uint16_t*>(W);
   if (orient == BSP_ORIENT_C && cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && aligned_to(keep, 8)) {
-    const long long ctas = (static_cast<long long>(rows) * (cols / 8) + 255) / 256;
-    const dim3 grid(static_cast<unsigned>(ctas));
-    if (ctas * 256 < (1LL << 32)) BSP_CUDA_TRY(launch_pdl(apply_mask_c_kernel<unsigned>, grid, dim3(256), 0, s, w, rows, cols, ldw, block, keep));
-    else BSP_CUDA_TRY(launch_pdl(apply_mask_c_kernel<unsigned long long>, grid, dim3(256), 0, s, w, rows, cols, ldw, block, keep));
+    const int chunks = cols / 8;
+    const long long ctas = (static_cast<long long>(rows) * chunks + 255) / 256;
+    if (rows <= 65535 && (chunks >= 32 || rows < 2048)) {
+      const dim3 grid((chunks + 255) / 256, rows), threads(chunks >= 256 ? 256 : (chunks + 31) / 32 * 32);
+      BSP_CUDA_TRY(launch_pdl(apply_mask_c_kernel<false, unsigned>, grid, threads, 0, s, w, rows, cols, ldw, block, keep));
+    } else if (ctas * 256 < (1LL << 32)) {
+      BSP_CUDA_TRY(launch_pdl(apply_mask_c_kernel<true, unsigned>, dim3(static_cast<unsigned>(ctas)), dim3(256), 0, s, w, rows, cols, ldw, block, keep));
+    } else {
+      BSP_CUDA_TRY(launch_pdl(apply_mask_c_kernel<true, unsigned long long>, dim3(static_cast<unsigned>(ctas)), dim3(256), 0, s, w, rows, cols, ldw, block, keep));
+    }
     return BSP_OK;
   }
   Geometry G{rows, cols, ldw, block, orient, 0, 0, 1};

@@ -39,6 +39,18 @@ def test_percentile_select(rows, cols, block, orient, ties):
         assert np.float32(t.item()) == np.float32(O.percentile_threshold(w, block, "CR"[orient], rate)), rate
 
 
+# a row per CTA and pieces numbered through: on both sides of 2048 rows and of 32 pieces a row; any geometry on both sides of
+# a CTA per SM
+@pytest.mark.parametrize("rows,cols,block,orient", [(2047, 248, 1, 0), (2048, 248, 2, 0), (2048, 256, 2, 0), (65536, 256, 256, 0),
+                                                    (40, 2056, 8, 0), (148, 256, 4, 1), (149, 256, 4, 1), (300, 129, 3, 0)])
+def test_mask_on_both_sides_of_its_rules(rows, cols, block, orient):
+    w, o = weights(f"m{rows}x{cols}", rows, cols), "CR"[orient]
+    keep = O.keep_flags(w, block, o, float(np.median(O.group_norms(w[:512] if orient == 0 else w, block, o))))
+    wd = to_dev(w).clone()
+    bsp.bsp_apply_mask(wd, block, orient, torch.from_numpy(keep.astype(np.uint8)).to(DEV))
+    assert np.array_equal(bits_of(wd), si.zero_groups(w, keep, block, o))
+
+
 def test_percentile_of_a_streamed_batch():
     """More items than the streaming sums need (six per SM) and more matrices than one launch takes: matrices with a
     histogram (16384 groups and more) among ones without, so that a CTA crosses from either kind to either; one cut into
