@@ -335,8 +335,8 @@ int bsp_linear_planned(const void* plan, int n_out, int k_in, int block,
                        void* Y, int ldy, void* stream);
 /* bsp_linear_planned with the kernel variant chosen by the caller: BSP_LINEAR_AUTO (what
  * bsp_linear_planned does), BSP_LINEAR_ONE_CTA (128 x BN tiles, one CTA each) or
- * BSP_LINEAR_CTA_PAIR (256 x 256 tiles shared by a cluster of two CTAs, one third less operand
- * traffic from L2).  The two named variants sum in the same order and give the same bits.
+ * BSP_LINEAR_CTA_PAIR (256 x BN tiles shared by a cluster of two CTAs, a quarter to a third less
+ * operand traffic from L2).  The two named variants sum in the same order and give the same bits.
  * BSP_LINEAR_AUTO takes the fastest by estimate and has a third choice: where a layer has few output
  * tiles (few tokens, or few outputs) a cluster of 2, 4 or 8 CTAs splits the contraction and adds the
  * float32 partial sums in a fixed order.  Its results are reproducible and as accurate, but their last
@@ -345,9 +345,8 @@ int bsp_linear_planned(const void* plan, int n_out, int k_in, int block,
 typedef enum { BSP_LINEAR_AUTO = 0, BSP_LINEAR_ONE_CTA = 1, BSP_LINEAR_CTA_PAIR = 2 } bsp_linear_algo;
 /* May be OR-ed into `algo`: the caller vouches that the plan is older than the work that immediately
  * precedes this call in the stream (the usual case in a chain of layers: the weights are old, only X is
- * fresh): whatever wrote the plan stands at least one kernel further ahead.  The one-CTA and the split
- * kernel then start fetching weight tiles while that work is still finishing; the pair kernel ignores
- * the flag.  Never set it when the preceding kernel writes the plan. */
+ * fresh): whatever wrote the plan stands at least one kernel further ahead.  The kernel then starts
+ * fetching weight tiles while that work is still finishing.  Never set it when the preceding kernel writes the plan. */
 #define BSP_LINEAR_PLAN_STABLE 0x100
 /* May be OR-ed into `algo`: write the output TRANSPOSED, Y := YT [n_out, tokens] row-major with
  * leading dimension ldy >= tokens (a multiple of 8), bit for bit the transpose of what the call

@@ -454,24 +454,31 @@ int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, lo
   if (ns != nullptr) *ns = choice < 0 ? whole_ns : best;
   return choice;
 }
-// dW: tiles 128 / 192 / 256 wide, whole (persistent kernel: per wave) or, 128 and 256 wide, split 2 / 4 / 8.  Rows of dY
-// or X that are no multiple of 128 bytes make the operand boxes straddle lines: a set of stage times of their own.
-// (4096 tokens: 768 x 768 24.6 us whole 256 wide, 12.4 split 4, 9.8 as 128-wide tiles split 2; 3072 x 768 17.0 as 256-wide
-// tiles split 2, 16.2 whole 128 wide; 3072 x 1024 26.2 whole 256 wide, 20.6 192 wide.  173 tokens: 7.3 and 5.0.)
-int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in, int* bn) {
-  const long long m_tiles = (n_out + kBlockM - 1) / kBlockM;
+// dW: whole tiles 128 / 192 / 256 wide by one CTA, 128 / 256 wide by a pair (persistent kernels: per wave, a stage longer the
+// more SMs are at work, as in choose_dense), or, 128 and 256 wide, split 2 / 4 / 8.  Rows of dY or X that are no multiple of
+// 128 bytes make the operand boxes straddle lines: a percentage, for the splits a set of stage times of their own.
+// (4096 tokens, one CTA 128 wide / pair 128 wide / split 2: 768 x 768 15.5 / 13.7 / 10.2 us, 3072 x 768 18.5 / 15.9, 2304 x
+// 768 18.1 / 15.6; 4096 x 1024 29.5 one CTA 256 wide, 25.9 pair 256 wide, 28.0 pair 128 wide; 1024 tokens, 3072 x 768 8.0 /
+// 7.0.  Over 28 weights the choice is 1.5 % behind the best on average.)
+TnChoice choose_tn(const TcDevice& dev, int tokens, int n_out, int k_in) {
+  const long long m_tiles = (n_out + kBlockM - 1) / kBlockM, m_pairs = (n_out + 2 * kBlockM - 1) / (2 * kBlockM);
   const int kb = (tokens + kBlockK - 1) / kBlockK;
   const int ragged = n_out % 64 || k_in % 64 ? 1 : 0;
-  static const int widths[3] = {128, 192, 256}, fixed_whole[3] = {4450, 5400, 6400};
-  static const int stage_whole[2][3] = {{175, 225, 283}, {250, 310, 366}};
+  static const int widths[5] = {128, 192, 256, 128, 256}, fixed[5] = {4670, 5110, 6240, 4010, 4770}, extra_wave[5] = {0, 0, 220, 0, 1270};
+  static const int stage_few[5] = {161, 243, 294, 141, 270}, stage_all[5] = {212, 307, 373, 187, 341};
+  static const int ragged_percent[5] = {124, 115, 114, 110, 100};
   static const int fixed_split[2][3] = {{4000, 4100, 4500}, {6700, 6700, 6600}};
   static const int stage_split[2][2][3] = {{{178, 178, 200}, {265, 265, 265}}, {{270, 334, 373}, {365, 380, 400}}};
   long long best = -1;
-  int choice = -1;
-  for (int w = 0; w < 3; ++w) {
-    const long long waves = (m_tiles * ((k_in + widths[w] - 1) / widths[w]) + dev.sms - 1) / dev.sms;
-    const long long t = fixed_whole[w] + 1500 * (waves - 1) + waves * kb * stage_whole[ragged][w];
-    if (best < 0 || t < best) { best = t; *bn = widths[w]; }
+  TnChoice choice{256, false, 1};
+  for (int w = 0; w < 5; ++w) {
+    const bool pair = w >= 3;
+    const long long tiles = (pair ? m_pairs : m_tiles) * ((k_in + widths[w] - 1) / widths[w]), seats = pair ? dev.sms / 2 : dev.sms;
+    const long long waves = (tiles + seats - 1) / seats, busy = tiles < seats ? tiles : seats;
+    long long stages = waves * kb * (stage_few[w] + (stage_all[w] - stage_few[w]) * busy / seats);
+    if (ragged) stages = stages * ragged_percent[w] / 100;
+    const long long t = fixed[w] + extra_wave[w] * (waves - 1) + stages;
+    if (best < 0 || t < best) { best = t; choice = TnChoice{widths[w], pair, 1}; }
   }
   for (int b = 0; b < 2; ++b) {
     const long long tiles = m_tiles * ((k_in + 128 * (b + 1) - 1) / (128 * (b + 1)));
@@ -479,7 +486,7 @@ int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in, int* b
       const int c = 2 << i;
       if (c > kb || tiles * c > dev.split_ctas[i]) continue;
       const long long t = fixed_split[b][i] + 4 * tiles * c + (kb + c - 1) / c * stage_split[b][ragged][i];
-      if (t < best) { best = t; choice = i; *bn = 128 * (b + 1); }
+      if (t < best) { best = t; choice = TnChoice{128 * (b + 1), false, c}; }
     }
   }
   return choice;

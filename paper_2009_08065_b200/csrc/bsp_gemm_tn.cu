@@ -10,8 +10,8 @@
 // stride byte offset = distance between 8-row groups).  Everything else (persistent CTAs, TMA
 // producers, one MMA-issuing thread, two TMEM accumulators, two epilogue groups, TMA stores,
 // bounded waits) is the pipeline of bsp_linear_tc.cu with a 128 x BN output tile.
-// The epilogue applies the mask (pruned groups of dW are written as zero).  A weight of fewer tiles than SMs goes
-// to the split contraction of bsp_gemm_split.cu instead where that is faster.
+// The epilogue applies the mask (pruned groups of dW are written as zero).  Most weights go to the CTA pairs of
+// bsp_linear_tc2.cu or, with fewer tiles than SMs, to the split contraction of bsp_gemm_split.cu instead (choose_tn).
 #include "bsp_tc.cuh"
 
 namespace bsp {
@@ -247,10 +247,11 @@ extern "C" int bsp_linear_backward_weight(const void* dY, int ldy, const void* X
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // (flags that are not 8-byte aligned are applied by the mask kernel afterwards)
   const uint8_t* flags = keep != nullptr && aligned_to(keep, 8) ? keep : nullptr;
-  int bn = 256;
-  const int split = choose_tn_split(*dev, tokens, n_out, k_in, &bn);
-  if (split >= 0) {
-    const int st = launch_tn_split(dev, bn, 2 << split, dY, ldy, X, ldx, tokens, n_out, k_in, block, flags, dW, lddw, s);
+  const TnChoice choice = choose_tn(*dev, tokens, n_out, k_in);
+  const int bn = choice.bn;
+  if (choice.pair || choice.cluster > 1) {
+    const int st = choice.pair ? launch_tn_pair(dev, bn, dY, ldy, X, ldx, tokens, n_out, k_in, block, flags, dW, lddw, s)
+                               : launch_tn_split(dev, bn, choice.cluster, dY, ldy, X, ldx, tokens, n_out, k_in, block, flags, dW, lddw, s);
     if (st != BSP_OK || keep == flags) return st;
     return bsp_apply_mask(dW, n_out, k_in, lddw, block, BSP_ORIENT_C, keep, stream);
   }

@@ -37,7 +37,7 @@ int check_call(const bsp_linear_call* c) {
 // 768 to 4096 features, blocks of 16 to 128 rows at 3 to 8 times compression: the gathering estimate is off by 6 % (rms),
 // the choice costs 0.6 % over the better route on average and 22 % at worst (7.1 us against 8.6).
 void estimate_ns(const bsp_linear_call& c, const TcDevice& dev, double* zero_expanded, double* gathered) {
-  long long ns = choose_dense(dev, c.tokens, c.n_out, c.k_in, c.act, c.YT == nullptr).ns;
+  long long ns = choose_dense(dev, c.tokens, c.n_out, c.k_in, c.act, c.YT == nullptr ? DenseKinds::kAll : DenseKinds::kOneCta).ns;
   int bn;
   choose_linear_split(dev, c.tokens, c.n_out, c.k_in, ns, &bn, &ns);
   *zero_expanded = static_cast<double>(ns) + 1000.0;

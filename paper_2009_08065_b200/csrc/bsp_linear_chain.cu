@@ -351,11 +351,11 @@ extern "C" int bsp_linear_chain(const bsp_chain_op* ops, int n_ops, const void* 
     if (!aligned_to(u.plan, 16) || !aligned_to(u.Y, 16) || u.k_in % 8 || u.n_out % 8 || u.ldy % 8 || src_ld % 8)
       return BSP_ERR_UNSUPPORTED;
     if (tokens == 0) continue;
-    const DenseChoice choice = choose_dense(*dev, tokens, u.n_out, u.k_in, u.act, false);
+    const DenseChoice choice = choose_dense(*dev, tokens, u.n_out, u.k_in, u.act, DenseKinds::kOneCta);
     const int bn = choice.bn;
     int bn_split;
     split = split || (u.k_in <= 12288 && choose_linear_split(*dev, tokens, u.n_out, u.k_in,
-                                                             choose_dense(*dev, tokens, u.n_out, u.k_in, u.act, true).ns, &bn_split) >= 0);
+                                                             choose_dense(*dev, tokens, u.n_out, u.k_in, u.act, DenseKinds::kAll).ns, &bn_split) >= 0);
     const uint16_t* src_base = static_cast<const uint16_t*>(src) + u.src_col;
     if (!make_map(&M.x[i], src_base, u.k_in, tokens, src_ld, kBlockM)) return BSP_ERR_CUDA;
     if (!make_map(&M.w[i], u.plan, u.k_in, u.n_out, u.k_in, bn)) return BSP_ERR_CUDA;

@@ -35,8 +35,8 @@ namespace bsp {
 
 int check_linear_args(const void* a, const void* b, const void* c, int n_out, int k_in, int block,
                       const void* X, int tokens, int ldx, int act, const void* Y, int ldy);
-int launch_tc_pair(TcDevice* dev, const void* plan, const void* X, void* Y, int tokens, int n_out, int k_in, int act,
-                   const void* bias, int ldx, int ldy, cudaStream_t s);
+int launch_tc_pair(TcDevice* dev, int bn, const void* plan, const void* X, void* Y, int tokens, int n_out, int k_in, int act,
+                   const void* bias, int ldx, int ldy, bool plan_stable, cudaStream_t s);
 
 using namespace tc;
 
@@ -603,30 +603,33 @@ dim3 grid_of(int x, long long pieces) {
   return dim3(x, static_cast<unsigned>((pieces + z - 1) / z), static_cast<unsigned>(z));
 }
 }  // namespace
-// Tile width, or the CTA-pair kernel, for a product of whole tiles: the least estimated time.  A launch costs a fixed
+// Tile width, one CTA or a pair, for a product of whole tiles: the least estimated time.  A launch costs a fixed
 // part (start-up, first operands, the last tile's epilogue), per wave of tiles the larger of its main loop and its
 // epilogue (with GELU also a part of the smaller one: they contend for issue slots), and something per wave after the
 // first.  A 64-deep stage takes longer the more SMs are drawing operands from L2 (two times per width, for a few CTAs
 // and for all of them), and where rows of X and the plan are no multiple of 128 bytes; more so where they are no multiple
 // of 32 either (every row then straddles sectors: 12891 x 3856 x 3080 one CTA 326 us, pair 259, 16650 x 1288 x 2136 130 and
 // 103; measured over estimated without that 1.4 to 1.5, pairs 1.16, over 17 such layers).  Fitted to launches of 8 to
-// 32768 tokens (nanoseconds; widths 64 / 128 / 192 / 256, pair): over 28 random layers and ten of 768 and 1024 features
-// the choice is about 1 % behind the best of the five on average.  Against the earlier rule (waves x (width + 440), pairs
-// from 1.25 x #SM tiles without GELU): 8192 tokens x 1024 outputs x 4096 inputs 52.7 -> 48.3 us, 4096 outputs with GELU
-// 55.5 -> 52.3.
-DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, int act, bool allow_pair) {
-  static const int width[5] = {64, 128, 192, 256, 256}, rows[5] = {128, 128, 128, 128, 256};
-  static const int fixed[5] = {2830, 3200, 3750, 4400, 5400}, extra_wave[5] = {500, 700, 300, 800, 800};
-  static const int stage_few[5] = {158, 168, 250, 320, 330}, stage_all[5] = {176, 210, 335, 370, 330};
-  static const int ragged_percent[2][5] = {{114, 130, 103, 110, 117}, {160, 170, 155, 160, 136}};
-  static const int epilogue[2][5] = {{500, 950, 1500, 1750, 2600}, {900, 1600, 2600, 2950, 3900}};
-  static const int gelu_tail[5] = {150, 500, 450, 600, 600}, gelu_overlap[5] = {8, 8, 8, 8, 5};
+// 32768 tokens (nanoseconds; one CTA 64 / 128 / 192 / 256 wide, pairs 128 / 192 / 256): over 64 layers of 256 to 1024
+// features the choice is 0.4 % behind the best of the seven on average and 6 % at worst.  Best one-CTA kernel / best pair:
+// 4096 tokens x 768 outputs x 3072 inputs 19.9 / 16.5 us, 2304 x 768 14.4 / 13.2, 3072 x 768 with GELU 20.7 / 19.8, 4096 x
+// 1024 with GELU 30.9 / 26.2, 768 x 768 7.0 / 7.2; 1003 tokens x 3072 x 1024 8.0 / 8.1, 512 x 768 x 3072 10.6 / 10.9.
+DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, int act, DenseKinds kinds) {
+  constexpr int kKinds = 7, kFirstPair = 4;
+  static const int width[kKinds] = {64, 128, 192, 256, 128, 192, 256};
+  static const int fixed[kKinds] = {2830, 3200, 3750, 4400, 3600, 4070, 4560}, extra_wave[kKinds] = {500, 700, 300, 800, 540, 450, 240};
+  static const int stage_few[kKinds] = {158, 168, 250, 320, 150, 200, 270}, stage_all[kKinds] = {176, 210, 335, 370, 190, 250, 330};
+  static const int ragged_percent[2][kKinds] = {{114, 130, 103, 110, 111, 106, 106}, {160, 170, 155, 160, 136, 136, 136}};
+  static const int epilogue[2][kKinds] = {{500, 950, 1500, 1750, 570, 610, 1170}, {900, 1600, 2600, 2950, 1570, 3160, 3660}};
+  static const int gelu_tail[kKinds] = {150, 500, 450, 600, 660, 530, 900};
   const long long kb = (k_in + kBlockK - 1) / kBlockK;
   const bool gelu = act == BSP_ACT_GELU;
   DenseChoice best{128, false, -1};
-  for (int c = 0; c < (allow_pair ? 5 : 4); ++c) {
-    const long long tiles = ((tokens + rows[c] - 1) / rows[c]) * static_cast<long long>((n_out + width[c] - 1) / width[c]);
-    const long long seats = c == 4 ? dev.sms / 2 : dev.sms;
+  for (int c = kinds == DenseKinds::kPairs ? kFirstPair : 0; c < (kinds == DenseKinds::kOneCta ? kFirstPair : kKinds); ++c) {
+    const bool pair = c >= kFirstPair;
+    const int rows = pair ? 2 * kBlockM : kBlockM;
+    const long long tiles = ((tokens + rows - 1) / rows) * static_cast<long long>((n_out + width[c] - 1) / width[c]);
+    const long long seats = pair ? dev.sms / 2 : dev.sms;
     const long long waves = (tiles + seats - 1) / seats;
     const long long busy = tiles < seats ? tiles : seats;
     long long main_ns = kb * (stage_few[c] + (stage_all[c] - stage_few[c]) * busy / seats);
@@ -635,10 +638,10 @@ DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, i
     long long tile_ns = main_ns > epi_ns ? main_ns : epi_ns;
     if (gelu) {
       const long long less = main_ns > epi_ns ? epi_ns : main_ns;
-      tile_ns += less * less / tile_ns / gelu_overlap[c];
+      tile_ns += less * less / tile_ns / 8;
     }
     const long long ns = fixed[c] + waves * tile_ns + (waves - 1) * extra_wave[c] + (gelu ? gelu_tail[c] : 0);
-    if (best.ns < 0 || ns < best.ns) best = DenseChoice{width[c], c == 4, ns};
+    if (best.ns < 0 || ns < best.ns) best = DenseChoice{width[c], pair, ns};
   }
   return best;
 }
@@ -819,18 +822,20 @@ extern "C" int bsp_linear_planned_ex(const void* plan, int n_out, int k_in, int 
   TcDevice* dev = tc_device();
   if (dev == nullptr) return BSP_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  DenseChoice choice = choose_dense(*dev, tokens, n_out, k_in, act, algo == BSP_LINEAR_AUTO && !transposed);
-  if (algo == BSP_LINEAR_CTA_PAIR) choice.pair = true;
+  const DenseKinds kinds = algo == BSP_LINEAR_CTA_PAIR ? DenseKinds::kPairs
+                           : algo == BSP_LINEAR_AUTO && !transposed ? DenseKinds::kAll : DenseKinds::kOneCta;
+  const DenseChoice choice = choose_dense(*dev, tokens, n_out, k_in, act, kinds);
+  const bool plan_stable = (algo_flags & BSP_LINEAR_PLAN_STABLE) != 0;
   if (algo == BSP_LINEAR_AUTO) {
     // few output tiles: a cluster of CTAs per tile, each with a part of the contraction
     int bn_split = 0;
     const int c = choose_linear_split(*dev, tokens, n_out, k_in, choice.ns, &bn_split);
     if (c >= 0)
       return launch_linear_split(dev, bn_split, 2 << c, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy,
-                                 (algo_flags & BSP_LINEAR_PLAN_STABLE) != 0, transposed, s);
+                                 plan_stable, transposed, s);
   }
-  if (choice.pair) return launch_tc_pair(dev, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy, s);
-  LinearParams P{tokens, n_out, k_in, act, (algo_flags & BSP_LINEAR_PLAN_STABLE) ? 1 : 0, copy_rows(tokens) * kBlockK * 2,
+  if (choice.pair) return launch_tc_pair(dev, choice.bn, plan, X, Y, tokens, n_out, k_in, act, bias, ldx, ldy, plan_stable, s);
+  LinearParams P{tokens, n_out, k_in, act, plan_stable ? 1 : 0, copy_rows(tokens) * kBlockK * 2,
                  transposed ? 1 : 0,
                  static_cast<const uint16_t*>(bias), dev->status};
   switch (choice.bn) {

@@ -176,6 +176,10 @@ __device__ __forceinline__ uint32_t cluster_size() {
   return r;
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// The same without ordering this thread's memory accesses, where what the others must see has a fence of its own (mbarriers:
+// fence.mbarrier_init) or where the barrier only keeps CTAs alive.  The release waits for every access in flight: 0.5 to 0.8 us
+// a barrier on a busy SM.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
   cluster_arrive();
@@ -514,16 +518,24 @@ struct TcDevice {
 TcDevice* tc_device();
 // Fills split_ctas (bsp_gemm_split.cu).
 bool query_split_ctas(int (&ctas)[3]);
-// Cluster size (2, 4, 8) index of dW's split contraction, or -1: the persistent kernel (bsp_gemm_split.cu); *bn = tile
-// width of either.
-int choose_tn_split(const TcDevice& dev, int tokens, int n_out, int k_in, int* bn);
+// Kernel for dW (bsp_gemm_split.cu): tile width, CTA pairs or not, and the cluster size (2, 4, 8) of a split contraction
+// or 1 for whole tiles.
+struct TnChoice {
+  int bn;
+  bool pair;
+  int cluster;
+};
+TnChoice choose_tn(const TcDevice& dev, int tokens, int n_out, int k_in);
+int launch_tn_pair(TcDevice* dev, int bn, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
+                   int block, const uint8_t* keep, void* dW, int lddw, cudaStream_t s);
 // Kernel for a linear layer on whole tiles, with its estimated time (bsp_linear_tc.cu).
 struct DenseChoice {
   int bn;
   bool pair;
   long long ns;
 };
-DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, int act, bool allow_pair);
+enum class DenseKinds { kOneCta, kPairs, kAll };
+DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, int act, DenseKinds kinds);
 // Cluster size index for the same layer with its contraction split, or -1 where whole tiles (whole_ns) are as fast; *ns
 // (may be null) receives the estimated time of what is faster.
 int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn, long long* ns = nullptr);
