@@ -117,7 +117,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_holder;
-  cluster_arrive();                              // this CTA runs and its mbarriers exist
+  cluster_arrive_relaxed();                      // this CTA runs and its mbarriers exist (fenced above)
 
   // The weights of a stable plan are older than the kernel before this one: their producer does not wait, and
   // leaves the signal to the warps that do (see launch_pdl).
@@ -213,8 +213,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   }
   __syncwarp();
   cluster_wait();                                // the others run
-  if constexpr (kTn) {                                 // and no longer need their stages
-    cluster_arrive();
+  if constexpr (kTn) {                                 // and no longer need their stages: their epilogue warps have seen the last MMA complete
+    cluster_arrive_relaxed();
     cluster_wait();
   }
 
@@ -355,7 +355,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 template <int BN, int C, bool kTn>
 int launch_split(TcDevice* dev, const CUtensorMap& map_a, const CUtensorMap& map_b, SplitParams P, cudaStream_t s) {
   CUtensorMap map_y;
-  if (P.transposed) map_y = map_a;                                   // (not used)
+  if (P.transposed || BN / C < 64) map_y = map_a;                    // (not used)
   else if (!make_map(&map_y, P.Y, P.cols, P.rows, P.ldy, kBlockM, kEpiCols)) return BSP_ERR_CUDA;
   constexpr int kStage = (kBlockM + BN) * kBlockK * 2;
   constexpr int kTail = 1024 + 160 + BN / C * 4 + 32;                // alignment slack, barriers, bias

@@ -501,12 +501,14 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
     tc::cluster_sync();
   }
   if (rank != 0) {
-    tc::cluster_sync();                                          // CTA 0 has read this CTA's list
+    tc::cluster_arrive_relaxed();
+    tc::cluster_wait();                                          // CTA 0 has read this CTA's list
     return;
   }
   // the next digit over the listed keys or all of them; then a warp ranks the few keys that are left, or the last
   // digit has bins of its own
   __syncthreads();
+  tc::cluster_arrive_relaxed();                                  // (the lists have been read: the other CTAs may leave)
   auto over_keys = [&](int above, uint32_t upper, auto f) {
     if (found != 0xffffffffu) {
       for (uint32_t i = threadIdx.x; i < found; i += kSelThreads)
@@ -542,7 +544,7 @@ select_kernel(const __grid_constant__ SelectBatchT<N> B) {
     p = pick_bin<kBins3>(hist + kBins2, p.want, s_sum, s_pick);
     if (threadIdx.x == 0) *J.out = threshold_of((prefix << kBits3) | p.bin);
   }
-  tc::cluster_sync();
+  tc::cluster_wait();
 }
 
 // ------------------------------------------------------------ select where counts do not fit 32 bits (select_large)
