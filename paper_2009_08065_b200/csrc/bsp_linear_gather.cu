@@ -264,6 +264,54 @@ __device__ __forceinline__ void mma_gather_stage(uint32_t d_tmem, uint64_t a_des
       : "memory");
 }
 
+// A 32-row piece of a TRANSPOSED output, [32 output rows][128 tokens].  The accumulator is read as 8 x 8 fragments (a lane
+// holds two neighbouring output rows of a token), which stmatrix stores transposed: four instructions a warp and piece
+// where the row-per-thread form of piece_store_transposed stores 32 16-bit values per thread.  The staging buffer is two
+// halves of 64 tokens with the 128-byte swizzle, so that the eight rows of a fragment fall on different banks.  The
+// epilogue of such a layer is bound by issue slots (58 % busy with four groups): 4096 x 1024 in 128-row blocks at 8x with
+// GELU, 8192 tokens, 32.6 -> 30.7 us.
+struct FragmentPiece {
+  uint32_t v[32];            // [16-token half][8 output rows: 4][token, token + 8 by two output rows]
+  uint32_t bias[4];          // of this lane's two rows of each 8
+};
+__device__ __forceinline__ void fragment_load(uint32_t taddr, uint32_t bias_smem, int lane, FragmentPiece& p) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(p.v[16 * h]), "=r"(p.v[16 * h + 1]), "=r"(p.v[16 * h + 2]), "=r"(p.v[16 * h + 3]), "=r"(p.v[16 * h + 4]),
+          "=r"(p.v[16 * h + 5]), "=r"(p.v[16 * h + 6]), "=r"(p.v[16 * h + 7]), "=r"(p.v[16 * h + 8]), "=r"(p.v[16 * h + 9]),
+          "=r"(p.v[16 * h + 10]), "=r"(p.v[16 * h + 11]), "=r"(p.v[16 * h + 12]), "=r"(p.v[16 * h + 13]), "=r"(p.v[16 * h + 14]),
+          "=r"(p.v[16 * h + 15])
+        : "r"(taddr + (static_cast<uint32_t>(16 * h) << 16))
+        : "memory");
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(p.bias[j]) : "r"(bias_smem + 16u * j + 4u * (lane & 3)));
+  tmem_load_wait();
+  tmem_loaded<32>(p.v);
+}
+__device__ __forceinline__ void fragment_store(const FragmentPiece& p, int act, uint32_t buf, int quad, int lane) {
+  // lane i of eight gives the address of output row 8 j + i; the four fragments of a store are the warp's 32 tokens
+  const uint32_t i = lane & 7, chunk = static_cast<uint32_t>((quad & 1) * 4 + (lane >> 3));
+  const uint32_t dst = buf + static_cast<uint32_t>(quad >> 1) * (kEpiStage / 2) + i * 128u + ((chunk ^ i) << 4);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const unsigned long long bias = pack_f32x2(__uint_as_float(p.bias[j] << 16), __uint_as_float(p.bias[j] & 0xffff0000u));
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t* v = &p.v[16 * (q >> 1) + 4 * j + 2 * (q & 1)];
+      float f0, f1;
+      unpack_f32x2(add_f32x2(pack_f32x2(__uint_as_float(v[0]), __uint_as_float(v[1])), bias), f0, f1);
+      if (act == BSP_ACT_GELU) gelu_erf_pair(f0, f1);
+      w[q] = pack_bf16x2(f0, f1);
+    }
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(dst + j * 1024u), "r"(w[0]), "r"(w[1]),
+                 "r"(w[2]), "r"(w[3]));
+  }
+}
+
 // Named barriers of the epilogue groups: 1 + g, and 5 + g with a vote.
 __device__ __forceinline__ void gather_group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory"); }
 // The 128 threads of an epilogue group agree on whether all of their waits succeeded; also
@@ -481,22 +529,39 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
         for (int c0 = 0; c0 < D; c0 += kEpiCols) {
           const uint32_t buf = buf0 + (piece_no % kBuffers) * kEpiStage;
           ++piece_no;
-          EpiloguePiece piece;
-          piece_load(taddr + c0, smem_u32(my_bias + c0), piece);
-          if (issuer) tma_store_wait_read<kBuffers - 1>();   // the store that last used this buffer has read it
-          gather_group_sync(group);
-          if (c0 + kEpiCols >= D) {               // this warp's last read of the accumulator
-            tcgen05_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty_bar(group));
+          auto acquire = [&] {                      // the buffer; and, after the last piece, the accumulator goes back
+            if (issuer) tma_store_wait_read<kBuffers - 1>();   // the store that last used this buffer has read it
+            gather_group_sync(group);
+            if (c0 + kEpiCols >= D) {
+              tcgen05_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(acc_empty_bar(group));
+            }
+          };
+          if (P.transposed) {
+            FragmentPiece piece;
+            fragment_load(taddr + c0, smem_u32(my_bias + c0), lane, piece);
+            acquire();
+            fragment_store(piece, P.act, buf, quad, lane);
+          } else {
+            EpiloguePiece piece;
+            piece_load(taddr + c0, smem_u32(my_bias + c0), piece);
+            acquire();
+            piece_store(piece, P.act, buf + static_cast<uint32_t>(row) * 64u, static_cast<uint32_t>((row >> 1) & 3));
           }
-          if (P.transposed) piece_store_transposed(piece, P.act, buf, row);
-          else piece_store(piece, P.act, buf + static_cast<uint32_t>(row) * 64u, static_cast<uint32_t>((row >> 1) & 3));
           fence_async_smem();
           gather_group_sync(group);
           if (issuer) {
-            if (P.transposed) tma_store_2d(&map_y, m * kBlockM, rb * D + c0, buf);
-            else tma_store_2d(&map_y, rb * D + c0, m * kBlockM, buf);
+            if (P.transposed) {
+              // (two boxes of 64 tokens, one bulk group; a tile may end within its first half)
+              if (m * kBlockM + 64 < P.tokens)
+                asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+                             ::"l"(reinterpret_cast<uint64_t>(&map_y)), "r"(m * kBlockM + 64), "r"(rb * D + c0), "r"(buf + kEpiStage / 2)
+                             : "memory");
+              tma_store_2d(&map_y, m * kBlockM, rb * D + c0, buf);
+            } else {
+              tma_store_2d(&map_y, rb * D + c0, m * kBlockM, buf);
+            }
           }
         }
       } else {
@@ -565,7 +630,7 @@ int launch_gather_groups(TcDevice* dev, const GatherParams& P, cudaStream_t s) {
   CUtensorMap map_y = map_xt;       // (blocks of 16 rows store without it)
   if (Cfg::kStaged) {
     if (P.transposed) {
-      if (!make_map(&map_y, P.Y, P.tokens, P.n_out, P.ldy, kEpiCols, kBlockM)) return BSP_ERR_CUDA;
+      if (!make_map(&map_y, P.Y, P.tokens, P.n_out, P.ldy, kEpiCols)) return BSP_ERR_CUDA;   // 64 tokens
     } else if (!make_map(&map_y, P.Y, P.n_out, P.tokens, P.ldy, kBlockM, kEpiCols)) {
       return BSP_ERR_CUDA;
     }

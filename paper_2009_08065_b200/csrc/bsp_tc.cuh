@@ -541,8 +541,9 @@ DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, i
 int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn, long long* ns = nullptr);
 int launch_linear_split(TcDevice* dev, int bn, int c, const void* plan, const void* X, void* Y, int tokens, int n_out, int k_in,
                         int act, const void* bias, int ldx, int ldy, bool plan_stable, bool transposed, cudaStream_t s);
-// How bsp_linear_gathered cuts a layer: runs of rb_per_chunk consecutive row-blocks x 128-token tiles, enough of them for
-// about six per SM, runs as long as that allows.
+// How bsp_linear_gathered cuts a layer: runs of rb_per_chunk consecutive row-blocks x 128-token tiles.  Runs as long as six
+// of them per SM allow, or shorter, down to half of that, where the busiest CTA then has fewer row-blocks (4096 outputs in
+// 128-row blocks, 8192 tokens: 15 in runs of three, 14 in runs of two).
 struct GatherUnits {
   int m_tiles, n_chunks, rb_per_chunk;
 };
@@ -552,8 +553,13 @@ inline GatherUnits gather_units(int tokens, int n_blocks, int sms) {
   int n_chunks = (6 * sms + u.m_tiles - 1) / u.m_tiles;
   if (n_chunks < 1) n_chunks = 1;
   if (n_chunks > n_blocks) n_chunks = n_blocks;
-  u.rb_per_chunk = (n_blocks + n_chunks - 1) / n_chunks;
-  u.n_chunks = (n_blocks + u.rb_per_chunk - 1) / u.rb_per_chunk;
+  const int longest = (n_blocks + n_chunks - 1) / n_chunks;
+  long long least = -1;
+  for (int run = longest; run >= 1 && 2 * run >= longest; --run) {
+    const int chunks = (n_blocks + run - 1) / run;
+    const long long busiest = (static_cast<long long>(u.m_tiles) * chunks + sms - 1) / sms * run;
+    if (least < 0 || busiest < least) { least = busiest; u.rb_per_chunk = run; u.n_chunks = chunks; }
+  }
   return u;
 }
 int launch_tn_split(TcDevice* dev, int bn, int c, const void* dY, int ldy, const void* X, int ldx, int tokens, int n_out, int k_in,
