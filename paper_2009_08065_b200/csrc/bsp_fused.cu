@@ -25,6 +25,7 @@ struct BatchT {
   float eps;
   int parts;                // stage 1 without flags: CTAs per row-block, each with part_chunks of its 8-column pieces
   int part_chunks;
+  int early;                // stage 1: CTAs that can be waiting for the previous kernel
   int first_block[N + 1];   // CTA index of each job's first row-block
   FusedJob job[N];
 };
@@ -52,6 +53,10 @@ fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
   const FusedJob& J = B.job[j];
   const int b = cta - B.first_block[j];
   const int q_end = kParts ? min(J.cols >> 3, q0 + B.part_chunks) : J.cols >> 3;
+  // (the rows of the CTAs that wait for the previous kernel, often a clearing one, come to L2 meanwhile: see prefetch_bytes)
+  if (static_cast<int>(blockIdx.x) < B.early)
+    for (int r = threadIdx.x; r < B.block; r += blockDim.x)
+      prefetch_bytes(J.W + (static_cast<size_t>(b) * B.block + r) * J.ldw + (q0 << 3), static_cast<uint32_t>(q_end - q0) * 16u);
   pdl_wait();
   pdl_launch_dependents();
   const bool want_flags = J.flags != nullptr;
@@ -350,6 +355,7 @@ int launch_stage1(const FusedJob* jobs, int n_jobs, int block, float eps, int sq
     B.parts = (chunks + 127) / 128;
     B.part_chunks = 128;
   }
+  B.early = 2 * sms;
   auto* kernel = block >= 32 && N == 1 ? (B.parts > 1 ? fused_stage1_kernel<N, N == 1, N == 1> : fused_stage1_kernel<N, false, N == 1>)
                                        : (B.parts > 1 ? fused_stage1_kernel<N, N == 1, false> : fused_stage1_kernel<N, false, false>);
   BSP_CUDA_TRY(launch_pdl(kernel, dim3(total * B.parts), dim3(threads), 0, s, B));
@@ -365,6 +371,7 @@ int launch_stage2(const FusedJob* jobs, int n_jobs, int block, cudaStream_t s) {
   B.squared = 0;
   B.parts = 1;
   B.part_chunks = 0;
+  B.early = 0;
   int splits = 1;
   size_t smem = 0;
   for (int i = 0; i < n_jobs; ++i) {
