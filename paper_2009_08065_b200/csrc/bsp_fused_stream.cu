@@ -113,8 +113,9 @@ __device__ __forceinline__ Item locate(const Batch& B, int item) {
   return I;
 }
 
-// Rows of an item into a shared-memory buffer, one bulk copy per row (called by one warp).
-template <class Batch>
+// Rows of an item into a shared-memory buffer, one bulk copy per row (called by one warp).  kPassing: they are not read
+// again where the layout is a matrix of its own, and leave L2 first.
+template <bool kPassing, class Batch>
 __device__ __forceinline__ void issue_rows(const Batch& B, const Item& I, uint32_t dst, uint32_t bar, int lane) {
   const FusedJob& J = B.job[I.jn].j;
   const int d = B.block;
@@ -122,12 +123,30 @@ __device__ __forceinline__ void issue_rows(const Batch& B, const Item& I, uint32
   if (lane == 0) mbar_arrive_expect_tx(bar, row_bytes * static_cast<uint32_t>(d));
   __syncwarp();
   const uint16_t* wblk = J.W + static_cast<size_t>(I.b) * d * J.ldw + I.c0;
+  if (kPassing && J.plan != nullptr && J.plan != J.W) {
+    uint64_t first;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+    for (int r = lane; r < d; r += 32)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                   ::"r"(dst + static_cast<uint32_t>(r) * row_bytes),
+                     "l"(reinterpret_cast<uint64_t>(wblk + static_cast<size_t>(r) * J.ldw)), "r"(row_bytes), "r"(bar), "l"(first)
+                   : "memory");
+    return;
+  }
   for (int r = lane; r < d; r += 32) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst + static_cast<uint32_t>(r) * row_bytes),
                    "l"(reinterpret_cast<uint64_t>(wblk + static_cast<size_t>(r) * J.ldw)), "r"(row_bytes), "r"(bar)
                  : "memory");
   }
+}
+
+// A store of an output that this launch does not read again.  The ticket variant's outputs (twice the weights and more) leave
+// L2 ahead of the weights that are still to be read, which the percentile's sums often left there.
+template <bool kPassing, class T>
+__device__ __forceinline__ void put(T* p, T v) {
+  if (kPassing) __stcs(p, v);
+  else *p = v;
 }
 
 // Published word of an item as it is now (ready bit set or not).
@@ -214,7 +233,8 @@ __global__ void __launch_bounds__(kStreamThreads, 8)
 fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
   extern __shared__ __align__(128) uint8_t s_raw[];
   __shared__ __align__(8) uint64_t s_bar;
-  __shared__ int s_item;
+  __shared__ Item s_item;
+  __shared__ int s_ticket;
   __shared__ int s_cnt[8];
   __shared__ double s_pen[8];
   __shared__ int s_warp[32];
@@ -245,7 +265,7 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
     // One wave: the rows are asked for before the wait for the clearing kernel.  That kernel is an
     // ordinary launch, so whatever wrote W earlier in the stream had finished before it began, and
     // this grid was started after that; only the published counts depend on the clearing itself.
-    if (direct) issue_rows(B, I, smem_u32(s_raw), bar, lane);
+    if (direct) issue_rows<false>(B, I, smem_u32(s_raw), bar, lane);
   }
   if (threadIdx.x == 0) {
     // launched with programmatic stream serialization: everything above overlapped the clearing
@@ -261,12 +281,12 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
         const unsigned long long t0 = tc::global_timer_ns();
         while (tc::global_timer_ns() - t0 < delay) __nanosleep(100);
       }
-      s_item = atomicAdd(B.ticket, 1);
+      s_ticket = atomicAdd(B.ticket, 1);
     }
   }
   __syncthreads();
   if (!direct) {
-    item = s_item;
+    item = s_ticket;
     if (item >= B.total_items) return;
     I = locate(B, item);
   }
@@ -276,7 +296,7 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
   // counter overlaps those writes.
   uint32_t parity = 0u;
   for (;;) {
-    if (warp == 0 && !direct) issue_rows(B, I, smem_u32(s_raw), bar, lane);
+    if (warp == 0 && !direct) issue_rows<!kOneWave>(B, I, smem_u32(s_raw), bar, lane);
     const StreamJob& O = B.job[I.jn];
     const FusedJob& J = O.j;
     const int b = I.b, q = I.q, c0 = I.c0, pc = I.pc, local = I.local;
@@ -303,20 +323,11 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
     const bool in_place = J.plan != nullptr && J.plan == J.W;
     int changes = 0;                         // in-place mode: a pruned group that still holds a non-zero weight
     for (int k = threadIdx.x; k < chunks; k += blockDim.x) {
-      float acc[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+      SumSq8 sums;
 #pragma unroll 4
-      for (int r = 0; r < d; ++r) {
-        const uint4 v = *reinterpret_cast<const uint4*>(s_w + r * pc + (k << 3));
-        const uint32_t w32[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float lo = __uint_as_float(w32[i] << 16), hi = __uint_as_float(w32[i] & 0xffff0000u);
-          acc[2 * i] = __fmaf_rn(lo, lo, acc[2 * i]);
-          acc[2 * i + 1] = __fmaf_rn(hi, hi, acc[2 * i + 1]);
-        }
-      }
+      for (int r = 0; r < d; ++r) sums.add(*reinterpret_cast<const uint4*>(s_w + r * pc + (k << 3)));
+      float acc[8];
+      sums.get(acc);
       uint32_t lo = 0, hi = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -339,12 +350,12 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
           fresh[i] = reciprocal(base[i] + B.eps);
         }
         if (J.norms) {
-          *reinterpret_cast<float4*>(J.norms + g0) = make_float4(n[0], n[1], n[2], n[3]);
-          *reinterpret_cast<float4*>(J.norms + g0 + 4) = make_float4(n[4], n[5], n[6], n[7]);
+          put<!kOneWave>(reinterpret_cast<float4*>(J.norms + g0), make_float4(n[0], n[1], n[2], n[3]));
+          put<!kOneWave>(reinterpret_cast<float4*>(J.norms + g0 + 4), make_float4(n[4], n[5], n[6], n[7]));
         }
         if (J.gamma_out) {
-          *reinterpret_cast<float4*>(J.gamma_out + g0) = make_float4(fresh[0], fresh[1], fresh[2], fresh[3]);
-          *reinterpret_cast<float4*>(J.gamma_out + g0 + 4) = make_float4(fresh[4], fresh[5], fresh[6], fresh[7]);
+          put<!kOneWave>(reinterpret_cast<float4*>(J.gamma_out + g0), make_float4(fresh[0], fresh[1], fresh[2], fresh[3]));
+          put<!kOneWave>(reinterpret_cast<float4*>(J.gamma_out + g0 + 4), make_float4(fresh[4], fresh[5], fresh[6], fresh[7]));
         }
         if (want_pen) {
           if (J.gamma_in) {
@@ -393,24 +404,26 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
         if (bit) s_idx[p++] = static_cast<uint16_t>((k << 3) + i);
       }
     }
-    // execution layout: the rows with the pruned columns zeroed, one warp per row, 16-byte stores.
+    // execution layout: the rows with the pruned columns zeroed, a warp every n_warps-th row, 16-byte stores; the masks of a
+    // lane's eight columns are made once for all of its rows.
     // When the job's plan IS its W (in-place mode, Algorithm 2's W = W * Mask), only 8-column pieces
     // that hold a weight of a pruned group are written: W read once, and written only where it changes
     // (an item whose pruned groups are all zero already skips the pass).
     if (J.plan != nullptr && (!in_place || rewrite)) {
       const size_t pld = in_place ? static_cast<size_t>(J.ldw) : static_cast<size_t>(J.cols);
-      for (int r = warp; r < d; r += n_warps) {
-        uint16_t* pdst = J.plan + (static_cast<size_t>(b) * d + r) * pld + c0;
-        for (int k = lane; k < chunks; k += 32) {
-          const uint4 w = *reinterpret_cast<const uint4*>(s_w + r * pc + (k << 3));
-          const uint2 f = *reinterpret_cast<const uint2*>(s_flag + (k << 3));
-          uint4 m;   // a flag byte is 0 or 1: flag * 0xffff masks the matching 16-bit element
-          m.x = w.x & (((f.x & 0xffu) * 0xffffu) | (((f.x >> 8) & 0xffu) * 0xffff0000u));
-          m.y = w.y & ((((f.x >> 16) & 0xffu) * 0xffffu) | (((f.x >> 24) & 0xffu) * 0xffff0000u));
-          m.z = w.z & (((f.y & 0xffu) * 0xffffu) | (((f.y >> 8) & 0xffu) * 0xffff0000u));
-          m.w = w.w & ((((f.y >> 16) & 0xffu) * 0xffffu) | (((f.y >> 24) & 0xffu) * 0xffff0000u));
-          if (!in_place || ((m.x ^ w.x) | (m.y ^ w.y) | (m.z ^ w.z) | (m.w ^ w.w)) != 0u)
-            *reinterpret_cast<uint4*>(pdst + (k << 3)) = m;
+      uint16_t* pblk = J.plan + static_cast<size_t>(b) * d * pld + c0;
+      for (int k = lane; k < chunks; k += 32) {
+        const uint2 f = *reinterpret_cast<const uint2*>(s_flag + (k << 3));
+        const uint32_t lo = f.x * 0xffu, hi = f.y * 0xffu;     // a flag byte is 0 or 1: 0 or 0xff
+        const uint4 mask = make_uint4(__byte_perm(lo, 0u, 0x1100), __byte_perm(lo, 0u, 0x3322), __byte_perm(hi, 0u, 0x1100),
+                                      __byte_perm(hi, 0u, 0x3322));
+        const uint16_t* src = s_w + warp * pc + (k << 3);
+        uint16_t* dst = pblk + static_cast<size_t>(warp) * pld + (k << 3);
+#pragma unroll 4
+        for (int r = warp; r < d; r += n_warps, src += n_warps * pc, dst += n_warps * pld) {
+          const uint4 w = *reinterpret_cast<const uint4*>(src);
+          const uint4 m = make_uint4(w.x & mask.x, w.y & mask.y, w.z & mask.z, w.w & mask.w);
+          if (!in_place || ((m.x ^ w.x) | (m.y ^ w.y) | (m.z ^ w.z) | (m.w ^ w.w)) != 0u) put<!kOneWave>(reinterpret_cast<uint4*>(dst), m);
         }
       }
     }
@@ -517,9 +530,9 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
     }
     // no wait from here on: take the next item (the answer is only looked at after the writes below)
     int next_item = 0;
-    if (!direct && threadIdx.x == 0) next_item = atomicAdd(B.ticket, 1);
+    if (!direct && warp == n_warps - 1 && lane == 0) next_item = atomicAdd(B.ticket, 1);
     if (kc > 0) {
-      for (int p = threadIdx.x; p < kc; p += blockDim.x) J.idx[base + p] = c0 + s_idx[p];
+      for (int p = threadIdx.x; p < kc; p += blockDim.x) put<!kOneWave>(J.idx + base + p, static_cast<int32_t>(c0 + s_idx[p]));
       // packed tile: row r of the block occupies vals[tile0 + r*kc_block, +kc_block); this part fills
       // positions [off_in_block, off_in_block + kc) of every row.
       const long long tile0 = static_cast<long long>(d) * block_base;
@@ -570,7 +583,7 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const int rr = r + u * n_warps;
-              if (rr < d) o[static_cast<size_t>(rr) * row_words] = w[u];
+              if (rr < d) put<!kOneWave>(o + static_cast<size_t>(rr) * row_words, w[u]);
             }
           }
         }
@@ -588,11 +601,18 @@ fused_stream_kernel(const __grid_constant__ StreamBatchT<N> B) {
       }
     }
     if (direct) break;
-    if (threadIdx.x == 0) s_item = next_item;
-    __syncthreads();                         // everybody is done with the row buffer and the lists; s_item is there
-    item = s_item;
+    if (warp == n_warps - 1) {               // one warp looks the next item up for all of them
+      next_item = __shfl_sync(0xffffffffu, next_item, 0);
+      if (next_item < B.total_items) {
+        const Item next = locate(B, next_item);
+        if (lane == 0) s_item = next;
+      }
+      if (lane == 0) s_ticket = next_item;
+    }
+    __syncthreads();                         // everybody is done with the row buffer and the lists; the next item is there
+    item = s_ticket;
     if (item >= B.total_items) break;
-    I = locate(B, item);
+    I = s_item;
     parity ^= 1u;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the buffer's readers are done before the copies write it
   }

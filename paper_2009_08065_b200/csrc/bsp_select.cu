@@ -213,20 +213,11 @@ sums_stream_kernel(const __grid_constant__ SelectBatchT<N> B) {
     const uint16_t* s_w = reinterpret_cast<const uint16_t*>(s_raw + static_cast<size_t>(slot) * buf_bytes);
     const bool count = J.head != nullptr;
     for (int k = threadIdx.x; k < (pc >> 3); k += kSumThreads) {
-      float acc[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+      SumSq8 sums;
 #pragma unroll 8
-      for (int r = 0; r < d; ++r) {                           // rows in increasing order: the defined decision quantity
-        const uint4 v = *reinterpret_cast<const uint4*>(s_w + r * pc + (k << 3));
-        const uint32_t w32[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float lo = __uint_as_float(w32[i] << 16), hi = __uint_as_float(w32[i] & 0xffff0000u);
-          acc[2 * i] = __fmaf_rn(lo, lo, acc[2 * i]);
-          acc[2 * i + 1] = __fmaf_rn(hi, hi, acc[2 * i + 1]);
-        }
-      }
+      for (int r = 0; r < d; ++r) sums.add(*reinterpret_cast<const uint4*>(s_w + r * pc + (k << 3)));   // rows in increasing order: the defined decision quantity
+      float acc[8];
+      sums.get(acc);
       float4* dst = reinterpret_cast<float4*>(J.S + static_cast<size_t>(b) * J.cols + c0 + (k << 3));
       dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
       dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
