@@ -331,27 +331,32 @@ struct SumSq8 {
 // save registers (54 instead of 92 here), which makes several trips to memory of one; a barrier of the warp keeps the loads
 // ahead of it.  Norms of the matrices of a 1024-wide layer, in an iteration of reweighted training: 24.5 -> 20.8 us, the
 // iteration 106.2 -> 102.5.  Not in kernels whose threads have 32 to 40 registers (the keep-count select: spills).
-template <int ROWS, bool kTogether>
+// kPast: the rows are not kept in L1.
+template <int ROWS, bool kTogether, bool kPast>
 __device__ __forceinline__ void sumsq8_rows(const uint16_t* p, int ldw, SumSq8& acc) {
   uint4 v[ROWS];
 #pragma unroll
-  for (int u = 0; u < ROWS; ++u) v[u] = ld_global(reinterpret_cast<const uint4*>(p + static_cast<size_t>(u) * ldw));
+  for (int u = 0; u < ROWS; ++u) {
+    const uint4* src = reinterpret_cast<const uint4*>(p + static_cast<size_t>(u) * ldw);
+    if (kPast) asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[u].x), "=r"(v[u].y), "=r"(v[u].z), "=r"(v[u].w) : "l"(src) : "memory");
+    else v[u] = ld_global(src);
+  }
   if (kTogether && ROWS > 1) __syncwarp(__activemask());
 #pragma unroll
   for (int u = 0; u < ROWS; ++u) acc.add(v[u]);     // rows in increasing order: the chains stay sequential
 }
 // kTall: 32 rows in flight instead of 16, for blocks of 32 rows and more (such a matrix has few of them, and a thread's
 // rows are a chain of trips to memory; not for the others, since it takes 156 registers).
-template <bool kTall = false, bool kTogether = true>
+template <bool kTall = false, bool kTogether = true, bool kPast = false>
 __device__ __forceinline__ void sumsq8(const uint16_t* p, int d, int ldw, float (&acc)[8]) {
   SumSq8 sums;
   int r = 0;
   if (kTall)
-    for (; r + 32 <= d; r += 32) sumsq8_rows<32, kTogether>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 512 bytes in flight
-  for (; r + 16 <= d; r += 16) sumsq8_rows<16, kTogether>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 256 bytes in flight
-  if (!kTall && r + 8 <= d) { sumsq8_rows<8, kTogether>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 8; }
-  for (; r + 4 <= d; r += 4) sumsq8_rows<4, kTogether>(p + static_cast<size_t>(r) * ldw, ldw, sums);
-  for (; r < d; ++r) sumsq8_rows<1, kTogether>(p + static_cast<size_t>(r) * ldw, ldw, sums);
+    for (; r + 32 <= d; r += 32) sumsq8_rows<32, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 512 bytes in flight
+  for (; r + 16 <= d; r += 16) sumsq8_rows<16, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 256 bytes in flight
+  if (!kTall && r + 8 <= d) { sumsq8_rows<8, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 8; }
+  for (; r + 4 <= d; r += 4) sumsq8_rows<4, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);
+  for (; r < d; ++r) sumsq8_rows<1, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);
   sums.get(acc);
 }
 
