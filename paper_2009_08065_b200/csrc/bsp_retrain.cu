@@ -115,16 +115,16 @@ masked_adam_kernel(AdamArgs A) {
 // the block's index list (2 bytes per entry) in shared memory, 16 bytes per load with all of a thread's loads
 // in flight (at the usual rates every 32-byte sector of a row holds a kept column, so whole rows are read
 // anyway), and gathers from there, two positions per 4-byte store.  HBM-bound in total, latency-bound per
-// matrix: four rows per CTA give a 768 x 768 matrix 192 CTAs, and the list travels beside the rows.  12 layers of four
+// matrix: up to four rows per CTA, fewer where there would be less than two CTAs per SM, and the list travels beside the rows.  12 layers of four
 // matrices, on average: 5.3 us gathering from global memory, 2.9 us.
 constexpr int kRepackRows = 4, kRepackThreads = 256, kRepackLoads = 6, kRepackMaxCols = 3072;
 __global__ void __launch_bounds__(kRepackThreads)
-repack_vec_kernel(const uint16_t* W, int cols, int ldw, int block, const int32_t* blk_ptr,
+repack_vec_kernel(const uint16_t* W, int cols, int ldw, int block, int rows_per, const int32_t* blk_ptr,
                   const int32_t* idx, uint16_t* vals) {
-  extern __shared__ __align__(16) uint16_t s_rows[];             // [kRepackRows][cols], then the list [cols]
-  const int b = blockIdx.x, r_lo = blockIdx.y * kRepackRows, n_rows = min(kRepackRows, block - r_lo);
+  extern __shared__ __align__(16) uint16_t s_rows[];             // [rows_per][cols], then the list [cols]
+  const int b = blockIdx.x, r_lo = blockIdx.y * rows_per, n_rows = min(rows_per, block - r_lo);
   const int chunks = cols >> 3;
-  uint16_t* s_list = s_rows + kRepackRows * cols;
+  uint16_t* s_list = s_rows + rows_per * cols;
   if (threadIdx.x == 0) prefetch_line(blk_ptr + b);
   if (static_cast<int>(threadIdx.x) < n_rows)
     prefetch_bytes(W + (static_cast<size_t>(b) * block + r_lo + threadIdx.x) * ldw, static_cast<uint32_t>(cols) * 2u);
@@ -285,13 +285,20 @@ extern "C" int bsp_repack_values(const void* W, int rows, int cols, int ldw, int
   if (grid.y > 65535) return BSP_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint16_t* w = static_cast<const uint16_t*>(W);
-  const size_t smem = static_cast<size_t>(cols) * (kRepackRows + 1) * 2;
   // Staged rows, where several CTAs fit an SM and have all of their rows.  Behind the Adam step, staged / gathered from
   // global memory: 4096 x 1024 in 16-row blocks 4.0 / 5.7 us, 768 x 3072 5.5 / 5.2, 8192 x 4096 49 / 26, 5344 x 920 in single
   // rows 11.2 / 10.2; 6042 x 2128 in pairs, by itself, 10.7 / 7.5.
   if (cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && cols <= kRepackMaxCols && block >= kRepackRows) {
-    BSP_CUDA_TRY(launch_pdl(repack_vec_kernel, grid, dim3(kRepackThreads), smem, s, w, cols, ldw, block, blk_ptr, idx,
-                            static_cast<uint16_t*>(vals)));
+    // Two CTAs per SM, or rows of their own: between the Adam steps of a stack (768 x 768 and 768 x 3072 have 192 CTAs of four
+    // rows) a call is then bound by half as long a chain of loads and stores.  Retraining 12 layers of 768 features 617 -> 601
+    // us, five of 400 in 8-row blocks 131 -> 127; single rows for every matrix 660, two 616.
+    int sms = 0;
+    BSP_TRY(sm_count(&sms));
+    int rows_per = kRepackRows;
+    while (rows_per > 1 && static_cast<long long>(nb) * ((block + rows_per - 1) / rows_per) < 2LL * sms) rows_per >>= 1;
+    const dim3 pieces(nb, (block + rows_per - 1) / rows_per);
+    BSP_CUDA_TRY(launch_pdl(repack_vec_kernel, pieces, dim3(kRepackThreads), static_cast<size_t>(cols) * (rows_per + 1) * 2, s, w, cols, ldw,
+                            block, rows_per, blk_ptr, idx, static_cast<uint16_t*>(vals)));
   } else {
     BSP_CUDA_TRY(launch_pdl(repack_kernel, grid, dim3(256), 0, s, w, ldw, block, blk_ptr, idx, static_cast<uint16_t*>(vals)));
   }
