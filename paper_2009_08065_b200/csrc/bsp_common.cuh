@@ -327,13 +327,38 @@ struct SumSq8 {
     for (int i = 0; i < 4; ++i) asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[2 * i]), "=f"(acc[2 * i + 1]) : "l"(pair[i]));
   }
 };
+// The same without register pairs, for kernels whose threads have 32 to 40 registers (the keep-count select would spill).
+struct SumSq8Few {
+  float acc8[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  __device__ __forceinline__ void add(const uint4& v) {
+    const uint32_t w32[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float lo = __uint_as_float(w32[i] << 16), hi = __uint_as_float(w32[i] & 0xffff0000u);
+      acc8[2 * i] = __fmaf_rn(lo, lo, acc8[2 * i]);
+      acc8[2 * i + 1] = __fmaf_rn(hi, hi, acc8[2 * i + 1]);
+    }
+  }
+  __device__ __forceinline__ void get(float (&acc)[8]) const {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = acc8[i];
+  }
+};
+template <bool kTogether>
+struct SumSq8Of {
+  using type = SumSq8;
+};
+template <>
+struct SumSq8Of<false> {
+  using type = SumSq8Few;
+};
 // kTogether: every load is issued before the first is used.  Left to itself the compiler interleaves loads and arithmetic to
 // save registers (54 instead of 92 here), which makes several trips to memory of one; a barrier of the warp keeps the loads
 // ahead of it.  Norms of the matrices of a 1024-wide layer, in an iteration of reweighted training: 24.5 -> 20.8 us, the
-// iteration 106.2 -> 102.5.  Not in kernels whose threads have 32 to 40 registers (the keep-count select: spills).
+// iteration 106.2 -> 102.5.  Not in kernels of few registers.
 // kPast: the rows are not kept in L1.
 template <int ROWS, bool kTogether, bool kPast>
-__device__ __forceinline__ void sumsq8_rows(const uint16_t* p, int ldw, SumSq8& acc) {
+__device__ __forceinline__ void sumsq8_rows(const uint16_t* p, int ldw, typename SumSq8Of<kTogether>::type& acc) {
   uint4 v[ROWS];
 #pragma unroll
   for (int u = 0; u < ROWS; ++u) {
@@ -349,7 +374,7 @@ __device__ __forceinline__ void sumsq8_rows(const uint16_t* p, int ldw, SumSq8& 
 // rows are a chain of trips to memory; not for the others, since it takes 156 registers).
 template <bool kTall = false, bool kTogether = true, bool kPast = false>
 __device__ __forceinline__ void sumsq8(const uint16_t* p, int d, int ldw, float (&acc)[8]) {
-  SumSq8 sums;
+  typename SumSq8Of<kTogether>::type sums;
   int r = 0;
   if (kTall)
     for (; r + 32 <= d; r += 32) sumsq8_rows<32, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 512 bytes in flight
