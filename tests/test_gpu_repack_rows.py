@@ -12,7 +12,8 @@ from gpu_util import DEV, bits_of, to_dev
 pytestmark = pytest.mark.gpu
 
 
-# 1, 3 and 30 row-blocks: single rows; 40 of 16 rows and 75 of 5: pairs; 100 of 16, 200 of 7 and 300 of 4: four rows
+# at 3072 columns 1, 3 and 30 row-blocks: single rows; 40 of 16 rows and 75 of 5: pairs; 100 of 16, 200 of 7 and 300 of 4: four
+# rows, as for narrower matrices
 @pytest.mark.parametrize("blocks,block", [(1, 16), (3, 5), (30, 4), (40, 16), (75, 5), (100, 16), (200, 7), (300, 4)])
 @pytest.mark.parametrize("cols,kept", [(8, 3), (264, 88), (3072, 771)])
 def test_repack_by_rows_per_cta(blocks, block, cols, kept):
