@@ -57,6 +57,7 @@ struct GatherCfg {
   static constexpr int kStageB = D * 128;                       // d rows of 64 bf16
   static constexpr int kStage = kGStageA + kStageB;
   static constexpr bool kStaged = D >= kEpiCols;                // outputs leave through staging buffers and TMA stores
+  static constexpr bool kFragments = GROUPS == 4;               // transposed pieces by fragments (see FragmentPiece)
   static constexpr int kStaging = kStaged ? kEpiBytes : 0;     // four buffers, shared out among the groups
   static constexpr int kFixed = 1024 /*alignment slack*/ + 512 /*barriers, stage bytes*/ + GROUPS * D * 2 /*bias, a block per group*/ + kStaging;
   static constexpr int kStagesRaw = (kSmemLimit - kFixed) / kStage;
@@ -269,7 +270,8 @@ __device__ __forceinline__ void mma_gather_stage(uint32_t d_tmem, uint64_t a_des
 // where the row-per-thread form of piece_store_transposed stores 32 16-bit values per thread.  The staging buffer is two
 // halves of 64 tokens with the 128-byte swizzle, so that the eight rows of a fragment fall on different banks.  The
 // epilogue of such a layer is bound by issue slots (58 % busy with four groups): 4096 x 1024 in 128-row blocks at 8x with
-// GELU, 8192 tokens, 32.6 -> 30.7 us.
+// GELU, 8192 tokens, 32.6 -> 30.7 us.  With two groups, which are not, a piece by itself takes longer (336 tokens, two linears
+// of 896 features: 15.5 -> 15.7 us).
 struct FragmentPiece {
   uint32_t v[32];            // [16-token half][8 output rows: 4][token, token + 8 by two output rows]
   uint32_t bias[4];          // of this lane's two rows of each 8
@@ -538,7 +540,7 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
               if (lane == 0) mbar_arrive(acc_empty_bar(group));
             }
           };
-          if (P.transposed) {
+          if (Cfg::kFragments && P.transposed) {
             FragmentPiece piece;
             fragment_load(taddr + c0, smem_u32(my_bias + c0), lane, piece);
             acquire();
@@ -547,14 +549,15 @@ linear_gather_kernel(const __grid_constant__ CUtensorMap map_xt, const __grid_co
             EpiloguePiece piece;
             piece_load(taddr + c0, smem_u32(my_bias + c0), piece);
             acquire();
-            piece_store(piece, P.act, buf + static_cast<uint32_t>(row) * 64u, static_cast<uint32_t>((row >> 1) & 3));
+            if (!Cfg::kFragments && P.transposed) piece_store_transposed(piece, P.act, buf, row);
+            else piece_store(piece, P.act, buf + static_cast<uint32_t>(row) * 64u, static_cast<uint32_t>((row >> 1) & 3));
           }
           fence_async_smem();
           gather_group_sync(group);
           if (issuer) {
             if (P.transposed) {
               // (two boxes of 64 tokens, one bulk group; a tile may end within its first half)
-              if (m * kBlockM + 64 < P.tokens)
+              if (Cfg::kFragments && m * kBlockM + 64 < P.tokens)
                 asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
                              ::"l"(reinterpret_cast<uint64_t>(&map_y)), "r"(m * kBlockM + 64), "r"(rb * D + c0), "r"(buf + kEpiStage / 2)
                              : "memory");
@@ -630,7 +633,7 @@ int launch_gather_groups(TcDevice* dev, const GatherParams& P, cudaStream_t s) {
   CUtensorMap map_y = map_xt;       // (blocks of 16 rows store without it)
   if (Cfg::kStaged) {
     if (P.transposed) {
-      if (!make_map(&map_y, P.Y, P.tokens, P.n_out, P.ldy, kEpiCols)) return BSP_ERR_CUDA;   // 64 tokens
+      if (!make_map(&map_y, P.Y, P.tokens, P.n_out, P.ldy, kEpiCols, Cfg::kFragments ? 64 : kBlockM)) return BSP_ERR_CUDA;
     } else if (!make_map(&map_y, P.Y, P.n_out, P.tokens, P.ldy, kBlockM, kEpiCols)) {
       return BSP_ERR_CUDA;
     }

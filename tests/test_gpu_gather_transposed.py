@@ -1,6 +1,7 @@
 """GPU parity of the gathering kernel's transposed output at the ends of its pieces: token counts within the first and the
-second 64 of a 128-token tile and on their edges, each block height, row-blocks that do not divide by a run.  Bit for bit
-the transpose of what the kernel writes otherwise."""
+second 64 of a 128-token tile and on their edges, each block height, row-blocks that do not divide by a run.  The last
+shapes, with GELU and many row-blocks, leave as fragments (four epilogue groups).  Bit for bit the transpose of what the
+kernel writes otherwise."""
 import pytest
 import torch
 
@@ -11,9 +12,12 @@ from gpu_util import DEV, to_dev
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d,n_out,k_in", [(32, 352, 264), (64, 960, 136), (128, 1408, 200)])
-@pytest.mark.parametrize("tokens", [8, 56, 64, 72, 128, 136, 1000])
-@pytest.mark.parametrize("act", [0, 1])
+SMALL = [(d, n, k, t, act) for d, n, k in ((32, 352, 264), (64, 960, 136), (128, 1408, 200))
+         for t in (8, 56, 64, 72, 128, 136, 1000) for act in (0, 1)]
+MANY = [(64, 2624, 72, 3720, 1), (64, 2624, 72, 3784, 1), (64, 2624, 136, 3776, 1), (128, 5248, 72, 3848, 1), (128, 5248, 72, 3904, 1)]
+
+
+@pytest.mark.parametrize("d,n_out,k_in,tokens,act", SMALL + MANY)
 def test_transposed_pieces(d, n_out, k_in, tokens, act):
     spec = si.LinearSpec(f"gt{d}", n_out, k_in, bool(act), 4.0, d)
     wp, _ = si.make_pruned_weight(93, spec)
