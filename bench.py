@@ -622,7 +622,7 @@ def other_workloads(device, peaks, args):
 
 
 TRAFFIC_PROFILE = os.path.join("profiles", "linear_tc_kernel_bert_base_T4096.md")
-TRAFFIC_SOURCES = ("paper_2009_08065_b200/csrc/bsp_linear_tc.cu", "paper_2009_08065_b200/csrc/bsp_tc.cuh")
+TRAFFIC_SOURCES = tuple("paper_2009_08065_b200/csrc/" + f for f in ("bsp_linear_tc.cu", "bsp_linear_tc2.cu", "bsp_tc.cuh"))
 
 
 def profiled_traffic():
@@ -854,7 +854,7 @@ def run_cuda(args):
             "gpu_launches": args.steps * sum(layer.weight_side_launches + k for k in range(n_lin + 1)),
             "clocks": clocks.summary(),
             "roofline": {
-                "kernel": "linear_tc_kernel (bsp_linear_planned_ex), the four launches of a step",
+                "kernel": "gemm_pair_kernel / linear_tc_kernel (bsp_linear_planned_ex), the four launches of a step",
                 "bound": "hbm" if hbm_binds else "tensor",
                 "achieved": round(ach_gbs if hbm_binds else ach_tf, 2),
                 "peak": hbm_peak if hbm_binds else peak, "unit": "GB/s" if hbm_binds else "TFLOP/s",
