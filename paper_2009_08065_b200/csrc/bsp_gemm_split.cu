@@ -98,18 +98,62 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   const int m0 = (tile / P.n_tiles) * kBlockM, n0 = (tile % P.n_tiles) * BN;
   const int quads = (min(kBlockM, P.rows - m0) + 31) >> 5;   // quarters of the tile with rows that exist
 
-  if (threadIdx.x == 0) {
-    *timed_out = 0u;
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
-    for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1); }
-    mbar_init(acc_bar, 1);
-    mbar_init(recv_bar, 1);
-    mbar_arrive_expect_tx(recv_bar, static_cast<uint32_t>((C - 1) * quads * 32 * W * 4));   // what the others will send
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 1) {
+  const int kb0 = static_cast<int>(static_cast<long long>(P.k_blocks) * rank / C);
+  const int kb1 = static_cast<int>(static_cast<long long>(P.k_blocks) * (rank + 1) / C);
+  const int ahead = min(S, kb1 - kb0);                 // stages that are filled without waiting for one to be free
+  auto load_a = [&](int kb, int stage) {
+    const uint32_t dst = smem_base + stage * kStage;
+    if constexpr (kTn) {
+      tma_stage_load(dst, &map_a, m0, kb * kBlockK, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
+      tma_load_2d_elect(dst + kAtomGroup, &map_a, m0 + 64, kb * kBlockK, full_bar(stage));
+    } else {
+      tma_stage_load(dst, &map_a, kb * kBlockK, m0, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
+    }
+  };
+  auto load_b = [&](int kb, int stage) {
+    const uint32_t dst = smem_base + stage * kStage + kStageA;
+    if constexpr (kTn) {
+      tma_stage_load(dst, &map_b, n0, kb * kBlockK, full_bar(stage), kStageB);
+#pragma unroll
+      for (int g = 1; g < BN / 64; ++g) tma_load_2d_elect(dst + g * kAtomGroup, &map_b, n0 + 64 * g, kb * kBlockK, full_bar(stage));
+    } else {
+      tma_stage_load(dst, &map_b, kb * kBlockK, n0, full_bar(stage), kStageB);
+    }
+  };
+
+  // The producers fill the first stages before the CTA meets: a cluster that found its SMs still taken by the kernel before
+  // starts late, and its set-up (0.5 us) would lie ahead of its first operands (four linears of 768 features with 8 tokens 14.5
+  // -> 14.1 us, an expansion and one linear with 128 tokens 6.47 -> 6.27).  The weights of a stable plan are older than
+  // the kernel before this one: their producer does not wait, and leaves the signal to the warps that do (see launch_pdl).
+  if (warp == 0) {
+    if (lane == 0) {
+      *timed_out = 0u;
+      for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1); }
+      mbar_init(acc_bar, 1);
+      mbar_init(recv_bar, 1);
+      mbar_arrive_expect_tx(recv_bar, static_cast<uint32_t>((C - 1) * quads * 32 * W * 4));   // what the others will send
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    asm volatile("bar.arrive 6, 64;" ::: "memory");    // the mbarriers exist
+    pdl_wait();
+    pdl_launch_dependents();
+    for (int i = 0; i < ahead; ++i) load_a(kb0 + i, i);
+  } else if (warp == 10) {
+    if (lane == 0) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_y)) : "memory");
+    }
+    __syncwarp();
+    asm volatile("bar.sync 6, 64;" ::: "memory");
+    if (!P.plan_stable) {
+      pdl_wait();
+      pdl_launch_dependents();
+    }
+    for (int i = 0; i < ahead; ++i) load_b(kb0 + i, i);
+  } else if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -118,49 +162,20 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_holder;
   cluster_arrive_relaxed();                      // this CTA runs and its mbarriers exist (fenced above)
-
-  // The weights of a stable plan are older than the kernel before this one: their producer does not wait, and
-  // leaves the signal to the warps that do (see launch_pdl).
-  if (!(P.plan_stable && warp == 10)) {
+  if (warp != 0 && warp != 10) {
     pdl_wait();
     pdl_launch_dependents();
   }
 
-  const int kb0 = static_cast<int>(static_cast<long long>(P.k_blocks) * rank / C);
-  const int kb1 = static_cast<int>(static_cast<long long>(P.k_blocks) * (rank + 1) / C);
-
-  if (warp == 0) {
-    // ---------------------------------------------------------------- TMA producer of the A tiles
-    int stage = 0;
-    uint32_t phase = 0;
+  if (warp == 0 || warp == 10) {
+    // ---------------------------------------------------------------- TMA producers of the A and the B tiles, further stages
+    int stage = ahead == S ? 0 : ahead;
+    uint32_t phase = ahead == S ? 1u : 0u;
     bool ok = true;
-    for (int kb = kb0; kb < kb1; ++kb) {
+    for (int kb = kb0 + ahead; kb < kb1; ++kb) {
       if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
-      const uint32_t dst = smem_base + stage * kStage;
-      if constexpr (kTn) {
-        tma_stage_load(dst, &map_a, m0, kb * kBlockK, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
-        tma_load_2d_elect(dst + kAtomGroup, &map_a, m0 + 64, kb * kBlockK, full_bar(stage));
-      } else {
-        tma_stage_load(dst, &map_a, kb * kBlockK, m0, full_bar(stage), static_cast<uint32_t>(P.a_bytes));
-      }
-      if (++stage == S) { stage = 0; phase ^= 1u; }
-    }
-    if (!ok && lane == 0) record_timeout(P.status, timed_out);
-  } else if (warp == 10) {
-    // ---------------------------------------------------------------- TMA producer of the B tiles
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int kb = kb0; kb < kb1; ++kb) {
-      if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, P.status)) { ok = false; break; }
-      const uint32_t dst = smem_base + stage * kStage + kStageA;
-      if constexpr (kTn) {
-        tma_stage_load(dst, &map_b, n0, kb * kBlockK, full_bar(stage), kStageB);
-#pragma unroll
-        for (int g = 1; g < BN / 64; ++g) tma_load_2d_elect(dst + g * kAtomGroup, &map_b, n0 + 64 * g, kb * kBlockK, full_bar(stage));
-      } else {
-        tma_stage_load(dst, &map_b, kb * kBlockK, n0, full_bar(stage), kStageB);
-      }
+      if (warp == 0) load_a(kb, stage);
+      else load_b(kb, stage);
       if (++stage == S) { stage = 0; phase ^= 1u; }
     }
     if (!ok && lane == 0) record_timeout(P.status, timed_out);
