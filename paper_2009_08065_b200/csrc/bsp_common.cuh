@@ -379,6 +379,9 @@ __device__ __forceinline__ void sumsq8(const uint16_t* p, int d, int ldw, float 
   if (kTall)
     for (; r + 32 <= d; r += 32) sumsq8_rows<32, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 512 bytes in flight
   for (; r + 16 <= d; r += 16) sumsq8_rows<16, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 256 bytes in flight
+  // (12 rows in one trip, not 8 and 4: pruning 768 x 768 in 12-row blocks 20.5 -> 20.1 us; 9 to 15 as far as they exist took 30
+  // registers more and 0.4 us of a layer's milestone)
+  if (kTogether && !kTall && r + 12 <= d) { sumsq8_rows<12, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 12; }
   if (!kTall && r + 8 <= d) { sumsq8_rows<8, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 8; }
   for (; r + 4 <= d; r += 4) sumsq8_rows<4, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);
   for (; r < d; ++r) sumsq8_rows<1, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);
