@@ -124,7 +124,9 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   // The producers fill the first stages before the CTA meets: a cluster that found its SMs still taken by the kernel before
   // starts late, and its set-up (0.5 us) would lie ahead of its first operands (four linears of 768 features with 8 tokens 14.5
   // -> 14.1 us, an expansion and one linear with 128 tokens 6.47 -> 6.27).  The weights of a stable plan are older than
-  // the kernel before this one: their producer does not wait, and leaves the signal to the warps that do (see launch_pdl).
+  // the kernel before this one: their producer does not wait (see launch_pdl).  The signal is left to the warp that allocates
+  // this CTA's tensor memory, behind the allocation: a dependent that sat down on this SM before it could take that memory
+  // first, and then wait for this grid while this CTA waits for the memory.
   if (warp == 0) {
     if (lane == 0) {
       *timed_out = 0u;
@@ -138,7 +140,6 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __syncwarp();
     asm volatile("bar.arrive 6, 64;" ::: "memory");    // the mbarriers exist
     pdl_wait();
-    pdl_launch_dependents();
     for (int i = 0; i < ahead; ++i) load_a(kb0 + i, i);
   } else if (warp == 10) {
     if (lane == 0) {
@@ -148,24 +149,20 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     }
     __syncwarp();
     asm volatile("bar.sync 6, 64;" ::: "memory");
-    if (!P.plan_stable) {
-      pdl_wait();
-      pdl_launch_dependents();
-    }
+    if (!P.plan_stable) pdl_wait();
     for (int i = 0; i < ahead; ++i) load_b(kb0 + i, i);
   } else if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    pdl_wait();
+    pdl_launch_dependents();
   }
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_holder;
   cluster_arrive_relaxed();                      // this CTA runs and its mbarriers exist (fenced above)
-  if (warp != 0 && warp != 10) {
-    pdl_wait();
-    pdl_launch_dependents();
-  }
+  if (warp > 1 && warp != 10) pdl_wait();
 
   if (warp == 0 || warp == 10) {
     // ---------------------------------------------------------------- TMA producers of the A and the B tiles, further stages

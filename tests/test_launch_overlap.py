@@ -51,6 +51,22 @@ def test_no_read_only_loads(file, name, params, body):
     assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", params), f"{file}: {name}"
 
 
+def test_tensor_memory_is_allocated_before_the_signal():
+    """A dependent grid that is let in before a CTA has its tensor memory could take that memory and then wait for the CTA."""
+    seen = set()
+    for file, name, _, body in kernels():
+        signal = re.search(r"pdl_launch_dependents|griddepcontrol\.launch_dependents", body)
+        if "tcgen05.alloc" not in body or signal is None:
+            continue
+        # behind the meeting of the warps that follows the allocation, or behind the allocation in the allocating warp itself
+        alloc = body.index("tcgen05.alloc")
+        between = body[alloc:signal.start()]
+        assert signal.start() > alloc and ("__syncthreads();" in between or "}" not in re.sub(r"\{[^{}]*\}", "", between)), f"{file}: {name}"
+        seen.add(name)
+    assert {"linear_tc_kernel", "gemm_pair_kernel", "gemm_split_kernel", "linear_gather_kernel", "gemm_tn_kernel",
+            "linear_chain_kernel"} <= seen
+
+
 def test_shared_helpers():
     src = strip_comments(open(os.path.join(CSRC, "bsp_common.cuh")).read())
     assert "__ldg(" not in src
