@@ -116,6 +116,18 @@ inline bool fused_shape_ok(const void* W, int rows, int cols, int ldw, int block
   return cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && cols <= kFusedMaxCols && rows / block <= kFusedMaxBlocks;
 }
 
+// Rows of one trip to memory (see sumsq8) for a launch of `ctas` CTAs that sum row-blocks of `block` rows, of which `per_sm16`
+// and `per_sm32` fit an SM with 16 and 32 rows in flight.  The longest trip while all CTAs run at once, with an eighth to
+// spare for those of the launch before; shorter ones where that leaves CTAs waiting for a seat, or where there are no rows
+// for it.  Norms, trips of 16 or 32 for all blocks / by this rule: 8192 x 3072 in single rows 77.7 / 42.2 us, in 8-row blocks
+// 17.6 / 14.2, in 32-row blocks 13.8 / 11.1; 768 x 3072 in 2-row blocks 5.2 / 3.6; percentile of 12 matrices of 512 x 512 in
+// 8-row blocks 11.2 / 9.8, of 40 of 512 x 64 in 32-row blocks 10.6 / 8.4.
+inline int rows_per_trip(int block, long long ctas, int per_sm16, int per_sm32, int sms) {
+  if (block < 8) return 4;
+  if (block >= 32 && ctas <= static_cast<long long>(sms) * per_sm32 * 7 / 8) return 32;
+  return ctas <= static_cast<long long>(sms) * per_sm16 * 7 / 8 ? 16 : 8;
+}
+
 // Widest vector load (in elements: 8, 4 or 1) that reads whole orientation-R groups: rows of `block`
 // contiguous elements starting at multiples of `block` in a row of leading dimension ldw.
 inline int contig_vec(const void* W, int ldw, int block) {
@@ -353,9 +365,9 @@ struct SumSq8Of<false> {
   using type = SumSq8Few;
 };
 // kTogether: every load is issued before the first is used.  Left to itself the compiler interleaves loads and arithmetic to
-// save registers (54 instead of 92 here), which makes several trips to memory of one; a barrier of the warp keeps the loads
-// ahead of it.  Norms of the matrices of a 1024-wide layer, in an iteration of reweighted training: 24.5 -> 20.8 us, the
-// iteration 106.2 -> 102.5.  Not in kernels of few registers.
+// save registers (54 instead of 90 here), which makes several trips to memory of one; a barrier of the warp keeps the loads
+// ahead of it (each thread names the threads that it is converged with, and they all come to it).  Norms of the matrices of a
+// 1024-wide layer, in an iteration of reweighted training: 24.5 -> 20.8 us, the iteration 106.2 -> 102.5.
 // kPast: the rows are not kept in L1.
 template <int ROWS, bool kTogether, bool kPast>
 __device__ __forceinline__ void sumsq8_rows(const uint16_t* p, int ldw, typename SumSq8Of<kTogether>::type& acc) {
@@ -370,19 +382,25 @@ __device__ __forceinline__ void sumsq8_rows(const uint16_t* p, int ldw, typename
 #pragma unroll
   for (int u = 0; u < ROWS; ++u) acc.add(v[u]);     // rows in increasing order: the chains stay sequential
 }
-// kTall: 32 rows in flight instead of 16, for blocks of 32 rows and more (such a matrix has few of them, and a thread's
-// rows are a chain of trips to memory; not for the others, since it takes 156 registers).
-template <bool kTall = false, bool kTogether = true, bool kPast = false>
+// kTrip: rows of one trip to memory, all of them in flight.  A row takes four registers, so a longer trip leaves fewer CTAs on
+// an SM: 4 rows 56 registers in the norms' kernel, 8 rows 64, 16 rows 90, 32 rows 156 (see rows_per_trip).  0: as the compiler
+// likes, for kernels of few registers.
+template <int kTrip, bool kPast = false>
 __device__ __forceinline__ void sumsq8(const uint16_t* p, int d, int ldw, float (&acc)[8]) {
+  constexpr bool kTogether = kTrip > 0;
+  constexpr int kMost = kTogether ? kTrip : 16;
   typename SumSq8Of<kTogether>::type sums;
   int r = 0;
-  if (kTall)
+  if (kMost >= 32)
     for (; r + 32 <= d; r += 32) sumsq8_rows<32, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 512 bytes in flight
-  for (; r + 16 <= d; r += 16) sumsq8_rows<16, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 256 bytes in flight
+  if (kMost >= 16)
+    for (; r + 16 <= d; r += 16) sumsq8_rows<16, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);   // 256 bytes in flight
   // (12 rows in one trip, not 8 and 4: pruning 768 x 768 in 12-row blocks 20.5 -> 20.1 us; 9 to 15 as far as they exist took 30
   // registers more and 0.4 us of a layer's milestone)
-  if (kTogether && !kTall && r + 12 <= d) { sumsq8_rows<12, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 12; }
-  if (!kTall && r + 8 <= d) { sumsq8_rows<8, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 8; }
+  if (kTogether && kMost == 16 && r + 12 <= d) { sumsq8_rows<12, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 12; }
+  if (kMost == 16 && r + 8 <= d) { sumsq8_rows<8, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums); r += 8; }
+  if (kMost == 8)
+    for (; r + 8 <= d; r += 8) sumsq8_rows<8, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);
   for (; r + 4 <= d; r += 4) sumsq8_rows<4, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);
   for (; r < d; ++r) sumsq8_rows<1, kTogether, kPast>(p + static_cast<size_t>(r) * ldw, ldw, sums);
   sums.get(acc);

@@ -42,8 +42,10 @@ __device__ __forceinline__ int find_job(const BatchT<N>& B, int cta) {
 }
 
 // (kParts as a template parameter: with the ranges as run-time values whole row-blocks took up to 2 us longer)
-template <int N, bool kParts, bool kTall>
-__global__ void __launch_bounds__(256)
+// Short blocks: 56 registers, which 288 threads of four CTAs leave, and not the 58 that the compiler would take: ten CTAs of 96
+// threads per SM instead of twelve made a second wave of 1536 (6144 x 768 in 4-row blocks 3.2 -> 3.7 us).
+template <int N, bool kParts, int kTrip>
+__global__ void __launch_bounds__(kTrip == 4 && !kParts ? 288 : 256, kTrip == 4 && !kParts ? 4 : 0)
 fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
   __shared__ int s_cnt[8];
   __shared__ double s_pen[8];
@@ -73,7 +75,7 @@ fused_stage1_kernel(const __grid_constant__ BatchT<N> B) {
   float pen = 0.0f;
   for (int q = q0 + threadIdx.x; q < q_end; q += blockDim.x) {
     float acc[8];
-    sumsq8<kTall>(J.W + static_cast<size_t>(b) * B.block * J.ldw + (q << 3), B.block, J.ldw, acc);
+    sumsq8<kTrip>(J.W + static_cast<size_t>(b) * B.block * J.ldw + (q << 3), B.block, J.ldw, acc);
     const size_t g0 = static_cast<size_t>(b) * J.cols + (q << 3);
     if (want_flags) {
       uint32_t lo = 0, hi = 0;
@@ -333,6 +335,12 @@ void fill_batch(BatchT<N>& B, const FusedJob* jobs, int n_jobs, int block, int* 
   B.first_block[n_jobs] = *total;
 }
 
+template <int N, bool kParts>
+auto* stage1_kernel(int trip) {
+  return trip == 4 ? fused_stage1_kernel<N, kParts, 4> : trip == 8 ? fused_stage1_kernel<N, kParts, 8>
+         : trip == 16 ? fused_stage1_kernel<N, kParts, 16> : fused_stage1_kernel<N, kParts, N == 1 ? 32 : 16>;
+}
+
 template <int N>
 int launch_stage1(const FusedJob* jobs, int n_jobs, int block, float eps, int squared, cudaStream_t s) {
   BatchT<N> B;
@@ -356,8 +364,10 @@ int launch_stage1(const FusedJob* jobs, int n_jobs, int block, float eps, int sq
     B.part_chunks = 128;
   }
   B.early = 2 * sms;
-  auto* kernel = block >= 32 && N == 1 ? (B.parts > 1 ? fused_stage1_kernel<N, N == 1, N == 1> : fused_stage1_kernel<N, false, N == 1>)
-                                       : (B.parts > 1 ? fused_stage1_kernel<N, N == 1, false> : fused_stage1_kernel<N, false, false>);
+  // (warps per SM: 21 with 16 rows in flight, 12 with 32)
+  const int warps = threads / 32;
+  const int trip = rows_per_trip(block, static_cast<long long>(total) * B.parts, 21 / warps, N == 1 ? 12 / warps : 0, sms);
+  auto* kernel = B.parts > 1 ? stage1_kernel<N, N == 1>(trip) : stage1_kernel<N, false>(trip);
   BSP_CUDA_TRY(launch_pdl(kernel, dim3(total * B.parts), dim3(threads), 0, s, B));
   return BSP_OK;
 }

@@ -138,7 +138,7 @@ flags_topk_kernel(const uint16_t* W, Geometry G, int keep_count,
   if (G.orient == BSP_ORIENT_C && G.vec == 8) {
     for (int q = threadIdx.x; q < (n >> 3); q += T) {
       float acc[8];
-      sumsq8<false, false>(W + static_cast<size_t>(b) * G.block * G.ldw + (q << 3), G.block, G.ldw, acc);
+      sumsq8<0>(W + static_cast<size_t>(b) * G.block * G.ldw + (q << 3), G.block, G.ldw, acc);
 #pragma unroll
       for (int i = 0; i < 8; ++i) s_key[(q << 3) + i] = __float_as_uint(acc[i]);
     }

@@ -122,7 +122,7 @@ grad_c_vec8_kernel(GradArgs A) {
     for (int i = 0; i < 8; ++i) factor[i] = 2.0f * A.scale * gam[i];
   } else {
     float acc[8];
-    sumsq8(p, A.block, A.ldw, acc);
+    sumsq8<16>(p, A.block, A.ldw, acc);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float n = __fsqrt_rn(acc[i]);

@@ -98,7 +98,7 @@ __device__ __forceinline__ void add_bins(const uint32_t* hist, uint32_t* head) {
 // wait for the zeros.  A warp of its own waits early and lets the select take its seats.
 // Orientation C, one CTA per row-block of every matrix, or per column range of one.
 // (kParts as a template parameter: with the ranges as run-time values whole row-blocks took up to 2 us longer)
-template <int N, bool kParts, bool kTall>
+template <int N, bool kParts, int kTrip>
 __global__ void __launch_bounds__(kSumThreads + 32)
 sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
   __shared__ __align__(16) uint32_t hist[kBins1];
@@ -119,7 +119,7 @@ sums_c_kernel(const __grid_constant__ SelectBatchT<N> B) {
   } else if (J.vec) {
     for (int q = (c0 >> 3) + threadIdx.x; q < (c_end >> 3); q += kSumThreads) {
       float acc[8];
-      sumsq8<kTall>(wblk + (q << 3), B.block, J.ldw, acc);
+      sumsq8<kTrip>(wblk + (q << 3), B.block, J.ldw, acc);
       float4* dst = reinterpret_cast<float4*>(out + (q << 3));
       dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
       dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
@@ -271,7 +271,7 @@ sums_flat_kernel(const __grid_constant__ SelectBatchT<N> B) {
       if (c < all) {
         const int b = c / chunks, k = c - b * chunks;
         float acc[8];
-        sumsq8<false, true, kPast>(J.W + static_cast<size_t>(b) * B.block * J.ldw + (k << 3), B.block, J.ldw, acc);
+        sumsq8<16, kPast>(J.W + static_cast<size_t>(b) * B.block * J.ldw + (k << 3), B.block, J.ldw, acc);
         float4* dst = reinterpret_cast<float4*>(J.S + static_cast<size_t>(c) * 8);
         dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
         dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
@@ -734,6 +734,12 @@ int launch_select(const SelectBatchT<N>& B, int sms, cudaStream_t s) {
   return BSP_OK;
 }
 
+template <int N, bool kParts>
+auto* sums_kernel(int trip) {
+  return trip == 4 ? sums_c_kernel<N, kParts, 4> : trip == 8 ? sums_c_kernel<N, kParts, 8> : trip == 16 ? sums_c_kernel<N, kParts, 16>
+                                                                                                      : sums_c_kernel<N, kParts, 32>;
+}
+
 // Sums of a batch in orientation C, where every matrix can be read in 16-byte pieces: warps on their own from 54 KB per SM on
 // where an item of the streaming kernel would be 16 KB or less on average, streaming where there are several items for every
 // CTA; one CTA per row-block otherwise (its single trip to memory is what a small batch needs: one layer of 256 features 9.9
@@ -795,8 +801,8 @@ int launch_sums_c(SelectBatchT<N>& B, int sms, cudaStream_t s) {
     B.first_block[i] = at;
     at += J.n_blocks * J.parts;
   }
-  auto* kernel = B.block >= 32 ? (parts ? sums_c_kernel<N, true, true> : sums_c_kernel<N, false, true>)
-                               : (parts ? sums_c_kernel<N, true, false> : sums_c_kernel<N, false, false>);
+  const int trip = rows_per_trip(B.block, at, 4, 2, sms);     // (CTAs of five warps with 88 and 152 registers)
+  auto* kernel = parts ? sums_kernel<N, true>(trip) : sums_kernel<N, false>(trip);
   BSP_CUDA_TRY(launch_pdl(kernel, dim3(at), dim3(kSumThreads + 32), 0, s, B));
   return BSP_OK;
 }
