@@ -115,7 +115,7 @@ masked_adam_kernel(AdamArgs A) {
 // the block's index list (2 bytes per entry) in shared memory, 16 bytes per load with all of a thread's loads
 // in flight (at the usual rates every 32-byte sector of a row holds a kept column, so whole rows are read
 // anyway), and gathers from there, two positions per 4-byte store.  HBM-bound in total, latency-bound per
-// matrix: up to four rows per CTA, fewer of wide matrices of few row-blocks, and the list travels beside the rows.  12 layers of four
+// matrix: four rows per CTA, two of wide matrices of few row-blocks, and the list travels beside the rows.  12 layers of four
 // matrices, on average: 5.3 us gathering from global memory, 2.9 us.
 constexpr int kRepackRows = 4, kRepackThreads = 256, kRepackLoads = 6, kRepackMaxCols = 3072;
 __global__ void __launch_bounds__(kRepackThreads)
@@ -289,16 +289,17 @@ extern "C" int bsp_repack_values(const void* W, int rows, int cols, int ldw, int
   // global memory: 4096 x 1024 in 16-row blocks 4.0 / 5.7 us, 768 x 3072 5.5 / 5.2, 8192 x 4096 49 / 26, 5344 x 920 in single
   // rows 11.2 / 10.2; 6042 x 2128 in pairs, by itself, 10.7 / 7.5.
   if (cols % 8 == 0 && ldw % 8 == 0 && aligned_to(W, 16) && cols <= kRepackMaxCols && block >= kRepackRows) {
-    // Two CTAs per SM, as far as a CTA keeps 1536 elements (a chunk of eight for most of its threads): between the Adam steps
-    // of a stack (768 x 768 and 768 x 3072 have 192 CTAs of four rows) a call is then bound by a shorter chain of loads and
-    // stores.  Four rows for all / this rule: retraining 12 layers of 768 features 598 -> 583 us, 9 of 336 in 8-row blocks
-    // 195.0 -> 188.0, 6 of 592 222.2 -> 215.4; halved for narrow rows as well 583, 196.6, 215.8, and 12 of 256 in 8-row
-    // blocks 216 -> 227.
+    // Two rows where four of them give fewer than two CTAs per SM and two are 1536 elements (a chunk of eight for most of the
+    // threads): between the Adam steps of a stack (768 x 768 and 768 x 3072 have 192 CTAs of four rows) a call is then bound by
+    // a shorter chain of loads and stores.  Four rows / two, behind the Adam step: 768 x 768 in 16-row blocks 6.65 / 6.31 us,
+    // 1024 x 1024 10.9 / 10.5, 992 x 2528 19.0 / 17.9; calls by themselves, one behind the other: the matrices of 12 layers of
+    // 512 features 2.84 / 2.60 on average, of 768 3.03 / 2.98, but one shape again and again out of L2 768 x 768 2.1 / 2.4, 1024 x
+    // 1024 2.5 / 3.0.  Single rows are no better behind Adam and cost by themselves (480 x 1920 in four, two and one 9.64 / 9.38 /
+    // 9.52 and 2.38 / 2.23 / 2.75), and so do two rows of narrow matrices (12 layers of 256 features 216 -> 227).
     int sms = 0;
     BSP_TRY(sm_count(&sms));
-    int rows_per = kRepackRows;
-    while (rows_per > 1 && rows_per / 2 * cols >= 1536 && static_cast<long long>(nb) * ((block + rows_per - 1) / rows_per) < 2LL * sms)
-      rows_per >>= 1;
+    const bool two = 2 * cols >= 1536 && static_cast<long long>(nb) * ((block + kRepackRows - 1) / kRepackRows) < 2LL * sms;
+    const int rows_per = two ? kRepackRows / 2 : kRepackRows;
     const dim3 pieces(nb, (block + rows_per - 1) / rows_per);
     BSP_CUDA_TRY(launch_pdl(repack_vec_kernel, pieces, dim3(kRepackThreads), static_cast<size_t>(cols) * (rows_per + 1) * 2, s, w, cols, ldw,
                             block, rows_per, blk_ptr, idx, static_cast<uint16_t*>(vals)));

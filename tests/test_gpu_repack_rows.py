@@ -1,4 +1,4 @@
-"""GPU parity of the re-packed values at the numbers of rows that a CTA takes (four, two or one, by the number of
+"""GPU parity of the re-packed values at the numbers of rows that a CTA takes (four or two, by the number of
 row-blocks), with row-blocks that they do not divide, odd and even kept counts, and empty blocks.  Bits are moved, so the
 result is exact."""
 import numpy as np
@@ -12,9 +12,9 @@ from gpu_util import DEV, bits_of, to_dev
 pytestmark = pytest.mark.gpu
 
 
-# at 3072 columns 1, 3 and 30 row-blocks: single rows; 40 of 16 rows and 75 of 5: pairs; 100 of 16, 200 of 7 and 300 of 4: four
-# rows, as for narrower matrices
-@pytest.mark.parametrize("blocks,block", [(1, 16), (3, 5), (30, 4), (40, 16), (75, 5), (100, 16), (200, 7), (300, 4)])
+# at 3072 columns 1, 3, 30 and 75 row-blocks: two rows, of five rows two and two and one; 40 of 16 and 70 of 7 as well; 100 of 16,
+# 200 of 7 and 300 of 4: four rows, as for narrower matrices
+@pytest.mark.parametrize("blocks,block", [(1, 16), (3, 5), (30, 4), (40, 16), (75, 5), (70, 7), (100, 16), (200, 7), (300, 4)])
 @pytest.mark.parametrize("cols,kept", [(8, 3), (264, 88), (3072, 771)])
 def test_repack_by_rows_per_cta(blocks, block, cols, kept):
     rng = np.random.default_rng(blocks * 1000 + cols)
