@@ -466,40 +466,56 @@ int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, lo
   if (ns != nullptr) *ns = choice < 0 ? whole_ns : best;
   return choice;
 }
-// dW: whole tiles 128 / 192 / 256 wide by one CTA, 128 / 256 wide by a pair (persistent kernels: per wave, a stage longer the
-// more SMs are at work, as in choose_dense), or, 128 and 256 wide, split 2 / 4 / 8.  Rows of dY or X that are no multiple of
-// 128 bytes make the operand boxes straddle lines: a percentage, for the splits a set of stage times of their own.
+// dW: whole tiles 128 / 192 / 256 wide by one CTA, 128 / 256 wide by a pair, or, 128 and 256 wide, split 2 / 4 / 8.  Whole
+// tiles as in choose_dense: a fixed part, per wave the larger of the main loop (a stage longer the more SMs are at work) and
+// the epilogue, which binds with few tokens, and something per wave after the first.  Rows of dY or X that are no multiple of
+// 128 bytes make that operand's boxes straddle lines, of 32 bytes sectors as well: percentages of the stage.  Operands beyond
+// what L2 holds make the narrow tiles, which read them more often, a tenth slower.
 // (4096 tokens, one CTA 128 wide / pair 128 wide / split 2: 768 x 768 15.5 / 13.7 / 10.2 us, 3072 x 768 18.5 / 15.9, 2304 x
-// 768 18.1 / 15.6; 4096 x 1024 29.5 one CTA 256 wide, 25.9 pair 256 wide, 28.0 pair 128 wide; 1024 tokens, 3072 x 768 8.0 /
-// 7.0.  Over 28 weights the choice is 1.5 % behind the best on average.)
+// 768 18.1 / 15.6; 4096 x 1024 31.9 and 28.4, pair 256 wide 26.3; 136 tokens, 2640 x 880 5.7 / 7.1; 36 tokens, 3648 x 2640 14.0
+// / 14.3, one CTA 192 wide 12.6; 7858 tokens, 1496 x 880 51.3 / 43.4, split 2 of 256 wide 36.5.  Over 467 weights of 1 to 15455
+// tokens, 281 of them of encoder layers of 256 to 1024 features, the choice is 0.4 % behind the best on average and 12 % at
+// worst.)
 TnChoice choose_tn(const TcDevice& dev, int tokens, int n_out, int k_in) {
+  struct Whole {
+    int width;
+    bool pair;
+    int fixed, epilogue, extra_wave, stage_few, stage_all, ragged_dy[3], ragged_x[3];     // percent by row_class
+  };
+  struct Split {
+    int width, c, fixed, per_cta, stage, ragged_dy[3], ragged_x[3];
+  };
+  static const Whole whole[5] = {{128, false, 4520, 770, 1470, 196, 194, {0, 14, 56}, {0, 14, 38}},
+                                 {192, false, 5400, 940, 2350, 249, 291, {0, 8, 36}, {0, 12, 33}},
+                                 {256, false, 6670, 900, 3270, 310, 346, {0, 6, 28}, {0, 6, 30}},
+                                 {128, true, 3800, 880, 1530, 166, 165, {0, 11, 62}, {0, 4, 20}},
+                                 {256, true, 5010, 1740, 2490, 277, 324, {0, 2, 17}, {0, 0, 7}}};
+  static const Split split[6] = {{128, 2, 3830, 5, 206, {0, 16, 53}, {0, 8, 45}},  {128, 4, 3860, 8, 211, {0, 8, 51}, {0, 11, 38}},
+                                 {128, 8, 3700, 10, 237, {0, 4, 55}, {0, 3, 30}},  {256, 2, 6240, 8, 337, {0, 2, 19}, {0, 9, 54}},
+                                 {256, 4, 5460, 14, 363, {0, 2, 13}, {0, 7, 55}},  {256, 8, 5850, 14, 408, {0, 0, 23}, {0, 2, 33}}};
+  auto row_class = [](int elements) { return elements % 64 == 0 ? 0 : elements % 16 == 0 ? 1 : 2; };
+  const int dy = row_class(n_out), x = row_class(k_in);
   const long long m_tiles = (n_out + kBlockM - 1) / kBlockM, m_pairs = (n_out + 2 * kBlockM - 1) / (2 * kBlockM);
   const int kb = (tokens + kBlockK - 1) / kBlockK;
-  const int ragged = n_out % 64 || k_in % 64 ? 1 : 0;
-  static const int widths[5] = {128, 192, 256, 128, 256}, fixed[5] = {4670, 5110, 6240, 4010, 4770}, extra_wave[5] = {0, 0, 220, 0, 1270};
-  static const int stage_few[5] = {161, 243, 294, 141, 270}, stage_all[5] = {212, 307, 373, 187, 341};
-  static const int ragged_percent[5] = {124, 115, 114, 110, 100};
-  static const int fixed_split[2][3] = {{4000, 4100, 4500}, {6700, 6700, 6600}};
-  static const int stage_split[2][2][3] = {{{178, 178, 200}, {265, 265, 265}}, {{270, 334, 373}, {365, 380, 400}}};
+  const bool beyond_l2 = 2LL * tokens * (n_out + k_in) > 100000000LL;
   long long best = -1;
   TnChoice choice{256, false, 1};
-  for (int w = 0; w < 5; ++w) {
-    const bool pair = w >= 3;
-    const long long tiles = (pair ? m_pairs : m_tiles) * ((k_in + widths[w] - 1) / widths[w]), seats = pair ? dev.sms / 2 : dev.sms;
+  for (const Whole& w : whole) {
+    const long long tiles = (w.pair ? m_pairs : m_tiles) * ((k_in + w.width - 1) / w.width), seats = w.pair ? dev.sms / 2 : dev.sms;
     const long long waves = (tiles + seats - 1) / seats, busy = tiles < seats ? tiles : seats;
-    long long stages = waves * kb * (stage_few[w] + (stage_all[w] - stage_few[w]) * busy / seats);
-    if (ragged) stages = stages * ragged_percent[w] / 100;
-    const long long t = fixed[w] + extra_wave[w] * (waves - 1) + stages;
-    if (best < 0 || t < best) { best = t; choice = TnChoice{widths[w], pair, 1}; }
+    int percent = 100 + w.ragged_dy[dy] + w.ragged_x[x];
+    if (w.width == 128 && w.pair && dy == 2 && x == 2) percent += 30;
+    if (w.width == 128 && beyond_l2) percent += 10;
+    const long long loop = kb * (w.stage_few + (w.stage_all - w.stage_few) * busy / seats) * percent / 100;
+    const long long t = w.fixed + waves * (loop > w.epilogue ? loop : w.epilogue) + w.extra_wave * (waves - 1);
+    if (best < 0 || t < best) { best = t; choice = TnChoice{w.width, w.pair, 1}; }
   }
-  for (int b = 0; b < 2; ++b) {
-    const long long tiles = m_tiles * ((k_in + 128 * (b + 1) - 1) / (128 * (b + 1)));
-    for (int i = 0; i < 3; ++i) {
-      const int c = 2 << i;
-      if (c > kb || tiles * c > dev.split_ctas[i]) continue;
-      const long long t = fixed_split[b][i] + 4 * tiles * c + (kb + c - 1) / c * stage_split[b][ragged][i];
-      if (t < best) { best = t; choice = TnChoice{128 * (b + 1), false, c}; }
-    }
+  for (int i = 0; i < 6; ++i) {
+    const Split& p = split[i];
+    const long long tiles = m_tiles * ((k_in + p.width - 1) / p.width);
+    if (p.c > kb || tiles * p.c > dev.split_ctas[i % 3]) continue;
+    const long long t = p.fixed + p.per_cta * tiles * p.c + (kb + p.c - 1) / p.c * p.stage * (100 + p.ragged_dy[dy] + p.ragged_x[x]) / 100;
+    if (t < best) { best = t; choice = TnChoice{p.width, false, p.c}; }
   }
   return choice;
 }

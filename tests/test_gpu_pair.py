@@ -32,10 +32,12 @@ def test_pair_linear_matches_one_cta(tokens, n_out, k_in, act):
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
 
 
-# tiles 256 x 128 and (700 x 4000 x 1000, 600 x 1000 x 4000) 256 x 256; flags in the epilogue, by the mask kernel, none
+# by pairs 256 x 128 (1000 x 2312 x 776 and the next four) and 256 x 256, and by one CTA with tiles 128 (65 x 1128 x 1816), 192
+# (the first two, 1 x 1328 x 2168) and 256 wide (40 x 2104 x 4136); flags in the epilogue, by the mask kernel, none
 @pytest.mark.parametrize("tokens,n_out,k_in,block", [
     (1, 2056, 1032, 8), (64, 2304, 1032, 16), (129, 1800, 1800, 3), (300, 3080, 1544, 8), (1000, 2312, 776, 8),
-    (700, 4000, 1000, 32), (600, 1000, 4000, 8)])
+    (1, 2552, 2248, 8), (129, 1080, 568, 3), (65, 1448, 3520, 8), (40, 2456, 2720, 8),
+    (700, 4000, 1000, 32), (600, 1000, 4000, 8), (64, 2200, 1640, 8), (65, 1128, 1816, 8), (1, 1328, 2168, 8), (40, 2104, 4136, 8)])
 @pytest.mark.parametrize("flags", ["aligned", "unaligned", "none"])
 def test_pair_weight_gradient(tokens, n_out, k_in, block, flags):
     dy = si.normal_bf16(92, f"dy{tokens}", (tokens, n_out), 1.0)
