@@ -32,22 +32,32 @@ int check_call(const bsp_linear_call* c) {
 
 // Estimated nanoseconds of the two routes.  Zero-expanded: what the kernel choice of bsp_linear_planned_ex expects, and a
 // microsecond that it leaves out for all of its kernels alike.  Gathering: a launch, and per row-block that the busiest CTA
-// works through 86 ns for every 16 kept columns (the TMA row gather is the bound, whatever the block height) and 213 ns per
-// 32 rows of the block for its epilogue, 301 with GELU.  Fitted to 185 launches of both routes, 128 to 32768 tokens,
-// 768 to 4096 features, blocks of 16 to 128 rows at 3 to 8 times compression: the gathering estimate is off by 6 % (rms),
-// the choice costs 0.6 % over the better route on average and 22 % at worst (7.1 us against 8.6).
+// works through 87 ns for every 16 kept columns (the TMA row gather is the bound, whatever the block height; a stage that a
+// row-block leaves with one group of 16 takes the time of two) and, per 32 rows of the block, its epilogue: 213 ns, with GELU
+// 400 by two epilogue groups, by four 300, or 260 where these write transposed pieces.  Fitted to 562 layers by both routes,
+// 64 to 32768 tokens, 224 to 4096 features, blocks of 16 to 128 rows at 2 to 10 times compression: the gathering estimate is
+// off by 6 % (rms), the choice costs 0.2 % over the better route on average and 11 % at worst (8192 tokens, 768 x 768 in 64-row
+// blocks at 5x 11.3 us zero-expanded, 12.5 gathered).  With 301 ns for every GELU and 3 % in favour of the zero-expanded route
+// it was 0.5 % and 27 %: 368 tokens, 800 x 3000 in 32-row blocks at 4.9x 9.5 us and 7.5; 32768 tokens, 3072 x 1024 in 128-row
+// blocks at 3x 127 and 116.
 void estimate_ns(const bsp_linear_call& c, const TcDevice& dev, double* zero_expanded, double* gathered) {
   long long ns = choose_dense(dev, c.tokens, c.n_out, c.k_in, c.act, c.YT == nullptr ? DenseKinds::kAll : DenseKinds::kOneCta).ns;
   int bn;
   choose_linear_split(dev, c.tokens, c.n_out, c.k_in, ns, &bn, &ns);
   *zero_expanded = static_cast<double>(ns) + 1000.0;
   const long long blocks = c.n_out / c.block;
-  const double kept_per_block = c.kept_weights >= 0 ? static_cast<double>(c.kept_weights) / c.block / blocks : c.k_in;
-  const double groups = kept_per_block > 16.0 ? ceil(kept_per_block / 16.0) : 1.0;
-  const double block_ns = 86.0 * groups + (c.act == BSP_ACT_GELU ? 301.0 : 213.0) * (c.block > 32 ? c.block / 32 : 1);
   const GatherUnits u = gather_units(c.tokens, static_cast<int>(blocks), dev.sms);
+  const double kept_per_block = c.kept_weights >= 0 ? static_cast<double>(c.kept_weights) / c.block / blocks : c.k_in;
+  double groups = kept_per_block > 16.0 ? ceil(kept_per_block / 16.0) : 1.0;
+  if (fmod(groups, 4.0) == 1.0) groups += 1.0;
+  double epilogue = 213.0;
+  if (c.act == BSP_ACT_GELU) {
+    const bool four = gather_four_groups(c.block, c.act, u.m_tiles * blocks, dev.sms);
+    epilogue = !four ? 400.0 : c.YT != nullptr ? 260.0 : 300.0;
+  }
+  const double block_ns = 87.0 * groups + epilogue * (c.block > 32 ? c.block / 32 : 1);
   const long long units = static_cast<long long>(u.m_tiles) * u.n_chunks;
-  *gathered = 4900.0 + static_cast<double>((units + dev.sms - 1) / dev.sms * u.rb_per_chunk) * block_ns;
+  *gathered = 4550.0 + static_cast<double>((units + dev.sms - 1) / dev.sms * u.rb_per_chunk) * block_ns;
 }
 
 int choose(const bsp_linear_call& c) {
@@ -65,7 +75,7 @@ int choose(const bsp_linear_call& c) {
   if (dev == nullptr) dev = &host;
   double tz, tg;
   estimate_ns(c, *dev, &tz, &tg);
-  return tg * 1.03 < tz ? BSP_ROUTE_GATHERED : BSP_ROUTE_ZERO_EXPANDED;
+  return tg < tz ? BSP_ROUTE_GATHERED : BSP_ROUTE_ZERO_EXPANDED;
 }
 
 int run_route(const bsp_linear_call& c, int route, cudaStream_t s) {

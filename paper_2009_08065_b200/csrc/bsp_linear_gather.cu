@@ -644,14 +644,11 @@ int launch_gather_groups(TcDevice* dev, const GatherParams& P, cudaStream_t s) {
   return BSP_OK;
 }
 
-// Four epilogue groups where GELU makes a row-block's epilogue longer than its stages and a CTA has several
-// row-blocks to take turns with: 4096 x 1024 in 128-row blocks at 8x and 8192 tokens 35 us with two groups, 30 with
-// four; without GELU, or with a few row-blocks per CTA, the smaller CTA starts sooner (0.3 to 1 us).
 template <int D>
 int launch_gather(TcDevice* dev, const GatherParams& P, cudaStream_t s) {
-  const long long blocks = static_cast<long long>(P.m_tiles) * P.n_blocks;
-  return D >= 64 && P.act == BSP_ACT_GELU && blocks >= 8LL * dev->sms ? launch_gather_groups<D, 4>(dev, P, s)
-                                                                      : launch_gather_groups<D, 2>(dev, P, s);
+  if constexpr (D >= 64)
+    if (gather_four_groups(D, P.act, static_cast<long long>(P.m_tiles) * P.n_blocks, dev->sms)) return launch_gather_groups<D, 4>(dev, P, s);
+  return launch_gather_groups<D, 2>(dev, P, s);
 }
 
 bool gather_block_ok(int block) { return block == 16 || block == 32 || block == 64 || block == 128; }

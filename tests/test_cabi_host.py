@@ -193,6 +193,24 @@ def _fake_call(n, k, d, c, tokens=32768, act=0, z=True, g=True):
     return call
 
 
+def test_route_choice_where_one_route_is_far_ahead():
+    """Sizes at which an estimate fitted to older kernels took the slower route."""
+    def route(n, k, d, c, tokens, act=0, transposed=False):
+        call = _fake_call(n, k, d, c, tokens=tokens, act=act)
+        if transposed:
+            call.Y, call.YT, call.ldyt = None, call.Y, tokens
+        return bsp.bsp_linear_route(call)
+    # 116 us against 127: QKV of a large batch
+    assert route(3072, 1024, 128, 3.0, 32768) == bsp.ROUTE_GATHERED
+    # 27.3 us against 23.1: 65 kept columns, a stage of 64 and one of the last
+    assert route(640, 640, 32, 640 / 65, 22760, transposed=True) == bsp.ROUTE_ZERO_EXPANDED
+    # 18.2 us against 17.2: GELU in rows by two groups; transposed by four it is 87.6 against 97.4 at eight times the tokens
+    assert route(4096, 1024, 128, 3.0, 2048, act=1) == bsp.ROUTE_ZERO_EXPANDED
+    assert route(4096, 1024, 128, 3.0, 16384, act=1, transposed=True) == bsp.ROUTE_GATHERED
+    # 6.5 us against 7.9: 768 x 3072 at 512 tokens, no split fits
+    assert route(768, 3072, 32, 8.0, 512, transposed=True) == bsp.ROUTE_GATHERED
+
+
 def test_route_choice_follows_the_measured_crossovers():
     """bsp_linear_route is host-only: with both routes possible it takes the gathering kernel where it was measured
     to win on B200 (64-row blocks from 5x to 8x on, 128-row blocks earlier) and the zero-expanded route elsewhere."""
