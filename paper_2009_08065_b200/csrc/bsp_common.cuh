@@ -174,7 +174,9 @@ inline int sm_count(int* sms) {
 //   - data older than the direct predecessor, where the library itself launched that predecessor: W and the sums
 //     behind the percentile's clearing kernel (bsp_select.cu), W in the second packing stage (bsp_fused.cu);
 //   - the weights of a plan that the caller vouches for (BSP_LINEAR_PLAN_STABLE): the weight warp of
-//     linear_tc_kernel and gemm_split_kernel, which does not wait and therefore does not signal either.
+//     linear_tc_kernel, gemm_pair_kernel and gemm_split_kernel, which does not wait and therefore does not signal either.
+// A kernel that allocates tensor memory signals behind its allocation: a dependent CTA that took the memory first would wait for
+// this grid, and this grid for the memory.
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};

@@ -271,7 +271,8 @@ __device__ __forceinline__ void mma_gather_stage(uint32_t d_tmem, uint64_t a_des
 // halves of 64 tokens with the 128-byte swizzle, so that the eight rows of a fragment fall on different banks.  The
 // epilogue of such a layer is bound by issue slots (58 % busy with four groups): 4096 x 1024 in 128-row blocks at 8x with
 // GELU, 8192 tokens, 32.6 -> 30.7 us.  With two groups, which are not, a piece by itself takes longer (336 tokens, two linears
-// of 896 features: 15.5 -> 15.7 us).
+// of 896 features: 15.5 -> 15.7 us).  With 128-row blocks the kernel stands at the 80 registers that 672 threads leave and
+// spills 16 bytes a thread; that is counted in the figures.
 struct FragmentPiece {
   uint32_t v[32];            // [16-token half][8 output rows: 4][token, token + 8 by two output rows]
   uint32_t bias[4];          // of this lane's two rows of each 8

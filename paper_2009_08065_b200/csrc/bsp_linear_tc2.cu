@@ -2,7 +2,8 @@
 //
 // The one-CTA kernels (bsp_linear_tc.cu, bsp_gemm_tn.cu) stream (128 + BN) x 64 operand elements from L2 per
 // 128 x BN x 64 block of multiply-adds, and at BERT shapes it is this L2 -> SM traffic, not the tensor pipe, that
-// binds: 16 to 17 TB/s over all SMs, whatever the tile.  Here two CTAs of a cluster share one 256 x BN output
+// binds: they move 15 to 17 TB/s over all SMs (131 bytes per ns and SM, 19 TB/s, is the most that was seen, by the 256 x 128
+// tiles of the weight gradient).  Here two CTAs of a cluster share one 256 x BN output
 // tile: each loads its own 128 rows of A and HALF of the BN rows of B, and one tcgen05.mma.cta_group::2 (M = 256)
 // issued by the leader CTA reads both CTAs' shared memory and writes rows 0..127 / 128..255 of the accumulator
 // into the two CTAs' tensor memories.  Per CTA that is (128 + BN / 2) x 64 elements per block: a third less

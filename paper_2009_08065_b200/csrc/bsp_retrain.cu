@@ -295,7 +295,8 @@ extern "C" int bsp_repack_values(const void* W, int rows, int cols, int ldw, int
     // 1024 x 1024 10.9 / 10.5, 992 x 2528 19.0 / 17.9; calls by themselves, one behind the other: the matrices of 12 layers of
     // 512 features 2.84 / 2.60 on average, of 768 3.03 / 2.98, but one shape again and again out of L2 768 x 768 2.1 / 2.4, 1024 x
     // 1024 2.5 / 3.0.  Single rows are no better behind Adam and cost by themselves (480 x 1920 in four, two and one 9.64 / 9.38 /
-    // 9.52 and 2.38 / 2.23 / 2.75), and so do two rows of narrow matrices (12 layers of 256 features 216 -> 227).
+    // 9.52 and 2.38 / 2.23 / 2.75), and so do two rows of narrow matrices (12 layers of 256 features 216 -> 227);
+    // 704 x 704, just below the line, would gain what 768 x 768 does (6.65 / 6.26).
     int sms = 0;
     BSP_TRY(sm_count(&sms));
     const bool two = 2 * cols >= 1536 && static_cast<long long>(nb) * ((block + kRepackRows - 1) / kRepackRows) < 2LL * sms;

@@ -52,7 +52,7 @@ template <int N>
 struct SelectBatchT {
   int n_jobs, block;
   int cleared;                      // the kernel before the sums is the clearing one
-  int max_part_cols, total_items;   // streaming sums kernel (its items), persistent one (its pieces)
+  int max_part_cols, total_items;   // sums_stream_kernel (its items), sums_flat_kernel (its pieces)
   int* status;
   int first_block[N];        // (row-blocks x parts before the job's own) apart from the wide records: a search stays within a few lines of the constant cache
   SelectJob job[N];
@@ -743,8 +743,11 @@ auto* sums_kernel(int trip) {
 // Sums of a batch in orientation C, where every matrix can be read in 16-byte pieces: warps on their own from 54 KB per SM on
 // where an item of the streaming kernel would be 16 KB or less on average, streaming where there are several items for every
 // CTA; one CTA per row-block otherwise (its single trip to memory is what a small batch needs: one layer of 256 features 9.9
-// us, 10.4 by warps).  From 324 KB per SM on the rows pass L1 by (12 layers of 640 features in 8-row blocks, with the
-// preparation behind, 139 -> 134 us; 12 of 256 44.3 -> 45.4).
+// us, 10.4 by warps).  From 324 KB per SM on the rows pass L1 by.  Percentiles of 8-row blocks, with the preparation behind them,
+// streamed / by warps through L1 / past it: 4 layers of 512 features (166 KB per SM) 45.7 / 43.3 / 43.6 us, 12 of 400 (304 KB)
+// 80.6 / 72.3 / 73.3, 4 of 768 (374) 71.9 / 72.3 / 73.3, 6 of 640 (389) 83.4 / 83.3 / 82.8, 12 of 576 (630) 129.3 / 115.6 /
+// 114.5, 12 of 640 (778) 143.0 / 141.4 / 134.6, 12 of 768 (1121) 184.5 / 185.5 / 176.2; in 16-row blocks 12 of 256 (125) 37.1 /
+// 34.0 / 34.3.
 template <int N>
 int launch_sums_c(SelectBatchT<N>& B, int sms, cudaStream_t s) {
   const int max_cols = kSumRowBytes / (2 * B.block) / 8 * 8;

@@ -32,6 +32,31 @@ def test_pair_linear_matches_one_cta(tokens, n_out, k_in, act):
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
 
 
+# Each linear reads what the one before it is still storing, while its weights are fetched at once: up to six tiles per pair, and
+# one tile behind them.
+@pytest.mark.parametrize("tokens", [600, 6000])
+def test_pair_chain_with_early_weights(tokens):
+    widths = [776, 2304, 1032, 3072, 256, 768]
+    x = to_dev(si.normal_bf16(93, f"cx{tokens}", (tokens, widths[0]), 1.0))
+    plans = [to_dev(si.normal_bf16(93, f"cw{i}", (n, k), 0.02)).view(torch.uint8).reshape(-1) for i, (k, n) in enumerate(zip(widths, widths[1:]))]
+
+    def chain(flags, rounds):
+        out = []
+        for _ in range(rounds):
+            ys = [torch.full((tokens, n), 0x7FC0, dtype=torch.int16, device=DEV) for n in widths[1:]]
+            src = x
+            for i, y in enumerate(ys):
+                bsp.bsp_linear_planned_ex(plans[i], widths[i + 1], widths[i], 8, src, None, i % 2, y, bsp.LINEAR_CTA_PAIR | flags)
+                src = y
+            out.append(ys)
+        return out
+
+    want = chain(0, 1)[0]
+    got = chain(bsp.LINEAR_PLAN_STABLE, 8)
+    bsp.bsp_linear_status()
+    assert all(torch.equal(a, b) for ys in got for a, b in zip(ys, want))
+
+
 # by pairs 256 x 128 (1000 x 2312 x 776 and the next four) and 256 x 256, and by one CTA with tiles 128 (65 x 1128 x 1816), 192
 # (the first two, 1 x 1328 x 2168) and 256 wide (40 x 2104 x 4136); flags in the epilogue, by the mask kernel, none
 @pytest.mark.parametrize("tokens,n_out,k_in,block", [

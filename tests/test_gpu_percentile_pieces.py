@@ -13,13 +13,35 @@ from gpu_util import DEV, bits_of, to_dev
 pytestmark = pytest.mark.gpu
 
 
+MIN_BYTES, PAST_L1_BYTES, ITEM_BYTES, ROW_BYTES = 54 * 1024, 324 * 1024, 16 * 1024, 24 * 1024    # the first two per SM
+
+
+def streamed_items(block, shapes):
+    """Items that the streaming kernel would have: row-blocks, cut into equal column ranges where they exceed 24 KB."""
+    most = ROW_BYTES // (2 * block) // 8 * 8
+    total = 0
+    for n, k in shapes:
+        parts = -(-k // most)
+        width = (-(-k // parts) + 7) // 8 * 8
+        total += n // block * -(-k // width)
+    return total
+
+
+# (the last two are large enough for the rows to pass L1 by)
 @pytest.mark.parametrize("block,shapes", [
-    (1, [(2000, 1032), (3, 8), (1500, 1416), (97, 264)]),
-    (3, [(3000, 528), (6, 8), (2001, 1032), (1500, 264)]),
-    (8, [(4096, 256), (8, 8), (8200, 264), (4096, 400), (64, 1032)]),
-    (21, [(2100, 368), (4200, 272), (21, 8), (6300, 360)]),
-    (8, [(8192, 1000)] * 3 + [(16, 72)])])
+    (1, [(2400, 1032), (3, 8), (1900, 1416), (97, 264)]),
+    (3, [(3000, 528), (6, 8), (3201, 1032), (1500, 264)]),
+    (8, [(4096, 256), (8, 8), (8200, 264), (4096, 400), (1024, 1032)]),
+    (13, [(4160, 520), (13, 8), (5200, 264), (2600, 400), (26, 1032)]),
+    (21, [(2100, 368), (4200, 272), (21, 8), (9450, 360)]),
+    (8, [(8192, 1000)] * 4 + [(16, 72)]),
+    (15, [(9000, 400), (15, 8)] + [(9000, 392)] * 7)])
 def test_batched_percentile_in_pieces(block, shapes):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    total = sum(2 * n * k for n, k in shapes)
+    large = shapes[0][0] >= 8192
+    assert 1.05 * MIN_BYTES * sms <= total <= ITEM_BYTES * streamed_items(block, shapes)
+    assert total >= 1.05 * PAST_L1_BYTES * sms if large else total <= PAST_L1_BYTES * sms / 1.05
     jobs, rates, weights = [], [], []
     for i, (n, k) in enumerate(shapes):
         w = si.normal_bf16(96, f"pp{block}.{i}", (n, k), 0.02)

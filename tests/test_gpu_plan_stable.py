@@ -8,8 +8,6 @@ from gpu_util import DEV
 
 pytestmark = pytest.mark.gpu
 
-STABLE = bsp.LINEAR_AUTO | bsp.LINEAR_PLAN_STABLE
-
 
 def packed(g, n_out, k_in, block):
     w = (torch.randn(n_out, k_in, generator=g, device=DEV) * 0.02).bfloat16()
@@ -18,11 +16,13 @@ def packed(g, n_out, k_in, block):
     return pk
 
 
-# 8 tokens: both linears split over clusters; 300: whole tiles.  Layout A belongs to a small linear that is ready to
-# start its weights at once, layout B is the larger one that its writer may still be storing.
-@pytest.mark.parametrize("tokens", [8, 300])
+# 8 tokens: both linears split over clusters; 300: whole tiles; "pair": pairs of CTAs, with one tile each and with several.
+# Layout A belongs to a small linear that is ready to start its weights at once, layout B is the larger one that its writer may
+# still be storing.
+@pytest.mark.parametrize("tokens,kernel", [(8, bsp.LINEAR_AUTO), (300, bsp.LINEAR_AUTO), (300, bsp.LINEAR_CTA_PAIR), (4096, bsp.LINEAR_CTA_PAIR)],
+                         ids=["8", "300", "300-pair", "4096-pair"])
 @pytest.mark.parametrize("writer", ["plan", "adam"])
-def test_layouts_written_two_calls_before(tokens, writer):
+def test_layouts_written_two_calls_before(tokens, kernel, writer):
     g = torch.Generator(device=DEV)
     g.manual_seed(tokens)
     shapes = [(256, 256), (3072, 3072)]                       # (n_out, k_in) of A and B
@@ -52,15 +52,15 @@ def test_layouts_written_two_calls_before(tokens, writer):
         torch.cuda.synchronize()
         want.append([torch.zeros(tokens, n, dtype=torch.bfloat16, device=DEV) for n, _ in shapes])
         for i in range(2):
-            linear(i, want[v][i], bsp.LINEAR_AUTO)
+            linear(i, want[v][i], kernel)
         torch.cuda.synchronize()
     assert not torch.equal(want[0][1], want[1][1])
-    rounds = 60
+    rounds = 60 if tokens < 4096 else 15                      # (outputs of 27 MB a round)
     got = [[torch.zeros_like(t) for t in want[0]] for _ in range(rounds)]
     for r in range(rounds):
         layouts(r % versions)
-        linear(0, got[r][0], STABLE)
-        linear(1, got[r][1], STABLE)
+        linear(0, got[r][0], kernel | bsp.LINEAR_PLAN_STABLE)
+        linear(1, got[r][1], kernel | bsp.LINEAR_PLAN_STABLE)
     bsp.bsp_linear_status()
     for r in range(rounds):
         for i in range(2):
