@@ -608,8 +608,9 @@ dim3 grid_of(int x, long long pieces) {
 // epilogue (with GELU also a part of the smaller one: they contend for issue slots), and something per wave after the
 // first.  A 64-deep stage takes longer the more SMs are drawing operands from L2 (two times per width, for a few CTAs
 // and for all of them), and where rows of X and the plan are no multiple of 128 bytes; more so where they are no multiple
-// of 32 either (every row then straddles sectors: 12891 x 3856 x 3080 one CTA 326 us, pair 259, 16650 x 1288 x 2136 130 and
-// 103; measured over estimated without that 1.4 to 1.5, pairs 1.16, over 17 such layers).  Fitted to launches of 8 to
+// of 32 either (every row then straddles sectors, the narrow tiles' most: 12891 x 3856 x 3080 with GELU by one CTA 256 wide 325
+// us, by pairs 128, 192 and 256 wide 328, 279 and 260; over 120 such layers the choice is 0.2 % behind the best on average and 7 %
+// at worst).  Fitted to launches of 8 to
 // 32768 tokens (nanoseconds; one CTA 64 / 128 / 192 / 256 wide, pairs 128 / 192 / 256): over 64 layers of 256 to 1024
 // features the choice is 0.4 % behind the best of the seven on average and 6 % at worst.  Best one-CTA kernel / best pair:
 // 4096 tokens x 768 outputs x 3072 inputs 19.9 / 16.5 us, 2304 x 768 14.4 / 13.2, 3072 x 768 with GELU 20.7 / 19.8, 4096 x
@@ -619,7 +620,7 @@ DenseChoice choose_dense(const TcDevice& dev, int tokens, int n_out, int k_in, i
   static const int width[kKinds] = {64, 128, 192, 256, 128, 192, 256};
   static const int fixed[kKinds] = {2830, 3200, 3750, 4400, 3600, 4070, 4560}, extra_wave[kKinds] = {500, 700, 300, 800, 540, 450, 240};
   static const int stage_few[kKinds] = {158, 168, 250, 320, 150, 200, 270}, stage_all[kKinds] = {176, 210, 335, 370, 190, 250, 330};
-  static const int ragged_percent[2][kKinds] = {{114, 130, 103, 110, 111, 106, 106}, {160, 170, 155, 160, 136, 136, 136}};
+  static const int ragged_percent[2][kKinds] = {{114, 130, 103, 110, 111, 106, 106}, {165, 192, 170, 167, 173, 155, 135}};
   static const int epilogue[2][kKinds] = {{500, 950, 1500, 1750, 570, 610, 1170}, {900, 1600, 2600, 2950, 1570, 3160, 3660}};
   static const int gelu_tail[kKinds] = {150, 500, 450, 600, 660, 530, 900};
   const long long kb = (k_in + kBlockK - 1) / kBlockK;
