@@ -978,7 +978,10 @@ def run_case(args):
     weight-side call on its four matrices, --case prepare_stack the same call on the 72 matrices of a BERT-base
     stack (inputs larger than L2), --case gather the gathering linear kernel on a BERT-large FFN-up point
     (16384 tokens, 1024 -> 4096, 64-row blocks, 5x), --case split a linear of 8 tokens (3072 -> 768), whose contraction
-    is split over clusters, --case percentile the threshold of a 3072 x 768 matrix of 16-row blocks."""
+    is split over clusters, --case percentile the threshold of a 3072 x 768 matrix of 16-row blocks, --case
+    percentile_stack the thresholds of 72 matrices of 640 features in 8-row blocks, --case gather_t the gathering
+    linear of 8192 tokens, 1024 -> 4096, 128-row blocks, 8x, with its output transposed, --case dweight the weight
+    gradient of 4096 tokens for 3072 x 768."""
     import torch
     torch.cuda.set_device(0)
     device = torch.device("cuda", 0)
@@ -991,9 +994,9 @@ def run_case(args):
         bsp.bsp_linear_status()
         print("case prepare_stack: 3 calls done")
         return
-    if args.case == "gather":
+    if args.case in ("gather", "gather_t"):
         import paper_2009_08065_b200 as bsp
-        T, N, K, d, c = 16384, 4096, 1024, 64, 5.0
+        T, N, K, d, c = (16384, 4096, 1024, 64, 5.0) if args.case == "gather" else (8192, 4096, 1024, 128, 8.0)
         gen = torch.Generator(device=device)
         gen.manual_seed(si.DEFAULT_SEED)
         X = torch.randn(T, K, device=device, generator=gen).to(torch.bfloat16)
@@ -1008,11 +1011,40 @@ def run_case(args):
         gplan = torch.empty(bsp.bsp_linear_gather_plan_bytes(N, K, d), dtype=torch.uint8, device=device)
         bsp.bsp_linear_gather_plan(pk, gplan)
         bias = (torch.randn(N, device=device, generator=gen) * 0.02).to(torch.bfloat16)
-        Y = torch.empty(T, N, dtype=torch.bfloat16, device=device)
+        transposed = args.case == "gather_t"
+        Y = torch.empty((N, T) if transposed else (T, N), dtype=torch.bfloat16, device=device)
         for _ in range(3):
-            bsp.bsp_linear_gathered(gplan, N, K, d, XT, bias, 1, Y)
+            bsp.bsp_linear_gathered_ex(gplan, N, K, d, XT, bias, 1, Y, transposed)
         bsp.bsp_linear_status()
-        print("case gather: 3 launches done")
+        print(f"case {args.case}: 3 launches done")
+        return
+    if args.case == "dweight":
+        import paper_2009_08065_b200 as bsp
+        T, N, K = 4096, 3072, 768
+        gen = torch.Generator(device=device)
+        gen.manual_seed(si.DEFAULT_SEED)
+        dY = (torch.randn(T, N, device=device, generator=gen) * 1e-3).to(torch.bfloat16)
+        X = torch.randn(T, K, device=device, generator=gen).to(torch.bfloat16)
+        keep = (torch.rand(N // 16, K, device=device, generator=gen) < 1.0 / 3.0).to(torch.uint8)
+        dW = torch.empty(N, K, dtype=torch.bfloat16, device=device)
+        for _ in range(4):
+            bsp.bsp_linear_backward_weight(dY, X, 16, keep, dW)
+        bsp.bsp_linear_status()
+        print("case dweight: 4 launches done")
+        return
+    if args.case == "percentile_stack":
+        import paper_2009_08065_b200 as bsp
+        gen = torch.Generator(device=device)
+        gen.manual_seed(si.DEFAULT_SEED)
+        jobs = []
+        for n, k in [(640, 640)] * 48 + [(2560, 640)] * 12 + [(640, 2560)] * 12:
+            W = (torch.randn(n, k, device=device, generator=gen) * 0.02).to(torch.bfloat16)
+            jobs.append(bsp.LayerJob(W=W, out=bsp.PackedMatrix.allocate(n, k, 8, bsp.ORIENT_C, device), threshold=0.0,
+                                     threshold_dev=torch.zeros(1, device=device)))
+        for _ in range(4):
+            bsp.bsp_percentile_threshold_batched(jobs, 8, [4.0] * len(jobs))
+        bsp.bsp_linear_status()
+        print("case percentile_stack: 4 calls done")
         return
     if args.case in ("split", "percentile"):
         import paper_2009_08065_b200 as bsp
@@ -1065,7 +1097,8 @@ def main():
     ap.add_argument("--steps", type=int, default=200)
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", choices=["cuda", "reference"], default="cuda")
-    ap.add_argument("--case", choices=["qkv", "attn_out", "ffn_up", "ffn_down", "prepare", "prepare_stack", "gather", "split", "percentile"],
+    ap.add_argument("--case", choices=["qkv", "attn_out", "ffn_up", "ffn_down", "prepare", "prepare_stack", "gather", "gather_t", "split", "percentile", "percentile_stack",
+                                       "dweight"],
                     default=None,
                     help="run a few launches of one call for a profiler and exit")
     ap.add_argument("--sweep", choices=["bert_large"], default=None,

@@ -444,7 +444,8 @@ bool query_split_ctas(int (&ctas)[3]) {
 //   and 2 per CTA
 // (768 outputs x 3072 inputs: 10.0 us whole, split 8 ways 3.8 us at 8 tokens and 4.6 us at 128; 768 x 768: 4.5 whole, 2.8
 // split 4 ways at 8 tokens; 1024 x 4096 at 1003 tokens: 13.4 whole, 10.6 as 128-wide tiles split 2; 304 x 304: 3.2 and
-// 2.6 at 8 tokens, not split at 1003.)
+// 2.6 at 8 tokens, not split at 1003.  Over 163 layers of 1 to 1500 tokens the choice among whole tiles and the six splits is
+// 0.9 % behind the best on average and 10 % at worst: 4 tokens, 432 x 1728 3.4 us as 128-wide tiles split 8, 3.1 as 64-wide ones.)
 int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, long long whole_ns, int* bn, long long* ns) {
   const long long m_tiles = (tokens + kBlockM - 1) / kBlockM;
   const int kb = (k_in + kBlockK - 1) / kBlockK;
