@@ -468,33 +468,37 @@ int choose_linear_split(const TcDevice& dev, int tokens, int n_out, int k_in, lo
   return choice;
 }
 // dW: whole tiles 128 / 192 / 256 wide by one CTA, 128 / 256 wide by a pair, or, 128 and 256 wide, split 2 / 4 / 8.  Whole
-// tiles as in choose_dense: a fixed part, per wave the larger of the main loop (a stage longer the more SMs are at work) and
-// the epilogue, which binds with few tokens, and something per wave after the first.  Rows of dY or X that are no multiple of
-// 128 bytes make that operand's boxes straddle lines, of 32 bytes sectors as well: percentages of the stage.  Operands beyond
-// what L2 holds make the narrow tiles, which read them more often, a tenth slower.
+// tiles as in choose_dense: a fixed part, per wave the larger of the main loop and the epilogue, which binds with few tokens, and
+// something per wave after the first; a stage takes longer the more SMs are at work in a single wave, and a little less where
+// waves follow one another and drift apart.  Rows of dY or X that are no multiple of 128 bytes make that operand's boxes straddle
+// lines, of 64 more of them and of 32 sectors as well: percentages of the stage.  Operands beyond what L2 holds make the narrow
+// tiles, which read them more often, a tenth slower.
 // (4096 tokens, one CTA 128 wide / pair 128 wide / split 2: 768 x 768 15.5 / 13.7 / 10.2 us, 3072 x 768 18.5 / 15.9, 2304 x
 // 768 18.1 / 15.6; 4096 x 1024 31.9 and 28.4, pair 256 wide 26.3; 136 tokens, 2640 x 880 5.7 / 7.1; 36 tokens, 3648 x 2640 14.0
-// / 14.3, one CTA 192 wide 12.6; 7858 tokens, 1496 x 880 51.3 / 43.4, split 2 of 256 wide 36.5.  Over 467 weights of 1 to 15455
-// tokens, 281 of them of encoder layers of 256 to 1024 features, the choice is 0.4 % behind the best on average and 12 % at
-// worst.)
+// / 14.3, one CTA 192 wide 12.6; 7858 tokens, 1496 x 880 51.3 / 43.4, split 2 of 256 wide 36.5; 6145 tokens, 880 x 880 split 2 of
+// 128 wide 18.7, split 4 of 256 wide 17.2.  Over 767 weights of 1 to 15455 tokens, most of them of encoder layers of 256 to 1024
+// features, the choice is 0.2 % behind the best on average and 7 % at worst.)
 TnChoice choose_tn(const TcDevice& dev, int tokens, int n_out, int k_in) {
   struct Whole {
     int width;
     bool pair;
-    int fixed, epilogue, extra_wave, stage_few, stage_all, ragged_dy[3], ragged_x[3];     // percent by row_class
+    int fixed, epilogue, extra_wave, stage_few, stage_full, stage_waves, ragged_dy[4], ragged_x[4];     // percent by row_class
   };
   struct Split {
-    int width, c, fixed, per_cta, stage, ragged_dy[3], ragged_x[3];
+    int width, c, fixed, per_cta, stage, ragged_dy[4], ragged_x[4];
   };
-  static const Whole whole[5] = {{128, false, 4520, 770, 1470, 196, 194, {0, 14, 56}, {0, 14, 38}},
-                                 {192, false, 5400, 940, 2350, 249, 291, {0, 8, 36}, {0, 12, 33}},
-                                 {256, false, 6670, 900, 3270, 310, 346, {0, 6, 28}, {0, 6, 30}},
-                                 {128, true, 3800, 880, 1530, 166, 165, {0, 11, 62}, {0, 4, 20}},
-                                 {256, true, 5010, 1740, 2490, 277, 324, {0, 2, 17}, {0, 0, 7}}};
-  static const Split split[6] = {{128, 2, 3830, 5, 206, {0, 16, 53}, {0, 8, 45}},  {128, 4, 3860, 8, 211, {0, 8, 51}, {0, 11, 38}},
-                                 {128, 8, 3700, 10, 237, {0, 4, 55}, {0, 3, 30}},  {256, 2, 6240, 8, 337, {0, 2, 19}, {0, 9, 54}},
-                                 {256, 4, 5460, 14, 363, {0, 2, 13}, {0, 7, 55}},  {256, 8, 5850, 14, 408, {0, 0, 23}, {0, 2, 33}}};
-  auto row_class = [](int elements) { return elements % 64 == 0 ? 0 : elements % 16 == 0 ? 1 : 2; };
+  static const Whole whole[5] = {{128, false, 4461, 623, 1780, 173, 218, 183, {0, 9, 16, 67}, {0, 8, 14, 20}},
+                                 {192, false, 5366, 967, 2370, 234, 325, 283, {0, 6, 8, 42}, {0, 4, 7, 19}},
+                                 {256, false, 6562, 949, 3365, 268, 378, 346, {0, 2, 9, 29}, {0, 2, 7, 19}},
+                                 {128, true, 3858, 790, 1695, 152, 187, 165, {0, 4, 16, 47}, {0, 3, 10, 13}},
+                                 {256, true, 4972, 1706, 2537, 259, 337, 300, {0, 0, 0, 18}, {0, 0, 0, 14}}};
+  static const Split split[6] = {{128, 2, 3776, 5, 211, {0, 9, 17, 46}, {0, 3, 13, 49}},
+                                 {128, 4, 3820, 8, 210, {0, 3, 14, 50}, {0, 14, 12, 38}},
+                                 {128, 8, 3631, 10, 234, {0, 8, 15, 50}, {0, 0, 6, 30}},
+                                 {256, 2, 5350, 10, 363, {0, 4, 5, 19}, {0, 0, 6, 40}},
+                                 {256, 4, 4699, 22, 364, {0, 0, 8, 12}, {0, 4, 7, 61}},
+                                 {256, 8, 5251, 16, 406, {0, 0, 4, 42}, {0, 0, 7, 35}}};
+  auto row_class = [](int elements) { return elements % 64 == 0 ? 0 : elements % 32 == 0 ? 1 : elements % 16 == 0 ? 2 : 3; };
   const int dy = row_class(n_out), x = row_class(k_in);
   const long long m_tiles = (n_out + kBlockM - 1) / kBlockM, m_pairs = (n_out + 2 * kBlockM - 1) / (2 * kBlockM);
   const int kb = (tokens + kBlockK - 1) / kBlockK;
@@ -503,11 +507,12 @@ TnChoice choose_tn(const TcDevice& dev, int tokens, int n_out, int k_in) {
   TnChoice choice{256, false, 1};
   for (const Whole& w : whole) {
     const long long tiles = (w.pair ? m_pairs : m_tiles) * ((k_in + w.width - 1) / w.width), seats = w.pair ? dev.sms / 2 : dev.sms;
-    const long long waves = (tiles + seats - 1) / seats, busy = tiles < seats ? tiles : seats;
+    const long long waves = (tiles + seats - 1) / seats;
+    const long long stage = waves > 1 ? w.stage_waves : w.stage_few + (w.stage_full - w.stage_few) * tiles / seats;
     int percent = 100 + w.ragged_dy[dy] + w.ragged_x[x];
-    if (w.width == 128 && w.pair && dy == 2 && x == 2) percent += 30;
+    if (w.width == 128 && w.pair && dy == 3 && x == 3) percent += 30;
     if (w.width == 128 && beyond_l2) percent += 10;
-    const long long loop = kb * (w.stage_few + (w.stage_all - w.stage_few) * busy / seats) * percent / 100;
+    const long long loop = kb * stage * percent / 100;
     const long long t = w.fixed + waves * (loop > w.epilogue ? loop : w.epilogue) + w.extra_wave * (waves - 1);
     if (best < 0 || t < best) { best = t; choice = TnChoice{w.width, w.pair, 1}; }
   }
@@ -515,7 +520,7 @@ TnChoice choose_tn(const TcDevice& dev, int tokens, int n_out, int k_in) {
     const Split& p = split[i];
     const long long tiles = m_tiles * ((k_in + p.width - 1) / p.width);
     if (p.c > kb || tiles * p.c > dev.split_ctas[i % 3]) continue;
-    const long long t = p.fixed + p.per_cta * tiles * p.c + (kb + p.c - 1) / p.c * p.stage * (100 + p.ragged_dy[dy] + p.ragged_x[x]) / 100;
+    const long long t = p.fixed + p.per_cta * tiles * p.c + static_cast<long long>((kb + p.c - 1) / p.c) * p.stage * (100 + p.ragged_dy[dy] + p.ragged_x[x]) / 100;
     if (t < best) { best = t; choice = TnChoice{p.width, false, p.c}; }
   }
   return choice;
